@@ -183,8 +183,8 @@ typedef struct gks_config {
     int32_t ilu_fuse_first; /* GKS_PC_ILU_SWEEP with ilu_sweeps > 0: 1 (default) the
                               block-diagonal pass z^0 = P r is folded into the first
                               forward sweep (each cell forms its lower neighbours'
-                              z^0 itself); 0 a separate pass.  Same arithmetic, same
-                              results                                                  */
+                              z^0 itself; GKS_FP64: on small meshes only); 0 a
+                              separate pass.  Same arithmetic, same results            */
     int32_t flux_split;    /* mixed precision without the Prandtl correction: 1 (default)
                               half of the warps of the persistent face flux kernel
                               form the FP64 part (values, interface state, collision
@@ -196,8 +196,9 @@ typedef struct gks_config {
     int32_t ilu_sweep_pairs; /* GKS_PC_ILU_SWEEP with the per-cell equations: 1 (default)
                               a pair of consecutive backward sweeps runs in one
                               launch, each cell forming its upper neighbours'
-                              first-sweep values itself; 0 one sweep per launch.
-                              Same arithmetic, same results                         */
+                              first-sweep values itself (GKS_MIXED; GKS_FP64 runs
+                              one sweep per launch either way); 0 one sweep per
+                              launch.  Same arithmetic, same results                */
     int32_t spmv_dots;     /* mixed precision with basis_fp32 and the per-cell equations:
                               1 (default) the operator kernel of an Arnoldi step also
                               forms the Gram-Schmidt products with the basis (the new

@@ -18,6 +18,7 @@
 #include <type_traits>
 
 #include "gks_internal.h"
+#include "gks_solve64.cuh"
 #include "gks_wait.cuh"
 
 namespace gks {
@@ -978,7 +979,7 @@ __global__ void __launch_bounds__(kBlock) k_ilu_bwd_sf(DeviceMesh d, const TP *_
 // first sweep, so the results are the same bit for bit.  One launch instead of
 // two reads each cell's factors and z once and writes x once; the neighbours'
 // data mostly comes from L2 (a neighbour is a few hundred to a thousand cells
-// away in RCM order).  Measured at 1M cells (ncu, one launch): 101 us against
+// away in RCM order).  Mixed precision only.  Measured at 1M cells (ncu, one launch): 101 us against
 // 55 + 59 us for the two sweeps.  The same fusion of the forward pair (which
 // also has to form the neighbours' neighbours' z^0 = P r) took 195 us against
 // 69 + 56 us, its three levels of dependent gathers exposed, and is not used.
@@ -988,7 +989,7 @@ __global__ void __launch_bounds__(kBlock) k_ilu_bwd_sf(DeviceMesh d, const TP *_
 // x^{q+2} = B(B(x^q)) with B(x)_i = z_i + P_i sum_{j>i} O_ij x_j: two backward
 // sweeps in one launch (x^q = xin; x^0 = z).
 template <typename TZ, typename TM, typename TP>
-__global__ void __launch_bounds__(kBlock, sizeof(TM) == 4 ? 3 : 2) k_ilu_bwd2(DeviceMesh d, const TP *__restrict__ Pg,
+__global__ void __launch_bounds__(kBlock, 3) k_ilu_bwd2(DeviceMesh d, const TP *__restrict__ Pg,
                                                       const TP *__restrict__ alg, const TP *__restrict__ exg,
                                                       const TP *__restrict__ eyg, const TZ *z, const TZ *xin,
                                                       TZ *xout)
@@ -1211,7 +1212,8 @@ __global__ void k_orth_update(DeviceMesh d, const TB *__restrict__ V, TB *__rest
 // out[s][q] (op) sum_{b in case(s)} part[b][v(s)][q], q < nq; op 0 store, 1 add,
 // 2 store sqrt.  With vn given, also co[s][q] = sum / vn[s][q]^2 (the
 // Gram-Schmidt coefficient of the unnormalised basis vector q).  One block of
-// kReduceThreads per (q, s): grid (nq, ns).
+// kReduceThreads per (q, s): grid (nq, ns).  rs: partial-sum rows per cell block
+// (the FP64 solve writes several on small meshes).
 constexpr int kReduceThreads = 256;
 
 // sum of at(b) over b = b0 + t, b0 + t + kReduceThreads, ... < b1 (t the
@@ -1239,13 +1241,14 @@ __device__ __forceinline__ double strided_sum(int b0, int b1, F &&at)
 }
 
 __global__ void __launch_bounds__(kReduceThreads) k_reduce(const double *__restrict__ part,
-                                                           const int32_t *__restrict__ seg, int pstride, double *out,
-                                                           int ostride, int op, const double *__restrict__ vn = nullptr,
-                                                           int vstride = 0, double *co = nullptr, int cstride = 0)
+                                                           const int32_t *__restrict__ seg, int rs, int pstride,
+                                                           double *out, int ostride, int op,
+                                                           const double *__restrict__ vn = nullptr, int vstride = 0,
+                                                           double *co = nullptr, int cstride = 0)
 {
     __shared__ double sh[kReduceThreads / 32];
     const int q = blockIdx.x, sy = blockIdx.y, c = sy >> 2, v = sy & 3;
-    const int b0 = seg[c], b1 = seg[c + 1];
+    const int b0 = rs * seg[c], b1 = rs * seg[c + 1];
     double acc = strided_sum(b0, b1, [&](int b) { return part[((int64_t)b * NV + v) * pstride + q]; });
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
     if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
@@ -1263,117 +1266,153 @@ __global__ void __launch_bounds__(kReduceThreads) k_reduce(const double *__restr
     }
 }
 
-// h[s][q] += h2[s][q], q <= j (second Gram-Schmidt pass)
-__global__ void k_hadd(double *hc, int hstride, const double *__restrict__ h2, int h2stride, int j, int ns)
-{
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < ns * (j + 1); t += gridDim.x * blockDim.x) {
-        const int sy = t / (j + 1), q = t % (j + 1);
-        hc[sy * hstride + q] += h2[sy * h2stride + q];
-    }
-}
-
-// Arnoldi index j of system sy (running systems only): the new Hessenberg
-// column from the raw sums hc, the earlier rotations applied, a new rotation,
-// the rotated residual g and the stopping test.
-__device__ __forceinline__ void givens_step(int sy, int j, int m, const double *__restrict__ hc, int hstride,
+// Arnoldi index j of system sy (running systems only), by one warp: the new
+// Hessenberg column from the raw sums hc (plus h2 of the second Gram-Schmidt
+// pass, if given), the earlier rotations applied, a new rotation, the rotated
+// residual g and the stopping test.  An FP64 division holds the pipe for 285 ns
+// whatever the number of lanes in it, so the column's divisions are done by the
+// lanes together and only the chain of rotations (four FP64 instructions each)
+// is serial; one thread for all of it took 9.6 us per launch with the reduction
+// (5.2 us this way, at Arnoldi indices 0-9).
+__device__ __forceinline__ void givens_step(int sy, int j, int m, const double *__restrict__ hc,
+                                            const double *__restrict__ h2, int h2stride, int hstride, double hnext,
                                             double *vn, double *H, double *cs, double *sn, double *g, int32_t *ctl,
                                             int ns, const double *__restrict__ bnorm,
-                                            const double *__restrict__ beta, double rtol, double eta, int maxit)
+                                            const double *__restrict__ beta, double rtol, double eta, int maxit,
+                                            double (*sh)[kMaxRestart + 1])
 {
-    if (!ctl[kCtlRunning * ns + sy]) return;
+    const int lane = threadIdx.x & 31;
     // Hessenberg column of the normalised basis: h_kj = <V_k, u_j> / (vn_k vn_j),
     // h_{j+1,j} = |V_{j+1}| / vn_j; the new vector's norm becomes vn_{j+1}
-    double h[kMaxRestart + 1];
+    double *h = sh[0], *c0 = sh[1], *s0 = sh[2], *hr = sh[3];
     const double nj = vn[sy * (m + 1) + j];
-    for (int k = 0; k <= j; ++k) h[k] = hc[sy * hstride + k] / (vn[sy * (m + 1) + k] * nj);
-    const double hnext = hc[sy * hstride + j + 1];
-    h[j + 1] = hnext / nj;
-    vn[sy * (m + 1) + j + 1] = hnext;
-    for (int k = 0; k < j; ++k) {
-        const double c = cs[sy * m + k], s = sn[sy * m + k];
-        const double t0 = h[k], t1 = h[k + 1];
-        h[k] = c * t0 + s * t1;
-        h[k + 1] = -s * t0 + c * t1;
+    for (int k = lane; k <= j + 1; k += 32) {
+        const double a = k <= j ? hc[sy * hstride + k] + (h2 ? h2[sy * h2stride + k] : 0.0) : hnext;
+        h[k] = a / (k <= j ? vn[sy * (m + 1) + k] * nj : nj);
+        if (k < j) {
+            c0[k] = cs[sy * m + k];
+            s0[k] = sn[sy * m + k];
+        }
     }
-    const double dd = hypot(h[j], h[j + 1]);
-    const double c = dd > 0.0 ? h[j] / dd : 1.0, s = dd > 0.0 ? h[j + 1] / dd : 0.0;
+    __syncwarp();
+    const double gj = g[sy * (m + 1) + j], bn = bnorm[sy], be = beta[sy];
+    const int it = ctl[kCtlIters * ns + sy] + 1;
+    double t0 = h[0];
+#pragma unroll 4
+    for (int k = 0; k < j; ++k) {
+        const double c = c0[k], s = s0[k], t1 = h[k + 1];
+        const double u = c * t0 + s * t1;
+        t0 = c * t1 - s * t0;
+        if (lane == 0) hr[k] = u;
+    }
+    const double t1 = h[j + 1];
+    // hypot where the squares leave FP64's range
+    const double d2 = t0 * t0 + t1 * t1;
+    double id, dd;
+    if (d2 > 1e-280 && d2 < 1e280) {
+        id = rsqrt(d2);
+        dd = d2 * id;
+    } else {
+        dd = hypot(t0, t1);
+        id = dd > 0.0 ? 1.0 / dd : 0.0;
+    }
+    const double c = dd > 0.0 ? t0 * id : 1.0, s = dd > 0.0 ? t1 * id : 0.0;
+    __syncwarp();
+    for (int k = lane; k < j; k += 32) H[((int64_t)sy * (m + 1) + k) * m + j] = hr[k];
+    if (lane != 0) return;
+    H[((int64_t)sy * (m + 1) + j) * m + j] = dd;
+    vn[sy * (m + 1) + j + 1] = hnext;
     cs[sy * m + j] = c;
     sn[sy * m + j] = s;
-    h[j] = dd;
-    for (int k = 0; k <= j; ++k) H[((int64_t)sy * (m + 1) + k) * m + j] = h[k];
-    const double gj = g[sy * (m + 1) + j];
     g[sy * (m + 1) + j + 1] = -s * gj;
     g[sy * (m + 1) + j] = c * gj;
     ctl[kCtlJv * ns + sy] = j + 1;
-    ctl[kCtlIters * ns + sy] += 1;
+    ctl[kCtlIters * ns + sy] = it;
     // stop the cycle at the target, or (mixed precision, eta > 0) once the inner
     // residual has dropped by eta: the FP64 refinement residual then restarts it
-    const double gn = fabs(g[sy * (m + 1) + j + 1]);
-    if (gn <= rtol * bnorm[sy] || gn <= eta * beta[sy] || !(hnext > 0.0) || ctl[kCtlIters * ns + sy] >= maxit ||
-        j + 1 == m)
+    const double gn = fabs(s * gj);
+    if (gn <= rtol * bn || gn <= eta * be || !(hnext > 0.0) || it >= maxit || j + 1 == m)
         ctl[kCtlRunning * ns + sy] = 0;
 }
 
-// The last reduction of an Arnoldi index (|V_{j+1}| of system blockIdx.y into
-// hc[.][j + 1], as k_reduce with op 2) followed by that system's Givens step
-// in thread 0, which saves a launch per index.
+// The last reduction of an Arnoldi index (|V_{j+1}| of system blockIdx.y, the
+// square root of the summed partials) followed by that system's Givens step,
+// which saves a launch per index.
 __global__ void __launch_bounds__(kReduceThreads) k_norm_givens(const double *__restrict__ part,
-                                                                const int32_t *__restrict__ seg, int pstride, int j,
-                                                                int m, double *hc, int hstride, double *vn, double *H,
+                                                                const int32_t *__restrict__ seg, int rs, int pstride,
+                                                                int j, int m, const double *hc, int hstride,
+                                                                const double *h2, int h2stride, double *vn, double *H,
                                                                 double *cs, double *sn, double *g, int32_t *ctl,
                                                                 int ns, const double *__restrict__ bnorm,
                                                                 const double *__restrict__ beta, double rtol,
                                                                 double eta, int maxit)
 {
     __shared__ double sh[kReduceThreads / 32];
+    __shared__ double shg[4][kMaxRestart + 1];
     const int sy = blockIdx.y, c = sy >> 2, v = sy & 3;
-    const int b0 = seg[c], b1 = seg[c + 1];
+    if (!ctl[kCtlRunning * ns + sy]) return;
+    const int b0 = rs * seg[c], b1 = rs * seg[c + 1];
     double acc = strided_sum(b0, b1, [&](int b) { return part[((int64_t)b * NV + v) * pstride]; });
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
     if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        acc = 0.0;
-        for (int w = 0; w < kReduceThreads / 32; ++w) acc += sh[w];
-        hc[sy * hstride + j + 1] = sqrt(acc);
-        givens_step(sy, j, m, hc, hstride, vn, H, cs, sn, g, ctl, ns, bnorm, beta, rtol, eta, maxit);
-    }
+    if (threadIdx.x >= 32) return;
+    acc = 0.0;
+    for (int w = 0; w < kReduceThreads / 32; ++w) acc += sh[w];
+    givens_step(sy, j, m, hc, h2, h2stride, hstride, sqrt(acc), vn, H, cs, sn, g, ctl, ns, bnorm, beta, rtol, eta,
+                maxit, shg);
 }
 
-// y = H^{-1} g on the first jv columns (upper triangular after the rotations).
-__global__ void k_backsolve(int m, const double *__restrict__ H, const double *__restrict__ g, double *y,
-                            const int32_t *__restrict__ ctl, int ns)
-{
-    const int sy = blockIdx.x * blockDim.x + threadIdx.x;
-    if (sy >= ns) return;
-    const int jv = ctl[kCtlJv * ns + sy];
-    for (int k = jv - 1; k >= 0; --k) {
-        double s = g[sy * (m + 1) + k];
-        for (int q = k + 1; q < jv; ++q) s -= H[((int64_t)sy * (m + 1) + k) * m + q] * y[sy * m + q];
-        y[sy * m + k] = s / H[((int64_t)sy * (m + 1) + k) * m + k];
-    }
-}
-
-// y_k /= vn_k: coefficients of the unnormalised preconditioned vectors
+// End of a cycle, one warp per system: y = H^{-1} g on the first jv columns
+// (upper triangular after the rotations), column by column, the lanes holding
+// the right-hand side (the diagonal's reciprocals are formed together); then
+// y_k /= vn_k, the coefficients of the unnormalised preconditioned vectors.
 // With sexp given (FP32 basis, rows [current][next] exponents e of the scale
 // 2^-e of the first basis vector): y is also scaled by 2^-e of the current
 // cycle (the combination adds 2^e sum y_k Z_k, so its FP32 sums stay near unit
 // size), and the next residual's exponent comes from the cycle's estimate
 // |g_jv| of its norm (at least 1e-3 rtol |b|).
 // y32 (optional): an FP32 copy of the result for the FP32 combination.
-__global__ void k_scale_y(int m, double *y, const double *__restrict__ vn, const int32_t *__restrict__ ctl, int ns,
-                          const double *__restrict__ g = nullptr, const double *__restrict__ bnorm = nullptr,
-                          double rtol = 0.0, int32_t *sexp = nullptr, float *y32 = nullptr)
+// One thread per system took 13-17 us for ten columns in two launches.
+constexpr int kSolveWarps = 4;      // systems per block
+__global__ void __launch_bounds__(32 * kSolveWarps)
+    k_cycle_solve(int m, const double *__restrict__ H, const double *__restrict__ g, double *__restrict__ y,
+                  const double *__restrict__ vn, const int32_t *__restrict__ ctl, int ns,
+                  const double *__restrict__ bnorm, double rtol, int32_t *sexp, float *y32)
 {
-    const int sy = blockIdx.x * blockDim.x + threadIdx.x;
+    const int sy = blockIdx.x * kSolveWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (sy >= ns) return;
     const int jv = ctl[kCtlJv * ns + sy];
+    if (jv <= 0) return;
+    // lane l holds the entries l and l + 32 (jv <= kMaxRestart = 64)
+    const double *Hs = H + (int64_t)sy * (m + 1) * m;
+    double rh[2], iv[2], sc[2];
     const double f = sexp ? pow2(-sexp[sy]) : 1.0;
-    for (int k = 0; k < jv; ++k) {
-        y[sy * m + k] = sexp ? y[sy * m + k] / vn[sy * (m + 1) + k] * f : y[sy * m + k] / vn[sy * (m + 1) + k];
-        if (y32) y32[sy * m + k] = float(y[sy * m + k]);
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        const int k = lane + 32 * q;
+        rh[q] = k < jv ? g[sy * (m + 1) + k] : 0.0;
+        iv[q] = k < jv ? 1.0 / Hs[(int64_t)k * m + k] : 0.0;
+        sc[q] = k < jv ? f / vn[sy * (m + 1) + k] : 0.0;
     }
-    if (sexp && jv > 0) {
+    for (int k = jv - 1; k >= 0; --k) {
+        const bool hi = k >= 32;
+        const double yk = __shfl_sync(0xffffffffu, hi ? rh[1] * iv[1] : rh[0] * iv[0], k & 31);
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int r = lane + 32 * q;
+            if (r < k) rh[q] = fma(-Hs[(int64_t)r * m + k], yk, rh[q]);
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        const int k = lane + 32 * q;
+        if (k >= jv) continue;
+        const double yk = rh[q] * iv[q] * sc[q];
+        y[sy * m + k] = yk;
+        if (y32) y32[sy * m + k] = float(yk);
+    }
+    if (sexp && lane == 0) {
         const double est = fmax(fabs(g[sy * (m + 1) + jv]), 1e-3 * rtol * bnorm[sy]);
         if (est > 0.0 && est < 1e300) sexp[ns + sy] = max(-1000, ilogb(est));
     }
@@ -1385,7 +1424,7 @@ __global__ void k_scale_y(int m, double *y, const double *__restrict__ vn, const
 // the inner tolerance; the next FP64 residual measures what is left) and added
 // to x in FP64, so the FP64 pipe sees one add per value instead of one
 // conversion and one FMA per value and Krylov vector.  With sexp given (FP32
-// basis): y carries 2^-e of the cycle (see k_scale_y) and the sum is scaled
+// basis): y carries 2^-e of the cycle (see k_cycle_solve) and the sum is scaled
 // back by 2^e in FP64 (exact).
 // y32 (FP32 Z only, optional): the FP32 copy of y, read instead of converting
 // y per thread; the scaled value 2^e acc is formed exactly on the integer pipe
@@ -1703,7 +1742,7 @@ gks_status precond_t(gks_mesh *m, const TP *Pg, const TP *alg, const TP *exg, co
         const bool fuse = ns > 0 && m->cfg.ilu_fuse_first;
         // two backward sweeps per launch where a pair follows (the per-cell
         // equations; same results as one sweep per launch)
-        const bool pairs = !rev.a && m->cfg.ilu_sweep_pairs;   // backward relation only
+        const bool pairs = std::is_same_v<TZ, float> && !rev.a && m->cfg.ilu_sweep_pairs;   // backward relation only
         const int nf = fuse ? ns : ns + 1;   // forward launches
         TZ *za = (nf % 2 == 1) ? tA : dst;   // buffers chosen so that z ends in tA
         TZ *zb = (nf % 2 == 1) ? dst : tA;
@@ -1725,9 +1764,13 @@ gks_status precond_t(gks_mesh *m, const TP *Pg, const TP *alg, const TP *exg, co
             TZ *xa = za;                                    // x^0 = z (in za)
             TZ *xb = (nb % 2 == 1) ? dst : (za == tB ? tA : tB);
             for (int q = 0; q < nb; ++q) {
-                if (q < npair) {
-                    k_ilu_bwd2<TZ, TM, TP><<<nblocks(T), kBlock, 0, s>>>(d, Pg, alg, exg, eyg, za, xa, xb);
-                    note_launch();
+                if constexpr (std::is_same_v<TZ, float>) {
+                    if (q < npair) {
+                        k_ilu_bwd2<TZ, TM, TP><<<nblocks(T), kBlock, 0, s>>>(d, Pg, alg, exg, eyg, za, xa, xb);
+                        note_launch();
+                    } else {
+                        bwd(T, nullptr, za, xa, xb);
+                    }
                 } else {
                     bwd(T, nullptr, za, xa, xb);
                 }
@@ -1740,10 +1783,147 @@ gks_status precond_t(gks_mesh *m, const TP *Pg, const TP *alg, const TP *exg, co
     return GKS_OK;
 }
 
+// The sweeps of the FP64 solve of the per-cell equations (a thread per cell and
+// variable): dst = M^{-1} src with the arithmetic of the sweeps of precond_t.
+// Sweeps that only feed another sweep form the rows 0 and 1 alone; their
+// results alternate between dst and t2 so that the last one is in t2, and the
+// full z is in t3 (or dst without backward sweeps).
+//
+// The block-diagonal pass is folded into the first forward sweep (ilu_fuse_first;
+// the same results bit for bit) where a launch costs more than the FP64 work it
+// repeats, up to kFuse64 triangles: ten steps take 6,307 against 6,403 us at 800
+// triangles, 8,839 against 8,949 at 6,400, 9,933 against 9,909 at 20,000.
+constexpr int64_t kFuse64 = 16000;
+
+gks_status precond64(gks_mesh *m, const double *src, double *dst, cudaStream_t s)
+{
+    const DeviceMesh &d = m->d;
+    Work &k = m->wk;
+    const int64_t T = d.T;
+    const unsigned g = (unsigned)((T + 31) / 32);
+    const int32_t *run = k.ctl + kCtlRunning * k.ns;
+    const int ns = m->cfg.ilu_sweeps, nsb = m->cfg.ilu_sweeps_bwd < 0 ? ns : m->cfg.ilu_sweeps_bwd;
+    const bool fuse = ns > 0 && m->cfg.ilu_fuse_first && T <= kFuse64;
+    double *z = nsb > 0 ? k.t3 : dst;
+    // buffer of the q-th of n intermediate results
+    auto mid = [&](int q, int n) { return (n - 1 - q) % 2 == 0 ? k.t2 : dst; };
+    auto fwd = [&](int nb, bool full, const double *zin, double *zout) {
+#define F64(NB, FULL) k64_fwd<NB, FULL><<<g, kW64, 0, s>>>(T, d.nb, d.P, d.off, d.blk_case, run, src, zin, zout)
+        if (nb == 0) full ? F64(0, true) : F64(0, false);
+        else if (nb == 1) full ? F64(1, true) : F64(1, false);
+        else full ? F64(2, true) : F64(2, false);
+#undef F64
+        note_launch();
+    };
+    // forward: z^0 = P r (a launch of its own unless folded in), z^{q+1} = F(z^q)
+    const int nf = fuse ? ns : ns + 1;                    // launches
+    const double *prev = nullptr;
+    for (int q = 0; q < nf; ++q) {
+        const bool last = q + 1 == nf;
+        double *out = last ? z : mid(q, nf - 1);
+        fwd(q == 0 ? (fuse ? 2 : 0) : 1, last, prev, out);
+        prev = out;
+    }
+    // backward: x^0 = z, x^{q+1} = B(x^q)
+    const double *x = z;
+    for (int q = 0; q < nsb; ++q) {
+        const bool last = q + 1 == nsb;
+        double *out = last ? dst : mid(q, nsb - 1);
+        if (last) k64_bwd<true><<<g, kW64, 0, s>>>(T, d.nb, d.P, d.off, d.blk_case, run, z, x, out);
+        else k64_bwd<false><<<g, kW64, 0, s>>>(T, d.nb, d.P, d.off, d.blk_case, run, z, x, out);
+        note_launch();
+        x = out;
+    }
+    GKS_CUDA(cudaGetLastError());
+    return GKS_OK;
+}
+
+// Launches of the FP64 solve with m->wk.c64 cells per thread.
+template <typename F>
+void with_cells64(int c, F &&f)
+{
+    switch (c) {
+    case 1: f(std::integral_constant<int, 1>{}); break;
+    case 2: f(std::integral_constant<int, 2>{}); break;
+    case 4: f(std::integral_constant<int, 4>{}); break;
+    default: f(std::integral_constant<int, 8>{}); break;
+    }
+    note_launch();
+}
+
+inline unsigned rows64(const gks_mesh *m) { return (unsigned)(m->wk.nblk * (kRows64 / m->wk.c64)); }
+
+// dynamic shared memory of the product kernels at Arnoldi index j
+inline size_t acc64(int j, int stride) { return sizeof(double) * 4 * (j + 1) * stride; }
+
+// Beyond 48 KiB (restart lengths above 45) the kernels have to ask for it.
+gks_status solve64_shared_limit(int mm)
+{
+    auto set = [&](auto C) -> gks_status {
+        constexpr int c = decltype(C)::value;
+        GKS_CUDA(cudaFuncSetAttribute(k64_apply_dots<c>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)acc64(mm - 1, kAccStride)));
+        GKS_CUDA(cudaFuncSetAttribute(k64_update_dots<c>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)acc64(mm - 1, kAccStride + 1)));
+        return GKS_OK;
+    };
+    gks_status st = set(std::integral_constant<int, 1>{});
+    if (st == GKS_OK) st = set(std::integral_constant<int, 2>{});
+    if (st == GKS_OK) st = set(std::integral_constant<int, 4>{});
+    if (st == GKS_OK) st = set(std::integral_constant<int, 8>{});
+    return st;
+}
+
+void solve64_rhs(gks_mesh *m, int ps, cudaStream_t q)
+{
+    const DeviceMesh &d = m->d;
+    with_cells64(m->wk.c64, [&](auto C) {
+        k64_rhs<decltype(C)::value><<<rows64(m), kW64, 0, q>>>(d.T, d.nb, d.a0, m->wk.w, m->wk.b, m->wk.part, ps);
+    });
+}
+
+void solve64_resid(gks_mesh *m, double *V0, int ps, cudaStream_t q)
+{
+    const DeviceMesh &d = m->d;
+    with_cells64(m->wk.c64, [&](auto C) {
+        k64_resid<decltype(C)::value><<<rows64(m), kW64, 0, q>>>(d.T, d.nb, d.D, d.off, m->wk.x, m->wk.b, V0,
+                                                               m->wk.part, ps);
+    });
+}
+
+void solve64_apply_dots(gks_mesh *m, const double *z, const double *V, double *y, int j, int ps, cudaStream_t q)
+{
+    const DeviceMesh &d = m->d;
+    with_cells64(m->wk.c64, [&](auto C) {
+        k64_apply_dots<decltype(C)::value><<<rows64(m), kW64, acc64(j, kAccStride), q>>>(
+            d.T, d.nb, d.D, d.off, d.blk_case, m->wk.ctl + kCtlRunning * m->wk.ns, z, y, V, j, m->wk.part, ps);
+    });
+}
+
+void solve64_update_dots(gks_mesh *m, const double *V, double *w, int j, int ps, cudaStream_t q)
+{
+    const DeviceMesh &d = m->d;
+    with_cells64(m->wk.c64, [&](auto C) {
+        k64_update_dots<decltype(C)::value><<<rows64(m), kW64, acc64(j, kAccStride + 1), q>>>(
+            d.T, d.blk_case, m->wk.ctl + kCtlRunning * m->wk.ns, V, w, j, m->wk.hco, ps, m->wk.part, ps);
+    });
+}
+
+void solve64_update_norm(gks_mesh *m, const double *V, double *w, int j, int ps, cudaStream_t q)
+{
+    const DeviceMesh &d = m->d;
+    with_cells64(m->wk.c64, [&](auto C) {
+        k64_update_norm<decltype(C)::value><<<rows64(m), kW64, 0, q>>>(
+            d.T, d.blk_case, m->wk.ctl + kCtlRunning * m->wk.ns, V, w, j, m->wk.hco, ps, m->wk.part, ps);
+    });
+}
+
 template <typename TR>
 gks_status precond(gks_mesh *m, const TR *src, double *dst, cudaStream_t s)
 {
     DeviceMesh &d = m->d;
+    if constexpr (std::is_same_v<TR, double>)
+        if (m->wk.c64 && m->cfg.precond == GKS_PC_ILU_SWEEP) return precond64(m, src, dst, s);
     return precond_t<TR, double, double>(m, d.P, d.alpha, d.ex, d.ey, src, dst, m->wk.t2, m->wk.t3, nullptr, s,
                                          {d.alr, d.exr, d.eyr, d.bdg});
 }
@@ -2068,6 +2248,12 @@ gks_status cls_solve_t(gks_mesh *m, TB *V, cudaStream_t s, int32_t *iters, doubl
     // refinement sweep then measures the true error
     const double eta = mixed ? m->cfg.inner_rtol : 0.0;
     gks_status st;
+    // the FP64 solve of the per-cell equations: a thread per cell and variable
+    // (gks_solve64.cuh), C64 cells per thread, rs partial-sum rows per cell block
+    const int C64 = k.c64, rs = C64 ? kRows64 / C64 : 1;
+    if (C64 && mm > 45) {
+        if ((st = solve64_shared_limit(mm)) != GKS_OK) return st;
+    }
 
     // FP32 basis: first basis vector scaled by a power of two; exponents per
     // system, [current cycle][next residual]
@@ -2097,6 +2283,11 @@ gks_status cls_solve_t(gks_mesh *m, TB *V, cudaStream_t s, int32_t *iters, doubl
     // the FP32-basis solve forms b in double-FP32 arithmetic when the weights fit
     const bool rhs_df = std::is_same<TB, float>::value && d.a0p;
     auto residual = [&](cudaStream_t q) -> gks_status {
+        if (C64) {
+            solve64_resid(m, reinterpret_cast<double *>(V), ps, q);
+            GKS_CUDA(cudaGetLastError());
+            return GKS_OK;
+        }
         if (std::is_same<TB, float>::value && d.D2) {
             if (d.SR2)
                 k_resid_df<true><<<4 * nb, kBlock, 0, q>>>(d, d.D2, d.S2, k.x, reinterpret_cast<float *>(V), k.b,
@@ -2119,14 +2310,18 @@ gks_status cls_solve_t(gks_mesh *m, TB *V, cudaStream_t s, int32_t *iters, doubl
             k_sf_begin<<<1, 32, 0, q>>>(k.sf_ctl, 1);      // a new solve: clear the wait error
             note_launch();
         }
-        if (rhs_df)
-            k_rhs_df<<<nb, kBlock, 0, q>>>(d, d.a0p, k.w, k.b, k.part, ps);
-        else
-            k_rhs<<<nb, kBlock, 0, q>>>(d, k.w, k.b, k.part, ps);
-        note_launch();
+        if (C64) {
+            solve64_rhs(m, ps, q);
+        } else {
+            if (rhs_df)
+                k_rhs_df<<<nb, kBlock, 0, q>>>(d, d.a0p, k.w, k.b, k.part, ps);
+            else
+                k_rhs<<<nb, kBlock, 0, q>>>(d, k.w, k.b, k.part, ps);
+            note_launch();
+        }
         if (sx) {
             // the FP32 basis stores its first vector scaled by a power of two 2^-e
-            k_reduce<<<dim3(1, ns), kReduceThreads, 0, q>>>(k.part + 1, d.case_blk, ps, k.hcol + 1, ps, 0);
+            k_reduce<<<dim3(1, ns), kReduceThreads, 0, q>>>(k.part + 1, d.case_blk, rs, ps, k.hcol + 1, ps, 0);
             note_launch();
             k_sigma<<<sblocks(ns), 128, 0, q>>>(k.hcol, ps, k.bnorm, k.sexp, ns); note_launch();
         }
@@ -2134,7 +2329,7 @@ gks_status cls_solve_t(gks_mesh *m, TB *V, cudaStream_t s, int32_t *iters, doubl
         slot = prof_start(m, kProfResid, q);
         // residual r = b - K x, written straight into the basis slot V_0 (v_0 = V_0 / beta)
         if (const gks_status r = residual(q); r != GKS_OK) return r;
-        k_reduce<<<dim3(sx ? 1 : 2, ns), kReduceThreads, 0, q>>>(k.part, d.case_blk, ps, k.hcol, ps, 0);
+        k_reduce<<<dim3(sx ? 1 : 2, ns), kReduceThreads, 0, q>>>(k.part, d.case_blk, rs, ps, k.hcol, ps, 0);
         note_launch();
         prof_stop(m, slot, q);
         slot = prof_start(m, kProfCtl, q);
@@ -2172,32 +2367,45 @@ gks_status cls_solve_t(gks_mesh *m, TB *V, cudaStream_t s, int32_t *iters, doubl
             }
         } else if (mixed) {
             spmv32(q, k.Z32 + j * vs, vj1);
+        } else if (C64) {
+            // with the first Gram-Schmidt products
+            solve64_apply_dots(m, k.Z + j * vs, reinterpret_cast<const double *>(V), reinterpret_cast<double *>(vj1),
+                               j, ps, q);
         } else {
             spmv64(q, k.Z + j * vs, vj1, 0, nullptr, nullptr);
         }
-        note_launch();
+        if (!C64) note_launch();
         prof_stop(m, slot, q);
         slot = prof_start(m, kProfOrth, q);
         // classical Gram-Schmidt: twice in FP64 mode; once in the mixed mode, whose
         // cycles only reduce the residual by inner_rtol before an FP64 restart
-        if (!fused_dots && (st = dots<TB>(m, V, vj1, j, k.part, ps, q)) != GKS_OK) return st;
-        k_reduce<<<dim3(j + 1, ns), kReduceThreads, 0, q>>>(k.part, d.case_blk, ps, k.hcol, ps, 0, k.vn, mm + 1,
+        if (!fused_dots && !C64 && (st = dots<TB>(m, V, vj1, j, k.part, ps, q)) != GKS_OK) return st;
+        k_reduce<<<dim3(j + 1, ns), kReduceThreads, 0, q>>>(k.part, d.case_blk, rs, ps, k.hcol, ps, 0, k.vn, mm + 1,
                                                              k.hco, ps);
         note_launch();
-        launch_orth_update<TB>(d, nb, q, V, vj1, j, k.hco, ps, k.ctl, ns, k.part, ps, mixed ? 1 : 0);
-        note_launch();
+        if (C64) {
+            solve64_update_dots(m, reinterpret_cast<const double *>(V), reinterpret_cast<double *>(vj1), j, ps, q);
+        } else {
+            launch_orth_update<TB>(d, nb, q, V, vj1, j, k.hco, ps, k.ctl, ns, k.part, ps, mixed ? 1 : 0);
+            note_launch();
+        }
         if (!mixed) {
-            if ((st = dots<TB>(m, V, vj1, j, k.part, ps, q)) != GKS_OK) return st;
-            k_reduce<<<dim3(j + 1, ns), kReduceThreads, 0, q>>>(k.part, d.case_blk, ps, k.y, mm, 0, k.vn, mm + 1,
+            // the second pass
+            if (!C64 && (st = dots<TB>(m, V, vj1, j, k.part, ps, q)) != GKS_OK) return st;
+            k_reduce<<<dim3(j + 1, ns), kReduceThreads, 0, q>>>(k.part, d.case_blk, rs, ps, k.y, mm, 0, k.vn, mm + 1,
                                                                  k.hco, ps);
             note_launch();
-            launch_orth_update<TB>(d, nb, q, V, vj1, j, k.hco, ps, k.ctl, ns, k.part, ps, 1); note_launch();
-            k_hadd<<<sblocks(ns * (j + 1)), 128, 0, q>>>(k.hcol, ps, k.y, mm, j, ns); note_launch();
+            if (C64) {
+                solve64_update_norm(m, reinterpret_cast<const double *>(V), reinterpret_cast<double *>(vj1), j, ps, q);
+            } else {
+                launch_orth_update<TB>(d, nb, q, V, vj1, j, k.hco, ps, k.ctl, ns, k.part, ps, 1);
+                note_launch();
+            }
         }
         // |V_{j+1}| and the Givens step of every system
-        k_norm_givens<<<dim3(1, ns), kReduceThreads, 0, q>>>(k.part, d.case_blk, ps, j, mm, k.hcol, ps, k.vn, k.H,
-                                                              k.cs, k.sn, k.g, k.ctl, ns, k.bnorm, k.beta, rtol, eta,
-                                                              maxit);
+        k_norm_givens<<<dim3(1, ns), kReduceThreads, 0, q>>>(k.part, d.case_blk, rs, ps, j, mm, k.hcol, ps,
+                                                              mixed ? nullptr : k.y, mm, k.vn, k.H, k.cs, k.sn, k.g,
+                                                              k.ctl, ns, k.bnorm, k.beta, rtol, eta, maxit);
         note_launch();
         prof_stop(m, slot, q);
         GKS_CUDA(cudaGetLastError());
@@ -2205,19 +2413,21 @@ gks_status cls_solve_t(gks_mesh *m, TB *V, cudaStream_t s, int32_t *iters, doubl
     };
     auto restart_body = [&](cudaStream_t q) -> gks_status {
         int slot = prof_start(m, kProfCorr, q);
-        k_backsolve<<<sblocks(ns), 128, 0, q>>>(mm, k.H, k.g, k.y, k.ctl, ns); note_launch();
-        k_scale_y<<<sblocks(ns), 128, 0, q>>>(mm, k.y, k.vn, k.ctl, ns, k.g, k.bnorm, rtol, sx,
-                                               mixed ? k.y32 : nullptr);
+        k_cycle_solve<<<(ns + kSolveWarps - 1) / kSolveWarps, 32 * kSolveWarps, 0, q>>>(
+            mm, k.H, k.g, k.y, k.vn, k.ctl, ns, k.bnorm, rtol, sx, mixed ? k.y32 : nullptr);
         note_launch();
         if (mixed)
             k_combine_z<float><<<dim3(nb, NV), kBlock, 0, q>>>(d, k.Z32, k.y, mm, k.ctl, ns, k.x, sx, k.y32);
+        else if (C64)
+            k64_combine<<<(unsigned)((T + 31) / 32), kW64, 0, q>>>(T, d.blk_case, k.Z, k.y, mm, k.ctl + kCtlJv * ns,
+                                                                  k.x);
         else
             k_combine_z<double><<<dim3(nb, NV), kBlock, 0, q>>>(d, k.Z, k.y, mm, k.ctl, ns, k.x);
         note_launch();
         prof_stop(m, slot, q);
         slot = prof_start(m, kProfResid, q);
         if (const gks_status r = residual(q); r != GKS_OK) return r;
-        k_reduce<<<dim3(1, ns), kReduceThreads, 0, q>>>(k.part, d.case_blk, ps, k.hcol, ps, 0); note_launch();
+        k_reduce<<<dim3(1, ns), kReduceThreads, 0, q>>>(k.part, d.case_blk, rs, ps, k.hcol, ps, 0); note_launch();
         prof_stop(m, slot, q);
         slot = prof_start(m, kProfCtl, q);
         k_start<<<sblocks(ns), 128, 0, q>>>(k.hcol, ps, k.bnorm, k.beta, k.vn, mm, k.ctl, ns, k.done, rtol, maxit,
@@ -2402,6 +2612,22 @@ gks_status cls_solve(gks_mesh *m, cudaStream_t s, int32_t *iters, double *relres
     if (const gks_status st = launch_warm(m, s); st != GKS_OK) return st;
     return k.V32 ? cls_solve_t<float>(m, k.V32, s, iters, relres, converged)
                  : cls_solve_t<double>(m, k.V, s, iters, relres, converged);
+}
+
+void plan_solve64(gks_mesh *m, int *rows)
+{
+    m->wk.c64 = cells64(m->d.T);
+    *rows = kRows64 / m->wk.c64;
+}
+
+gks_status launch_off64(gks_mesh *m)
+{
+    const DeviceMesh &d = m->d;
+    if (d.T == 0) return GKS_OK;
+    k64_off<<<nblocks(d.T), kBlock>>>(d.T, d.alpha, d.ex, d.ey, d.off);
+    note_launch();
+    GKS_CUDA(cudaGetLastError());
+    return GKS_OK;
 }
 
 gks_status run_graph_launch(gks_mesh *m, int64_t max_steps, cudaStream_t s, bool *used)

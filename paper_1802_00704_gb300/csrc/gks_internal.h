@@ -69,6 +69,7 @@ struct DeviceMesh {
     // second-derivative equations (cls_M = 2): beta of the diagonal coupling of the
     // unknowns 3..5 with the neighbour's (plus the reverse one in the global system)
     double *bdg = nullptr;           // [3][T]; with alr.. allocated for either option (zeros if unused)
+    double *off = nullptr;           // [9][T] alpha, alpha dx, alpha dy per slot (FP64 solve, per-cell equations)
     double *a0 = nullptr;            // [3][5][T] weighted row 0 of A_ij (right-hand side)
     float *a0p = nullptr;            // [30][T] FP32 pairs of a0 (the 15 high parts, then the low parts)
     double *D = nullptr;             // [15][T] symmetric diagonal block, upper triangle row-major
@@ -112,6 +113,7 @@ struct Work {
     int m = 0;                       // restart length in use (the autotuner may lower it)
     int m_alloc = 0;                 // restart length the Krylov buffers were sized for
     int nblk = 0;                    // cell blocks (kBlock cells each)
+    int c64 = 0;                     // FP64 solve of the per-cell equations: cells per thread (0: other solves)
     int sm_count = 0;                // multiprocessors of the handle's device
     int ns = 4;                      // GMRES systems: 4 per case
     double *w = nullptr;             // [4][T] state (internal order)
@@ -138,7 +140,7 @@ struct Work {
     double *Z = nullptr;             // [m][20][T] M^{-1} V_k (FP64 path)
     float *Z32 = nullptr;            // [m][20][T] M^{-1} V_k (mixed path)
     double *flux = nullptr;          // [4][F]
-    double *part = nullptr;          // [nblk][4][m+2] partial sums per cell block
+    double *part = nullptr;          // [nblk * rows][4][m+2] partial sums (rows per cell block: 8 / c64, else 1)
     double *dpart = nullptr;         // [nblk][4] partial minima / sums
     // small GMRES state (device), one row per system
     double *H = nullptr;             // [ns][m+1][m]  (Givens-rotated Hessenberg)
@@ -266,6 +268,10 @@ struct CaseIn {
     const double *bc_state;
 };
 
+// cells per thread of the FP64 solve and its partial-sum rows per cell block; the
+// multiplied-out off-diagonal blocks d.off from d.alpha, d.ex, d.ey (gks_cls.cu)
+void plan_solve64(gks_mesh *m, int *rows);
+gks_status launch_off64(gks_mesh *m);
 // set-up (gks_setup.cu)
 gks_status build_batch(gks_mesh *m, const CaseIn *cases, int32_t n_cases);
 void free_mesh(gks_mesh *m);

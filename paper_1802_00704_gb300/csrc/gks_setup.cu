@@ -856,7 +856,13 @@ gks_status build_batch(gks_mesh *m, const CaseIn *cases, int32_t n_cases)
     } else {
         AL(Z, (size_t)mm * 20 * T);
     }
-    AL(part, (size_t)nblk * 4 * (mm + 2)); AL(dpart, (size_t)nblk * 4);
+    int rows = 1;
+    if (cfg.precision == GKS_FP64 && !ext) {
+        plan_solve64(m, &rows);
+        if ((st = dalloc(m, &d.off, (size_t)9 * T)) != GKS_OK) return st;
+        if ((st = launch_off64(m)) != GKS_OK) return st;
+    }
+    AL(part, (size_t)nblk * rows * 4 * (mm + 2)); AL(dpart, (size_t)nblk * 4);
     if (cfg.limiter) {
         AL(xl, 20 * T); AL(lflag, T);
     }

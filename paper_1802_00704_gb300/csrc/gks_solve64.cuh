@@ -1,0 +1,498 @@
+// Kernels of the FP64 reconstruction solve (per-cell equations), one thread per
+// cell and variable.
+//
+// GB300 runs FP64 at 1/64 of its FP32 rate: a warp's FP64 instruction holds its
+// SM sub-partition for 33 ns whatever its active lanes, so a kernel's time is
+// the number of FP64 instructions per thread times the warps per sub-partition
+// (608 of them).  A thread per cell (all four variables in it) left an
+// 800-triangle mesh with 25 warps of 640 instructions per preconditioner
+// application.  Here a warp takes 32 cells of one variable: four times the
+// warps with a quarter of the instructions each, no block-wide barrier, and the
+// warps of a variable whose system has stopped return at once.
+//
+// Three more things keep the instruction count down:
+//  - a sweep whose result only feeds another sweep forms the gradient rows 0
+//    and 1 of each cell alone, all that an off-diagonal block reads (10 of the
+//    25 products with the pivot inverse);
+//  - the off-diagonal blocks are stored multiplied out (off: alpha, alpha dx,
+//    alpha dy per slot), and only the lower (upper) slots of a cell enter the
+//    arithmetic of a triangular relation;
+//  - sums over cells start their FMA chains from the running sum in shared
+//    memory and are added across the lanes of a warp in transposed order, 7-31
+//    additions for all Arnoldi indices together instead of 5 for each.
+// Measured on GB300 (the solve's classes, per Arnoldi index, events around each
+// class): preconditioner with two sweeps each way 80 -> 25 us at 800 triangles
+// and 680 -> 448 us at 399,424; operator with the first Gram-Schmidt products and
+// the rest of the Gram-Schmidt passes 83 -> 46 us and 610 -> 528 us.  Two
+// backward sweeps in one launch, each thread forming its upper neighbours' first
+// sweep itself, were no faster at any size (6,323 against 6,307 us for ten steps
+// at 800 triangles, 10,285 against 9,933 at 20,000) and are not there.
+#pragma once
+
+#include "gks_internal.h"
+
+namespace gks {
+namespace {
+
+constexpr int kW64 = 128;              // threads per block: one warp per variable
+
+// Cells per thread (C) and partial-sum rows per kBlock-cell block (8 / C): more
+// cells per thread amortise the sums across lanes once the GPU is full of warps
+// (T / 8 of them with one cell per thread), fewer spread a small mesh over it.
+inline int cells64(int64_t T) { return T <= 40000 ? 1 : (T <= 80000 ? 2 : (T <= 160000 ? 4 : 8)); }
+constexpr int kRows64 = kBlock / 32;   // rows per cell block with one cell per thread
+
+// acc += O (g1, g2) for the stored block (a, ax, ay) = alpha (1, dx, dy)
+__device__ __forceinline__ void off_acc(double a, double ax, double ay, double g1, double g2, double *acc)
+{
+    acc[0] = fma(a, g1, acc[0]);
+    acc[1] = fma(a, g2, acc[1]);
+    acc[2] = fma(ax, g1, acc[2]);
+    acc[3] = fma(ay, g1, fma(ax, g2, acc[3]));
+    acc[4] = fma(ay, g2, acc[4]);
+}
+
+// The lower (UP = false: 0 <= j < i) or upper (j > i) neighbours of cell i, in
+// slot order: js[q], their slots ss[q], q < the returned number.
+template <bool UP>
+__device__ __forceinline__ int side_slots(const int32_t *__restrict__ nb, int64_t T, int64_t i, int *js, int *ss)
+{
+    int n = 0;
+    js[0] = js[1] = js[2] = (int)i;
+    ss[0] = ss[1] = ss[2] = 0;
+#pragma unroll
+    for (int s = 0; s < 3; ++s) {
+        const int j = nb[s * T + i];
+        if (!(UP ? j > (int)i : (j >= 0 && j < (int)i))) continue;
+        if (n == 0) { js[0] = j; ss[0] = s; }
+        else if (n == 1) { js[1] = j; ss[1] = s; }
+        else { js[2] = j; ss[2] = s; }
+        ++n;
+    }
+    return n;
+}
+
+struct Off64 {
+    double a, ax, ay;
+};
+
+__device__ __forceinline__ Off64 off_load(const double *__restrict__ off, int64_t T, int s, int64_t i)
+{
+    return {off[(3 * s) * T + i], off[(3 * s + 1) * T + i], off[(3 * s + 2) * T + i]};
+}
+
+// Multiplied-out off-diagonal blocks (set-up): off[3 s + (0, 1, 2)] = alpha (1, dx, dy)
+__global__ void k64_off(int64_t T, const double *__restrict__ al, const double *__restrict__ ex,
+                        const double *__restrict__ ey, double *__restrict__ off)
+{
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= T) return;
+#pragma unroll
+    for (int s = 0; s < 3; ++s) {
+        const double a = al[s * T + i];
+        off[(3 * s) * T + i] = a;
+        off[(3 * s + 1) * T + i] = a * ex[s * T + i];
+        off[(3 * s + 2) * T + i] = a * ey[s * T + i];
+    }
+}
+
+// What every kernel of the solve knows about its warp: the variable, the first
+// cell of the block, and whether the system still runs.
+struct Warp64 {
+    int lane, v, sys;
+    bool run;
+};
+
+__device__ __forceinline__ Warp64 warp64(const int32_t *__restrict__ blk_case, const int32_t *__restrict__ run,
+                                         int64_t cell0)
+{
+    Warp64 w;
+    w.lane = threadIdx.x & 31;
+    w.v = threadIdx.x >> 5;
+    w.sys = 4 * blk_case[cell0 / kBlock] + w.v;
+    w.run = !run || run[w.sys] != 0;
+    return w;
+}
+
+// Forward relation z_i = P_i (r_i + sum_{k<i} O_ik zin_k).  NB 0: no neighbours
+// (z = P r); 1: zin as given; 2: zin_k = P_k r_k formed here (the first sweep).
+// FULL: all five rows of z, else the rows 0 and 1 that the next sweep reads.
+template <int NB, bool FULL>
+__global__ void __launch_bounds__(kW64) k64_fwd(int64_t T, const int32_t *__restrict__ nb,
+                                                const double *__restrict__ P, const double *__restrict__ off,
+                                                const int32_t *__restrict__ blk_case, const int32_t *__restrict__ run,
+                                                const double *__restrict__ r, const double *__restrict__ zin,
+                                                double *__restrict__ zout)
+{
+    const int64_t c0 = blockIdx.x * (int64_t)32;
+    const Warp64 w = warp64(blk_case, run, c0);
+    const int64_t i = c0 + w.lane;
+    if (!w.run || i >= T) return;
+    const double *rv = r + (int64_t)w.v * 5 * T;
+    constexpr int NR = FULL ? 5 : 2;
+    double y[5], Pm[NR * 5];
+#pragma unroll
+    for (int k = 0; k < 5; ++k) y[k] = rv[k * T + i];
+#pragma unroll
+    for (int k = 0; k < NR * 5; ++k) Pm[k] = P[k * T + i];
+    if (NB) {
+        int js[3], ss[3];
+        const int n = side_slots<false>(nb, T, i, js, ss);
+        // the loads of all neighbours first, then the sums
+        Off64 o[3];
+        double z[3][2], rj[NB == 2 ? 3 : 1][5], pj[NB == 2 ? 3 : 1][10];
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+            if (q < n) {
+                const int64_t j = js[q];
+                o[q] = off_load(off, T, ss[q], i);
+                if (NB == 2) {
+#pragma unroll
+                    for (int k = 0; k < 5; ++k) rj[q][k] = rv[k * T + j];
+#pragma unroll
+                    for (int k = 0; k < 10; ++k) pj[q][k] = P[k * T + j];
+                } else {
+#pragma unroll
+                    for (int a = 0; a < 2; ++a) z[q][a] = zin[(w.v * 5 + a) * T + j];
+                }
+            }
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+            if (q < n) {
+                if (NB == 2)
+#pragma unroll
+                    for (int a = 0; a < 2; ++a) {
+                        double t = 0.0;
+#pragma unroll
+                        for (int c = 0; c < 5; ++c) t = fma(pj[q][a * 5 + c], rj[q][c], t);
+                        z[q][a] = t;
+                    }
+                off_acc(o[q].a, o[q].ax, o[q].ay, z[q][0], z[q][1], y);
+            }
+    }
+#pragma unroll
+    for (int a = 0; a < NR; ++a) {
+        double s = 0.0;
+#pragma unroll
+        for (int c = 0; c < 5; ++c) s = fma(Pm[a * 5 + c], y[c], s);
+        zout[(w.v * 5 + a) * T + i] = s;
+    }
+}
+
+// Backward relation x_i = z_i + P_i sum_{j>i} O_ij xin_j (rows 0 and 1 alone
+// unless FULL)
+template <bool FULL>
+__global__ void __launch_bounds__(kW64) k64_bwd(int64_t T, const int32_t *__restrict__ nb,
+                                                const double *__restrict__ P, const double *__restrict__ off,
+                                                const int32_t *__restrict__ blk_case, const int32_t *__restrict__ run,
+                                                const double *__restrict__ z, const double *__restrict__ xin,
+                                                double *__restrict__ xout)
+{
+    const int64_t c0 = blockIdx.x * (int64_t)32;
+    const Warp64 w = warp64(blk_case, run, c0);
+    const int64_t i = c0 + w.lane;
+    if (!w.run || i >= T) return;
+    constexpr int NR = FULL ? 5 : 2;
+    double y[5] = {0.0, 0.0, 0.0, 0.0, 0.0}, zi[NR], Pm[NR * 5];
+#pragma unroll
+    for (int k = 0; k < NR; ++k) zi[k] = z[(w.v * 5 + k) * T + i];
+#pragma unroll
+    for (int k = 0; k < NR * 5; ++k) Pm[k] = P[k * T + i];
+    int js[3], ss[3];
+    const int n = side_slots<true>(nb, T, i, js, ss);
+    Off64 o[3];
+    double x[3][2];
+#pragma unroll
+    for (int q = 0; q < 3; ++q)
+        if (q < n) {
+            o[q] = off_load(off, T, ss[q], i);
+#pragma unroll
+            for (int a = 0; a < 2; ++a) x[q][a] = xin[(w.v * 5 + a) * T + js[q]];
+        }
+#pragma unroll
+    for (int q = 0; q < 3; ++q)
+        if (q < n) off_acc(o[q].a, o[q].ax, o[q].ay, x[q][0], x[q][1], y);
+#pragma unroll
+    for (int a = 0; a < NR; ++a) {
+        double s = zi[a];
+#pragma unroll
+        for (int c = 0; c < 5; ++c) s = fma(Pm[a * 5 + c], y[c], s);
+        xout[(w.v * 5 + a) * T + i] = s;
+    }
+}
+
+// acc = (K x)_i of variable v: diagonal block minus the off-diagonal ones
+__device__ __forceinline__ void apply64(int64_t T, const int32_t *__restrict__ nb, const double *__restrict__ D,
+                                        const double *__restrict__ off, const double *__restrict__ xv, int64_t i,
+                                        double *acc)
+{
+    int j[3];
+    Off64 o[3];
+    double g[3][2], Dm[15], x[5];
+#pragma unroll
+    for (int s = 0; s < 3; ++s) j[s] = nb[s * T + i];
+#pragma unroll
+    for (int l = 0; l < 5; ++l) x[l] = xv[l * T + i];
+#pragma unroll
+    for (int q = 0; q < 15; ++q) Dm[q] = D[q * T + i];
+#pragma unroll
+    for (int s = 0; s < 3; ++s) {
+        // a missing neighbour has a zero block; it reads the cell's own values
+        const int64_t n = j[s] >= 0 ? j[s] : i;
+        o[s] = off_load(off, T, s, i);
+        g[s][0] = -xv[n];
+        g[s][1] = -xv[T + n];
+    }
+    constexpr int kIdx[5][5] = {{0, 1, 2, 3, 4}, {1, 5, 6, 7, 8}, {2, 6, 9, 10, 11}, {3, 7, 10, 12, 13},
+                                {4, 8, 11, 13, 14}};
+#pragma unroll
+    for (int a = 0; a < 5; ++a) {
+        acc[a] = Dm[kIdx[a][0]] * x[0];
+#pragma unroll
+        for (int c = 1; c < 5; ++c) acc[a] = fma(Dm[kIdx[a][c]], x[c], acc[a]);
+    }
+#pragma unroll
+    for (int s = 0; s < 3; ++s) off_acc(o[s].a, o[s].ax, o[s].ay, g[s][0], g[s][1], acc);
+}
+
+// Sums over the lanes of a warp of the rows acc[k][lane] (k < K, row stride 33),
+// written to out[k]: each row is split among 32 / (rows per pass) lanes, which
+// add its entries in order and then each other's sums.
+constexpr int kAccStride = 33;
+
+__device__ __forceinline__ void warp_rows(const double *acc, int K, int lane, double *__restrict__ out)
+{
+    const int g = K <= 4 ? 8 : (K <= 8 ? 4 : (K <= 16 ? 2 : 1));
+    const int sub = lane % g;
+    for (int k0 = 0; k0 < K; k0 += 32 / g) {
+        const int k = k0 + lane / g;
+        double s = 0.0;
+        if (k < K)
+            for (int t = sub; t < 32; t += g) s += acc[k * kAccStride + t];
+        for (int o = g >> 1; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (sub == 0 && k < K) out[k] = s;
+    }
+}
+
+// One value per lane summed over the warp (lane 0 gets it)
+__device__ __forceinline__ double warp_sum(double s)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    return s;
+}
+
+// y = K z and the products <V_k, y>, k <= j, of the first Gram-Schmidt pass:
+// part[row][v][k] over the 32 C cells of the block.  Dynamic shared memory:
+// 4 (j + 1) kAccStride doubles.
+template <int C>
+__global__ void __launch_bounds__(kW64) k64_apply_dots(int64_t T, const int32_t *__restrict__ nb,
+                                                       const double *__restrict__ D, const double *__restrict__ off,
+                                                       const int32_t *__restrict__ blk_case,
+                                                       const int32_t *__restrict__ run, const double *__restrict__ z,
+                                                       double *__restrict__ y, const double *__restrict__ V, int j,
+                                                       double *__restrict__ part, int ps)
+{
+    extern __shared__ double sh64[];
+    const int64_t c0 = blockIdx.x * (int64_t)(32 * C);
+    const Warp64 w = warp64(blk_case, run, c0);
+    if (!w.run) return;
+    const int K = j + 1;
+    double *acc = sh64 + w.v * K * kAccStride;
+    for (int k = 0; k < K; ++k) acc[k * kAccStride + w.lane] = 0.0;
+    const int64_t vo = (int64_t)w.v * 5 * T, vs = 20 * T;
+    for (int c = 0; c < C; ++c) {
+        const int64_t i = c0 + 32 * c + w.lane;
+        if (i >= T) break;
+        double u[5];
+        apply64(T, nb, D, off, z + vo, i, u);
+#pragma unroll
+        for (int l = 0; l < 5; ++l) y[vo + l * T + i] = u[l];
+#pragma unroll 4
+        for (int k = 0; k < K; ++k) {
+            const double *vk = V + k * vs + vo + i;
+            double s = acc[k * kAccStride + w.lane];
+#pragma unroll
+            for (int l = 0; l < 5; ++l) s = fma(vk[l * T], u[l], s);
+            acc[k * kAccStride + w.lane] = s;
+        }
+    }
+    __syncwarp();
+    warp_rows(acc, K, w.lane, part + ((int64_t)blockIdx.x * 4 + w.v) * ps);
+}
+
+// w -= sum_k h_k V_k, then the products <V_k, w> of the second pass
+template <int C>
+__global__ void __launch_bounds__(kW64) k64_update_dots(int64_t T, const int32_t *__restrict__ blk_case,
+                                                        const int32_t *__restrict__ run,
+                                                        const double *__restrict__ V, double *__restrict__ wn, int j,
+                                                        const double *__restrict__ hc, int hstride,
+                                                        double *__restrict__ part, int ps)
+{
+    extern __shared__ double sh64[];
+    const int64_t c0 = blockIdx.x * (int64_t)(32 * C);
+    const Warp64 w = warp64(blk_case, run, c0);
+    if (!w.run) return;
+    const int K = j + 1;
+    double *acc = sh64 + w.v * K * (kAccStride + 1), *h = acc + K * kAccStride;
+    for (int k = w.lane; k < K; k += 32) h[k] = hc[w.sys * hstride + k];
+    for (int k = 0; k < K; ++k) acc[k * kAccStride + w.lane] = 0.0;
+    __syncwarp();
+    const int64_t vo = (int64_t)w.v * 5 * T, vs = 20 * T;
+    for (int c = 0; c < C; ++c) {
+        const int64_t i = c0 + 32 * c + w.lane;
+        if (i >= T) break;
+        double u[5];
+#pragma unroll
+        for (int l = 0; l < 5; ++l) u[l] = wn[vo + l * T + i];
+#pragma unroll 4
+        for (int k = 0; k < K; ++k) {
+            const double *vk = V + k * vs + vo + i;
+            const double hk = -h[k];
+#pragma unroll
+            for (int l = 0; l < 5; ++l) u[l] = fma(hk, vk[l * T], u[l]);
+        }
+#pragma unroll
+        for (int l = 0; l < 5; ++l) wn[vo + l * T + i] = u[l];
+#pragma unroll 4
+        for (int k = 0; k < K; ++k) {
+            const double *vk = V + k * vs + vo + i;
+            double s = acc[k * kAccStride + w.lane];
+#pragma unroll
+            for (int l = 0; l < 5; ++l) s = fma(vk[l * T], u[l], s);
+            acc[k * kAccStride + w.lane] = s;
+        }
+    }
+    __syncwarp();
+    warp_rows(acc, K, w.lane, part + ((int64_t)blockIdx.x * 4 + w.v) * ps);
+}
+
+// w -= sum_k h_k V_k and the partial |w|^2
+template <int C>
+__global__ void __launch_bounds__(kW64) k64_update_norm(int64_t T, const int32_t *__restrict__ blk_case,
+                                                        const int32_t *__restrict__ run,
+                                                        const double *__restrict__ V, double *__restrict__ wn, int j,
+                                                        const double *__restrict__ hc, int hstride,
+                                                        double *__restrict__ part, int ps)
+{
+    __shared__ double hs[4][kMaxRestart];
+    const int64_t c0 = blockIdx.x * (int64_t)(32 * C);
+    const Warp64 w = warp64(blk_case, run, c0);
+    if (!w.run) return;
+    const int K = j + 1;
+    for (int k = w.lane; k < K; k += 32) hs[w.v][k] = hc[w.sys * hstride + k];
+    __syncwarp();
+    const int64_t vo = (int64_t)w.v * 5 * T, vs = 20 * T;
+    double nr = 0.0;
+    for (int c = 0; c < C; ++c) {
+        const int64_t i = c0 + 32 * c + w.lane;
+        if (i >= T) break;
+        double u[5];
+#pragma unroll
+        for (int l = 0; l < 5; ++l) u[l] = wn[vo + l * T + i];
+#pragma unroll 4
+        for (int k = 0; k < K; ++k) {
+            const double *vk = V + k * vs + vo + i;
+            const double hk = -hs[w.v][k];
+#pragma unroll
+            for (int l = 0; l < 5; ++l) u[l] = fma(hk, vk[l * T], u[l]);
+        }
+#pragma unroll
+        for (int l = 0; l < 5; ++l) {
+            wn[vo + l * T + i] = u[l];
+            nr = fma(u[l], u[l], nr);
+        }
+    }
+    nr = warp_sum(nr);
+    if (w.lane == 0) part[((int64_t)blockIdx.x * 4 + w.v) * ps] = nr;
+}
+
+// Right-hand side b_i = sum_j a0_ij (w_j - w_i) and the partial |b|^2 (entry 1)
+template <int C>
+__global__ void __launch_bounds__(kW64) k64_rhs(int64_t T, const int32_t *__restrict__ nb,
+                                                const double *__restrict__ a0, const double *__restrict__ wst,
+                                                double *__restrict__ b, double *__restrict__ part, int ps)
+{
+    const int64_t c0 = blockIdx.x * (int64_t)(32 * C);
+    const int lane = threadIdx.x & 31, v = threadIdx.x >> 5;
+    const int64_t vo = (int64_t)v * 5 * T;
+    const double *wv = wst + v * T;
+    double nr = 0.0;
+    for (int c = 0; c < C; ++c) {
+        const int64_t i = c0 + 32 * c + lane;
+        if (i >= T) break;
+        const double wi = wv[i];
+        double du[3], a[3][5], s[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            const int j = nb[q * T + i];
+            du[q] = wv[j >= 0 ? j : i] - wi;       // no neighbour: 0
+#pragma unroll
+            for (int l = 0; l < 5; ++l) a[q][l] = a0[(q * 5 + l) * T + i];
+        }
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+#pragma unroll
+            for (int l = 0; l < 5; ++l) s[l] = fma(a[q][l], du[q], s[l]);
+#pragma unroll
+        for (int l = 0; l < 5; ++l) {
+            b[vo + l * T + i] = s[l];
+            nr = fma(s[l], s[l], nr);
+        }
+    }
+    nr = warp_sum(nr);
+    if (lane == 0) part[((int64_t)blockIdx.x * 4 + v) * ps + 1] = nr;
+}
+
+// Residual y = b - K x and the partial |y|^2 (entry 0)
+template <int C>
+__global__ void __launch_bounds__(kW64) k64_resid(int64_t T, const int32_t *__restrict__ nb,
+                                                  const double *__restrict__ D, const double *__restrict__ off,
+                                                  const double *__restrict__ x, const double *__restrict__ b,
+                                                  double *__restrict__ y, double *__restrict__ part, int ps)
+{
+    const int64_t c0 = blockIdx.x * (int64_t)(32 * C);
+    const int lane = threadIdx.x & 31, v = threadIdx.x >> 5;
+    const int64_t vo = (int64_t)v * 5 * T;
+    double nr = 0.0;
+    for (int c = 0; c < C; ++c) {
+        const int64_t i = c0 + 32 * c + lane;
+        if (i >= T) break;
+        double u[5];
+        apply64(T, nb, D, off, x + vo, i, u);
+#pragma unroll
+        for (int l = 0; l < 5; ++l) {
+            const double rv = b[vo + l * T + i] - u[l];
+            y[vo + l * T + i] = rv;
+            nr = fma(rv, rv, nr);
+        }
+    }
+    nr = warp_sum(nr);
+    if (lane == 0) part[((int64_t)blockIdx.x * 4 + v) * ps] = nr;
+}
+
+// x += sum_{k<jv} y_k Z_k at the end of a cycle
+__global__ void __launch_bounds__(kW64) k64_combine(int64_t T, const int32_t *__restrict__ blk_case,
+                                                    const double *__restrict__ Z, const double *__restrict__ y,
+                                                    int m, const int32_t *__restrict__ jvs, double *__restrict__ x)
+{
+    const int64_t c0 = blockIdx.x * (int64_t)32;
+    const Warp64 w = warp64(blk_case, nullptr, c0);
+    const int64_t i = c0 + w.lane;
+    const int jv = jvs[w.sys];
+    if (jv <= 0 || i >= T) return;
+    const int64_t vo = (int64_t)w.v * 5 * T, vs = 20 * T;
+    double acc[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+#pragma unroll 4
+    for (int k = 0; k < jv; ++k) {
+        const double yk = y[w.sys * m + k];
+        const double *zk = Z + k * vs + vo + i;
+#pragma unroll
+        for (int l = 0; l < 5; ++l) acc[l] = fma(yk, zk[l * T], acc[l]);
+    }
+#pragma unroll
+    for (int l = 0; l < 5; ++l) x[vo + l * T + i] += acc[l];
+}
+
+}  // namespace
+}  // namespace gks
