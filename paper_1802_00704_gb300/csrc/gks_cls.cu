@@ -3,8 +3,8 @@
 //
 // Four independent systems (rho, rho u, rho v, E) share one operator; every
 // kernel handles one cell and all four variables, so each block of the
-// operator is read once per application.  Vectors are SoA [var][dof][cell] in
-// RCM order.  GMRES (Saad & Schultz 1986) is right-preconditioned, uses
+// operator is read once per application.  FP64 vectors are [var][dof][cell] in
+// RCM order, FP32 vectors [dof][cell][var] (vload, vstore).  GMRES (Saad & Schultz 1986) is right-preconditioned, uses
 // classical Gram-Schmidt (twice, CGS2, in FP64 mode), and keeps per-variable
 // state on the device (running/converged masks); reductions go through
 // per-block partial sums and a fixed-order second pass, so results are
@@ -18,7 +18,7 @@
 #include <type_traits>
 
 #include "gks_internal.h"
-#include "gks_solve64.cuh"
+#include "gks_solve32.cuh"
 #include "gks_wait.cuh"
 
 namespace gks {
@@ -61,6 +61,12 @@ __device__ __forceinline__ double pow2(int e)
 {
     e = e < -1022 ? -1022 : (e > 1023 ? 1023 : e);
     return __longlong_as_double((long long)(e + 1023) << 52);
+}
+
+// 2^k in FP32 for k <= 0; 0 below FP32's normal range
+__device__ __forceinline__ float pow2f(int k)
+{
+    return k >= -126 ? __uint_as_float((unsigned)(127 + k) << 23) : 0.0f;
 }
 
 // Block reduction of NV values; thread 0 of the block gets the totals.
@@ -155,22 +161,20 @@ __device__ __forceinline__ void cell_apply(const DeviceMesh &d, const TM *__rest
         sax[s] = sa[s] * exg[s * T + i];
         say[s] = sa[s] * eyg[s * T + i];
     }
-    TM g[3][2 * NV];
+    TM g[3][2][NV];
 #pragma unroll
     for (int s = 0; s < 3; ++s)
 #pragma unroll
-        for (int v = 0; v < NV; ++v) {
-            g[s][2 * v] = TM(x[(v * ND + 0) * T + jn[s]]);
-            g[s][2 * v + 1] = TM(x[(v * ND + 1) * T + jn[s]]);
-        }
+        for (int a = 0; a < 2; ++a) vload(x, a, T, jn[s], g[s][a]);
     TM Dm[15];
 #pragma unroll
     for (int q = 0; q < 15; ++q) Dm[q] = Dg[q * T + i];
+    TM xo[ND][NV];
+#pragma unroll
+    for (int l = 0; l < ND; ++l) vload(x, l, T, i, xo[l]);
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
-        TM xv[ND];
-#pragma unroll
-        for (int l = 0; l < ND; ++l) xv[l] = TM(x[(v * ND + l) * T + i]);
+        const TM xv[ND] = {xo[0][v], xo[1][v], xo[2][v], xo[3][v], xo[4][v]};
         // symmetric 5x5 times vector
         acc[v * ND + 0] = Dm[0] * xv[0] + Dm[1] * xv[1] + Dm[2] * xv[2] + Dm[3] * xv[3] + Dm[4] * xv[4];
         acc[v * ND + 1] = Dm[1] * xv[0] + Dm[5] * xv[1] + Dm[6] * xv[2] + Dm[7] * xv[3] + Dm[8] * xv[4];
@@ -181,7 +185,7 @@ __device__ __forceinline__ void cell_apply(const DeviceMesh &d, const TM *__rest
 #pragma unroll
     for (int s = 0; s < 3; ++s)
 #pragma unroll
-        for (int v = 0; v < NV; ++v) oacc(sa[s], sax[s], say[s], g[s][2 * v], g[s][2 * v + 1], acc + v * ND);
+        for (int v = 0; v < NV; ++v) oacc(sa[s], sax[s], say[s], g[s][0][v], g[s][1][v], acc + v * ND);
     if (G) {
 #pragma unroll
         for (int s = 0; s < 3; ++s) {
@@ -189,11 +193,12 @@ __device__ __forceinline__ void cell_apply(const DeviceMesh &d, const TM *__rest
             const TM sr = has ? -arg[s * T + i] : TM(0);
             const TM srx = sr * exrg[s * T + i], sry = sr * eyrg[s * T + i];
             const TM sb = has ? -bdgg[s * T + i] : TM(0);
+            TM xn[ND][NV];
+#pragma unroll
+            for (int l = 0; l < ND; ++l) vload(x, l, T, jn[s], xn[l]);
 #pragma unroll
             for (int v = 0; v < NV; ++v) {
-                TM xj[ND];
-#pragma unroll
-                for (int l = 0; l < ND; ++l) xj[l] = TM(x[(v * ND + l) * T + jn[s]]);
+                const TM xj[ND] = {xn[0][v], xn[1][v], xn[2][v], xn[3][v], xn[4][v]};
                 racc(sr, srx, sry, xj, acc + v * ND);
 #pragma unroll
                 for (int l = 2; l < ND; ++l) acc[v * ND + l] = fma(sb, xj[l], acc[v * ND + l]);
@@ -225,19 +230,25 @@ __global__ void k_spmv(DeviceMesh d, const TM *__restrict__ Dg, const TM *__rest
         cell_apply<TX, TM, G>(d, Dg, alg, exg, eyg, x, i, acc, arg, exrg, eyrg, bdgg);
         if (mode == 0) {
 #pragma unroll
-            for (int q = 0; q < NX; ++q) y[q * T + i] = TY(acc[q]);
+            for (int l = 0; l < ND; ++l) {
+                const TY o[NV] = {TY(acc[l]), TY(acc[ND + l]), TY(acc[2 * ND + l]), TY(acc[3 * ND + l])};
+                vstore(y, l, T, i, o);
+            }
         } else {
             const int c = d.blk_case[blockIdx.x];
+            double sig[NV];
 #pragma unroll
-            for (int v = 0; v < NV; ++v) {
-                const double sig = sexp ? pow2(-sexp[4 * c + v]) : 1.0;
+            for (int v = 0; v < NV; ++v) sig[v] = sexp ? pow2(-sexp[4 * c + v]) : 1.0;
 #pragma unroll
-                for (int l = 0; l < ND; ++l) {
+            for (int l = 0; l < ND; ++l) {
+                TY o[NV];
+#pragma unroll
+                for (int v = 0; v < NV; ++v) {
                     const double rv = b[(v * ND + l) * T + i] - double(acc[v * ND + l]);
-                    const TY st = TY(rv * sig);
-                    y[(v * ND + l) * T + i] = st;
-                    nr[v] += double(st) * double(st);
+                    o[v] = TY(rv * sig[v]);
+                    nr[v] += double(o[v]) * double(o[v]);
                 }
+                vstore(y, l, T, i, o);
             }
         }
     }
@@ -245,96 +256,6 @@ __global__ void k_spmv(DeviceMesh d, const TM *__restrict__ Dg, const TM *__rest
         block_sum4(nr, sh);
         if (threadIdx.x == 0)
             for (int v = 0; v < NV; ++v) part[(blockIdx.x * NV + v) * pstride + 0] = nr[v];
-    }
-}
-
-// y = K z with the first Gram-Schmidt pass fused in (the FP32-basis inner
-// cycles): each thread keeps its cell's y_i in registers and forms the
-// products with V_0..V_j at the same cell, so the new basis vector is not read
-// back from HBM by a separate dot-product kernel.  part[blk][v][k] =
-// sum over the block's cells of <V_k, y>_v: FP32 products and warp sums (as
-// k_dots), each warp's sums widened to FP64 and added across the block's warps
-// in order.  Deterministic; a different summation order than k_dots, so the
-// iterates agree with the unfused path to rounding.  J > 0: the Arnoldi index
-// j = J - 1 is a compile-time constant, the products with all J basis vectors
-// are formed before one block-wide pass sums them (one barrier instead of two
-// per vector); the same operations in the same order as the loop over k.
-template <int J = 0>
-__global__ void __launch_bounds__(kBlock, 3)
-    k_spmv_dots(DeviceMesh d, const float *__restrict__ Dg, const float *__restrict__ alg,
-                const float *__restrict__ exg, const float *__restrict__ eyg, const float *__restrict__ x,
-                float *__restrict__ y, const float *__restrict__ V, int j, double *__restrict__ part, int pstride)
-{
-    __shared__ float sh[kBlock / 32][J > 0 ? J : 1][NV];
-    const int64_t T = d.T;
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    float acc[NX];
-#pragma unroll
-    for (int q = 0; q < NX; ++q) acc[q] = 0.0f;
-    if (i < T) {
-        cell_apply<float, float, false>(d, Dg, alg, exg, eyg, x, i, acc);
-#pragma unroll
-        for (int q = 0; q < NX; ++q) y[q * T + i] = acc[q];
-    }
-    const int64_t vs = (int64_t)NX * T;
-    if constexpr (J > 0) {
-        float sv[J][NV];
-#pragma unroll
-        for (int k = 0; k < J; ++k)
-#pragma unroll
-            for (int v = 0; v < NV; ++v) sv[k][v] = 0.0f;
-        if (i < T) {
-#pragma unroll
-            for (int k = 0; k < J; ++k) {
-                const float *vk = V + k * vs;
-#pragma unroll
-                for (int v = 0; v < NV; ++v)
-#pragma unroll
-                    for (int l = 0; l < ND; ++l) sv[k][v] = fmaf(vk[(v * ND + l) * T + i], acc[v * ND + l], sv[k][v]);
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < J; ++k)
-#pragma unroll
-            for (int v = 0; v < NV; ++v)
-                for (int o = 16; o > 0; o >>= 1) sv[k][v] += __shfl_down_sync(0xffffffffu, sv[k][v], o);
-        if (lane == 0)
-#pragma unroll
-            for (int k = 0; k < J; ++k)
-#pragma unroll
-                for (int v = 0; v < NV; ++v) sh[warp][k][v] = sv[k][v];
-        __syncthreads();
-        if (threadIdx.x < J * NV) {
-            const int k = threadIdx.x / NV, v = threadIdx.x % NV;
-            double t = 0.0;
-            for (int w = 0; w < kBlock / 32; ++w) t += double(sh[w][k][v]);
-            part[(blockIdx.x * NV + v) * pstride + k] = t;
-        }
-    } else {
-        for (int k = 0; k <= j; ++k) {
-            float sv[NV] = {0.0f, 0.0f, 0.0f, 0.0f};
-            if (i < T) {
-                const float *vk = V + k * vs;
-#pragma unroll
-                for (int v = 0; v < NV; ++v)
-#pragma unroll
-                    for (int l = 0; l < ND; ++l) sv[v] = fmaf(vk[(v * ND + l) * T + i], acc[v * ND + l], sv[v]);
-            }
-#pragma unroll
-            for (int v = 0; v < NV; ++v)
-                for (int o = 16; o > 0; o >>= 1) sv[v] += __shfl_down_sync(0xffffffffu, sv[v], o);
-            if (lane == 0)
-#pragma unroll
-                for (int v = 0; v < NV; ++v) sh[warp][0][v] = sv[v];
-            __syncthreads();
-            if (threadIdx.x < NV) {
-                double t = 0.0;
-                for (int w = 0; w < kBlock / 32; ++w) t += double(sh[w][0][threadIdx.x]);
-                part[(blockIdx.x * NV + threadIdx.x) * pstride + k] = t;
-            }
-            __syncthreads();
-        }
     }
 }
 
@@ -405,36 +326,65 @@ __device__ __noinline__ void resid64_cell(const DeviceMesh &d, const double *__r
     for (int l = 0; l < ND; ++l) out[l] = float((b[(v * ND + l) * d.T + i] - acc[v * ND + l]) * pow2(-e));
 }
 
-// V_0 = 2^-e (b - K x) in FP32 and partial |V_0|^2 (as k_spmv mode 1 with an
-// FP32 basis), in double-FP32 arithmetic: the operator as FP32 pairs D2 ([30][T]:
-// the 15 diagonal-block values, then their low parts) and S2 ([18][T]: sa,
-// sa dx, sa dy of each neighbour, then their low parts), 2^-e x and 2^-e b
-// split on the fly, so the sums come out scaled.  One thread per cell and
-// variable (the double-FP32 chains are latency-bound: many small threads hide
-// it better than one thread per cell); block q of the 1-D grid takes variable
-// q % 4 of cell block q / 4, so the four blocks of a cell block run together
-// and share the operator through L2.  A value outside the split range sends
-// the thread to the FP64 operator.  Each thread's five squares are summed in
-// FP32 (the scaled vector is near unit size).  G: global normal equations, the
-// transpose form from the reverse-slot pairs SR2 ([18][T], as S2) on all five
-// unknowns of each neighbour.
-template <bool G>
-__global__ void __launch_bounds__(kBlock, 4) k_resid_df(DeviceMesh d, const float *__restrict__ D2,
-                                                       const float *__restrict__ S2, const double *__restrict__ x,
-                                                       float *__restrict__ y, const double *__restrict__ b,
-                                                       double *__restrict__ part, int pstride,
-                                                       const int32_t *__restrict__ sexp,
-                                                       const float *__restrict__ SR2 = nullptr,
-                                                       const float *__restrict__ SB2 = nullptr)
+constexpr int kResidRows = NV;          // blocks (partial-sum rows) of the residual per cell block
+
+// (h, l) of every lane summed over the warp (lane 0 gets the pair)
+__device__ __forceinline__ void df_warp_sum(float &h, float &l)
 {
-    __shared__ double sh[kBlock / 32];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+        df_add(__shfl_down_sync(0xffffffffu, h, o), __shfl_down_sync(0xffffffffu, l, o), h, l);
+}
+
+// four floats of chunk q of cell i
+__device__ __forceinline__ void load4(const float4 *__restrict__ p, int q, int64_t T, int64_t i, float *o)
+{
+    const float4 t = p[q * T + i];
+    o[0] = t.x;
+    o[1] = t.y;
+    o[2] = t.z;
+    o[3] = t.w;
+}
+
+// V_0 = 2^-e (b - K x) in FP32 and partial |V_0|^2 (as k_spmv mode 1 with an
+// FP32 basis), in double-FP32 arithmetic: the operator as FP32 pairs D2
+// ([12][T][4]: the 15 diagonal-block values and their low parts, sa, sa dx, sa dy
+// of each neighbour and their low parts), 2^-e x and 2^-e b split on the fly, so
+// the sums come out scaled.  One thread per cell and
+// variable (the double-FP32 chains are latency-bound: many small threads hide
+// it better than one thread per cell), the four variables of a cell in
+// neighbouring lanes: one load serves the operator of eight cells for all four,
+// and V_0 is written in whole lines.  (With the variables in different blocks
+// of 256 cells the operator came from L2 four times; in different warps of a
+// block it was no faster.)  A value outside the split range sends
+// the thread to the FP64 operator.  Each thread's five squares are summed in
+// FP32 (the scaled vector is near unit size), the threads' sums to 48 bits.
+// act (NULL on a solve's first residual): a case without an active system keeps
+// its V_0 and norms.  G: global normal equations, the
+// transpose form from the reverse-slot pairs SR2 ([6][T][4]: 9 values and their
+// low parts, then -beta per slot and its low parts) on all five unknowns of each
+// neighbour.
+template <bool G>
+__global__ void __launch_bounds__(kBlock, 4) k_resid_df(const __grid_constant__ DeviceMesh d,
+                                                        const float4 *__restrict__ D2,
+                                                        const double *__restrict__ x, float *__restrict__ y,
+                                                        const double *__restrict__ b, double *__restrict__ part,
+                                                        int pstride, const int32_t *__restrict__ sexp,
+                                                        const int32_t *__restrict__ act,
+                                                        const float4 *__restrict__ SR2 = nullptr)
+{
+    __shared__ float2 sh[kBlock / 32][NV];
     const int64_t T = d.T;
-    const int v = blockIdx.x & 3;
-    const int64_t blk = blockIdx.x >> 2;
-    const int64_t i = blk * kBlock + threadIdx.x;
-    double nr = 0.0;
+    const int cs = d.blk_case[blockIdx.x / kResidRows];
+    if (act) {
+        const int4 r = reinterpret_cast<const int4 *>(act)[cs];
+        if ((r.x | r.y | r.z | r.w) == 0) return;
+    }
+    const int v = threadIdx.x & 3;
+    const int64_t i = blockIdx.x * (int64_t)(kBlock / NV) + (threadIdx.x >> 2);
+    float nh = 0.0f, nl = 0.0f;
     if (i < T) {
-        const int e = sexp[4 * d.blk_case[blk] + v];
+        const int e = sexp[4 * cs + v];
         int64_t jn[3];
 #pragma unroll
         for (int s = 0; s < 3; ++s) {
@@ -446,11 +396,11 @@ __global__ void __launch_bounds__(kBlock, 4) k_resid_df(DeviceMesh d, const floa
         // in the same order
         constexpr int NG = G ? ND : 2;                    // neighbour unknowns used
         double xv[ND], gv[3][NG], bv[ND];
-        float dp[30], op[18], rp[G ? 18 : 1], bp[G ? 6 : 1];
+        float dp[48], rp[G ? 24 : 1];
 #pragma unroll
         for (int l = 0; l < ND; ++l) xv[l] = x[(v * ND + l) * T + i];
 #pragma unroll
-        for (int q = 0; q < 30; ++q) dp[q] = D2[q * T + i];
+        for (int q = 0; q < 8; ++q) load4(D2, q, T, i, dp + 4 * q);
         bool ok = true;
         float xh[ND], xl[ND], gh[3][NG], gl[3][NG], ah[ND], al[ND], out[ND];
 #pragma unroll
@@ -470,13 +420,11 @@ __global__ void __launch_bounds__(kBlock, 4) k_resid_df(DeviceMesh d, const floa
 #pragma unroll
             for (int l = 0; l < NG; ++l) gv[s][l] = x[(v * ND + l) * T + jn[s]];
 #pragma unroll
-        for (int q = 0; q < 18; ++q) op[q] = S2[q * T + i];
-        if (G) {
+        for (int q = 8; q < 12; ++q) load4(D2, q, T, i, dp + 4 * q);
+        const float *op = dp + 30, *bp = rp + (G ? 18 : 0);
+        if (G)
 #pragma unroll
-            for (int q = 0; q < 18; ++q) rp[q] = SR2[q * T + i];
-#pragma unroll
-            for (int q = 0; q < 6; ++q) bp[q] = SB2[q * T + i];
-        }
+            for (int q = 0; q < 6; ++q) load4(SR2, q, T, i, rp + 4 * q);
 #pragma unroll
         for (int l = 0; l < ND; ++l) bv[l] = b[(v * ND + l) * T + i];
 #pragma unroll
@@ -517,18 +465,19 @@ __global__ void __launch_bounds__(kBlock, 4) k_resid_df(DeviceMesh d, const floa
         float sq = 0.0f;
 #pragma unroll
         for (int l = 0; l < ND; ++l) {
-            y[(v * ND + l) * T + i] = out[l];
+            y[(l * T + i) * NV + v] = out[l];
             sq = __fmaf_rn(out[l], out[l], sq);
         }
-        nr = double(sq);
+        nh = sq;
     }
-    for (int o = 16; o > 0; o >>= 1) nr += __shfl_down_sync(0xffffffffu, nr, o);
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = nr;
+    // over the warp's eight cells, then the warps
+#pragma unroll
+    for (int o = 16; o >= NV; o >>= 1) df_add(__shfl_down_sync(0xffffffffu, nh, o), __shfl_down_sync(0xffffffffu, nl, o), nh, nl);
+    if ((threadIdx.x & 31) < NV) sh[threadIdx.x >> 5][threadIdx.x & 31] = make_float2(nh, nl);
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int w = 0; w < kBlock / 32; ++w) t += sh[w];
-        part[(blk * NV + v) * pstride + 0] = t;
+    if (threadIdx.x < NV) {
+        for (int w = 1; w < kBlock / 32; ++w) df_add(sh[w][threadIdx.x].x, sh[w][threadIdx.x].y, nh, nl);
+        part[((int64_t)blockIdx.x * NV + threadIdx.x) * pstride] = double(nh) + double(nl);
     }
 }
 
@@ -547,30 +496,36 @@ __device__ __forceinline__ double f2d_pow2(float f, int e)
 }
 
 // The right-hand side of k_rhs in double-FP32 arithmetic (the FP32-basis
-// solve).  GB300's FP64 pipe made the FP64 kernel (92 FP64 operations per
-// cell) its bottleneck; here a cell and variable take the power of two 2^e of
-// their largest difference w_j - w_i (formed in FP64), split the scaled
-// differences on the integer pipe, multiply them exactly by the weights as FP32
-// pairs a0p ([30][T]: the 15 high parts, then the low parts) and sum with
-// compensation (df_mac); the normalised pair (high + low, 48 bits) is widened
-// on the integer pipe and added in FP64: 32 FP64 operations per cell, b to
-// about 2^-48 relative at any magnitude.  A difference that does not split
-// (not finite) sends the cell to FP64.  part[blk][v][1] gets the block's |b|^2:
-// the scaled high parts squared in FP32, rescaled to the warp's largest 2^e,
-// summed in FP32 within the warp and in FP64 across warps.
-__global__ void __launch_bounds__(kBlock, 3) k_rhs_df(DeviceMesh d, const float *__restrict__ a0p,
-                                                      const double *__restrict__ w, double *__restrict__ b,
-                                                      double *__restrict__ part, int pstride)
+// solve), one thread per cell and variable.  GB300's FP64 pipe made the FP64
+// kernel (92 FP64 operations per cell) its bottleneck; here a cell and variable
+// take the power of two 2^e of their largest difference w_j - w_i (formed in
+// FP64), split the scaled differences on the integer pipe, multiply them exactly
+// by the weights as FP32 pairs a0p ([30][T]: the 15 high parts, then the low
+// parts) and sum with compensation (df_mac); the normalised pair (high + low, 48
+// bits) is widened on the integer pipe and added in FP64: 8 FP64 instructions
+// per cell and variable, b to about 2^-48 relative at any magnitude.  A
+// difference that does not split (not finite) sends the thread to FP64.
+// part[row][v][1] gets the |b|^2 of the block's 32 C cells: the scaled high
+// parts squared in FP32, the lanes' sums kept to 48 bits with a power of two of
+// their own, rescaled to the warp's largest at the end.  The four warps of a
+// block take the four variables of the same cells (the weights come from L1).
+template <int C>
+__global__ void __launch_bounds__(kW32) k_rhs_df(DeviceMesh d, const float *__restrict__ a0p,
+                                                 const double *__restrict__ w, double *__restrict__ b,
+                                                 double *__restrict__ part, int pstride)
 {
-    __shared__ double sh[(kBlock / 32) * NV];
-    const int64_t T = d.T;
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    float ss[NV] = {0.0f, 0.0f, 0.0f, 0.0f};      // scaled |b|^2 of this cell
-    int ev[NV] = {-1022, -1022, -1022, -1022};    // the scales 2^e
-    if (i < T) {
-        double wi[NV], du[3][NV];
+    const int64_t T = d.T, c0 = blockIdx.x * (int64_t)(32 * C);
+    const int lane = threadIdx.x & 31, v = threadIdx.x >> 5;
+    const double *wv = w + v * T;
+    float nh = 0.0f, nl = 0.0f;                   // 2^(-2 ne) |b|^2 of this lane
+    int ne = -1022;
+    for (int c = 0; c < C; ++c) {
+        const int64_t i = c0 + 32 * c + lane;
+        if (i >= T) break;
         int js[3];
-        // the cell's weights first: their loads overlap the neighbour gathers
+#pragma unroll
+        for (int s = 0; s < 3; ++s) js[s] = d.nb[s * T + i];
+        // the cell's weights: their loads overlap the neighbour gathers
         float ah[3][ND], al[3][ND];
 #pragma unroll
         for (int s = 0; s < 3; ++s)
@@ -579,94 +534,70 @@ __global__ void __launch_bounds__(kBlock, 3) k_rhs_df(DeviceMesh d, const float 
                 ah[s][l] = a0p[(s * ND + l) * T + i];
                 al[s][l] = a0p[(15 + s * ND + l) * T + i];
             }
-#pragma unroll
-        for (int v = 0; v < NV; ++v) wi[v] = w[v * T + i];
-#pragma unroll
-        for (int s = 0; s < 3; ++s) {
-            js[s] = d.nb[s * T + i];
-#pragma unroll
-            for (int v = 0; v < NV; ++v) du[s][v] = js[s] >= 0 ? w[v * T + js[s]] - wi[v] : 0.0;
-        }
-#pragma unroll
-        for (int v = 0; v < NV; ++v) {
-            int em = 1;
-#pragma unroll
-            for (int s = 0; s < 3; ++s) {
-                const int E = (int)(((unsigned)__double2hiint(du[s][v]) >> 20) & 0x7FFu);
-                em = E > em ? E : em;
-            }
-            ev[v] = (em == 2047 ? 1023 : em) - 1023;
-        }
-        // with 2^e the largest difference of its variable, a difference fails to
-        // split only when it is not finite: that sends the cell to FP64
+        const double wi = wv[i];
+        double du[3];
+        int em = 1;
         bool ok = true;
 #pragma unroll
-        for (int s = 0; s < 3; ++s)
-#pragma unroll
-            for (int v = 0; v < NV; ++v) ok &= isfinite(du[s][v]);
+        for (int s = 0; s < 3; ++s) {
+            du[s] = wv[js[s] >= 0 ? js[s] : i] - wi;       // no neighbour: 0
+            const int E = (int)(((unsigned)__double2hiint(du[s]) >> 20) & 0x7FFu);
+            em = E > em ? E : em;
+            ok &= E < 2047;
+        }
+        // with 2^e the largest difference, a difference fails to split only when
+        // it is not finite: that sends the thread to FP64
+        const int e = (em == 2047 ? 1023 : em) - 1023;
+        float ss = 0.0f;                                   // 2^(-2 e) |b|^2 of this cell
         if (ok) {
-            // one variable at a time (ten accumulators live, not forty); each sum
-            // runs over the neighbours in order, as the FP64 kernel's does
+            float sh_[ND], sl_[ND];
 #pragma unroll
-            for (int v = 0; v < NV; ++v) {
-                float sh_[ND], sl_[ND];
+            for (int l = 0; l < ND; ++l) sh_[l] = sl_[l] = 0.0f;
 #pragma unroll
-                for (int l = 0; l < ND; ++l) sh_[l] = sl_[l] = 0.0f;
+            for (int s = 0; s < 3; ++s) {
+                float dh, dl;
+                df_split(du[s], e, dh, dl);
 #pragma unroll
-                for (int s = 0; s < 3; ++s) {
-                    if (js[s] < 0) continue;
-                    float dh, dl;
-                    df_split(du[s][v], ev[v], dh, dl);
+                for (int l = 0; l < ND; ++l) df_mac(ah[s][l], al[s][l], dh, dl, sh_[l], sl_[l]);
+            }
 #pragma unroll
-                    for (int l = 0; l < ND; ++l) df_mac(ah[s][l], al[s][l], dh, dl, sh_[l], sl_[l]);
-                }
-#pragma unroll
-                for (int l = 0; l < ND; ++l) {
-                    // normalise (TwoSum): h + lo = sh + sl exactly
-                    const float h = __fadd_rn(sh_[l], sl_[l]);
-                    const float z = __fsub_rn(h, sh_[l]);
-                    const float lo = __fadd_rn(__fsub_rn(sh_[l], __fsub_rn(h, z)), __fsub_rn(sl_[l], z));
-                    b[(v * ND + l) * T + i] = f2d_pow2(h, ev[v]) + f2d_pow2(lo, ev[v]);
-                    ss[v] = __fmaf_rn(h, h, ss[v]);
-                }
+            for (int l = 0; l < ND; ++l) {
+                // normalise (TwoSum): h + lo = sh + sl exactly
+                const float h = __fadd_rn(sh_[l], sl_[l]);
+                const float z = __fsub_rn(h, sh_[l]);
+                const float lo = __fadd_rn(__fsub_rn(sh_[l], __fsub_rn(h, z)), __fsub_rn(sl_[l], z));
+                b[(v * ND + l) * T + i] = f2d_pow2(h, e) + f2d_pow2(lo, e);
+                ss = __fmaf_rn(h, h, ss);
             }
         } else {
             // FP64 as in k_rhs; the norm from the values scaled by 2^-e
-#pragma unroll
-            for (int v = 0; v < NV; ++v) {
-                double acc[ND] = {0.0, 0.0, 0.0, 0.0, 0.0};
-                for (int s = 0; s < 3; ++s) {
-                    if (js[s] < 0) continue;
-                    for (int l = 0; l < ND; ++l) acc[l] += d.a0[(s * ND + l) * T + i] * du[s][v];
-                }
-                for (int l = 0; l < ND; ++l) {
-                    b[(v * ND + l) * T + i] = acc[l];
-                    const float h = float(acc[l] * pow2(-ev[v]));
-                    ss[v] = __fmaf_rn(h, h, ss[v]);
-                }
+            double acc[ND] = {0.0, 0.0, 0.0, 0.0, 0.0};
+            for (int s = 0; s < 3; ++s) {
+                if (js[s] < 0) continue;
+                for (int l = 0; l < ND; ++l) acc[l] += d.a0[(s * ND + l) * T + i] * du[s];
+            }
+            for (int l = 0; l < ND; ++l) {
+                b[(v * ND + l) * T + i] = acc[l];
+                const float h = float(acc[l] * pow2(-e));
+                ss = __fmaf_rn(h, h, ss);
             }
         }
+        // to the larger of the two powers of two (terms below 2^-126 of it drop out)
+        const int m = max(e, ne);
+        const float f0 = pow2f(2 * (ne - m)), f1 = pow2f(2 * (e - m));
+        nh *= f0;
+        nl *= f0;
+        df_add(ss * f1, 0.0f, nh, nl);
+        ne = m;
     }
-    // |b|^2 = sum 2^(2e) ss: rescaled to the warp's largest e in FP32 (smaller
-    // terms that underflow are below 2^-126 of the largest), summed in FP32
-    // within the warp, widened once per warp and summed in FP64 across warps
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-        int em = ev[v];
-        for (int o = 16; o > 0; o >>= 1) em = max(em, __shfl_xor_sync(0xffffffffu, em, o));
-        const int k = 2 * (ev[v] - em);           // <= 0
-        float c = k >= -126 ? ss[v] * __uint_as_float((unsigned)(127 + k) << 23) : 0.0f;
-        for (int o = 16; o > 0; o >>= 1) c += __shfl_down_sync(0xffffffffu, c, o);
-        if (lane == 0) sh[warp * NV + v] = double(c) * pow2(em) * pow2(em);
-    }
-    __syncthreads();
-    if (threadIdx.x == 0)
-        for (int v = 0; v < NV; ++v) {
-            double t = 0.0;
-            for (int k = 0; k < kBlock / 32; ++k) t += sh[k * NV + v];
-            part[(blockIdx.x * NV + v) * pstride + 1] = t;
-        }
+    int m = ne;
+    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+    const float f = pow2f(2 * (ne - m));
+    nh *= f;
+    nl *= f;
+    df_warp_sum(nh, nl);
+    if (lane == 0)
+        part[((int64_t)blockIdx.x * NV + v) * pstride + 1] = (double(nh) + double(nl)) * pow2(m) * pow2(m);
 }
 
 // Forward block-ILU relation for the listed rows (or all rows when rows == nullptr):
@@ -683,15 +614,6 @@ __global__ void __launch_bounds__(kBlock, 3) k_rhs_df(DeviceMesh d, const float 
 // preconditioner), widened to TM on load.
 // G: global normal equations, the transpose form with the reverse-slot
 // coefficients arg, exrg, eyrg on all five unknowns of the neighbour.
-// a neighbour's value: through L2 in the sync-free solves (written by another
-// block of the same launch), a plain load otherwise
-template <bool SF, typename T>
-__device__ __forceinline__ T ldx(const T *p)
-{
-    if constexpr (SF) return __ldcg(p);
-    else return *p;
-}
-
 // A bounded wait of the sync-free solves gives up after 1 s (a correct solve
 // waits a few microseconds per level).
 constexpr uint64_t kWaitLimitNs = 1000000000ull;
@@ -711,13 +633,16 @@ __device__ __forceinline__ void ilu_fwd_row(const DeviceMesh &d, const TP *__res
     const int64_t T = d.T;
     TM y[NX];
 #pragma unroll
-    for (int k = 0; k < NX; ++k) y[k] = TM(r[k * T + i]);
+    for (int l = 0; l < ND; ++l) {
+        TM t[NV];
+        vload(r, l, T, i, t);
+        if (rcopy) vstore(rcopy, l, T, i, t);
+#pragma unroll
+        for (int v = 0; v < NV; ++v) y[v * ND + l] = t[v];
+    }
     TM Pm[25];
 #pragma unroll
     for (int k = 0; k < 25; ++k) Pm[k] = TM(Pg[k * T + i]);
-    if (rcopy)
-#pragma unroll
-        for (int k = 0; k < NX; ++k) rcopy[k * T + i] = TZ(y[k]);
     if (SF) {
         // every lower neighbour's tag first (one round trip for all of them)
         const int32_t *wf[3];
@@ -742,9 +667,9 @@ __device__ __forceinline__ void ilu_fwd_row(const DeviceMesh &d, const TP *__res
             const TM sa = TM(alg[s * T + i]), sax = sa * TM(exg[s * T + i]), say = sa * TM(eyg[s * T + i]);
             TM zn[NV][NA];
             if (use_nb == 2) {
-                TM rj[NX];
+                TM rj[ND][NV];
 #pragma unroll
-                for (int k = 0; k < NX; ++k) rj[k] = TM(r[k * T + j]);
+                for (int l = 0; l < ND; ++l) vload(r, l, T, j, rj[l]);
 #pragma unroll
                 for (int a = 0; a < NA; ++a) {
                     TM pa[ND];
@@ -754,20 +679,19 @@ __device__ __forceinline__ void ilu_fwd_row(const DeviceMesh &d, const TP *__res
                     for (int v = 0; v < NV; ++v) {
                         TM t = TM(0);
 #pragma unroll
-                        for (int c = 0; c < ND; ++c) t = fma(pa[c], rj[v * ND + c], t);
+                        for (int c = 0; c < ND; ++c) t = fma(pa[c], rj[c][v], t);
                         zn[v][a] = TM(TZ(t));
                     }
                 }
-            } else if (SF) {
-#pragma unroll
-                for (int v = 0; v < NV; ++v)
-#pragma unroll
-                    for (int a = 0; a < NA; ++a) zn[v][a] = TM(__ldcg(zin + (v * ND + a) * T + j));
             } else {
 #pragma unroll
-                for (int v = 0; v < NV; ++v)
+                for (int a = 0; a < NA; ++a) {
+                    TM t[NV];
+                    if constexpr (SF) vload_cg(zin, a, T, j, t);
+                    else vload(zin, a, T, j, t);
 #pragma unroll
-                    for (int a = 0; a < NA; ++a) zn[v][a] = TM(zin[(v * ND + a) * T + j]);
+                    for (int v = 0; v < NV; ++v) zn[v][a] = t[v];
+                }
             }
             if (!lower) continue;
 #pragma unroll
@@ -785,14 +709,16 @@ __device__ __forceinline__ void ilu_fwd_row(const DeviceMesh &d, const TP *__res
         }
     }
 #pragma unroll
-    for (int v = 0; v < NV; ++v)
+    for (int a = 0; a < ND; ++a) {
+        TM o[NV];
 #pragma unroll
-        for (int a = 0; a < ND; ++a) {
-            TM s = TM(0);
+        for (int v = 0; v < NV; ++v) {
+            o[v] = TM(0);
 #pragma unroll
-            for (int c = 0; c < ND; ++c) s = fma(Pm[a * ND + c], y[v * ND + c], s);
-            zout[(v * ND + a) * T + i] = TZ(s);
+            for (int c = 0; c < ND; ++c) o[v] = fma(Pm[a * ND + c], y[v * ND + c], o[v]);
         }
+        vstore(zout, a, T, i, o);
+    }
     if (SF) publish(sf_flag + i, sf_tag);
 }
 
@@ -822,12 +748,11 @@ __device__ __forceinline__ void ilu_bwd_row(const DeviceMesh &d, const TP *__res
                                             int32_t *sf_flag, int32_t sf_tag, int32_t *sf_err)
 {
     const int64_t T = d.T;
-    TM zi[NX], y[NX];
+    TM zi[ND][NV], y[NX];
 #pragma unroll
-    for (int k = 0; k < NX; ++k) {
-        zi[k] = TM(z[k * T + i]);
-        y[k] = TM(0);
-    }
+    for (int l = 0; l < ND; ++l) vload(z, l, T, i, zi[l]);
+#pragma unroll
+    for (int k = 0; k < NX; ++k) y[k] = TM(0);
     TM Pm[25];
 #pragma unroll
     for (int k = 0; k < 25; ++k) Pm[k] = TM(Pg[k * T + i]);
@@ -846,18 +771,21 @@ __device__ __forceinline__ void ilu_bwd_row(const DeviceMesh &d, const TP *__res
         const int j = d.nb[s * T + i];
         if (j <= i) continue;
         const TM sa = TM(alg[s * T + i]), sax = sa * TM(exg[s * T + i]), say = sa * TM(eyg[s * T + i]);
+        constexpr int NA = G ? ND : 2;       // rows of a neighbour that its block reaches
+        TM xn[NA][NV];
 #pragma unroll
-        for (int v = 0; v < NV; ++v)
-            oacc(sa, sax, say, TM(ldx<SF>(xin + (v * ND + 0) * T + j)), TM(ldx<SF>(xin + (v * ND + 1) * T + j)),
-                 y + v * ND);
-        if (G) {
+        for (int a = 0; a < NA; ++a) {
+            if constexpr (SF) vload_cg(xin, a, T, j, xn[a]);
+            else vload(xin, a, T, j, xn[a]);
+        }
+#pragma unroll
+        for (int v = 0; v < NV; ++v) oacc(sa, sax, say, xn[0][v], xn[1][v], y + v * ND);
+        if constexpr (G) {
             const TM sr = TM(arg[s * T + i]), srx = sr * TM(exrg[s * T + i]), sry = sr * TM(eyrg[s * T + i]);
             const TM sb = TM(bdgg[s * T + i]);
 #pragma unroll
             for (int v = 0; v < NV; ++v) {
-                TM xj[ND];
-#pragma unroll
-                for (int l = 0; l < ND; ++l) xj[l] = TM(ldx<SF>(xin + (v * ND + l) * T + j));
+                const TM xj[ND] = {xn[0][v], xn[1][v], xn[2][v], xn[3][v], xn[4][v]};
                 racc(sr, srx, sry, xj, y + v * ND);
 #pragma unroll
                 for (int l = 2; l < ND; ++l) y[v * ND + l] = fma(sb, xj[l], y[v * ND + l]);
@@ -865,14 +793,16 @@ __device__ __forceinline__ void ilu_bwd_row(const DeviceMesh &d, const TP *__res
         }
     }
 #pragma unroll
-    for (int v = 0; v < NV; ++v)
+    for (int a = 0; a < ND; ++a) {
+        TM o[NV];
 #pragma unroll
-        for (int a = 0; a < ND; ++a) {
-            TM s = zi[v * ND + a];
+        for (int v = 0; v < NV; ++v) {
+            o[v] = zi[a][v];
 #pragma unroll
-            for (int c = 0; c < ND; ++c) s = fma(Pm[a * ND + c], y[v * ND + c], s);
-            xout[(v * ND + a) * T + i] = TZ(s);
+            for (int c = 0; c < ND; ++c) o[v] = fma(Pm[a * ND + c], y[v * ND + c], o[v]);
         }
+        vstore(xout, a, T, i, o);
+    }
     if (SF) publish(sf_flag + i, sf_tag);
 }
 
@@ -972,97 +902,6 @@ __global__ void __launch_bounds__(kBlock) k_ilu_bwd_sf(DeviceMesh d, const TP *_
     }
 }
 
-// ---- two backward preconditioner sweeps per launch: the second sweep of a
-// cell needs its upper neighbours' first-sweep values, which each thread forms
-// itself from the neighbours' own data (factors, z, and their upper
-// neighbours' values), with exactly the arithmetic and roundings of a separate
-// first sweep, so the results are the same bit for bit.  One launch instead of
-// two reads each cell's factors and z once and writes x once; the neighbours'
-// data mostly comes from L2 (a neighbour is a few hundred to a thousand cells
-// away in RCM order).  Mixed precision only.  Measured at 1M cells (ncu, one launch): 101 us against
-// 55 + 59 us for the two sweeps.  The same fusion of the forward pair (which
-// also has to form the neighbours' neighbours' z^0 = P r) took 195 us against
-// 69 + 56 us, its three levels of dependent gathers exposed, and is not used.
-// Per-cell equations only (the global normal equations' reverse slots keep one
-// sweep per launch).
-
-// x^{q+2} = B(B(x^q)) with B(x)_i = z_i + P_i sum_{j>i} O_ij x_j: two backward
-// sweeps in one launch (x^q = xin; x^0 = z).
-template <typename TZ, typename TM, typename TP>
-__global__ void __launch_bounds__(kBlock, 3) k_ilu_bwd2(DeviceMesh d, const TP *__restrict__ Pg,
-                                                      const TP *__restrict__ alg, const TP *__restrict__ exg,
-                                                      const TP *__restrict__ eyg, const TZ *z, const TZ *xin,
-                                                      TZ *xout)
-{
-    const int64_t T = d.T;
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= T) return;
-    TM y[NX];
-#pragma unroll
-    for (int k = 0; k < NX; ++k) y[k] = TM(0);
-#pragma unroll 1
-    for (int s = 0; s < 3; ++s) {
-        const int j = d.nb[s * T + i];
-        if (j <= i) continue;
-        const TM sa = TM(alg[s * T + i]), sax = sa * TM(exg[s * T + i]), say = sa * TM(eyg[s * T + i]);
-        // the first sweep at j, rows 0 and 1: x^{q+1}_j = z_j + P_j sum_{k>j} O_jk x^q_k
-        TM yj[NX];
-#pragma unroll
-        for (int q = 0; q < NX; ++q) yj[q] = TM(0);
-        // the three slots' loads issued together (a slot that is not an upper
-        // neighbour of j reads j's own values, discarded); only the sums are
-        // conditional, in slot order
-#pragma unroll
-        for (int s2 = 0; s2 < 3; ++s2) {
-            const int kn = d.nb[s2 * T + j];
-            const bool upper = kn > j;
-            const int64_t k = upper ? kn : j;
-            const TM sb = TM(alg[s2 * T + j]), sbx = sb * TM(exg[s2 * T + j]), sby = sb * TM(eyg[s2 * T + j]);
-            TM xk[NV][2];
-#pragma unroll
-            for (int v = 0; v < NV; ++v) {
-                xk[v][0] = TM(xin[(v * ND + 0) * T + k]);
-                xk[v][1] = TM(xin[(v * ND + 1) * T + k]);
-            }
-            if (!upper) continue;
-#pragma unroll
-            for (int v = 0; v < NV; ++v) oacc(sb, sbx, sby, xk[v][0], xk[v][1], yj + v * ND);
-        }
-        TM x1[NV][2];
-#pragma unroll
-        for (int a = 0; a < 2; ++a) {
-            TM pa[ND];
-#pragma unroll
-            for (int c = 0; c < ND; ++c) pa[c] = TM(Pg[(a * ND + c) * T + j]);
-#pragma unroll
-            for (int v = 0; v < NV; ++v) {
-                TM t = TM(z[(v * ND + a) * T + j]);
-#pragma unroll
-                for (int c = 0; c < ND; ++c) t = fma(pa[c], yj[v * ND + c], t);
-                x1[v][a] = TM(TZ(t));
-            }
-        }
-#pragma unroll
-        for (int v = 0; v < NV; ++v) oacc(sa, sax, say, x1[v][0], x1[v][1], y + v * ND);
-    }
-    // the cell's own factor and z last, after the gathers (fewer values live
-    // while the neighbours' first sweep is formed)
-    TM Pm[25], zi[NX];
-#pragma unroll
-    for (int k = 0; k < 25; ++k) Pm[k] = TM(Pg[k * T + i]);
-#pragma unroll
-    for (int k = 0; k < NX; ++k) zi[k] = TM(z[k * T + i]);
-#pragma unroll
-    for (int v = 0; v < NV; ++v)
-#pragma unroll
-        for (int a = 0; a < ND; ++a) {
-            TM t = zi[v * ND + a];
-#pragma unroll
-            for (int c = 0; c < ND; ++c) t = fma(Pm[a * ND + c], y[v * ND + c], t);
-            xout[(v * ND + a) * T + i] = TZ(t);
-        }
-}
-
 // Partial dot products <V_k, w> of the four variables over one block of
 // kBlock cells: grid (k, block), blockIdx.x = k so that the j + 1 blocks of a
 // cell block run together and read w once from HBM.  64 threads per variable,
@@ -1104,6 +943,27 @@ __global__ void __launch_bounds__(kDotThreads, 3) k_dots(int64_t T, int64_t nblk
     }
 }
 
+// The same for an FP32 basis ([dof][cell][variable]): a thread per cell, FP32
+// within a warp (160 products), FP64 across warps and blocks.
+__global__ void __launch_bounds__(kBlock) k_dots32(int64_t T, const float *__restrict__ V,
+                                                   const float *__restrict__ w, double *__restrict__ part, int pstride)
+{
+    __shared__ float sh[kBlock / 32][1][4];
+    const int64_t b = blockIdx.x, i = b * kBlock + threadIdx.x;
+    const int k = blockIdx.y;
+    float sv[1][4] = {};
+    if (i < T)
+#pragma unroll
+        for (int l = 0; l < ND; ++l) {
+            float a[NV], u[NV];
+            vload(V + (int64_t)k * NX * T, l, T, i, a);
+            vload(w, l, T, i, u);
+#pragma unroll
+            for (int v = 0; v < NV; ++v) sv[0][v] = fmaf(a[v], u[v], sv[0][v]);
+        }
+    block_rows32<1>(sv, sh, part, pstride, k);
+}
+
 // w -= sum_{k<=j} c[s][k] V_k for running systems s = case * 4 + v (c: the
 // Gram-Schmidt coefficients of the unnormalised basis), w = 0 for the others;
 // optional partial |w|^2 per block.  The arithmetic is in the basis precision
@@ -1131,53 +991,46 @@ __global__ void k_orth_update(DeviceMesh d, const TB *__restrict__ V, TB *__rest
     TB nrm[NV] = {0, 0, 0, 0};
     if (J > 0 && i < T) {
         bool run[NV];
-        TB wv[NV][ND], vk[NV][J > 0 ? J : 1][ND];
+        TB wv[ND][NV], vk[J > 0 ? J : 1][ND][NV];
 #pragma unroll
-        for (int v = 0; v < NV; ++v) {
-            run[v] = ctl[kCtlRunning * ns + 4 * c + v] != 0;
+        for (int v = 0; v < NV; ++v) run[v] = ctl[kCtlRunning * ns + 4 * c + v] != 0;
 #pragma unroll
-            for (int l = 0; l < ND; ++l) wv[v][l] = w[(v * ND + l) * T + i];
+        for (int l = 0; l < ND; ++l) vload(w, l, T, i, wv[l]);
 #pragma unroll
-            for (int k = 0; k < J; ++k)
+        for (int k = 0; k < J; ++k)
 #pragma unroll
-                for (int l = 0; l < ND; ++l) vk[v][k][l] = V[k * vs + (v * ND + l) * T + i];
-        }
+            for (int l = 0; l < ND; ++l) vload(V + k * vs, l, T, i, vk[k][l]);
 #pragma unroll
-        for (int v = 0; v < NV; ++v) {
+        for (int l = 0; l < ND; ++l) {
 #pragma unroll
-            for (int k = 0; k < J; ++k)
+            for (int v = 0; v < NV; ++v) {
 #pragma unroll
-                for (int l = 0; l < ND; ++l) wv[v][l] = fma(-shc[v][k], vk[v][k][l], wv[v][l]);
-#pragma unroll
-            for (int l = 0; l < ND; ++l) {
-                const TB o = run[v] ? wv[v][l] : TB(0);
-                w[(v * ND + l) * T + i] = o;
-                nrm[v] = fma(o, o, nrm[v]);
+                for (int k = 0; k < J; ++k) wv[l][v] = fma(-shc[v][k], vk[k][l][v], wv[l][v]);
+                wv[l][v] = run[v] ? wv[l][v] : TB(0);
+                nrm[v] = fma(wv[l][v], wv[l][v], nrm[v]);
             }
+            vstore(w, l, T, i, wv[l]);
         }
     } else if (i < T) {
+        TB wv[ND][NV];
 #pragma unroll
-        for (int v = 0; v < NV; ++v) {
-            const int sy = 4 * c + v;
-            if (!ctl[kCtlRunning * ns + sy]) {
-#pragma unroll
-                for (int l = 0; l < ND; ++l) w[(v * ND + l) * T + i] = TB(0);
-                continue;
-            }
-            TB wv[ND];
-#pragma unroll
-            for (int l = 0; l < ND; ++l) wv[l] = w[(v * ND + l) * T + i];
-            for (int k = 0; k <= j; ++k) {
-                const TB hk = shc[v][k];
-                const TB *vk = V + k * vs;
-#pragma unroll
-                for (int l = 0; l < ND; ++l) wv[l] = fma(-hk, vk[(v * ND + l) * T + i], wv[l]);
-            }
+        for (int l = 0; l < ND; ++l) vload(w, l, T, i, wv[l]);
+        for (int k = 0; k <= j; ++k)
 #pragma unroll
             for (int l = 0; l < ND; ++l) {
-                w[(v * ND + l) * T + i] = wv[l];
-                nrm[v] = fma(wv[l], wv[l], nrm[v]);
+                TB t[NV];
+                vload(V + k * vs, l, T, i, t);
+#pragma unroll
+                for (int v = 0; v < NV; ++v) wv[l][v] = fma(-shc[v][k], t[v], wv[l][v]);
             }
+#pragma unroll
+        for (int l = 0; l < ND; ++l) {
+#pragma unroll
+            for (int v = 0; v < NV; ++v) {
+                wv[l][v] = ctl[kCtlRunning * ns + 4 * c + v] ? wv[l][v] : TB(0);
+                nrm[v] = fma(wv[l][v], wv[l][v], nrm[v]);
+            }
+            vstore(w, l, T, i, wv[l]);
         }
     }
     if (want_norm) {
@@ -1418,52 +1271,63 @@ __global__ void __launch_bounds__(32 * kSolveWarps)
     }
 }
 
-// x += sum_{k<jv} y_k Z_k with Z_k = M^{-1} V_k kept from the iterations
-// x += sum_k y[s][k] Z_k.  FP64 path: FP64 sums.  Mixed path (FP32 Z): the
-// correction of one inner cycle is formed in FP32 (it only has to be accurate to
-// the inner tolerance; the next FP64 residual measures what is left) and added
-// to x in FP64, so the FP64 pipe sees one add per value instead of one
-// conversion and one FMA per value and Krylov vector.  With sexp given (FP32
-// basis): y carries 2^-e of the cycle (see k_cycle_solve) and the sum is scaled
-// back by 2^e in FP64 (exact).
-// y32 (FP32 Z only, optional): the FP32 copy of y, read instead of converting
-// y per thread; the scaled value 2^e acc is formed exactly on the integer pipe
-// (f2d_pow2), so the FP64 pipe sees one add per value.
-template <typename TZ>
-__global__ void k_combine_z(DeviceMesh d, const TZ *__restrict__ Z, const double *__restrict__ y, int m,
-                            const int32_t *__restrict__ ctl, int ns, double *__restrict__ x,
-                            const int32_t *__restrict__ sexp = nullptr, const float *__restrict__ y32 = nullptr)
+// x += sum_k y[s][k] Z_k, k < jv, with Z_k = M^{-1} V_k kept from the iterations.
+// FP64 path (extended stencil; see k64_combine): FP64 sums, one variable per grid row.
+__global__ void k_combine_z(DeviceMesh d, const double *__restrict__ Z, const double *__restrict__ y, int m,
+                            const int32_t *__restrict__ ctl, int ns, double *__restrict__ x)
 {
     const int64_t T = d.T;
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= T) return;
-    const int v = blockIdx.y;                          // one variable per grid row
+    const int v = blockIdx.y;
     const int sy = 4 * d.blk_case[blockIdx.x] + v;
     const int jv = ctl[kCtlJv * ns + sy];
     if (jv <= 0) return;
     const int64_t vs = (int64_t)NX * T;
-    TZ acc[ND] = {0, 0, 0, 0, 0};
+    double acc[ND] = {0, 0, 0, 0, 0};
     for (int k = 0; k < jv; ++k) {
-        const TZ yk = y32 ? TZ(y32[sy * m + k]) : TZ(y[sy * m + k]);
+        const double yk = y[sy * m + k];
 #pragma unroll
         for (int l = 0; l < ND; ++l) acc[l] += yk * Z[k * vs + (v * ND + l) * T + i];
     }
-    if (sexp) {
-        const int e = sexp[sy];
-        if (std::is_same<TZ, float>::value) {
-            // 2^e acc as an FP64 value formed on the integer pipe (exact; no
-            // conversion instruction on the FP64 pipe), one FP64 add per value
 #pragma unroll
-            for (int l = 0; l < ND; ++l) x[(v * ND + l) * T + i] += f2d_pow2(float(acc[l]), e);
-        } else {
-            const double f = pow2(e);
+    for (int l = 0; l < ND; ++l) x[(v * ND + l) * T + i] += acc[l];
+}
+
+// Mixed path (FP32 Z): the correction of one inner cycle is formed in FP32 (it
+// only has to be accurate to the inner tolerance; the next FP64 residual measures
+// what is left) and added to x in FP64, so the FP64 pipe sees one add per value
+// instead of one conversion and one FMA per value and Krylov vector.  With sexp
+// given (FP32 basis): y carries 2^-e of the cycle (see k_cycle_solve) and the sum
+// is scaled back by 2^e exactly, on the integer pipe (f2d_pow2).  A thread per
+// cell and variable, the four variables of a cell in neighbouring lanes.
+__global__ void __launch_bounds__(kBlock) k_combine32(DeviceMesh d, const float *__restrict__ Z,
+                                                      const float *__restrict__ y32, int m,
+                                                      const int32_t *__restrict__ ctl, int ns,
+                                                      double *__restrict__ x, const int32_t *__restrict__ sexp)
+{
+    const int64_t T = d.T;
+    const int v = threadIdx.x & 3;
+    const int64_t i = blockIdx.x * (int64_t)(kBlock / NV) + (threadIdx.x >> 2);
+    if (i >= T) return;
+    const int sy = 4 * d.blk_case[blockIdx.x / NV] + v;
+    const int jv = ctl[kCtlJv * ns + sy];
+    if (jv <= 0) return;
+    const float *zv = Z + i * NV + v;
+    const int64_t ls = NV * T, vs = (int64_t)NX * T;
+    double xi[ND];
 #pragma unroll
-            for (int l = 0; l < ND; ++l) x[(v * ND + l) * T + i] += double(acc[l]) * f;
-        }
-    } else {
+    for (int l = 0; l < ND; ++l) xi[l] = x[(v * ND + l) * T + i];
+    float acc[ND] = {0, 0, 0, 0, 0};
+#pragma unroll 4
+    for (int k = 0; k < jv; ++k) {
+        const float yk = y32[sy * m + k];
 #pragma unroll
-        for (int l = 0; l < ND; ++l) x[(v * ND + l) * T + i] += double(acc[l]);
+        for (int l = 0; l < ND; ++l) acc[l] = fmaf(yk, zv[k * vs + l * ls], acc[l]);
     }
+    const int e = sexp ? sexp[sy] : 0;
+#pragma unroll
+    for (int l = 0; l < ND; ++l) x[(v * ND + l) * T + i] = xi[l] + (sexp ? f2d_pow2(acc[l], e) : double(acc[l]));
 }
 
 // Warm start of solve n (cases not done) from the last solutions
@@ -1481,6 +1345,7 @@ __global__ void k_warm(DeviceMesh d, double *__restrict__ x, double *__restrict_
     const int64_t T = d.T;
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= T) return;
+    const int q0 = blockIdx.y * ND;                  // one variable per grid row
     // n solves so far: the two history buffers swap roles after every solve, and
     // the extrapolation uses as many past solutions as exist
     const int64_t n = *nsolve;
@@ -1488,16 +1353,16 @@ __global__ void k_warm(DeviceMesh d, double *__restrict__ x, double *__restrict_
     double *__restrict__ xpp = (n & 1) ? h0 : h1;
     const int order = (max_order >= 2 && n >= 3) ? 2 : (n >= 2 ? 1 : 0);
     if (done[d.blk_case[blockIdx.x]]) {
-#pragma unroll 4
-        for (int q = 0; q < NX; ++q) {
+#pragma unroll
+        for (int q = q0; q < q0 + ND; ++q) {
             const double b = xp[q * T + i], c = xpp[q * T + i];
             xp[q * T + i] = c;
             xpp[q * T + i] = b;
         }
         return;
     }
-#pragma unroll 4
-    for (int q = 0; q < NX; ++q) {
+#pragma unroll
+    for (int q = q0; q < q0 + ND; ++q) {
         const double a = x[q * T + i];
         if (order == 2) x[q * T + i] = 3.0 * (a - xp[q * T + i]) + xpp[q * T + i];
         else if (order == 1) x[q * T + i] = 2.0 * a - xp[q * T + i];
@@ -1529,6 +1394,12 @@ __global__ void k_start(const double *__restrict__ sums, int sstride, double *bn
 {
     const int sy = blockIdx.x * blockDim.x + threadIdx.x;
     if (sy >= ns) return;
+    if (!first && !ctl[kCtlActive * ns + sy]) {
+        // a system that stopped keeps its solution, its residual and their norm
+        ctl[kCtlRunning * ns + sy] = 0;
+        ctl[kCtlJv * ns + sy] = 0;
+        return;
+    }
     // |b| comes with the first residual; restarts reuse it
     const double vn0 = sqrt(sums[sy * sstride + 0]);
     double be = vn0;
@@ -1740,9 +1611,6 @@ gks_status precond_t(gks_mesh *m, const TP *Pg, const TP *alg, const TP *exg, co
         const int nsb = m->cfg.ilu_sweeps_bwd < 0 ? ns : m->cfg.ilu_sweeps_bwd;
         // z^0 folded into the first sweep (ilu_fuse_first) or a pass of its own
         const bool fuse = ns > 0 && m->cfg.ilu_fuse_first;
-        // two backward sweeps per launch where a pair follows (the per-cell
-        // equations; same results as one sweep per launch)
-        const bool pairs = std::is_same_v<TZ, float> && !rev.a && m->cfg.ilu_sweep_pairs;   // backward relation only
         const int nf = fuse ? ns : ns + 1;   // forward launches
         TZ *za = (nf % 2 == 1) ? tA : dst;   // buffers chosen so that z ends in tA
         TZ *zb = (nf % 2 == 1) ? dst : tA;
@@ -1759,21 +1627,10 @@ gks_status precond_t(gks_mesh *m, const TP *Pg, const TP *alg, const TP *exg, co
         if (nsb == 0) {
             GKS_CUDA(cudaMemcpyAsync(dst, za, sizeof(TZ) * NX * T, cudaMemcpyDeviceToDevice, s));
         } else {
-            // launches: pairs of sweeps, then a single one if nsb is odd
-            const int npair = pairs ? nsb / 2 : 0, nb = npair + (nsb - 2 * npair);
             TZ *xa = za;                                    // x^0 = z (in za)
-            TZ *xb = (nb % 2 == 1) ? dst : (za == tB ? tA : tB);
-            for (int q = 0; q < nb; ++q) {
-                if constexpr (std::is_same_v<TZ, float>) {
-                    if (q < npair) {
-                        k_ilu_bwd2<TZ, TM, TP><<<nblocks(T), kBlock, 0, s>>>(d, Pg, alg, exg, eyg, za, xa, xb);
-                        note_launch();
-                    } else {
-                        bwd(T, nullptr, za, xa, xb);
-                    }
-                } else {
-                    bwd(T, nullptr, za, xa, xb);
-                }
+            TZ *xb = (nsb % 2 == 1) ? dst : (za == tB ? tA : tB);
+            for (int q = 0; q < nsb; ++q) {
+                bwd(T, nullptr, za, xa, xb);
                 xa = xb;
                 xb = (xb == dst) ? tB : dst;
             }
@@ -1838,9 +1695,9 @@ gks_status precond64(gks_mesh *m, const double *src, double *dst, cudaStream_t s
     return GKS_OK;
 }
 
-// Launches of the FP64 solve with m->wk.c64 cells per thread.
+// A launch with c cells per thread.
 template <typename F>
-void with_cells64(int c, F &&f)
+void with_cells(int c, F &&f)
 {
     switch (c) {
     case 1: f(std::integral_constant<int, 1>{}); break;
@@ -1877,24 +1734,24 @@ gks_status solve64_shared_limit(int mm)
 void solve64_rhs(gks_mesh *m, int ps, cudaStream_t q)
 {
     const DeviceMesh &d = m->d;
-    with_cells64(m->wk.c64, [&](auto C) {
+    with_cells(m->wk.c64, [&](auto C) {
         k64_rhs<decltype(C)::value><<<rows64(m), kW64, 0, q>>>(d.T, d.nb, d.a0, m->wk.w, m->wk.b, m->wk.part, ps);
     });
 }
 
-void solve64_resid(gks_mesh *m, double *V0, int ps, cudaStream_t q)
+void solve64_resid(gks_mesh *m, double *V0, const int32_t *act, int ps, cudaStream_t q)
 {
     const DeviceMesh &d = m->d;
-    with_cells64(m->wk.c64, [&](auto C) {
-        k64_resid<decltype(C)::value><<<rows64(m), kW64, 0, q>>>(d.T, d.nb, d.D, d.off, m->wk.x, m->wk.b, V0,
-                                                               m->wk.part, ps);
+    with_cells(m->wk.c64, [&](auto C) {
+        k64_resid<decltype(C)::value><<<rows64(m), kW64, 0, q>>>(d.T, d.nb, d.D, d.off, d.blk_case, act, m->wk.x,
+                                                               m->wk.b, V0, m->wk.part, ps);
     });
 }
 
 void solve64_apply_dots(gks_mesh *m, const double *z, const double *V, double *y, int j, int ps, cudaStream_t q)
 {
     const DeviceMesh &d = m->d;
-    with_cells64(m->wk.c64, [&](auto C) {
+    with_cells(m->wk.c64, [&](auto C) {
         k64_apply_dots<decltype(C)::value><<<rows64(m), kW64, acc64(j, kAccStride), q>>>(
             d.T, d.nb, d.D, d.off, d.blk_case, m->wk.ctl + kCtlRunning * m->wk.ns, z, y, V, j, m->wk.part, ps);
     });
@@ -1903,7 +1760,7 @@ void solve64_apply_dots(gks_mesh *m, const double *z, const double *V, double *y
 void solve64_update_dots(gks_mesh *m, const double *V, double *w, int j, int ps, cudaStream_t q)
 {
     const DeviceMesh &d = m->d;
-    with_cells64(m->wk.c64, [&](auto C) {
+    with_cells(m->wk.c64, [&](auto C) {
         k64_update_dots<decltype(C)::value><<<rows64(m), kW64, acc64(j, kAccStride + 1), q>>>(
             d.T, d.blk_case, m->wk.ctl + kCtlRunning * m->wk.ns, V, w, j, m->wk.hco, ps, m->wk.part, ps);
     });
@@ -1912,7 +1769,7 @@ void solve64_update_dots(gks_mesh *m, const double *V, double *w, int j, int ps,
 void solve64_update_norm(gks_mesh *m, const double *V, double *w, int j, int ps, cudaStream_t q)
 {
     const DeviceMesh &d = m->d;
-    with_cells64(m->wk.c64, [&](auto C) {
+    with_cells(m->wk.c64, [&](auto C) {
         k64_update_norm<decltype(C)::value><<<rows64(m), kW64, 0, q>>>(
             d.T, d.blk_case, m->wk.ctl + kCtlRunning * m->wk.ns, V, w, j, m->wk.hco, ps, m->wk.part, ps);
     });
@@ -1928,10 +1785,103 @@ gks_status precond(gks_mesh *m, const TR *src, double *dst, cudaStream_t s)
                                          {d.alr, d.exr, d.eyr, d.bdg});
 }
 
+void solve32_rhs(gks_mesh *m, int ps, cudaStream_t q)
+{
+    const unsigned g = (unsigned)(m->wk.nblk * (kRows64 / m->wk.c32));
+    with_cells(m->wk.c32, [&](auto C) {
+        k_rhs_df<decltype(C)::value><<<g, kW32, 0, q>>>(m->d, m->d.a0p, m->wk.w, m->wk.b, m->wk.part, ps);
+    });
+}
+
+void solve32_apply_dots(gks_mesh *m, const float *z, const float *V, float *y, int j, int ps, cudaStream_t q)
+{
+    const DeviceMesh &d = m->d;
+    const Work &k = m->wk;
+    const int32_t *run = k.ctl + kCtlRunning * k.ns;
+    const float4 *op = reinterpret_cast<const float4 *>(d.op32);
+#define A32(J) k32_apply_dots<J><<<k.nblk, kBlock, 0, q>>>(d.T, d.nb, op, d.blk_case, run, z, y, V, j, k.part, ps)
+    switch (j) {     // the first four Arnoldi indices unrolled (the inner cycles rarely go further)
+    case 0: A32(1); break;
+    case 1: A32(2); break;
+    case 2: A32(3); break;
+    case 3: A32(4); break;
+    default: A32(0);
+    }
+#undef A32
+    note_launch();
+}
+
+void solve32_update_norm(gks_mesh *m, const float *V, float *w, int j, int ps, cudaStream_t q)
+{
+    const DeviceMesh &d = m->d;
+    const Work &k = m->wk;
+    const int32_t *run = k.ctl + kCtlRunning * k.ns;
+#define U32(J) k32_update_norm<J><<<k.nblk, kBlock, 0, q>>>(d.T, d.blk_case, run, V, w, j, k.hco, ps, k.part, ps)
+    switch (j) {
+    case 0: U32(1); break;
+    case 1: U32(2); break;
+    case 2: U32(3); break;
+    case 3: U32(4); break;
+    default: U32(0);
+    }
+#undef U32
+    note_launch();
+}
+
+// The FP32 sweeps of the per-cell equations with packed factors (see precond64
+// for the buffers).  A wider source is rounded to FP32 once, in the
+// first pass, for the later sweeps.
+template <typename TR, typename TP>
+gks_status precond32s(gks_mesh *m, const TP *pk, const TR *src, float *dst, cudaStream_t s)
+{
+    const DeviceMesh &d = m->d;
+    Work &k = m->wk;
+    const int64_t T = d.T;
+    const unsigned g = (unsigned)((T + kW32 - 1) / kW32);
+    const int32_t *run = k.ctl + kCtlRunning * k.ns;
+    const int ns = m->cfg.ilu_sweeps, nsb = m->cfg.ilu_sweeps_bwd < 0 ? ns : m->cfg.ilu_sweeps_bwd;
+    const bool fuse = ns > 0 && m->cfg.ilu_fuse_first;
+    float *z = nsb > 0 ? k.t3_32 : dst;
+    auto mid = [&](int q, int n) { return (n - 1 - q) % 2 == 0 ? k.t2_32 : dst; };
+    float *rc = (sizeof(TR) > sizeof(float) && ns > 0) ? k.r32 : nullptr;
+    const int nf = fuse ? ns : ns + 1;                    // forward launches
+    const float *prev = nullptr;
+    for (int q = 0; q < nf; ++q) {
+        const bool last = q + 1 == nf;
+        float *out = last ? z : mid(q, nf - 1);
+#define F32(NB, FULL, TS, SRC, RC) \
+    k32_fwd<NB, FULL, TS, TP><<<g, kW32, 0, s>>>(T, d.nb, pk, d.blk_case, run, SRC, prev, out, RC)
+        if (q == 0 && fuse) last ? F32(2, true, TR, src, rc) : F32(2, false, TR, src, rc);
+        else if (q == 0) last ? F32(0, true, TR, src, rc) : F32(0, false, TR, src, rc);
+        else if (rc) last ? F32(1, true, float, rc, nullptr) : F32(1, false, float, rc, nullptr);
+        else last ? F32(1, true, TR, src, nullptr) : F32(1, false, TR, src, nullptr);
+#undef F32
+        note_launch();
+        prev = out;
+    }
+    // backward: pairs of sweeps (ilu_sweep_pairs), then a single one if nsb is odd
+    const int npair = m->cfg.ilu_sweep_pairs ? nsb / 2 : 0, nb = npair + (nsb - 2 * npair);
+    const float *x = z;
+    for (int q = 0; q < nb; ++q) {
+        const bool last = q + 1 == nb;
+        float *out = last ? dst : mid(q, nb - 1);
+#define B32(K, FULL) K<FULL, TP><<<g, kW32, 0, s>>>(T, d.nb, pk, d.blk_case, run, z, x, out)
+        if (q < npair) last ? B32(k32_bwd2, true) : B32(k32_bwd2, false);
+        else last ? B32(k32_bwd, true) : B32(k32_bwd, false);
+#undef B32
+        note_launch();
+        x = out;
+    }
+    GKS_CUDA(cudaGetLastError());
+    return GKS_OK;
+}
+
 template <typename TR>
 gks_status precond32(gks_mesh *m, const TR *src, float *dst, cudaStream_t s)
 {
     DeviceMesh &d = m->d;
+    if (m->cfg.precond == GKS_PC_ILU_SWEEP && d.pk16) return precond32s<TR, __half>(m, d.pk16, src, dst, s);
+    if (m->cfg.precond == GKS_PC_ILU_SWEEP && d.pk32) return precond32s<TR, float>(m, d.pk32, src, dst, s);
     if (d.P16)   // FP16 factors (ilu_fp16), FP32 arithmetic
         return precond_t<TR, float, float, __half>(m, d.P16, d.alpha16, d.ex16, d.ey16, src, dst, m->wk.t2_32,
                                                    m->wk.t3_32, m->wk.r32, s, {d.alr16, d.exr16, d.eyr16, d.bdg16});
@@ -2210,8 +2160,12 @@ template <typename TB>
 gks_status dots(gks_mesh *m, const TB *V, const TB *w, int j, double *part, int ps, cudaStream_t s)
 {
     const int64_t nblk = m->wk.nblk;
-    const dim3 g((unsigned)(j + 1), (unsigned)std::min<int64_t>(nblk, kDotMaxTiles));
-    k_dots<TB><<<g, kDotThreads, 0, s>>>(m->d.T, nblk, V, w, part, ps);
+    if constexpr (std::is_same_v<TB, float>) {
+        k_dots32<<<dim3((unsigned)nblk, (unsigned)(j + 1)), kBlock, 0, s>>>(m->d.T, V, w, part, ps);
+    } else {
+        const dim3 g((unsigned)(j + 1), (unsigned)std::min<int64_t>(nblk, kDotMaxTiles));
+        k_dots<TB><<<g, kDotThreads, 0, s>>>(m->d.T, nblk, V, w, part, ps);
+    }
     note_launch();
     GKS_CUDA(cudaGetLastError());
     return GKS_OK;
@@ -2250,7 +2204,7 @@ gks_status cls_solve_t(gks_mesh *m, TB *V, cudaStream_t s, int32_t *iters, doubl
     gks_status st;
     // the FP64 solve of the per-cell equations: a thread per cell and variable
     // (gks_solve64.cuh), C64 cells per thread, rs partial-sum rows per cell block
-    const int C64 = k.c64, rs = C64 ? kRows64 / C64 : 1;
+    const int C64 = k.c64;
     if (C64 && mm > 45) {
         if ((st = solve64_shared_limit(mm)) != GKS_OK) return st;
     }
@@ -2282,23 +2236,31 @@ gks_status cls_solve_t(gks_mesh *m, TB *V, cudaStream_t s, int32_t *iters, doubl
     };
     // the FP32-basis solve forms b in double-FP32 arithmetic when the weights fit
     const bool rhs_df = std::is_same<TB, float>::value && d.a0p;
-    auto residual = [&](cudaStream_t q) -> gks_status {
+    // the FP32 basis with the per-cell equations: the operator kernel also forms
+    // the Gram-Schmidt products
+    const bool fused_dots = std::is_same<TB, float>::value && !d.alr32 && m->cfg.spmv_dots;
+    // partial-sum rows per cell block of the kernels in use
+    const int rs64 = C64 ? kRows64 / C64 : 1, rs32 = k.c32 ? kRows64 / k.c32 : 1;
+    const int rs_rhs = C64 ? rs64 : (rhs_df ? rs32 : 1);
+    const int rs_res = C64 ? rs64 : (std::is_same<TB, float>::value && d.D2 ? kResidRows : 1);
+    const int rs = rs64;
+    auto residual = [&](cudaStream_t q, bool first) -> gks_status {
+        const int32_t *act = first ? nullptr : k.ctl + kCtlActive * ns;
         if (C64) {
-            solve64_resid(m, reinterpret_cast<double *>(V), ps, q);
-            GKS_CUDA(cudaGetLastError());
-            return GKS_OK;
-        }
-        if (std::is_same<TB, float>::value && d.D2) {
+            solve64_resid(m, reinterpret_cast<double *>(V), act, ps, q);
+        } else if (std::is_same<TB, float>::value && d.D2) {
+            float *v0 = reinterpret_cast<float *>(V);
+            const float4 *d2 = reinterpret_cast<const float4 *>(d.D2);
             if (d.SR2)
-                k_resid_df<true><<<4 * nb, kBlock, 0, q>>>(d, d.D2, d.S2, k.x, reinterpret_cast<float *>(V), k.b,
-                                                           k.part, ps, sxn, d.SR2, d.SB2);
+                k_resid_df<true><<<kResidRows * nb, kBlock, 0, q>>>(d, d2, k.x, v0, k.b, k.part, ps, sxn, act,
+                                                                   reinterpret_cast<const float4 *>(d.SR2));
             else
-                k_resid_df<false><<<4 * nb, kBlock, 0, q>>>(d, d.D2, d.S2, k.x, reinterpret_cast<float *>(V), k.b,
-                                                            k.part, ps, sxn);
+                k_resid_df<false><<<kResidRows * nb, kBlock, 0, q>>>(d, d2, k.x, v0, k.b, k.part, ps, sxn, act);
+            note_launch();
         } else {
             spmv64(q, k.x, V, 1, k.b, sxn);
+            note_launch();
         }
-        note_launch();
         GKS_CUDA(cudaGetLastError());
         return GKS_OK;
     };
@@ -2312,24 +2274,23 @@ gks_status cls_solve_t(gks_mesh *m, TB *V, cudaStream_t s, int32_t *iters, doubl
         }
         if (C64) {
             solve64_rhs(m, ps, q);
+        } else if (rhs_df) {
+            solve32_rhs(m, ps, q);
         } else {
-            if (rhs_df)
-                k_rhs_df<<<nb, kBlock, 0, q>>>(d, d.a0p, k.w, k.b, k.part, ps);
-            else
-                k_rhs<<<nb, kBlock, 0, q>>>(d, k.w, k.b, k.part, ps);
+            k_rhs<<<nb, kBlock, 0, q>>>(d, k.w, k.b, k.part, ps);
             note_launch();
         }
         if (sx) {
             // the FP32 basis stores its first vector scaled by a power of two 2^-e
-            k_reduce<<<dim3(1, ns), kReduceThreads, 0, q>>>(k.part + 1, d.case_blk, rs, ps, k.hcol + 1, ps, 0);
+            k_reduce<<<dim3(1, ns), kReduceThreads, 0, q>>>(k.part + 1, d.case_blk, rs_rhs, ps, k.hcol + 1, ps, 0);
             note_launch();
             k_sigma<<<sblocks(ns), 128, 0, q>>>(k.hcol, ps, k.bnorm, k.sexp, ns); note_launch();
         }
         prof_stop(m, slot, q);
         slot = prof_start(m, kProfResid, q);
         // residual r = b - K x, written straight into the basis slot V_0 (v_0 = V_0 / beta)
-        if (const gks_status r = residual(q); r != GKS_OK) return r;
-        k_reduce<<<dim3(sx ? 1 : 2, ns), kReduceThreads, 0, q>>>(k.part, d.case_blk, rs, ps, k.hcol, ps, 0);
+        if (const gks_status r = residual(q, true); r != GKS_OK) return r;
+        k_reduce<<<dim3(sx ? 1 : 2, ns), kReduceThreads, 0, q>>>(k.part, d.case_blk, rs_res, ps, k.hcol, ps, 0);
         note_launch();
         prof_stop(m, slot, q);
         slot = prof_start(m, kProfCtl, q);
@@ -2351,20 +2312,9 @@ gks_status cls_solve_t(gks_mesh *m, TB *V, cudaStream_t s, int32_t *iters, doubl
             return st;
         prof_stop(m, slot, q);
         slot = prof_start(m, kProfSpmv, q);
-        // the FP32 basis with the per-cell equations: the operator kernel also
-        // forms the first Gram-Schmidt products (k_spmv_dots)
-        const bool fused_dots = std::is_same<TB, float>::value && !d.alr32 && m->cfg.spmv_dots;
         if (fused_dots) {
-            float *yv = reinterpret_cast<float *>(vj1);
-            const float *Vf = reinterpret_cast<const float *>(V);
-            const float *zj = k.Z32 + j * vs;
-            switch (j) {     // the first four Arnoldi indices unrolled (the inner cycles rarely go further)
-            case 0: k_spmv_dots<1><<<nb, kBlock, 0, q>>>(d, d.D32, d.alpha32, d.ex32, d.ey32, zj, yv, Vf, j, k.part, ps); break;
-            case 1: k_spmv_dots<2><<<nb, kBlock, 0, q>>>(d, d.D32, d.alpha32, d.ex32, d.ey32, zj, yv, Vf, j, k.part, ps); break;
-            case 2: k_spmv_dots<3><<<nb, kBlock, 0, q>>>(d, d.D32, d.alpha32, d.ex32, d.ey32, zj, yv, Vf, j, k.part, ps); break;
-            case 3: k_spmv_dots<4><<<nb, kBlock, 0, q>>>(d, d.D32, d.alpha32, d.ex32, d.ey32, zj, yv, Vf, j, k.part, ps); break;
-            default: k_spmv_dots<<<nb, kBlock, 0, q>>>(d, d.D32, d.alpha32, d.ex32, d.ey32, zj, yv, Vf, j, k.part, ps);
-            }
+            solve32_apply_dots(m, k.Z32 + j * vs, reinterpret_cast<const float *>(V), reinterpret_cast<float *>(vj1),
+                               j, ps, q);
         } else if (mixed) {
             spmv32(q, k.Z32 + j * vs, vj1);
         } else if (C64) {
@@ -2374,7 +2324,7 @@ gks_status cls_solve_t(gks_mesh *m, TB *V, cudaStream_t s, int32_t *iters, doubl
         } else {
             spmv64(q, k.Z + j * vs, vj1, 0, nullptr, nullptr);
         }
-        if (!C64) note_launch();
+        if (!C64 && !fused_dots) note_launch();
         prof_stop(m, slot, q);
         slot = prof_start(m, kProfOrth, q);
         // classical Gram-Schmidt: twice in FP64 mode; once in the mixed mode, whose
@@ -2385,6 +2335,8 @@ gks_status cls_solve_t(gks_mesh *m, TB *V, cudaStream_t s, int32_t *iters, doubl
         note_launch();
         if (C64) {
             solve64_update_dots(m, reinterpret_cast<const double *>(V), reinterpret_cast<double *>(vj1), j, ps, q);
+        } else if (fused_dots) {
+            solve32_update_norm(m, reinterpret_cast<const float *>(V), reinterpret_cast<float *>(vj1), j, ps, q);
         } else {
             launch_orth_update<TB>(d, nb, q, V, vj1, j, k.hco, ps, k.ctl, ns, k.part, ps, mixed ? 1 : 0);
             note_launch();
@@ -2417,17 +2369,17 @@ gks_status cls_solve_t(gks_mesh *m, TB *V, cudaStream_t s, int32_t *iters, doubl
             mm, k.H, k.g, k.y, k.vn, k.ctl, ns, k.bnorm, rtol, sx, mixed ? k.y32 : nullptr);
         note_launch();
         if (mixed)
-            k_combine_z<float><<<dim3(nb, NV), kBlock, 0, q>>>(d, k.Z32, k.y, mm, k.ctl, ns, k.x, sx, k.y32);
+            k_combine32<<<NV * nb, kBlock, 0, q>>>(d, k.Z32, k.y32, mm, k.ctl, ns, k.x, sx);
         else if (C64)
             k64_combine<<<(unsigned)((T + 31) / 32), kW64, 0, q>>>(T, d.blk_case, k.Z, k.y, mm, k.ctl + kCtlJv * ns,
                                                                   k.x);
         else
-            k_combine_z<double><<<dim3(nb, NV), kBlock, 0, q>>>(d, k.Z, k.y, mm, k.ctl, ns, k.x);
+            k_combine_z<<<dim3(nb, NV), kBlock, 0, q>>>(d, k.Z, k.y, mm, k.ctl, ns, k.x);
         note_launch();
         prof_stop(m, slot, q);
         slot = prof_start(m, kProfResid, q);
-        if (const gks_status r = residual(q); r != GKS_OK) return r;
-        k_reduce<<<dim3(1, ns), kReduceThreads, 0, q>>>(k.part, d.case_blk, rs, ps, k.hcol, ps, 0); note_launch();
+        if (const gks_status r = residual(q, false); r != GKS_OK) return r;
+        k_reduce<<<dim3(1, ns), kReduceThreads, 0, q>>>(k.part, d.case_blk, rs_res, ps, k.hcol, ps, 0); note_launch();
         prof_stop(m, slot, q);
         slot = prof_start(m, kProfCtl, q);
         k_start<<<sblocks(ns), 128, 0, q>>>(k.hcol, ps, k.bnorm, k.beta, k.vn, mm, k.ctl, ns, k.done, rtol, maxit,
@@ -2531,7 +2483,7 @@ gks_status launch_warm(gks_mesh *m, cudaStream_t s)
     Work &k = m->wk;
     if (!m->cfg.warm_extrap) return GKS_OK;
     const int slot = prof_start(m, kProfCtl, s);
-    k_warm<<<(unsigned)k.nblk, kBlock, 0, s>>>(m->d, k.x, k.x_prev, k.x_prev2, k.done, k.nsolve, m->cfg.warm_extrap);
+    k_warm<<<dim3((unsigned)k.nblk, NV), kBlock, 0, s>>>(m->d, k.x, k.x_prev, k.x_prev2, k.done, k.nsolve, m->cfg.warm_extrap);
     note_launch();
     prof_stop(m, slot, s);
     GKS_CUDA(cudaGetLastError());
@@ -2614,18 +2566,35 @@ gks_status cls_solve(gks_mesh *m, cudaStream_t s, int32_t *iters, double *relres
                  : cls_solve_t<double>(m, k.V, s, iters, relres, converged);
 }
 
-void plan_solve64(gks_mesh *m, int *rows)
+void plan_solve(gks_mesh *m, int *rows)
 {
-    m->wk.c64 = cells64(m->d.T);
-    *rows = kRows64 / m->wk.c64;
+    const int c = cells64(m->d.T);
+    if (m->cfg.precision == GKS_FP64) m->wk.c64 = c;
+    else m->wk.c32 = c;
+    // the mixed path's residual has a row per quarter of a cell block
+    *rows = std::max(kRows64 / c, m->cfg.precision == GKS_MIXED ? kResidRows : 1);
 }
 
-gks_status launch_off64(gks_mesh *m)
+gks_status launch_pack(gks_mesh *m)
 {
     const DeviceMesh &d = m->d;
     if (d.T == 0) return GKS_OK;
-    k64_off<<<nblocks(d.T), kBlock>>>(d.T, d.alpha, d.ex, d.ey, d.off);
-    note_launch();
+    const unsigned g = nblocks(d.T);
+    if (d.off) {
+        k64_off<<<g, kBlock>>>(d.T, d.alpha, d.ex, d.ey, d.off);
+        note_launch();
+    }
+    if (d.op32) {
+        k32_pack_op<<<g, kBlock>>>(d.T, d.D32, d.alpha32, d.ex32, d.ey32, reinterpret_cast<float4 *>(d.op32));
+        note_launch();
+    }
+    if (d.pk16) {
+        k32_pack<__half><<<g, kBlock>>>(d.T, d.P16, d.alpha16, d.ex16, d.ey16, d.pk16);
+        note_launch();
+    } else if (d.pk32) {
+        k32_pack<float><<<g, kBlock>>>(d.T, d.P32, d.alpha32, d.ex32, d.ey32, d.pk32);
+        note_launch();
+    }
     GKS_CUDA(cudaGetLastError());
     return GKS_OK;
 }

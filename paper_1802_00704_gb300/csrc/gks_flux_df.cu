@@ -86,23 +86,25 @@ __device__ __forceinline__ void ghost_val_df(int tag, const double *bc, df nx, d
 }
 
 // y = (hi, lo) pairs of x: w2 [8][T] from w [4][T], x2 [40][T] from x [20][T]
-// (high parts of all rows first), by integer operations
+// (high parts of all rows first), by integer operations; four rows per thread,
+// grid row 0 the state, 1-5 the coefficients
 __global__ void k_to_df(const double *__restrict__ w, const double *__restrict__ x, float *__restrict__ w2,
                         float *__restrict__ x2, int64_t T)
 {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= T) return;
+    const int g = blockIdx.y;
+    const double *src = g ? x + (int64_t)(4 * (g - 1)) * T : w;
+    float *hi = g ? x2 + (int64_t)(4 * (g - 1)) * T : w2;
+    float *lo = hi + (g ? 20 : 4) * T;
+    double v[4];
 #pragma unroll
-    for (int v = 0; v < 4; ++v) {
-        const df p = dfm::split_double(w[v * T + i]);
-        w2[v * T + i] = p.hi;
-        w2[(4 + v) * T + i] = p.lo;
-    }
-#pragma unroll 4
-    for (int q = 0; q < 20; ++q) {
-        const df p = dfm::split_double(x[q * T + i]);
-        x2[q * T + i] = p.hi;
-        x2[(20 + q) * T + i] = p.lo;
+    for (int q = 0; q < 4; ++q) v[q] = src[q * T + i];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const df p = dfm::split_double(v[q]);
+        hi[q * T + i] = p.hi;
+        lo[q * T + i] = p.lo;
     }
 }
 
@@ -273,7 +275,7 @@ gks_status launch_flux_df(gks_mesh *m, const double *w, const double *x, double 
     const unsigned g = blocks(2 * m->d.F, kFluxBlock);
     {
         // FP32 pairs of the state and the coefficients, then the double-FP32 flux
-        k_to_df<<<blocks(m->d.T, kBlock), kBlock, 0, s>>>(w, x, m->wk.w2, m->wk.x2, m->d.T);
+        k_to_df<<<dim3(blocks(m->d.T, kBlock), 6), kBlock, 0, s>>>(w, x, m->wk.w2, m->wk.x2, m->d.T);
         note_launch();
         const lead::LeadConst lc = lead_const(c);
         const df pr_fac = dfm::from_double(1.0 / c.prandtl - 1.0);

@@ -81,6 +81,10 @@ struct DeviceMesh {
     // NULL when not asked for or a value is outside FP16's range)
     __half *P16 = nullptr, *alpha16 = nullptr, *ex16 = nullptr, *ey16 = nullptr;
     __half *alr16 = nullptr, *exr16 = nullptr, *eyr16 = nullptr, *bdg16 = nullptr;
+    // the per-cell equations' sweeps and operator: factors packed in chunks of eight values per
+    // cell (34 values, FP16 or FP32), the operator [6][T][4] (gks_solve32.cuh)
+    __half *pk16 = nullptr;
+    float *pk32 = nullptr, *op32 = nullptr;
     float *ih32 = nullptr;           // [T] 1 / h_i (mixed flux)
     // FP32 pairs (hi, lo) of the geometry for the double-FP32 flux (mixed precision)
     float *m2 = nullptr;             // [6][T] mxx, mxy, myy, then their low parts
@@ -89,11 +93,10 @@ struct DeviceMesh {
     float *flen2 = nullptr;          // [2][F] half the face length (Gauss weight 1/2), its low part
     // the operator as FP32 pairs hi + lo for the double-FP32 refinement residual
     // (mixed mode with an FP32 basis; NULL when a value is outside the pair range)
-    float *D2 = nullptr;             // [30][T] the 15 diagonal-block values, then their low parts
-    float *S2 = nullptr;             // [18][T] sa, sa dx, sa dy per neighbour slot (sa = -alpha, 0
-                                     //         without neighbour), then their low parts
-    float *SR2 = nullptr;            // [18][T] the same for the reverse slots (global normal equations)
-    float *SB2 = nullptr;            // [6][T] -beta per slot, then the low parts (second-derivative equations)
+    float *D2 = nullptr;             // [12][T][4] the 15 diagonal-block values, their low parts, sa, sa dx, sa dy
+                                     //         per neighbour slot (sa = -alpha, 0 without neighbour), their low parts
+    float *SR2 = nullptr;            // [6][T][4] sa, sa dx, sa dy of the reverse slots (global normal equations), their
+                                     //         low parts, -beta per slot (second-derivative equations), its low parts
     double *ox = nullptr, *oy = nullptr;  // [3][T] neighbour centroid in i's scaled frame (limiter)
     int32_t *kord = nullptr;         // [T] reconstruction order k_i of Eq. (28) (limiter)
     int32_t *cf = nullptr;           // [3][T] (face << 1) | side, -1 unused
@@ -114,6 +117,7 @@ struct Work {
     int m_alloc = 0;                 // restart length the Krylov buffers were sized for
     int nblk = 0;                    // cell blocks (kBlock cells each)
     int c64 = 0;                     // FP64 solve of the per-cell equations: cells per thread (0: other solves)
+    int c32 = 0;                     // FP32-basis solve: cells per thread of the right-hand side kernel
     int sm_count = 0;                // multiprocessors of the handle's device
     int ns = 4;                      // GMRES systems: 4 per case
     double *w = nullptr;             // [4][T] state (internal order)
@@ -134,13 +138,14 @@ struct Work {
     int32_t *lflag = nullptr;        // [T] 0 untouched, 1 limited, 2 reset to the average
     double *b = nullptr, *r = nullptr, *t2 = nullptr, *t3 = nullptr;  // [20][T]
     float *t2_32 = nullptr, *t3_32 = nullptr;  // [20][T] FP32 preconditioner work
-    float *r32 = nullptr;            // [20][T] FP32 copy of the preconditioner's source (sweeps)
+    float *r32 = nullptr;            // [20][T] FP32 copy of the preconditioner's source (sweeps); the FP32
+                                     //         vectors of the solve are [5][T][4]: dof, cell, variable
     double *V = nullptr;             // [(m+1)][20][T] Krylov basis, unnormalised: v_k = V_k / vn_k
     float *V32 = nullptr;            // the same stored in FP32 (mixed mode with basis_fp32; V unused)
     double *Z = nullptr;             // [m][20][T] M^{-1} V_k (FP64 path)
     float *Z32 = nullptr;            // [m][20][T] M^{-1} V_k (mixed path)
     double *flux = nullptr;          // [4][F]
-    double *part = nullptr;          // [nblk * rows][4][m+2] partial sums (rows per cell block: 8 / c64, else 1)
+    double *part = nullptr;          // [nblk * rows][4][m+2] partial sums (rows per cell block: plan_solve)
     double *dpart = nullptr;         // [nblk][4] partial minima / sums
     // small GMRES state (device), one row per system
     double *H = nullptr;             // [ns][m+1][m]  (Givens-rotated Hessenberg)
@@ -268,10 +273,10 @@ struct CaseIn {
     const double *bc_state;
 };
 
-// cells per thread of the FP64 solve and its partial-sum rows per cell block; the
-// multiplied-out off-diagonal blocks d.off from d.alpha, d.ex, d.ey (gks_cls.cu)
-void plan_solve64(gks_mesh *m, int *rows);
-gks_status launch_off64(gks_mesh *m);
+// cells per thread of the solve's kernels and its partial-sum rows per cell block;
+// the arrays d.off, d.op32, d.pk16 or d.pk32 (where allocated) from the uploaded ones (gks_cls.cu)
+void plan_solve(gks_mesh *m, int *rows);
+gks_status launch_pack(gks_mesh *m);
 // set-up (gks_setup.cu)
 gks_status build_batch(gks_mesh *m, const CaseIn *cases, int32_t n_cases);
 void free_mesh(gks_mesh *m);

@@ -795,28 +795,28 @@ gks_status build_batch(gks_mesh *m, const CaseIn *cases, int32_t n_cases)
                 hi = float(v);
                 lo = float(v - double(hi));
             };
-            std::vector<float> h_D2(30 * T), h_S2(18 * T), h_SR2(ext ? 18 * T : 0), h_SB2(ext ? 6 * T : 0);
+            // groups of four values per cell
+            auto at = [T](int q, int64_t i) { return ((q / 4) * T + i) * 4 + q % 4; };
+            std::vector<float> h_D2(48 * T), h_SR2(ext ? 24 * T : 0);
             for (int64_t i = 0; i < T; ++i) {
-                for (int q = 0; q < 15; ++q) pair(h_D[q * T + i], h_D2[q * T + i], h_D2[(15 + q) * T + i]);
+                for (int q = 0; q < 15; ++q) pair(h_D[q * T + i], h_D2[at(q, i)], h_D2[at(15 + q, i)]);
                 for (int s = 0; s < 3; ++s) {
                     const double sa = h_nb[s * T + i] >= 0 ? -h_alpha[s * T + i] : 0.0;
                     const double o[3] = {sa, sa * h_ex[s * T + i], sa * h_ey[s * T + i]};
                     for (int q = 0; q < 3; ++q)
-                        pair(o[q], h_S2[(3 * s + q) * T + i], h_S2[(9 + 3 * s + q) * T + i]);
+                        pair(o[q], h_D2[at(30 + 3 * s + q, i)], h_D2[at(39 + 3 * s + q, i)]);
                     if (ext) {
                         const double sr = h_nb[s * T + i] >= 0 ? -h_alr[s * T + i] : 0.0;
                         const double r[3] = {sr, sr * h_exr[s * T + i], sr * h_eyr[s * T + i]};
                         for (int q = 0; q < 3; ++q)
-                            pair(r[q], h_SR2[(3 * s + q) * T + i], h_SR2[(9 + 3 * s + q) * T + i]);
-                        pair(h_nb[s * T + i] >= 0 ? -h_bdg[s * T + i] : 0.0, h_SB2[s * T + i], h_SB2[(3 + s) * T + i]);
+                            pair(r[q], h_SR2[at(3 * s + q, i)], h_SR2[at(9 + 3 * s + q, i)]);
+                        pair(h_nb[s * T + i] >= 0 ? -h_bdg[s * T + i] : 0.0, h_SR2[at(18 + s, i)], h_SR2[at(21 + s, i)]);
                     }
                 }
             }
             if (in_range) {
-                UP(D2, h_D2); UP(S2, h_S2);
-                if (ext) {
-                    UP(SR2, h_SR2); UP(SB2, h_SB2);
-                }
+                UP(D2, h_D2);
+                if (ext) UP(SR2, h_SR2);
                 // pairs of the right-hand-side weights for the double-FP32 right-hand side
                 // (0 or 2^-50 <= |a0| <= 2^50: the low parts stay normal FP32 and the
                 // scaled squares of the norm stay below 2^128)
@@ -857,10 +857,17 @@ gks_status build_batch(gks_mesh *m, const CaseIn *cases, int32_t n_cases)
         AL(Z, (size_t)mm * 20 * T);
     }
     int rows = 1;
-    if (cfg.precision == GKS_FP64 && !ext) {
-        plan_solve64(m, &rows);
-        if ((st = dalloc(m, &d.off, (size_t)9 * T)) != GKS_OK) return st;
-        if ((st = launch_off64(m)) != GKS_OK) return st;
+    if (cfg.precision == GKS_MIXED || !ext) plan_solve(m, &rows);
+    if (!ext) {
+        if (cfg.precision == GKS_FP64) {
+            if ((st = dalloc(m, &d.off, (size_t)9 * T)) != GKS_OK) return st;
+        } else {
+            if ((st = dalloc(m, &d.op32, (size_t)24 * T)) != GKS_OK) return st;
+            if (cfg.precond == GKS_PC_ILU_SWEEP &&
+                (st = d.P16 ? dalloc(m, &d.pk16, (size_t)34 * T) : dalloc(m, &d.pk32, (size_t)34 * T)) != GKS_OK)
+                return st;
+        }
+        if ((st = launch_pack(m)) != GKS_OK) return st;
     }
     AL(part, (size_t)nblk * rows * 4 * (mm + 2)); AL(dpart, (size_t)nblk * 4);
     if (cfg.limiter) {

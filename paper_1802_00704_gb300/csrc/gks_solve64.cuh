@@ -444,15 +444,20 @@ __global__ void __launch_bounds__(kW64) k64_rhs(int64_t T, const int32_t *__rest
     if (lane == 0) part[((int64_t)blockIdx.x * 4 + v) * ps + 1] = nr;
 }
 
-// Residual y = b - K x and the partial |y|^2 (entry 0)
+// Residual y = b - K x and the partial |y|^2 (entry 0); act (NULL on a solve's
+// first residual): systems that are not active keep theirs
 template <int C>
 __global__ void __launch_bounds__(kW64) k64_resid(int64_t T, const int32_t *__restrict__ nb,
                                                   const double *__restrict__ D, const double *__restrict__ off,
-                                                  const double *__restrict__ x, const double *__restrict__ b,
-                                                  double *__restrict__ y, double *__restrict__ part, int ps)
+                                                  const int32_t *__restrict__ blk_case,
+                                                  const int32_t *__restrict__ act, const double *__restrict__ x,
+                                                  const double *__restrict__ b, double *__restrict__ y,
+                                                  double *__restrict__ part, int ps)
 {
     const int64_t c0 = blockIdx.x * (int64_t)(32 * C);
-    const int lane = threadIdx.x & 31, v = threadIdx.x >> 5;
+    const Warp64 w = warp64(blk_case, act, c0);
+    if (!w.run) return;
+    const int lane = w.lane, v = w.v;
     const int64_t vo = (int64_t)v * 5 * T;
     double nr = 0.0;
     for (int c = 0; c < C; ++c) {
