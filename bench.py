@@ -72,7 +72,7 @@ FLUX_SOURCES = {
                       "gks_erfcx_coef.h"),
     "mixed_flux_ws": ("gks_flux.cu", "gks_kinetic.cuh", "gks_face.cuh"),
     "mixed_flux": ("gks_flux.cu", "gks_kinetic.cuh", "gks_face.cuh"),
-    "flux": ("gks_flux.cu", "gks_kinetic.cuh", "gks_face.cuh"),
+    "flux": ("gks_flux.cu", "gks_kinetic64.cuh", "gks_face.cuh"),
 }
 
 

@@ -9,6 +9,7 @@
 
 #include "gks_face.cuh"
 #include "gks_kinetic.cuh"
+#include "gks_kinetic64.cuh"
 
 namespace gks {
 namespace {
@@ -77,7 +78,7 @@ __global__ void __launch_bounds__(kFluxBlock, MIXED ? 4 : 1) k_face_flux(DeviceM
                 const double bc[4] = {d.bc[f], d.bc[F + f], d.bc[2 * F + f], d.bc[3 * F + f]};
                 ghost(d.ftag[f], bc, nx, ny, gamma, wl, wr);
             }
-            ok = kin::gp_flux<double, HEAT, KIN>(wl, wr, dt, gamma, mu, tau2, fk, prandtl);
+            ok = kin64::gp_flux<double, HEAT, KIN>(wl, wr, dt, gamma, mu, tau2, fk, prandtl);
         }
         if (!ok) atomicOr(&status[cs], kStatusNonPhys);
         const double s = 0.5 * d.flen[f];      // Gauss weight 1/2 times the face length
@@ -302,7 +303,7 @@ __global__ void __launch_bounds__(kFluxBlock) k_point_flux(int64_t n, const doub
         b[k] = wr[24 * q + k];
     }
     const bool ok = MIXED ? kin::gp_flux_mixed<HEAT, KIN>(a, b, dt, gamma, mu, tau2, f, prandtl)
-                          : kin::gp_flux<double, HEAT, KIN>(a, b, dt, gamma, mu, tau2, f, prandtl);
+                          : kin64::gp_flux<double, HEAT, KIN>(a, b, dt, gamma, mu, tau2, f, prandtl);
     if (!ok && status) atomicOr(status, kStatusNonPhys);
 #pragma unroll
     for (int k = 0; k < 4; ++k) out[4 * q + k] = f[k];
