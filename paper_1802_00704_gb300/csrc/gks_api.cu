@@ -509,10 +509,8 @@ gks_status run_steps_async(gks_mesh *m, int64_t max_steps, cudaStream_t s)
     while (q < max_steps) {
         const int64_t chunk = std::min<int64_t>(kCheckEvery, max_steps - q);
         for (int64_t r = 0; r < chunk; ++r) {
-            if ((st = launch_cfl_dt(m, k.w, k.dt, s)) != GKS_OK) return st;
-            if ((st = launch_clip_only(m, s)) != GKS_OK) return st;
-            if ((st = cls_solve(m, s, nullptr, nullptr, nullptr)) != GKS_OK) return st;
-            if ((st = launch_acc_iters(m, s)) != GKS_OK) return st;
+            if ((st = launch_cfl_dt(m, k.w, k.dt, s, true)) != GKS_OK) return st;
+            if ((st = cls_solve(m, s, nullptr, nullptr, nullptr, true)) != GKS_OK) return st;
             if (m->cfg.limiter && (st = launch_limiter(m, k.w, k.x, s)) != GKS_OK) return st;
             if ((st = launch_flux(m, k.w, m->cfg.limiter ? k.xl : k.x, 0.0, k.dt, k.flux, s)) != GKS_OK) return st;
             if ((st = launch_update(m, k.w, k.flux, s)) != GKS_OK) return st;

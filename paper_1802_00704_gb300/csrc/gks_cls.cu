@@ -18,7 +18,7 @@
 #include <type_traits>
 
 #include "gks_internal.h"
-#include "gks_solve32.cuh"
+#include "gks_control.cuh"
 #include "gks_wait.cuh"
 
 namespace gks {
@@ -92,9 +92,8 @@ __device__ __forceinline__ void block_sum4(double *v, double *sh)
 }
 
 // r_i = sum_j a0_ij (ubar_j - ubar_i), Eq. (25) with b_ij = (ubar_j - ubar_i, 0, 0)
-// with partial sums of |b|^2 per block and variable in part[blk][v][1]
-__global__ void k_rhs(DeviceMesh d, const double *__restrict__ w, double *__restrict__ b, double *__restrict__ part,
-                      int pstride)
+// with partial sums of |b|^2 per block and variable in column 1 of part
+__global__ void k_rhs(DeviceMesh d, const double *__restrict__ w, double *__restrict__ b, double *__restrict__ part)
 {
     __shared__ double sh[32 * NV];
     const int64_t T = d.T;
@@ -132,7 +131,7 @@ __global__ void k_rhs(DeviceMesh d, const double *__restrict__ w, double *__rest
     }
     block_sum4(nb, sh);
     if (threadIdx.x == 0)
-        for (int v = 0; v < NV; ++v) part[(blockIdx.x * NV + v) * pstride + 1] = nb[v];
+        for (int v = 0; v < NV; ++v) part[(NV + v) * (int64_t)gridDim.x + blockIdx.x] = nb[v];
 }
 
 // acc = (K x)_i, the operator row of cell i applied to x (TM arithmetic).
@@ -217,7 +216,7 @@ template <typename TX, typename TM, typename TY, bool G = false>
 __global__ void k_spmv(DeviceMesh d, const TM *__restrict__ Dg, const TM *__restrict__ alg,
                        const TM *__restrict__ exg, const TM *__restrict__ eyg, const TX *__restrict__ x,
                        TY *__restrict__ y, int mode, const double *__restrict__ b, double *__restrict__ part,
-                       int pstride, const int32_t *__restrict__ sexp = nullptr, const TM *__restrict__ arg = nullptr,
+                       const int32_t *__restrict__ sexp = nullptr, const TM *__restrict__ arg = nullptr,
                        const TM *__restrict__ exrg = nullptr, const TM *__restrict__ eyrg = nullptr,
                        const TM *__restrict__ bdgg = nullptr)
 {
@@ -255,7 +254,7 @@ __global__ void k_spmv(DeviceMesh d, const TM *__restrict__ Dg, const TM *__rest
     if (mode >= 1) {
         block_sum4(nr, sh);
         if (threadIdx.x == 0)
-            for (int v = 0; v < NV; ++v) part[(blockIdx.x * NV + v) * pstride + 0] = nr[v];
+            for (int v = 0; v < NV; ++v) part[v * (int64_t)gridDim.x + blockIdx.x] = nr[v];
     }
 }
 
@@ -326,7 +325,7 @@ __device__ __noinline__ void resid64_cell(const DeviceMesh &d, const double *__r
     for (int l = 0; l < ND; ++l) out[l] = float((b[(v * ND + l) * d.T + i] - acc[v * ND + l]) * pow2(-e));
 }
 
-constexpr int kResidRows = NV;          // blocks (partial-sum rows) of the residual per cell block
+constexpr int kResidRows = NV;          // residual blocks (partial-sum rows) per cell block
 
 // (h, l) of every lane summed over the warp (lane 0 gets the pair)
 __device__ __forceinline__ void df_warp_sum(float &h, float &l)
@@ -369,7 +368,7 @@ __global__ void __launch_bounds__(kBlock, 4) k_resid_df(const __grid_constant__ 
                                                         const float4 *__restrict__ D2,
                                                         const double *__restrict__ x, float *__restrict__ y,
                                                         const double *__restrict__ b, double *__restrict__ part,
-                                                        int pstride, const int32_t *__restrict__ sexp,
+                                                        const int32_t *__restrict__ sexp,
                                                         const int32_t *__restrict__ act,
                                                         const float4 *__restrict__ SR2 = nullptr)
 {
@@ -477,7 +476,7 @@ __global__ void __launch_bounds__(kBlock, 4) k_resid_df(const __grid_constant__ 
     __syncthreads();
     if (threadIdx.x < NV) {
         for (int w = 1; w < kBlock / 32; ++w) df_add(sh[w][threadIdx.x].x, sh[w][threadIdx.x].y, nh, nl);
-        part[((int64_t)blockIdx.x * NV + threadIdx.x) * pstride] = double(nh) + double(nl);
+        part[threadIdx.x * (int64_t)gridDim.x + blockIdx.x] = double(nh) + double(nl);
     }
 }
 
@@ -505,14 +504,14 @@ __device__ __forceinline__ double f2d_pow2(float f, int e)
 // bits) is widened on the integer pipe and added in FP64: 8 FP64 instructions
 // per cell and variable, b to about 2^-48 relative at any magnitude.  A
 // difference that does not split (not finite) sends the thread to FP64.
-// part[row][v][1] gets the |b|^2 of the block's 32 C cells: the scaled high
+// Column 1 of part gets the |b|^2 of the block's 32 C cells: the scaled high
 // parts squared in FP32, the lanes' sums kept to 48 bits with a power of two of
 // their own, rescaled to the warp's largest at the end.  The four warps of a
 // block take the four variables of the same cells (the weights come from L1).
 template <int C>
 __global__ void __launch_bounds__(kW32) k_rhs_df(DeviceMesh d, const float *__restrict__ a0p,
                                                  const double *__restrict__ w, double *__restrict__ b,
-                                                 double *__restrict__ part, int pstride)
+                                                 double *__restrict__ part)
 {
     const int64_t T = d.T, c0 = blockIdx.x * (int64_t)(32 * C);
     const int lane = threadIdx.x & 31, v = threadIdx.x >> 5;
@@ -597,7 +596,7 @@ __global__ void __launch_bounds__(kW32) k_rhs_df(DeviceMesh d, const float *__re
     nl *= f;
     df_warp_sum(nh, nl);
     if (lane == 0)
-        part[((int64_t)blockIdx.x * NV + v) * pstride + 1] = (double(nh) + double(nl)) * pow2(m) * pow2(m);
+        part[(NV + v) * (int64_t)gridDim.x + blockIdx.x] = (double(nh) + double(nl)) * pow2(m) * pow2(m);
 }
 
 // Forward block-ILU relation for the listed rows (or all rows when rows == nullptr):
@@ -907,15 +906,14 @@ __global__ void __launch_bounds__(kBlock) k_ilu_bwd_sf(DeviceMesh d, const TP *_
 // cell block run together and read w once from HBM.  64 threads per variable,
 // four cells each (64 apart), all 40 loads issued before the sums (read-only
 // kernels need many bytes in flight); the warp sums then the two warps of a
-// variable give part[blk][v][k].  Fixed order: the sums are deterministic.
+// variable give part[k][v][blk].  Fixed order: the sums are deterministic.
 // TB: type of the stored basis.  An FP64 basis is multiplied and summed in
 // FP64; an FP32 basis (the inner cycles of the mixed mode) in FP32 within a
 // warp (640 products), each warp's sum then widened once and summed across
 // warps and blocks in FP64, so that the FP64 pipe sees almost nothing.
 template <typename TB>
 __global__ void __launch_bounds__(kDotThreads, 3) k_dots(int64_t T, int64_t nblk, const TB *__restrict__ V,
-                                                         const TB *__restrict__ w, double *__restrict__ part,
-                                                         int pstride)
+                                                         const TB *__restrict__ w, double *__restrict__ part)
 {
     constexpr int kPerVar = kDotThreads / NV;          // 64 threads (two warps) per variable
     constexpr int kCells = kBlock / kPerVar;           // 4 cells per thread
@@ -938,7 +936,7 @@ __global__ void __launch_bounds__(kDotThreads, 3) k_dots(int64_t T, int64_t nblk
         for (int o = 16; o > 0; o >>= 1) st += __shfl_down_sync(0xffffffffu, st, o);
         if (lane == 0) sh[warp] = double(st);
         __syncthreads();
-        if (threadIdx.x < NV) part[(b * NV + threadIdx.x) * pstride + k] = sh[2 * threadIdx.x] + sh[2 * threadIdx.x + 1];
+        if (threadIdx.x < NV) part[(k * NV + threadIdx.x) * nblk + b] = sh[2 * threadIdx.x] + sh[2 * threadIdx.x + 1];
         __syncthreads();
     }
 }
@@ -946,7 +944,7 @@ __global__ void __launch_bounds__(kDotThreads, 3) k_dots(int64_t T, int64_t nblk
 // The same for an FP32 basis ([dof][cell][variable]): a thread per cell, FP32
 // within a warp (160 products), FP64 across warps and blocks.
 __global__ void __launch_bounds__(kBlock) k_dots32(int64_t T, const float *__restrict__ V,
-                                                   const float *__restrict__ w, double *__restrict__ part, int pstride)
+                                                   const float *__restrict__ w, double *__restrict__ part)
 {
     __shared__ float sh[kBlock / 32][1][4];
     const int64_t b = blockIdx.x, i = b * kBlock + threadIdx.x;
@@ -961,7 +959,7 @@ __global__ void __launch_bounds__(kBlock) k_dots32(int64_t T, const float *__res
 #pragma unroll
             for (int v = 0; v < NV; ++v) sv[0][v] = fmaf(a[v], u[v], sv[0][v]);
         }
-    block_rows32<1>(sv, sh, part, pstride, k);
+    block_rows32<1>(sv, sh, part, k);
 }
 
 // w -= sum_{k<=j} c[s][k] V_k for running systems s = case * 4 + v (c: the
@@ -976,7 +974,7 @@ __global__ void __launch_bounds__(kBlock) k_dots32(int64_t T, const float *__res
 template <typename TB, int J = 0>
 __global__ void k_orth_update(DeviceMesh d, const TB *__restrict__ V, TB *__restrict__ w, int j,
                               const double *__restrict__ hc, int hstride, const int32_t *__restrict__ ctl, int ns,
-                              double *__restrict__ part, int pstride, int want_norm)
+                              double *__restrict__ part, int want_norm)
 {
     if (J > 0) j = J - 1;
     __shared__ double sh[32 * NV];
@@ -1056,218 +1054,7 @@ __global__ void k_orth_update(DeviceMesh d, const TB *__restrict__ V, TB *__rest
             block_sum4(nd, sh);
         }
         if (threadIdx.x == 0)
-            for (int v = 0; v < NV; ++v) part[(blockIdx.x * NV + v) * pstride + 0] = nd[v];
-    }
-}
-
-// Segmented sums over the partial-sum rows of each case (cell blocks,
-// seg[c]..seg[c+1]), fixed order:
-// out[s][q] (op) sum_{b in case(s)} part[b][v(s)][q], q < nq; op 0 store, 1 add,
-// 2 store sqrt.  With vn given, also co[s][q] = sum / vn[s][q]^2 (the
-// Gram-Schmidt coefficient of the unnormalised basis vector q).  One block of
-// kReduceThreads per (q, s): grid (nq, ns).  rs: partial-sum rows per cell block
-// (the FP64 solve writes several on small meshes).
-constexpr int kReduceThreads = 256;
-
-// sum of at(b) over b = b0 + t, b0 + t + kReduceThreads, ... < b1 (t the
-// thread), added in that order as the plain loop does, so the sum is the same
-// bit for bit; the loads are issued eight at a time, so a thread waits for a
-// few L2 round trips instead of one per term (a case's 4,000 cell blocks at 1M
-// are 16 terms per thread)
-template <typename F>
-__device__ __forceinline__ double strided_sum(int b0, int b1, F &&at)
-{
-    constexpr int U = 8;
-    double acc = 0.0;
-    for (int b = b0 + (int)threadIdx.x; b < b1; b += U * kReduceThreads) {
-        double t[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int bb = b + u * kReduceThreads;
-            t[u] = bb < b1 ? at(bb) : 0.0;
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-            if (b + u * kReduceThreads < b1) acc += t[u];
-    }
-    return acc;
-}
-
-__global__ void __launch_bounds__(kReduceThreads) k_reduce(const double *__restrict__ part,
-                                                           const int32_t *__restrict__ seg, int rs, int pstride,
-                                                           double *out, int ostride, int op,
-                                                           const double *__restrict__ vn = nullptr, int vstride = 0,
-                                                           double *co = nullptr, int cstride = 0)
-{
-    __shared__ double sh[kReduceThreads / 32];
-    const int q = blockIdx.x, sy = blockIdx.y, c = sy >> 2, v = sy & 3;
-    const int b0 = rs * seg[c], b1 = rs * seg[c + 1];
-    double acc = strided_sum(b0, b1, [&](int b) { return part[((int64_t)b * NV + v) * pstride + q]; });
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        acc = 0.0;
-        for (int w = 0; w < kReduceThreads / 32; ++w) acc += sh[w];
-        if (op == 0) out[sy * ostride + q] = acc;
-        else if (op == 1) out[sy * ostride + q] += acc;
-        else out[sy * ostride + q] = sqrt(acc);
-        if (co) {
-            const double n = vn[sy * vstride + q];
-            co[sy * cstride + q] = n > 0.0 ? acc / (n * n) : 0.0;
-        }
-    }
-}
-
-// Arnoldi index j of system sy (running systems only), by one warp: the new
-// Hessenberg column from the raw sums hc (plus h2 of the second Gram-Schmidt
-// pass, if given), the earlier rotations applied, a new rotation, the rotated
-// residual g and the stopping test.  An FP64 division holds the pipe for 285 ns
-// whatever the number of lanes in it, so the column's divisions are done by the
-// lanes together and only the chain of rotations (four FP64 instructions each)
-// is serial; one thread for all of it took 9.6 us per launch with the reduction
-// (5.2 us this way, at Arnoldi indices 0-9).
-__device__ __forceinline__ void givens_step(int sy, int j, int m, const double *__restrict__ hc,
-                                            const double *__restrict__ h2, int h2stride, int hstride, double hnext,
-                                            double *vn, double *H, double *cs, double *sn, double *g, int32_t *ctl,
-                                            int ns, const double *__restrict__ bnorm,
-                                            const double *__restrict__ beta, double rtol, double eta, int maxit,
-                                            double (*sh)[kMaxRestart + 1])
-{
-    const int lane = threadIdx.x & 31;
-    // Hessenberg column of the normalised basis: h_kj = <V_k, u_j> / (vn_k vn_j),
-    // h_{j+1,j} = |V_{j+1}| / vn_j; the new vector's norm becomes vn_{j+1}
-    double *h = sh[0], *c0 = sh[1], *s0 = sh[2], *hr = sh[3];
-    const double nj = vn[sy * (m + 1) + j];
-    for (int k = lane; k <= j + 1; k += 32) {
-        const double a = k <= j ? hc[sy * hstride + k] + (h2 ? h2[sy * h2stride + k] : 0.0) : hnext;
-        h[k] = a / (k <= j ? vn[sy * (m + 1) + k] * nj : nj);
-        if (k < j) {
-            c0[k] = cs[sy * m + k];
-            s0[k] = sn[sy * m + k];
-        }
-    }
-    __syncwarp();
-    const double gj = g[sy * (m + 1) + j], bn = bnorm[sy], be = beta[sy];
-    const int it = ctl[kCtlIters * ns + sy] + 1;
-    double t0 = h[0];
-#pragma unroll 4
-    for (int k = 0; k < j; ++k) {
-        const double c = c0[k], s = s0[k], t1 = h[k + 1];
-        const double u = c * t0 + s * t1;
-        t0 = c * t1 - s * t0;
-        if (lane == 0) hr[k] = u;
-    }
-    const double t1 = h[j + 1];
-    // hypot where the squares leave FP64's range
-    const double d2 = t0 * t0 + t1 * t1;
-    double id, dd;
-    if (d2 > 1e-280 && d2 < 1e280) {
-        id = rsqrt(d2);
-        dd = d2 * id;
-    } else {
-        dd = hypot(t0, t1);
-        id = dd > 0.0 ? 1.0 / dd : 0.0;
-    }
-    const double c = dd > 0.0 ? t0 * id : 1.0, s = dd > 0.0 ? t1 * id : 0.0;
-    __syncwarp();
-    for (int k = lane; k < j; k += 32) H[((int64_t)sy * (m + 1) + k) * m + j] = hr[k];
-    if (lane != 0) return;
-    H[((int64_t)sy * (m + 1) + j) * m + j] = dd;
-    vn[sy * (m + 1) + j + 1] = hnext;
-    cs[sy * m + j] = c;
-    sn[sy * m + j] = s;
-    g[sy * (m + 1) + j + 1] = -s * gj;
-    g[sy * (m + 1) + j] = c * gj;
-    ctl[kCtlJv * ns + sy] = j + 1;
-    ctl[kCtlIters * ns + sy] = it;
-    // stop the cycle at the target, or (mixed precision, eta > 0) once the inner
-    // residual has dropped by eta: the FP64 refinement residual then restarts it
-    const double gn = fabs(s * gj);
-    if (gn <= rtol * bn || gn <= eta * be || !(hnext > 0.0) || it >= maxit || j + 1 == m)
-        ctl[kCtlRunning * ns + sy] = 0;
-}
-
-// The last reduction of an Arnoldi index (|V_{j+1}| of system blockIdx.y, the
-// square root of the summed partials) followed by that system's Givens step,
-// which saves a launch per index.
-__global__ void __launch_bounds__(kReduceThreads) k_norm_givens(const double *__restrict__ part,
-                                                                const int32_t *__restrict__ seg, int rs, int pstride,
-                                                                int j, int m, const double *hc, int hstride,
-                                                                const double *h2, int h2stride, double *vn, double *H,
-                                                                double *cs, double *sn, double *g, int32_t *ctl,
-                                                                int ns, const double *__restrict__ bnorm,
-                                                                const double *__restrict__ beta, double rtol,
-                                                                double eta, int maxit)
-{
-    __shared__ double sh[kReduceThreads / 32];
-    __shared__ double shg[4][kMaxRestart + 1];
-    const int sy = blockIdx.y, c = sy >> 2, v = sy & 3;
-    if (!ctl[kCtlRunning * ns + sy]) return;
-    const int b0 = rs * seg[c], b1 = rs * seg[c + 1];
-    double acc = strided_sum(b0, b1, [&](int b) { return part[((int64_t)b * NV + v) * pstride]; });
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
-    __syncthreads();
-    if (threadIdx.x >= 32) return;
-    acc = 0.0;
-    for (int w = 0; w < kReduceThreads / 32; ++w) acc += sh[w];
-    givens_step(sy, j, m, hc, h2, h2stride, hstride, sqrt(acc), vn, H, cs, sn, g, ctl, ns, bnorm, beta, rtol, eta,
-                maxit, shg);
-}
-
-// End of a cycle, one warp per system: y = H^{-1} g on the first jv columns
-// (upper triangular after the rotations), column by column, the lanes holding
-// the right-hand side (the diagonal's reciprocals are formed together); then
-// y_k /= vn_k, the coefficients of the unnormalised preconditioned vectors.
-// With sexp given (FP32 basis, rows [current][next] exponents e of the scale
-// 2^-e of the first basis vector): y is also scaled by 2^-e of the current
-// cycle (the combination adds 2^e sum y_k Z_k, so its FP32 sums stay near unit
-// size), and the next residual's exponent comes from the cycle's estimate
-// |g_jv| of its norm (at least 1e-3 rtol |b|).
-// y32 (optional): an FP32 copy of the result for the FP32 combination.
-// One thread per system took 13-17 us for ten columns in two launches.
-constexpr int kSolveWarps = 4;      // systems per block
-__global__ void __launch_bounds__(32 * kSolveWarps)
-    k_cycle_solve(int m, const double *__restrict__ H, const double *__restrict__ g, double *__restrict__ y,
-                  const double *__restrict__ vn, const int32_t *__restrict__ ctl, int ns,
-                  const double *__restrict__ bnorm, double rtol, int32_t *sexp, float *y32)
-{
-    const int sy = blockIdx.x * kSolveWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (sy >= ns) return;
-    const int jv = ctl[kCtlJv * ns + sy];
-    if (jv <= 0) return;
-    // lane l holds the entries l and l + 32 (jv <= kMaxRestart = 64)
-    const double *Hs = H + (int64_t)sy * (m + 1) * m;
-    double rh[2], iv[2], sc[2];
-    const double f = sexp ? pow2(-sexp[sy]) : 1.0;
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-        const int k = lane + 32 * q;
-        rh[q] = k < jv ? g[sy * (m + 1) + k] : 0.0;
-        iv[q] = k < jv ? 1.0 / Hs[(int64_t)k * m + k] : 0.0;
-        sc[q] = k < jv ? f / vn[sy * (m + 1) + k] : 0.0;
-    }
-    for (int k = jv - 1; k >= 0; --k) {
-        const bool hi = k >= 32;
-        const double yk = __shfl_sync(0xffffffffu, hi ? rh[1] * iv[1] : rh[0] * iv[0], k & 31);
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            const int r = lane + 32 * q;
-            if (r < k) rh[q] = fma(-Hs[(int64_t)r * m + k], yk, rh[q]);
-        }
-    }
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-        const int k = lane + 32 * q;
-        if (k >= jv) continue;
-        const double yk = rh[q] * iv[q] * sc[q];
-        y[sy * m + k] = yk;
-        if (y32) y32[sy * m + k] = float(yk);
-    }
-    if (sexp && lane == 0) {
-        const double est = fmax(fabs(g[sy * (m + 1) + jv]), 1e-3 * rtol * bnorm[sy]);
-        if (est > 0.0 && est < 1e300) sexp[ns + sy] = max(-1000, ilogb(est));
+            for (int v = 0; v < NV; ++v) part[v * (int64_t)gridDim.x + blockIdx.x] = nd[v];
     }
 }
 
@@ -1370,105 +1157,12 @@ __global__ void k_warm(DeviceMesh d, double *__restrict__ x, double *__restrict_
     }
 }
 
-// Start (first = 1) or restart of every system: sums[s][0] = |r|^2,
-// sums[s][1] = |b|^2.  Systems of finished cases stay inactive.
-// Scale of the first residual of a solve: next exponent sexp[ns + s] = e with 2^-e B in [1, 2),
-// B = max(|b|, |b_prev|) (sums[s][1] = |b|^2, bnorm = |b| of the previous
-// solve, 0 at first): the warm start solved the previous system, so its
-// residual is of the order of B at most; e = 0 when B = 0.
-__global__ void k_sigma(const double *__restrict__ sums, int sstride, const double *__restrict__ bnorm,
-                        int32_t *sexp, int ns)
-{
-    const int sy = blockIdx.x * blockDim.x + threadIdx.x;
-    if (sy >= ns) return;
-    const double bn = fmax(sqrt(sums[sy * sstride + 1]), bnorm[sy]);
-    sexp[ns + sy] = bn > 0.0 && bn < 1e300 ? max(-1000, ilogb(bn)) : 0;
-}
-
-// sums[s][0] = |V_0|^2 of the stored first basis vector V_0 = 2^-e r (e: the
-// next exponent sexp[ns + s], which becomes the current one sexp[s]; e = 0
-// when sexp is NULL), sums[s][1] = |b|^2 (first solve of a step).
-__global__ void k_start(const double *__restrict__ sums, int sstride, double *bnorm, double *beta, double *vn, int m,
-                        int32_t *ctl, int ns, const int32_t *__restrict__ done, double rtol, int maxit, int first,
-                        int32_t *sexp = nullptr)
-{
-    const int sy = blockIdx.x * blockDim.x + threadIdx.x;
-    if (sy >= ns) return;
-    if (!first && !ctl[kCtlActive * ns + sy]) {
-        // a system that stopped keeps its solution, its residual and their norm
-        ctl[kCtlRunning * ns + sy] = 0;
-        ctl[kCtlJv * ns + sy] = 0;
-        return;
-    }
-    // |b| comes with the first residual; restarts reuse it
-    const double vn0 = sqrt(sums[sy * sstride + 0]);
-    double be = vn0;
-    if (sexp) {
-        be = vn0 * pow2(sexp[ns + sy]);
-        sexp[sy] = sexp[ns + sy];
-    }
-    const double bn = first ? sqrt(sums[sy * sstride + 1]) : bnorm[sy];
-    if (first) {
-        bnorm[sy] = bn;
-        ctl[kCtlIters * ns + sy] = 0;
-        ctl[kCtlActive * ns + sy] = !done[sy >> 2];
-    }
-    beta[sy] = be;
-    vn[sy * (m + 1)] = vn0;                            // V_0 = 2^-e r, v_0 = r / beta
-    const int act = ctl[kCtlActive * ns + sy] && bn > 0.0 && be > rtol * bn && ctl[kCtlIters * ns + sy] < maxit;
-    ctl[kCtlActive * ns + sy] = act;
-    ctl[kCtlRunning * ns + sy] = act;
-    ctl[kCtlJv * ns + sy] = 0;
-}
-
-// flags[0] = any active system, flags[1] = any running system (one block).
-__global__ void k_any(const int32_t *__restrict__ ctl, int ns, int32_t *flags)
-{
-    __shared__ int sh[2];
-    if (threadIdx.x < 2) sh[threadIdx.x] = 0;
-    __syncthreads();
-    int a = 0, r = 0;
-    for (int sy = threadIdx.x; sy < ns; sy += blockDim.x) {
-        a |= ctl[kCtlActive * ns + sy];
-        r |= ctl[kCtlRunning * ns + sy];
-    }
-    if (a) atomicOr(&sh[0], 1);
-    if (r) atomicOr(&sh[1], 1);
-    __syncthreads();
-    if (threadIdx.x < 2) flags[threadIdx.x] = sh[threadIdx.x];
-}
-
-// Condition of the device-controlled solve (one block): any system active
-// (which = 0, the cycle loop) or running (which = 1, the next Arnoldi index).
-// Thread 0 counts the run in ctr[slot] (slot >= 0) and sets the handle (set).
-// guard 1 starts the solve's cycle count; guard 2 counts a cycle and ends the
-// loop once more than limit cycles ran (each cycle takes at least one
-// iteration of every active system, which stops at maxit, so the limit
-// maxit + 1 is a backstop that a correct solve never reaches).
-__global__ void k_cond(const int32_t *__restrict__ ctl, int ns, int which, cudaGraphConditionalHandle h, int set,
-                       int64_t *ctr, int slot, int guard, int64_t limit)
-{
-    __shared__ int any;
-    if (threadIdx.x == 0) any = 0;
-    __syncthreads();
-    int a = 0;
-    for (int sy = threadIdx.x; sy < ns; sy += blockDim.x) a |= ctl[(which ? kCtlRunning : kCtlActive) * ns + sy];
-    if (a) atomicOr(&any, 1);
-    __syncthreads();
-    if (threadIdx.x != 0) return;
-    unsigned v = any ? 1u : 0u;
-    if (slot >= 0) ctr[slot] += 1;
-    if (guard == 1) ctr[kCtrGuard] = 0;
-    if (guard == 2 && ++ctr[kCtrGuard] > limit) v = 0u;
-    if (set) cudaGraphSetConditional(h, v);
-}
-
 // Condition of the device-controlled step loop (one block): any case not done,
 // and the loops of this launch (run_ctl[0]) below its limit (run_ctl[1]).
 // entry = 1 before the loop (no loops yet); otherwise at the end of a loop,
 // which it counts in run_ctl[0] and in ctr[kCtrRun].
-__global__ void k_run_cond(const int32_t *__restrict__ done, int n, int64_t *run_ctl, int64_t *ctr,
-                           cudaGraphConditionalHandle h, int entry)
+__global__ void k_run_cond(const int32_t *done, int n, int64_t *run_ctl, int64_t *ctr, cudaGraphConditionalHandle h,
+                           int entry)
 {
     __shared__ int any;
     if (threadIdx.x == 0) any = 0;
@@ -1487,15 +1181,8 @@ __global__ void k_run_cond(const int32_t *__restrict__ done, int n, int64_t *run
     cudaGraphSetConditional(h, (any && loops < run_ctl[1]) ? 1u : 0u);
 }
 
-// g = beta e_1 for active systems.
-__global__ void k_init_g(double *g, int m, const double *__restrict__ beta, const int32_t *__restrict__ ctl, int ns)
-{
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < ns * (m + 1); t += gridDim.x * blockDim.x) {
-        const int sy = t / (m + 1);
-        g[t] = (t % (m + 1) == 0 && ctl[kCtlActive * ns + sy]) ? beta[sy] : 0.0;
-    }
-}
-
+// x = 0 for systems with b = 0 (|b| compared as integers: an FP64 comparison per
+// thread took 10 us at 1M triangles)
 __global__ void k_zero_trivial(DeviceMesh d, double *__restrict__ x, const double *__restrict__ bnorm)
 {
     const int64_t T = d.T;
@@ -1504,7 +1191,8 @@ __global__ void k_zero_trivial(DeviceMesh d, double *__restrict__ x, const doubl
     const int c = d.blk_case[blockIdx.x];
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
-        if (bnorm[4 * c + v] > 0.0) continue;
+        const long long b = __double_as_longlong(bnorm[4 * c + v]);
+        if (b > 0 && b <= 0x7FF0000000000000ll) continue;      // |b| > 0
 #pragma unroll
         for (int l = 0; l < ND; ++l) x[(v * ND + l) * T + i] = 0.0;
     }
@@ -1513,13 +1201,15 @@ __global__ void k_zero_trivial(DeviceMesh d, double *__restrict__ x, const doubl
 // status[c] |= noconv for cases with a system that stopped above the tolerance,
 // and |= timeout for every active case if a wait of the sync-free ILU solves
 // gave up during the solve (sf_err, may be NULL); the solve count of the warm
-// start (k_warm) goes up by one
+// start (k_warm) goes up by one; in a run (acc) the solve's iterations it are
+// added to the sums acc
 __global__ void k_mark_noconv(const double *__restrict__ bnorm, const double *__restrict__ beta,
                               const int32_t *__restrict__ done, int ns, double rtol, int32_t *status,
-                              int64_t *nsolve, const int32_t *sf_err)
+                              int64_t *nsolve, const int32_t *sf_err, const int32_t *__restrict__ it, int64_t *acc)
 {
     const int sy = blockIdx.x * blockDim.x + threadIdx.x;
     if (sy == 0) ++*nsolve;
+    if (acc && sy < ns) acc[sy] += it[sy];
     if (sy >= ns || done[sy >> 2]) return;
     if (bnorm[sy] > 0.0 && beta[sy] > rtol * bnorm[sy]) atomicOr(&status[sy >> 2], kStatusNoConv);
     if (sf_err && *sf_err) atomicOr(&status[sy >> 2], kStatusTimeout);
@@ -1531,15 +1221,14 @@ inline unsigned nblocks(int64_t n) { return (unsigned)((n + kBlock - 1) / kBlock
 // (the inner cycles of the mixed mode rarely go further)
 template <typename TB>
 void launch_orth_update(const DeviceMesh &d, unsigned nb, cudaStream_t q, const TB *V, TB *w, int j,
-                        const double *hc, int hstride, const int32_t *ctl, int ns, double *part, int pstride,
-                        int want_norm)
+                        const double *hc, int hstride, const int32_t *ctl, int ns, double *part, int want_norm)
 {
     switch (j) {
-    case 0: k_orth_update<TB, 1><<<nb, kBlock, 0, q>>>(d, V, w, j, hc, hstride, ctl, ns, part, pstride, want_norm); break;
-    case 1: k_orth_update<TB, 2><<<nb, kBlock, 0, q>>>(d, V, w, j, hc, hstride, ctl, ns, part, pstride, want_norm); break;
-    case 2: k_orth_update<TB, 3><<<nb, kBlock, 0, q>>>(d, V, w, j, hc, hstride, ctl, ns, part, pstride, want_norm); break;
-    case 3: k_orth_update<TB, 4><<<nb, kBlock, 0, q>>>(d, V, w, j, hc, hstride, ctl, ns, part, pstride, want_norm); break;
-    default: k_orth_update<TB><<<nb, kBlock, 0, q>>>(d, V, w, j, hc, hstride, ctl, ns, part, pstride, want_norm);
+    case 0: k_orth_update<TB, 1><<<nb, kBlock, 0, q>>>(d, V, w, j, hc, hstride, ctl, ns, part, want_norm); break;
+    case 1: k_orth_update<TB, 2><<<nb, kBlock, 0, q>>>(d, V, w, j, hc, hstride, ctl, ns, part, want_norm); break;
+    case 2: k_orth_update<TB, 3><<<nb, kBlock, 0, q>>>(d, V, w, j, hc, hstride, ctl, ns, part, want_norm); break;
+    case 3: k_orth_update<TB, 4><<<nb, kBlock, 0, q>>>(d, V, w, j, hc, hstride, ctl, ns, part, want_norm); break;
+    default: k_orth_update<TB><<<nb, kBlock, 0, q>>>(d, V, w, j, hc, hstride, ctl, ns, part, want_norm);
     }
 }
 
@@ -1731,29 +1420,29 @@ gks_status solve64_shared_limit(int mm)
     return st;
 }
 
-void solve64_rhs(gks_mesh *m, int ps, cudaStream_t q)
+void solve64_rhs(gks_mesh *m, cudaStream_t q)
 {
     const DeviceMesh &d = m->d;
     with_cells(m->wk.c64, [&](auto C) {
-        k64_rhs<decltype(C)::value><<<rows64(m), kW64, 0, q>>>(d.T, d.nb, d.a0, m->wk.w, m->wk.b, m->wk.part, ps);
+        k64_rhs<decltype(C)::value><<<rows64(m), kW64, 0, q>>>(d.T, d.nb, d.a0, m->wk.w, m->wk.b, m->wk.part);
     });
 }
 
-void solve64_resid(gks_mesh *m, double *V0, const int32_t *act, int ps, cudaStream_t q)
+void solve64_resid(gks_mesh *m, double *V0, const int32_t *act, cudaStream_t q)
 {
     const DeviceMesh &d = m->d;
     with_cells(m->wk.c64, [&](auto C) {
         k64_resid<decltype(C)::value><<<rows64(m), kW64, 0, q>>>(d.T, d.nb, d.D, d.off, d.blk_case, act, m->wk.x,
-                                                               m->wk.b, V0, m->wk.part, ps);
+                                                               m->wk.b, V0, m->wk.part);
     });
 }
 
-void solve64_apply_dots(gks_mesh *m, const double *z, const double *V, double *y, int j, int ps, cudaStream_t q)
+void solve64_apply_dots(gks_mesh *m, const double *z, const double *V, double *y, int j, cudaStream_t q)
 {
     const DeviceMesh &d = m->d;
     with_cells(m->wk.c64, [&](auto C) {
         k64_apply_dots<decltype(C)::value><<<rows64(m), kW64, acc64(j, kAccStride), q>>>(
-            d.T, d.nb, d.D, d.off, d.blk_case, m->wk.ctl + kCtlRunning * m->wk.ns, z, y, V, j, m->wk.part, ps);
+            d.T, d.nb, d.D, d.off, d.blk_case, m->wk.ctl + kCtlRunning * m->wk.ns, z, y, V, j, m->wk.part);
     });
 }
 
@@ -1762,7 +1451,7 @@ void solve64_update_dots(gks_mesh *m, const double *V, double *w, int j, int ps,
     const DeviceMesh &d = m->d;
     with_cells(m->wk.c64, [&](auto C) {
         k64_update_dots<decltype(C)::value><<<rows64(m), kW64, acc64(j, kAccStride + 1), q>>>(
-            d.T, d.blk_case, m->wk.ctl + kCtlRunning * m->wk.ns, V, w, j, m->wk.hco, ps, m->wk.part, ps);
+            d.T, d.blk_case, m->wk.ctl + kCtlRunning * m->wk.ns, V, w, j, m->wk.hco, ps, m->wk.part);
     });
 }
 
@@ -1771,7 +1460,7 @@ void solve64_update_norm(gks_mesh *m, const double *V, double *w, int j, int ps,
     const DeviceMesh &d = m->d;
     with_cells(m->wk.c64, [&](auto C) {
         k64_update_norm<decltype(C)::value><<<rows64(m), kW64, 0, q>>>(
-            d.T, d.blk_case, m->wk.ctl + kCtlRunning * m->wk.ns, V, w, j, m->wk.hco, ps, m->wk.part, ps);
+            d.T, d.blk_case, m->wk.ctl + kCtlRunning * m->wk.ns, V, w, j, m->wk.hco, ps, m->wk.part);
     });
 }
 
@@ -1785,21 +1474,21 @@ gks_status precond(gks_mesh *m, const TR *src, double *dst, cudaStream_t s)
                                          {d.alr, d.exr, d.eyr, d.bdg});
 }
 
-void solve32_rhs(gks_mesh *m, int ps, cudaStream_t q)
+void solve32_rhs(gks_mesh *m, cudaStream_t q)
 {
     const unsigned g = (unsigned)(m->wk.nblk * (kRows64 / m->wk.c32));
     with_cells(m->wk.c32, [&](auto C) {
-        k_rhs_df<decltype(C)::value><<<g, kW32, 0, q>>>(m->d, m->d.a0p, m->wk.w, m->wk.b, m->wk.part, ps);
+        k_rhs_df<decltype(C)::value><<<g, kW32, 0, q>>>(m->d, m->d.a0p, m->wk.w, m->wk.b, m->wk.part);
     });
 }
 
-void solve32_apply_dots(gks_mesh *m, const float *z, const float *V, float *y, int j, int ps, cudaStream_t q)
+void solve32_apply_dots(gks_mesh *m, const float *z, const float *V, float *y, int j, cudaStream_t q)
 {
     const DeviceMesh &d = m->d;
     const Work &k = m->wk;
     const int32_t *run = k.ctl + kCtlRunning * k.ns;
     const float4 *op = reinterpret_cast<const float4 *>(d.op32);
-#define A32(J) k32_apply_dots<J><<<k.nblk, kBlock, 0, q>>>(d.T, d.nb, op, d.blk_case, run, z, y, V, j, k.part, ps)
+#define A32(J) k32_apply_dots<J><<<k.nblk, kBlock, 0, q>>>(d.T, d.nb, op, d.blk_case, run, z, y, V, j, k.part)
     switch (j) {     // the first four Arnoldi indices unrolled (the inner cycles rarely go further)
     case 0: A32(1); break;
     case 1: A32(2); break;
@@ -1816,7 +1505,7 @@ void solve32_update_norm(gks_mesh *m, const float *V, float *w, int j, int ps, c
     const DeviceMesh &d = m->d;
     const Work &k = m->wk;
     const int32_t *run = k.ctl + kCtlRunning * k.ns;
-#define U32(J) k32_update_norm<J><<<k.nblk, kBlock, 0, q>>>(d.T, d.blk_case, run, V, w, j, k.hco, ps, k.part, ps)
+#define U32(J) k32_update_norm<J><<<k.nblk, kBlock, 0, q>>>(d.T, d.blk_case, run, V, w, j, k.hco, ps, k.part)
     switch (j) {
     case 0: U32(1); break;
     case 1: U32(2); break;
@@ -1889,14 +1578,11 @@ gks_status precond32(gks_mesh *m, const TR *src, float *dst, cudaStream_t s)
                                        m->wk.r32, s, {d.alr32, d.exr32, d.eyr32, d.bdg32});
 }
 
-// Any active / any running system into the pinned host flags (no synchronisation).
+// The control kernels' words (any active, any running system) into the pinned
+// host flags (no synchronisation).
 gks_status enqueue_flags(gks_mesh *m, cudaStream_t s)
 {
-    const int slot = prof_start(m, kProfCtl, s);
-    k_any<<<1, kBlock, 0, s>>>(m->wk.ctl, m->wk.ns, m->wk.flags);
-    note_launch();
     GKS_CUDA(cudaMemcpyAsync(m->wk.h_flags, m->wk.flags, sizeof(int32_t) * 2, cudaMemcpyDeviceToHost, s));
-    prof_stop(m, slot, s);
     return GKS_OK;
 }
 
@@ -2074,56 +1760,40 @@ struct SolveEmbed {
 // The device-controlled solve as one executable graph (or, with emb, as nodes
 // of the caller's graph):
 //   start; c = any active
-//   while (c) { i_0 = any running
-//               if (i_0) { Arnoldi 0; i_1 = any running
-//                          if (i_1) { Arnoldi 1; ... if (i_{m-1}) { Arnoldi m-1 } } }
+//   while (c) { count the cycle; Arnoldi 0; i_1 = any running
+//               if (i_1) { Arnoldi 1; ... if (i_{m-1}) { Arnoldi m-1 } }
 //               restart; c = any active (and within the cycle limit) }
-// The condition kernels replace the host flags of the per-part graphs; the
-// conditions of an index are only evaluated once the one before it has run.
+// (a cycle starts with every active system running).  The conditions replace the
+// host flags of the per-part graphs; those of an index are only evaluated once
+// the one before it has run.
 template <typename SB, typename IB, typename RB>
 gks_status build_whole(gks_mesh *m, cudaStream_t s, SB &&start_body, IB &&iter_body, RB &&restart_body,
                        SolveEmbed *emb = nullptr)
 {
     SolveGraphs &G = *m->graphs;
     Work &k = m->wk;
-    const int ns = k.ns, mm = k.m;
+    const int mm = k.m;
     const int64_t limit = (int64_t)m->cfg.gmres_maxit + 1;
     if (const gks_status r = ensure_counters(m, s); r != GKS_OK) return r;
     int64_t *ctr = G.ctr;
-    const int32_t *ctl = k.ctl;
+    uint32_t *ticket = reinterpret_cast<uint32_t *>(k.flags + 3);
     cudaGraph_t top = emb ? emb->g : nullptr;
     if (!emb) GKS_CUDA(cudaGraphCreate(&top, 0));
     const size_t ndep = emb && emb->dep ? 1 : 0;
     gks_status st = GKS_OK;
     std::vector<int64_t> nl_iter(mm, 0);
-    int64_t nl_start = 0, nl_c0 = 0, nl_restart = 0;
+    int64_t nl_start = 0, nl_restart = 0;
     do {
-        cudaGraphConditionalHandle h_outer, h_next;
+        cudaGraphConditionalHandle h_outer, h_next = 0;
         if (cudaGraphConditionalHandleCreate(&h_outer, top, 0, 0) != cudaSuccess) { st = GKS_ECUDA; break; }
         cudaGraphNode_t sink, wnode, inode;
         cudaGraph_t wbody, ibody;
         st = capture_into(m, top, ndep ? &emb->dep : nullptr, ndep, &sink, &nl_start, [&](cudaStream_t q) -> gks_status {
-            gks_status r = start_body(q);
-            if (r != GKS_OK) return r;
-            k_cond<<<1, kBlock, 0, q>>>(ctl, ns, 0, h_outer, 1, ctr, -1, 1, limit); note_launch();
-            return GKS_OK;
+            return start_body(q, Cond{h_outer, ctr, 0, nullptr, ticket, 1, -1, 1});
         });
         if (st != GKS_OK || (st = add_cond(top, sink, h_outer, cudaGraphCondTypeWhile, &wnode, &wbody)) != GKS_OK)
             break;
-        if (cudaGraphConditionalHandleCreate(&h_next, wbody, 0, 0) != cudaSuccess) { st = GKS_ECUDA; break; }
-        st = capture_into(m, wbody, nullptr, 0, &sink, &nl_c0, [&](cudaStream_t q) -> gks_status {
-            k_cond<<<1, kBlock, 0, q>>>(ctl, ns, 1, h_next, 1, ctr, -1, 0, limit); note_launch();
-            return GKS_OK;
-        });
-        if (st != GKS_OK || (st = add_cond(wbody, sink, h_next, cudaGraphCondTypeIf, &inode, &ibody)) != GKS_OK)
-            break;
-        st = capture_into(m, wbody, &inode, 1, &sink, &nl_restart, [&](cudaStream_t q) -> gks_status {
-            gks_status r = restart_body(q);
-            if (r != GKS_OK) return r;
-            k_cond<<<1, kBlock, 0, q>>>(ctl, ns, 0, h_outer, 1, ctr, kCtrCycles, 2, limit); note_launch();
-            return GKS_OK;
-        });
-        if (st != GKS_OK) break;
+        ibody = wbody;
         for (int j = 0; j < mm && st == GKS_OK; ++j) {
             const bool more = j + 1 < mm;
             if (more && cudaGraphConditionalHandleCreate(&h_next, ibody, 0, 0) != cudaSuccess) {
@@ -2131,12 +1801,26 @@ gks_status build_whole(gks_mesh *m, cudaStream_t s, SB &&start_body, IB &&iter_b
                 break;
             }
             st = capture_into(m, ibody, nullptr, 0, &sink, &nl_iter[j], [&](cudaStream_t q) -> gks_status {
-                gks_status r = iter_body(q, j);
-                if (r != GKS_OK) return r;
-                k_cond<<<1, kBlock, 0, q>>>(ctl, ns, 1, h_next, more ? 1 : 0, ctr, j, 0, limit); note_launch();
-                return GKS_OK;
+                if (j == 0) {
+                    k_cycle_count<<<1, 32, 0, q>>>(ctr);
+                    note_launch();
+                }
+                return iter_body(q, j, Cond{h_next, ctr, 0, nullptr, ticket, more ? 1 : 0, j, 0});
             });
-            if (st == GKS_OK && more) st = add_cond(ibody, sink, h_next, cudaGraphCondTypeIf, &inode, &ibody);
+            if (st == GKS_OK && more) {
+                cudaGraph_t next;
+                st = add_cond(ibody, sink, h_next, cudaGraphCondTypeIf, &inode, &next);
+                ibody = next;
+            } else {
+                inode = sink;
+            }
+            if (st == GKS_OK && j == 0) {
+                // the rest of the loop's body after the first index (and those nested behind it)
+                cudaGraphNode_t tail;
+                st = capture_into(m, wbody, &inode, 1, &tail, &nl_restart, [&](cudaStream_t q) -> gks_status {
+                    return restart_body(q, Cond{h_outer, ctr, limit, nullptr, ticket, 1, -1, 0});
+                });
+            }
         }
         if (st != GKS_OK) break;
         if (emb) {
@@ -2150,21 +1834,22 @@ gks_status build_whole(gks_mesh *m, cudaStream_t s, SB &&start_body, IB &&iter_b
     cudaGetLastError();
     if (st != GKS_OK) return st;
     G.whole_start_launches = nl_start;
-    G.whole_cycle_launches = nl_c0 + nl_restart;
+    nl_iter[0] -= 1;                                     // k_cycle_count: counted with the cycle
+    G.whole_cycle_launches = nl_restart + 1;
     G.whole_iter_launches = nl_iter;
     return GKS_OK;
 }
 
-// part[blk][v][k] = partial <V_k, w>, k <= j, per cell block
+// part[k][v][blk] = partial <V_k, w>, k <= j, per cell block
 template <typename TB>
-gks_status dots(gks_mesh *m, const TB *V, const TB *w, int j, double *part, int ps, cudaStream_t s)
+gks_status dots(gks_mesh *m, const TB *V, const TB *w, int j, double *part, cudaStream_t s)
 {
     const int64_t nblk = m->wk.nblk;
     if constexpr (std::is_same_v<TB, float>) {
-        k_dots32<<<dim3((unsigned)nblk, (unsigned)(j + 1)), kBlock, 0, s>>>(m->d.T, V, w, part, ps);
+        k_dots32<<<dim3((unsigned)nblk, (unsigned)(j + 1)), kBlock, 0, s>>>(m->d.T, V, w, part);
     } else {
         const dim3 g((unsigned)(j + 1), (unsigned)std::min<int64_t>(nblk, kDotMaxTiles));
-        k_dots<TB><<<g, kDotThreads, 0, s>>>(m->d.T, nblk, V, w, part, ps);
+        k_dots<TB><<<g, kDotThreads, 0, s>>>(m->d.T, nblk, V, w, part);
     }
     note_launch();
     GKS_CUDA(cudaGetLastError());
@@ -2184,7 +1869,7 @@ inline unsigned sblocks(int n) { return (unsigned)((n + 127) / 128); }
 // closing kernel are built into the caller's graph instead of run.
 template <typename TB>
 gks_status cls_solve_t(gks_mesh *m, TB *V, cudaStream_t s, int32_t *iters, double *relres, int32_t *converged,
-                       SolveEmbed *emb = nullptr)
+                       bool acc, SolveEmbed *emb = nullptr)
 {
     DeviceMesh &d = m->d;
     Work &k = m->wk;
@@ -2220,19 +1905,19 @@ gks_status cls_solve_t(gks_mesh *m, TB *V, cudaStream_t s, int32_t *iters, doubl
     auto spmv64 = [&](cudaStream_t q, const double *xs, TB *y, int mode, const double *bb, const int32_t *se) {
         if (d.alr)
             k_spmv<double, double, TB, true><<<nb, kBlock, 0, q>>>(d, d.D, d.alpha, d.ex, d.ey, xs, y, mode, bb,
-                                                                   k.part, ps, se, d.alr, d.exr, d.eyr, d.bdg);
+                                                                   k.part, se, d.alr, d.exr, d.eyr, d.bdg);
         else
             k_spmv<double, double, TB, false><<<nb, kBlock, 0, q>>>(d, d.D, d.alpha, d.ex, d.ey, xs, y, mode, bb,
-                                                                    k.part, ps, se);
+                                                                    k.part, se);
     };
     auto spmv32 = [&](cudaStream_t q, const float *xs, TB *y) {
         if (d.alr32)
             k_spmv<float, float, TB, true><<<nb, kBlock, 0, q>>>(d, d.D32, d.alpha32, d.ex32, d.ey32, xs, y, 0,
-                                                                 nullptr, nullptr, 0, nullptr, d.alr32, d.exr32,
+                                                                 nullptr, nullptr, nullptr, d.alr32, d.exr32,
                                                                  d.eyr32, d.bdg32);
         else
             k_spmv<float, float, TB, false><<<nb, kBlock, 0, q>>>(d, d.D32, d.alpha32, d.ex32, d.ey32, xs, y, 0,
-                                                                  nullptr, nullptr, 0);
+                                                                  nullptr, nullptr);
     };
     // the FP32-basis solve forms b in double-FP32 arithmetic when the weights fit
     const bool rhs_df = std::is_same<TB, float>::value && d.a0p;
@@ -2247,15 +1932,15 @@ gks_status cls_solve_t(gks_mesh *m, TB *V, cudaStream_t s, int32_t *iters, doubl
     auto residual = [&](cudaStream_t q, bool first) -> gks_status {
         const int32_t *act = first ? nullptr : k.ctl + kCtlActive * ns;
         if (C64) {
-            solve64_resid(m, reinterpret_cast<double *>(V), act, ps, q);
+            solve64_resid(m, reinterpret_cast<double *>(V), act, q);
         } else if (std::is_same<TB, float>::value && d.D2) {
             float *v0 = reinterpret_cast<float *>(V);
             const float4 *d2 = reinterpret_cast<const float4 *>(d.D2);
             if (d.SR2)
-                k_resid_df<true><<<kResidRows * nb, kBlock, 0, q>>>(d, d2, k.x, v0, k.b, k.part, ps, sxn, act,
+                k_resid_df<true><<<rs_res * nb, kBlock, 0, q>>>(d, d2, k.x, v0, k.b, k.part, sxn, act,
                                                                    reinterpret_cast<const float4 *>(d.SR2));
             else
-                k_resid_df<false><<<kResidRows * nb, kBlock, 0, q>>>(d, d2, k.x, v0, k.b, k.part, ps, sxn, act);
+                k_resid_df<false><<<rs_res * nb, kBlock, 0, q>>>(d, d2, k.x, v0, k.b, k.part, sxn, act);
             note_launch();
         } else {
             spmv64(q, k.x, V, 1, k.b, sxn);
@@ -2264,46 +1949,52 @@ gks_status cls_solve_t(gks_mesh *m, TB *V, cudaStream_t s, int32_t *iters, doubl
         GKS_CUDA(cudaGetLastError());
         return GKS_OK;
     };
+    const Krylov kry = {mm, ns, k.H, k.cs, k.sn, k.g, k.y, k.vn, mixed ? k.y32 : nullptr, k.ctl, k.bnorm, k.beta, sx,
+                        rtol, eta, maxit};
+    auto cycle_begin = [&](cudaStream_t q, int first, const Cond &cd) {
+        k_cycle_begin<<<ns, kReduceThreads, 0, q>>>(kry, k.part, rs_res * (int64_t)nb, d.case_blk, rs_res,
+                                                        k.hcol + 1, ps, k.done, first, cd);
+        note_launch();
+    };
     // the three fixed launch sequences (the per-part graphs end each with the
-    // flags for the host, the whole-solve graph with a condition kernel)
-    auto start_body = [&](cudaStream_t q) -> gks_status {
+    // flags for the host; in the whole-solve graph their last kernels set the
+    // conditions)
+    uint32_t *ticket = reinterpret_cast<uint32_t *>(k.flags + 3);
+    const Cond host_active = {0, nullptr, 0, k.flags, ticket, 0, -1, 0};
+    const Cond host_running = {0, nullptr, 0, k.flags + 1, ticket, 0, -1, 0};
+    auto start_body = [&](cudaStream_t q, const Cond &cd) -> gks_status {
         int slot = prof_start(m, kProfCtl, q);
         if (m->cfg.precond == GKS_PC_ILU_EXACT) {
             k_sf_begin<<<1, 32, 0, q>>>(k.sf_ctl, 1);      // a new solve: clear the wait error
             note_launch();
         }
         if (C64) {
-            solve64_rhs(m, ps, q);
+            solve64_rhs(m, q);
         } else if (rhs_df) {
-            solve32_rhs(m, ps, q);
+            solve32_rhs(m, q);
         } else {
-            k_rhs<<<nb, kBlock, 0, q>>>(d, k.w, k.b, k.part, ps);
+            k_rhs<<<nb, kBlock, 0, q>>>(d, k.w, k.b, k.part);
             note_launch();
         }
         if (sx) {
             // the FP32 basis stores its first vector scaled by a power of two 2^-e
-            k_reduce<<<dim3(1, ns), kReduceThreads, 0, q>>>(k.part + 1, d.case_blk, rs_rhs, ps, k.hcol + 1, ps, 0);
+            k_sigma<<<ns, kReduceThreads, 0, q>>>(k.part, rs_rhs * (int64_t)nb, d.case_blk, rs_rhs, k.hcol + 1,
+                                                      ps, k.bnorm, k.sexp, ns);
             note_launch();
-            k_sigma<<<sblocks(ns), 128, 0, q>>>(k.hcol, ps, k.bnorm, k.sexp, ns); note_launch();
         }
         prof_stop(m, slot, q);
         slot = prof_start(m, kProfResid, q);
         // residual r = b - K x, written straight into the basis slot V_0 (v_0 = V_0 / beta)
         if (const gks_status r = residual(q, true); r != GKS_OK) return r;
-        k_reduce<<<dim3(sx ? 1 : 2, ns), kReduceThreads, 0, q>>>(k.part, d.case_blk, rs_res, ps, k.hcol, ps, 0);
-        note_launch();
         prof_stop(m, slot, q);
         slot = prof_start(m, kProfCtl, q);
-        k_start<<<sblocks(ns), 128, 0, q>>>(k.hcol, ps, k.bnorm, k.beta, k.vn, mm, k.ctl, ns, k.done, rtol, maxit,
-                                             1, sx);
-        note_launch();
+        cycle_begin(q, 1, cd);
         k_zero_trivial<<<nb, kBlock, 0, q>>>(d, k.x, k.bnorm); note_launch();
-        k_init_g<<<sblocks(ns * (mm + 1)), 128, 0, q>>>(k.g, mm, k.beta, k.ctl, ns); note_launch();
         prof_stop(m, slot, q);
         GKS_CUDA(cudaGetLastError());
         return GKS_OK;
     };
-    auto iter_body = [&](cudaStream_t q, int j) -> gks_status {
+    auto iter_body = [&](cudaStream_t q, int j, const Cond &cd) -> gks_status {
         TB *vj = V + j * vs, *vj1 = V + (j + 1) * vs;
         gks_status st;
         int slot = prof_start(m, kProfIlu, q);
@@ -2314,13 +2005,13 @@ gks_status cls_solve_t(gks_mesh *m, TB *V, cudaStream_t s, int32_t *iters, doubl
         slot = prof_start(m, kProfSpmv, q);
         if (fused_dots) {
             solve32_apply_dots(m, k.Z32 + j * vs, reinterpret_cast<const float *>(V), reinterpret_cast<float *>(vj1),
-                               j, ps, q);
+                               j, q);
         } else if (mixed) {
             spmv32(q, k.Z32 + j * vs, vj1);
         } else if (C64) {
             // with the first Gram-Schmidt products
             solve64_apply_dots(m, k.Z + j * vs, reinterpret_cast<const double *>(V), reinterpret_cast<double *>(vj1),
-                               j, ps, q);
+                               j, q);
         } else {
             spmv64(q, k.Z + j * vs, vj1, 0, nullptr, nullptr);
         }
@@ -2329,45 +2020,45 @@ gks_status cls_solve_t(gks_mesh *m, TB *V, cudaStream_t s, int32_t *iters, doubl
         slot = prof_start(m, kProfOrth, q);
         // classical Gram-Schmidt: twice in FP64 mode; once in the mixed mode, whose
         // cycles only reduce the residual by inner_rtol before an FP64 restart
-        if (!fused_dots && !C64 && (st = dots<TB>(m, V, vj1, j, k.part, ps, q)) != GKS_OK) return st;
-        k_reduce<<<dim3(j + 1, ns), kReduceThreads, 0, q>>>(k.part, d.case_blk, rs, ps, k.hcol, ps, 0, k.vn, mm + 1,
-                                                             k.hco, ps);
+        if (!fused_dots && !C64 && (st = dots<TB>(m, V, vj1, j, k.part, q)) != GKS_OK) return st;
+        k_reduce<<<dim3(j + 1, ns), kReduceThreads, 0, q>>>(k.part, rs * (int64_t)nb, d.case_blk, rs, k.hcol, ps, k.vn,
+                                                             mm + 1, k.hco, ps);
         note_launch();
         if (C64) {
             solve64_update_dots(m, reinterpret_cast<const double *>(V), reinterpret_cast<double *>(vj1), j, ps, q);
         } else if (fused_dots) {
             solve32_update_norm(m, reinterpret_cast<const float *>(V), reinterpret_cast<float *>(vj1), j, ps, q);
         } else {
-            launch_orth_update<TB>(d, nb, q, V, vj1, j, k.hco, ps, k.ctl, ns, k.part, ps, mixed ? 1 : 0);
+            launch_orth_update<TB>(d, nb, q, V, vj1, j, k.hco, ps, k.ctl, ns, k.part, mixed ? 1 : 0);
             note_launch();
         }
         if (!mixed) {
             // the second pass
-            if (!C64 && (st = dots<TB>(m, V, vj1, j, k.part, ps, q)) != GKS_OK) return st;
-            k_reduce<<<dim3(j + 1, ns), kReduceThreads, 0, q>>>(k.part, d.case_blk, rs, ps, k.y, mm, 0, k.vn, mm + 1,
-                                                                 k.hco, ps);
+            if (!C64 && (st = dots<TB>(m, V, vj1, j, k.part, q)) != GKS_OK) return st;
+            k_reduce<<<dim3(j + 1, ns), kReduceThreads, 0, q>>>(k.part, rs * (int64_t)nb, d.case_blk, rs, k.y, mm, k.vn,
+                                                                 mm + 1, k.hco, ps);
             note_launch();
             if (C64) {
                 solve64_update_norm(m, reinterpret_cast<const double *>(V), reinterpret_cast<double *>(vj1), j, ps, q);
             } else {
-                launch_orth_update<TB>(d, nb, q, V, vj1, j, k.hco, ps, k.ctl, ns, k.part, ps, 1);
+                launch_orth_update<TB>(d, nb, q, V, vj1, j, k.hco, ps, k.ctl, ns, k.part, 1);
                 note_launch();
             }
         }
-        // |V_{j+1}| and the Givens step of every system
-        k_norm_givens<<<dim3(1, ns), kReduceThreads, 0, q>>>(k.part, d.case_blk, rs, ps, j, mm, k.hcol, ps,
-                                                              mixed ? nullptr : k.y, mm, k.vn, k.H, k.cs, k.sn, k.g,
-                                                              k.ctl, ns, k.bnorm, k.beta, rtol, eta, maxit);
+        // |V_{j+1}| and the Givens step of every system (and the end of a single mesh's cycle)
+        k_arnoldi_end<<<ns, kReduceThreads, 0, q>>>(kry, k.part, rs * (int64_t)nb, d.case_blk, rs, j, k.hcol, ps,
+                                                        mixed ? nullptr : k.y, mm, cd);
         note_launch();
         prof_stop(m, slot, q);
         GKS_CUDA(cudaGetLastError());
         return GKS_OK;
     };
-    auto restart_body = [&](cudaStream_t q) -> gks_status {
+    auto restart_body = [&](cudaStream_t q, const Cond &cd) -> gks_status {
         int slot = prof_start(m, kProfCorr, q);
-        k_cycle_solve<<<(ns + kSolveWarps - 1) / kSolveWarps, 32 * kSolveWarps, 0, q>>>(
-            mm, k.H, k.g, k.y, k.vn, k.ctl, ns, k.bnorm, rtol, sx, mixed ? k.y32 : nullptr);
-        note_launch();
+        if (m->n_case > 1) {
+            k_cycle_solve<<<(ns + kSolveWarps - 1) / kSolveWarps, 32 * kSolveWarps, 0, q>>>(kry);
+            note_launch();
+        }
         if (mixed)
             k_combine32<<<NV * nb, kBlock, 0, q>>>(d, k.Z32, k.y32, mm, k.ctl, ns, k.x, sx);
         else if (C64)
@@ -2379,21 +2070,17 @@ gks_status cls_solve_t(gks_mesh *m, TB *V, cudaStream_t s, int32_t *iters, doubl
         prof_stop(m, slot, q);
         slot = prof_start(m, kProfResid, q);
         if (const gks_status r = residual(q, false); r != GKS_OK) return r;
-        k_reduce<<<dim3(1, ns), kReduceThreads, 0, q>>>(k.part, d.case_blk, rs_res, ps, k.hcol, ps, 0); note_launch();
         prof_stop(m, slot, q);
         slot = prof_start(m, kProfCtl, q);
-        k_start<<<sblocks(ns), 128, 0, q>>>(k.hcol, ps, k.bnorm, k.beta, k.vn, mm, k.ctl, ns, k.done, rtol, maxit,
-                                             0, sx);
-        note_launch();
-        k_init_g<<<sblocks(ns * (mm + 1)), 128, 0, q>>>(k.g, mm, k.beta, k.ctl, ns); note_launch();
+        cycle_begin(q, 0, cd);
         prof_stop(m, slot, q);
         GKS_CUDA(cudaGetLastError());
         return GKS_OK;
     };
     auto with_flags = [&](cudaStream_t q, gks_status r) { return r != GKS_OK ? r : enqueue_flags(m, q); };
-    auto start_part = [&](cudaStream_t q) { return with_flags(q, start_body(q)); };
-    auto iter_part = [&](cudaStream_t q, int j) { return with_flags(q, iter_body(q, j)); };
-    auto restart_part = [&](cudaStream_t q) { return with_flags(q, restart_body(q)); };
+    auto start_part = [&](cudaStream_t q) { return with_flags(q, start_body(q, host_active)); };
+    auto iter_part = [&](cudaStream_t q, int j) { return with_flags(q, iter_body(q, j, host_running)); };
+    auto restart_part = [&](cudaStream_t q) { return with_flags(q, restart_body(q, host_active)); };
 
     const bool use_graph = prepare_graphs(m);
     SolveGraphs *G = use_graph ? m->graphs : nullptr;
@@ -2408,7 +2095,8 @@ gks_status cls_solve_t(gks_mesh *m, TB *V, cudaStream_t s, int32_t *iters, doubl
         int64_t nl = 0;
         st = capture_into(m, emb->g, &emb->sink, 1, &emb->sink, &nl, [&](cudaStream_t q) -> gks_status {
             k_mark_noconv<<<sblocks(ns), 128, 0, q>>>(k.bnorm, k.beta, k.done, ns, rtol, k.status, k.nsolve,
-                                                         m->cfg.precond == GKS_PC_ILU_EXACT ? k.sf_ctl + 3 : nullptr);
+                                                      m->cfg.precond == GKS_PC_ILU_EXACT ? k.sf_ctl + 3 : nullptr,
+                                                      k.ctl + kCtlIters * ns, k.iters_acc);
             note_launch();
             GKS_CUDA(cudaGetLastError());
             return GKS_OK;
@@ -2451,7 +2139,8 @@ gks_status cls_solve_t(gks_mesh *m, TB *V, cudaStream_t s, int32_t *iters, doubl
         m->prof.residuals += 1;
     }
     k_mark_noconv<<<sblocks(ns), 128, 0, s>>>(k.bnorm, k.beta, k.done, ns, rtol, k.status, k.nsolve,
-                                              m->cfg.precond == GKS_PC_ILU_EXACT ? k.sf_ctl + 3 : nullptr);
+                                              m->cfg.precond == GKS_PC_ILU_EXACT ? k.sf_ctl + 3 : nullptr,
+                                              k.ctl + kCtlIters * ns, acc ? k.iters_acc : nullptr);
     note_launch();
     if (iters || relres || converged) {
         std::vector<int32_t> it(ns);
@@ -2521,19 +2210,17 @@ gks_status build_run(gks_mesh *m, cudaStream_t s)
         if (st != GKS_OK || (st = add_cond(top, sink, h, cudaGraphCondTypeWhile, &wnode, &body)) != GKS_OK) break;
         st = capture_into(m, body, nullptr, 0, &sink, &nl_a, [&](cudaStream_t q) -> gks_status {
             gks_status r;
-            if ((r = launch_cfl_dt(m, k.w, k.dt, q)) != GKS_OK) return r;
-            if ((r = launch_clip_only(m, q)) != GKS_OK) return r;
+            if ((r = launch_cfl_dt(m, k.w, k.dt, q, true)) != GKS_OK) return r;
             return launch_warm(m, q);
         });
         if (st != GKS_OK) break;
         e.g = body;
         e.dep = sink;
-        st = k.V32 ? cls_solve_t<float>(m, k.V32, s, nullptr, nullptr, nullptr, &e)
-                   : cls_solve_t<double>(m, k.V, s, nullptr, nullptr, nullptr, &e);
+        st = k.V32 ? cls_solve_t<float>(m, k.V32, s, nullptr, nullptr, nullptr, true, &e)
+                   : cls_solve_t<double>(m, k.V, s, nullptr, nullptr, nullptr, true, &e);
         if (st != GKS_OK) break;
         st = capture_into(m, body, &e.sink, 1, &sink, &nl_b, [&](cudaStream_t q) -> gks_status {
             gks_status r;
-            if ((r = launch_acc_iters(m, q)) != GKS_OK) return r;
             if (m->cfg.limiter && (r = launch_limiter(m, k.w, k.x, q)) != GKS_OK) return r;
             if ((r = launch_flux(m, k.w, m->cfg.limiter ? k.xl : k.x, 0.0, k.dt, k.flux, q)) != GKS_OK) return r;
             if ((r = launch_update(m, k.w, k.flux, q)) != GKS_OK) return r;
@@ -2558,12 +2245,12 @@ gks_status build_run(gks_mesh *m, cudaStream_t s)
 
 }  // namespace
 
-gks_status cls_solve(gks_mesh *m, cudaStream_t s, int32_t *iters, double *relres, int32_t *converged)
+gks_status cls_solve(gks_mesh *m, cudaStream_t s, int32_t *iters, double *relres, int32_t *converged, bool acc)
 {
     Work &k = m->wk;
     if (const gks_status st = launch_warm(m, s); st != GKS_OK) return st;
-    return k.V32 ? cls_solve_t<float>(m, k.V32, s, iters, relres, converged)
-                 : cls_solve_t<double>(m, k.V, s, iters, relres, converged);
+    return k.V32 ? cls_solve_t<float>(m, k.V32, s, iters, relres, converged, acc)
+                 : cls_solve_t<double>(m, k.V, s, iters, relres, converged, acc);
 }
 
 void plan_solve(gks_mesh *m, int *rows)
@@ -2571,7 +2258,7 @@ void plan_solve(gks_mesh *m, int *rows)
     const int c = cells64(m->d.T);
     if (m->cfg.precision == GKS_FP64) m->wk.c64 = c;
     else m->wk.c32 = c;
-    // the mixed path's residual has a row per quarter of a cell block
+    // the mixed path's residual has rows of its own
     *rows = std::max(kRows64 / c, m->cfg.precision == GKS_MIXED ? kResidRows : 1);
 }
 

@@ -145,7 +145,7 @@ struct Work {
     double *Z = nullptr;             // [m][20][T] M^{-1} V_k (FP64 path)
     float *Z32 = nullptr;            // [m][20][T] M^{-1} V_k (mixed path)
     double *flux = nullptr;          // [4][F]
-    double *part = nullptr;          // [nblk * rows][4][m+2] partial sums (rows per cell block: plan_solve)
+    double *part = nullptr;          // [m+2][4][nblk * rows] partial sums (rows per cell block: plan_solve)
     double *dpart = nullptr;         // [nblk][4] partial minima / sums
     // small GMRES state (device), one row per system
     double *H = nullptr;             // [ns][m+1][m]  (Givens-rotated Hessenberg)
@@ -160,7 +160,7 @@ struct Work {
     int32_t *ctl = nullptr;          // [kCtlFields][ns]
     int32_t *sexp = nullptr;         // [2][ns] FP32 basis: first basis vector stored as 2^-e r; e of the
                                      //         current cycle, then that of the next residual
-    int32_t *flags = nullptr;        // [4]: any active, any running, all cases done
+    int32_t *flags = nullptr;        // [4]: any active, any running, (unused), blocks done of a control kernel
     double *dt = nullptr;            // [ncase] step of each case (0: case inactive)
     double *tcase = nullptr;         // [ncase] time reached
     double *tfinal = nullptr;        // [ncase] end time (<= 0: none)
@@ -284,7 +284,9 @@ void free_mesh(gks_mesh *m);
 // CLS reconstruction (gks_cls.cu): rhs from m->wk.w, solution in m->wk.x.
 // Per system (case * 4 + variable, may be NULL): iterations, relative residuals;
 // *converged = 1 if every active system met the tolerance.
-gks_status cls_solve(gks_mesh *m, cudaStream_t s, int32_t *iters, double *relres, int32_t *converged);
+// acc: a step of a run, the iterations are added to the per-system sums.
+gks_status cls_solve(gks_mesh *m, cudaStream_t s, int32_t *iters, double *relres, int32_t *converged,
+                     bool acc = false);
 // The step loop of a run (CFL step clipped to the end times, CLS solve, limiter,
 // flux, update, per-case clocks) for at most max_steps loops as one launch of a
 // graph with device-side control; *used = false when graphs are off, the
@@ -305,7 +307,9 @@ gks_status launch_flux_df(gks_mesh *m, const double *w, const double *x, double 
                           double *flux, cudaStream_t s);
 gks_status launch_point_flux_df(int64_t n, const double *wl, const double *wr, double dt, const gks_config &cfg,
                                 double *out, int32_t *status, cudaStream_t s);
-gks_status launch_cfl_dt(gks_mesh *m, const double *w, double *dt_dev, cudaStream_t s);
+// CFL step per case; clip: clipped to the case's end time (0 once the case is done, which
+// marks it; the time is not advanced)
+gks_status launch_cfl_dt(gks_mesh *m, const double *w, double *dt_dev, cudaStream_t s, bool clip = false);
 gks_status launch_point_flux(int64_t n, const double *wl, const double *wr, double dt, const gks_config &cfg,
                              double *out, int32_t *status, cudaStream_t s);
 // gather (internal[v][i] = caller[v][perm[i]], padding untouched) or scatter
@@ -314,12 +318,9 @@ gks_status launch_permute(const double *src, double *dst, const int32_t *perm, i
 gks_status launch_steady_partial(gks_mesh *m, cudaStream_t s);
 // per-case step control for runs: dt = min(cfl dt, t_final - t) or 0 when done; t += dt
 gks_status launch_clip_dt(gks_mesh *m, cudaStream_t s);
-// the asynchronous step loop: dt of each case clipped to its end time (0 once
-// the case is done, time not advanced yet); after the step, a case whose status
-// is set stops, the others advance their time and step count
-gks_status launch_clip_only(gks_mesh *m, cudaStream_t s);
+// the asynchronous step loop after a step: a case whose status is set stops, the
+// others advance their time and step count
 gks_status launch_after_step(gks_mesh *m, cudaStream_t s);
-gks_status launch_acc_iters(gks_mesh *m, cudaStream_t s);
 // shock detector + DWBAP limiter: m->wk.xl from m->wk.x (gks_limiter.cu)
 gks_status launch_limiter(gks_mesh *m, const double *w, const double *x, cudaStream_t s);
 // caller-ordered copy of the limiter flags of the last launch_limiter

@@ -891,6 +891,7 @@ gks_status build_batch(gks_mesh *m, const CaseIn *cases, int32_t n_cases)
 #undef AL
     GKS_CUDA(cudaMemset(k.sf_ctl, 0, sizeof(int32_t) * 4));
     if (k.sf_flag) GKS_CUDA(cudaMemset(k.sf_flag, 0, sizeof(int32_t) * T));
+    GKS_CUDA(cudaMemset(k.flags, 0, sizeof(int32_t) * 4));
     GKS_CUDA(cudaMemset(k.nsolve, 0, sizeof(int64_t)));
     GKS_CUDA(cudaMemset(k.run_ctl, 0, sizeof(int64_t) * 4));
     GKS_CUDA(cudaMemset(k.x, 0, sizeof(double) * 20 * T));

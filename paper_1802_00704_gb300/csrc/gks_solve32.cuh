@@ -431,10 +431,9 @@ __device__ __forceinline__ void df_add(float x, float y, float &h, float &l)
 }
 
 // Block sums of K x 4 FP32 values per thread, sv[k][v]: FP32 within a warp (at
-// most 160 products each), added across the warps to 48 bits: part[row][v][k0 + k].
+// most 160 products each), added across the warps to 48 bits: part[k0 + k][v][row].
 template <int K>
-__device__ __forceinline__ void block_rows32(float (&sv)[K][4], float (*sh)[K][4], double *__restrict__ part, int ps,
-                                             int k0)
+__device__ __forceinline__ void block_rows32(float (&sv)[K][4], float (*sh)[K][4], double *__restrict__ part, int k0)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
@@ -458,7 +457,7 @@ __device__ __forceinline__ void block_rows32(float (&sv)[K][4], float (*sh)[K][4
         float h = 0.0f, l = 0.0f;
 #pragma unroll
         for (int w = 0; w < kBlock / 32; ++w) df_add(sh[w][k][v], 0.0f, h, l);
-        part[((int64_t)blockIdx.x * 4 + v) * ps + k0 + k] = double(h) + double(l);
+        part[((k0 + k) * 4 + v) * (int64_t)gridDim.x + blockIdx.x] = double(h) + double(l);
     }
 }
 
@@ -472,7 +471,7 @@ __global__ void __launch_bounds__(kBlock, 3) k32_apply_dots(int64_t T, const int
                                                             const int32_t *__restrict__ run,
                                                             const float *__restrict__ z, float *__restrict__ y,
                                                             const float *__restrict__ V, int j,
-                                                            double *__restrict__ part, int ps)
+                                                            double *__restrict__ part)
 {
     constexpr int N = J > 0 ? J : 2;
     __shared__ float sh[kBlock / 32][N][4];
@@ -500,7 +499,7 @@ __global__ void __launch_bounds__(kBlock, 3) k32_apply_dots(int64_t T, const int
                 }
             }
         if (J == 0 && k0 > 0) __syncthreads();
-        block_rows32<N>(sv, sh, part, ps, k0);
+        block_rows32<N>(sv, sh, part, k0);
     }
 }
 
@@ -511,7 +510,7 @@ __global__ void __launch_bounds__(kBlock) k32_update_norm(int64_t T, const int32
                                                           const int32_t *__restrict__ run,
                                                           const float *__restrict__ V, float *__restrict__ wn, int j,
                                                           const double *__restrict__ hc, int hstride,
-                                                          double *__restrict__ part, int ps)
+                                                          double *__restrict__ part)
 {
     if (J > 0) j = J - 1;
     __shared__ float sh[kBlock / 32][1][4];
@@ -563,7 +562,7 @@ __global__ void __launch_bounds__(kBlock) k32_update_norm(int64_t T, const int32
             vstore(wn, l, T, i, w[l]);
         }
     }
-    block_rows32<1>(nrm, sh, part, ps, 0);
+    block_rows32<1>(nrm, sh, part, 0);
 }
 
 }  // namespace

@@ -256,11 +256,11 @@ __device__ __forceinline__ void apply64(int64_t T, const int32_t *__restrict__ n
 }
 
 // Sums over the lanes of a warp of the rows acc[k][lane] (k < K, row stride 33),
-// written to out[k]: each row is split among 32 / (rows per pass) lanes, which
+// written to out[k os]: each row is split among 32 / (rows per pass) lanes, which
 // add its entries in order and then each other's sums.
 constexpr int kAccStride = 33;
 
-__device__ __forceinline__ void warp_rows(const double *acc, int K, int lane, double *__restrict__ out)
+__device__ __forceinline__ void warp_rows(const double *acc, int K, int lane, double *__restrict__ out, int64_t os)
 {
     const int g = K <= 4 ? 8 : (K <= 8 ? 4 : (K <= 16 ? 2 : 1));
     const int sub = lane % g;
@@ -270,7 +270,7 @@ __device__ __forceinline__ void warp_rows(const double *acc, int K, int lane, do
         if (k < K)
             for (int t = sub; t < 32; t += g) s += acc[k * kAccStride + t];
         for (int o = g >> 1; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (sub == 0 && k < K) out[k] = s;
+        if (sub == 0 && k < K) out[k * os] = s;
     }
 }
 
@@ -283,7 +283,7 @@ __device__ __forceinline__ double warp_sum(double s)
 }
 
 // y = K z and the products <V_k, y>, k <= j, of the first Gram-Schmidt pass:
-// part[row][v][k] over the 32 C cells of the block.  Dynamic shared memory:
+// part[k][v][row] over the 32 C cells of the block.  Dynamic shared memory:
 // 4 (j + 1) kAccStride doubles.
 template <int C>
 __global__ void __launch_bounds__(kW64) k64_apply_dots(int64_t T, const int32_t *__restrict__ nb,
@@ -291,7 +291,7 @@ __global__ void __launch_bounds__(kW64) k64_apply_dots(int64_t T, const int32_t 
                                                        const int32_t *__restrict__ blk_case,
                                                        const int32_t *__restrict__ run, const double *__restrict__ z,
                                                        double *__restrict__ y, const double *__restrict__ V, int j,
-                                                       double *__restrict__ part, int ps)
+                                                       double *__restrict__ part)
 {
     extern __shared__ double sh64[];
     const int64_t c0 = blockIdx.x * (int64_t)(32 * C);
@@ -318,7 +318,7 @@ __global__ void __launch_bounds__(kW64) k64_apply_dots(int64_t T, const int32_t 
         }
     }
     __syncwarp();
-    warp_rows(acc, K, w.lane, part + ((int64_t)blockIdx.x * 4 + w.v) * ps);
+    warp_rows(acc, K, w.lane, part + w.v * (int64_t)gridDim.x + blockIdx.x, 4 * (int64_t)gridDim.x);
 }
 
 // w -= sum_k h_k V_k, then the products <V_k, w> of the second pass
@@ -327,7 +327,7 @@ __global__ void __launch_bounds__(kW64) k64_update_dots(int64_t T, const int32_t
                                                         const int32_t *__restrict__ run,
                                                         const double *__restrict__ V, double *__restrict__ wn, int j,
                                                         const double *__restrict__ hc, int hstride,
-                                                        double *__restrict__ part, int ps)
+                                                        double *__restrict__ part)
 {
     extern __shared__ double sh64[];
     const int64_t c0 = blockIdx.x * (int64_t)(32 * C);
@@ -364,7 +364,7 @@ __global__ void __launch_bounds__(kW64) k64_update_dots(int64_t T, const int32_t
         }
     }
     __syncwarp();
-    warp_rows(acc, K, w.lane, part + ((int64_t)blockIdx.x * 4 + w.v) * ps);
+    warp_rows(acc, K, w.lane, part + w.v * (int64_t)gridDim.x + blockIdx.x, 4 * (int64_t)gridDim.x);
 }
 
 // w -= sum_k h_k V_k and the partial |w|^2
@@ -373,7 +373,7 @@ __global__ void __launch_bounds__(kW64) k64_update_norm(int64_t T, const int32_t
                                                         const int32_t *__restrict__ run,
                                                         const double *__restrict__ V, double *__restrict__ wn, int j,
                                                         const double *__restrict__ hc, int hstride,
-                                                        double *__restrict__ part, int ps)
+                                                        double *__restrict__ part)
 {
     __shared__ double hs[4][kMaxRestart];
     const int64_t c0 = blockIdx.x * (int64_t)(32 * C);
@@ -404,14 +404,14 @@ __global__ void __launch_bounds__(kW64) k64_update_norm(int64_t T, const int32_t
         }
     }
     nr = warp_sum(nr);
-    if (w.lane == 0) part[((int64_t)blockIdx.x * 4 + w.v) * ps] = nr;
+    if (w.lane == 0) part[w.v * (int64_t)gridDim.x + blockIdx.x] = nr;
 }
 
 // Right-hand side b_i = sum_j a0_ij (w_j - w_i) and the partial |b|^2 (entry 1)
 template <int C>
 __global__ void __launch_bounds__(kW64) k64_rhs(int64_t T, const int32_t *__restrict__ nb,
                                                 const double *__restrict__ a0, const double *__restrict__ wst,
-                                                double *__restrict__ b, double *__restrict__ part, int ps)
+                                                double *__restrict__ b, double *__restrict__ part)
 {
     const int64_t c0 = blockIdx.x * (int64_t)(32 * C);
     const int lane = threadIdx.x & 31, v = threadIdx.x >> 5;
@@ -441,7 +441,7 @@ __global__ void __launch_bounds__(kW64) k64_rhs(int64_t T, const int32_t *__rest
         }
     }
     nr = warp_sum(nr);
-    if (lane == 0) part[((int64_t)blockIdx.x * 4 + v) * ps + 1] = nr;
+    if (lane == 0) part[(4 + v) * (int64_t)gridDim.x + blockIdx.x] = nr;
 }
 
 // Residual y = b - K x and the partial |y|^2 (entry 0); act (NULL on a solve's
@@ -452,7 +452,7 @@ __global__ void __launch_bounds__(kW64) k64_resid(int64_t T, const int32_t *__re
                                                   const int32_t *__restrict__ blk_case,
                                                   const int32_t *__restrict__ act, const double *__restrict__ x,
                                                   const double *__restrict__ b, double *__restrict__ y,
-                                                  double *__restrict__ part, int ps)
+                                                  double *__restrict__ part)
 {
     const int64_t c0 = blockIdx.x * (int64_t)(32 * C);
     const Warp64 w = warp64(blk_case, act, c0);
@@ -473,7 +473,7 @@ __global__ void __launch_bounds__(kW64) k64_resid(int64_t T, const int32_t *__re
         }
     }
     nr = warp_sum(nr);
-    if (lane == 0) part[((int64_t)blockIdx.x * 4 + v) * ps] = nr;
+    if (lane == 0) part[v * (int64_t)gridDim.x + blockIdx.x] = nr;
 }
 
 // x += sum_{k<jv} y_k Z_k at the end of a cycle

@@ -124,9 +124,21 @@ __global__ void k_cfl_partial(DeviceMesh d, const double *__restrict__ w, double
     }
 }
 
-// out[c] = scale * min of the block minima of case c (one block per case)
+// dt of a case clipped to its end time; 0 for a case that is done or has
+// reached its end (which marks it done); the time is advanced after the step
+__device__ __forceinline__ double clip_step(double dt, double t, double tf, int32_t *done)
+{
+    if (*done || (tf > 0.0 && t >= tf * (1.0 - 1e-14))) {
+        *done = 1;
+        return 0.0;
+    }
+    return tf > 0.0 ? fmin(dt, tf - t) : dt;
+}
+
+// out[c] = scale * min of the block minima of case c (one block per case); with
+// done given, clipped to the case's end time
 __global__ void k_min_final(const double *__restrict__ part, const int32_t *__restrict__ case_blk, double scale,
-                            double *out)
+                            double *out, const double *__restrict__ t, const double *__restrict__ tf, int32_t *done)
 {
     __shared__ double sh[kBlock];
     const int c = blockIdx.x;
@@ -138,7 +150,10 @@ __global__ void k_min_final(const double *__restrict__ part, const int32_t *__re
         if (threadIdx.x < o) sh[threadIdx.x] = fmin(sh[threadIdx.x], sh[threadIdx.x + o]);
         __syncthreads();
     }
-    if (threadIdx.x == 0) out[c] = scale * sh[0];
+    if (threadIdx.x == 0) {
+        const double dt = scale * sh[0];
+        out[c] = done ? clip_step(dt, t[c], tf[c], done + c) : dt;
+    }
 }
 
 // Per-case step control: dt = min(cfl step, t_final - t), 0 once done; t += dt.
@@ -155,21 +170,6 @@ __global__ void k_clip_dt(double *dt, double *t, const double *__restrict__ tf, 
     t[c] += dt[c];
 }
 
-// dt of each case clipped to its end time; 0 for a case that is done or has
-// reached its end (which marks it done); the time is advanced after the step
-__global__ void k_clip_only(double *dt, const double *__restrict__ t, const double *__restrict__ tf, int32_t *done,
-                            int n)
-{
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= n) return;
-    if (done[c] || (tf[c] > 0.0 && t[c] >= tf[c] * (1.0 - 1e-14))) {
-        done[c] = 1;
-        dt[c] = 0.0;
-        return;
-    }
-    if (tf[c] > 0.0) dt[c] = fmin(dt[c], tf[c] - t[c]);
-}
-
 // after a step: a case with status bits set stops (done); every other case
 // that took a step advances its time, step count and last step
 __global__ void k_after_step(const double *__restrict__ dt, double *t, int32_t *done,
@@ -184,13 +184,6 @@ __global__ void k_after_step(const double *__restrict__ dt, double *t, int32_t *
     t[c] += dt[c];
     nstep[c] += 1;
     last_dt[c] = dt[c];
-}
-
-// acc[s] += iterations of system s in the last solve
-__global__ void k_acc_iters(const int32_t *__restrict__ it, int64_t *acc, int ns)
-{
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q < ns) acc[q] += it[q];
 }
 
 // Internal rows [nvar][n] <-> caller rows [nvar][nc]; padding (perm < 0) untouched.
@@ -261,12 +254,14 @@ gks_status launch_update(gks_mesh *m, double *w, const double *flux, cudaStream_
     return GKS_OK;
 }
 
-gks_status launch_cfl_dt(gks_mesh *m, const double *w, double *dt_dev, cudaStream_t s)
+gks_status launch_cfl_dt(gks_mesh *m, const double *w, double *dt_dev, cudaStream_t s, bool clip)
 {
     const unsigned nb = blocks(m->d.T, kBlock);
     const int slot = prof_start(m, kProfCtl, s);
     k_cfl_partial<<<nb, kBlock, 0, s>>>(m->d, w, m->cfg.gamma, m->cfg.mu, m->wk.dpart); note_launch();
-    k_min_final<<<m->d.ncase, kBlock, 0, s>>>(m->wk.dpart, m->d.case_blk, m->cfg.cfl, dt_dev); note_launch();
+    k_min_final<<<m->d.ncase, kBlock, 0, s>>>(m->wk.dpart, m->d.case_blk, m->cfg.cfl, dt_dev, m->wk.tcase,
+                                              m->wk.tfinal, clip ? m->wk.done : nullptr);
+    note_launch();
     prof_stop(m, slot, s);
     GKS_CUDA(cudaGetLastError());
     return GKS_OK;
@@ -288,28 +283,12 @@ gks_status launch_clip_dt(gks_mesh *m, cudaStream_t s)
     return GKS_OK;
 }
 
-gks_status launch_clip_only(gks_mesh *m, cudaStream_t s)
-{
-    const int n = m->d.ncase;
-    k_clip_only<<<(n + 127) / 128, 128, 0, s>>>(m->wk.dt, m->wk.tcase, m->wk.tfinal, m->wk.done, n); note_launch();
-    GKS_CUDA(cudaGetLastError());
-    return GKS_OK;
-}
-
 gks_status launch_after_step(gks_mesh *m, cudaStream_t s)
 {
     const int n = m->d.ncase;
     Work &k = m->wk;
     k_after_step<<<(n + 127) / 128, 128, 0, s>>>(k.dt, k.tcase, k.done, k.status, k.nstep, k.last_dt, n);
     note_launch();
-    GKS_CUDA(cudaGetLastError());
-    return GKS_OK;
-}
-
-gks_status launch_acc_iters(gks_mesh *m, cudaStream_t s)
-{
-    const int ns = m->wk.ns;
-    k_acc_iters<<<(ns + 127) / 128, 128, 0, s>>>(m->wk.ctl + kCtlIters * ns, m->wk.iters_acc, ns); note_launch();
     GKS_CUDA(cudaGetLastError());
     return GKS_OK;
 }
