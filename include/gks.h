@@ -216,11 +216,11 @@ typedef struct gks_config {
                               whose FP32 slope-carrying terms (the viscous stress)
                               would limit the agreement with the FP64 path         */
     int32_t flux_shape;    /* launch shape of the double-FP32 flux kernel: 0 (default)
-                              128 threads x 4 blocks per SM (128 registers), 1 x 3
-                              (168 registers), 2 x 2 (255 registers).  The same
-                              source, compiled once per shape, so results of two
-                              shapes may differ in the last bits; the autotuner's
-                              last stage picks one                                     */
+                              128 threads x 4 blocks per SM on small meshes, 256 x 2
+                              on large ones (128 registers), 1 256 x 2, 2 128 x 2
+                              (255 registers).  The same source, compiled once per
+                              shape, so results of two shapes may differ in the last
+                              bits; the autotuner's last stage picks one               */
     int32_t reserved;      /* must be 0                                                */
 } gks_config;
 
@@ -449,8 +449,7 @@ typedef struct gks_tune_result {
     int32_t ilu_sweeps_bwd;       /* chosen backward sweeps (-1: as ilu_sweeps)     */
     int32_t gmres_m;              /* chosen restart length (also in the config)     */
     int32_t flux_variant;         /* chosen launch shape of the double-FP32 flux
-                                     kernel: 0 128 threads x 4 blocks per SM (128
-                                     registers), 1 x 3 (168), 2 x 2 (255)          */
+                                     kernel (gks_config.flux_shape)                */
 } gks_tune_result;
 
 GKS_EXPORT gks_status gks_autotune(gks_mesh *mesh, const double *w, int32_t trial_steps, gks_tune_result *out,

@@ -114,8 +114,13 @@ __global__ void k_to_df(const double *__restrict__ w, const double *__restrict__
 // a face in neighbouring lanes, summed in pairs and written once in FP64.
 // HEAT: Prandtl correction (pr_fac = 1/Pr - 1); KIN: kinetic interface slopes.
 // NT threads per block, MINB blocks per SM: the register budget, 65536 /
-// (NT MINB) per thread (128 for the default 128 x 4, with some spills; the
-// autotuner also times 128 x 3 and 128 x 2).
+// (NT MINB) per thread (128 for 128 x 4 and 256 x 2, with some spills).  The
+// kernel is issue-bound with instruction fetch as its largest stall (100 KB of
+// straight code); larger blocks start together and share more fetches, smaller
+// ones fill the last wave better.  Measured on GB300 with the pairs' conversion
+// (us, 128 x 4 / 256 x 2 / 512 x 1): 1,426 / 1,236 / 1,292 at 1,000,000 triangles,
+// 211 / 201 / 227 at 131,000, 68.9 / 75.3 / 74.4 at 41,000; 168 registers (128 x 3,
+// 384 x 1) 1,375 and 1,392 at 1,000,000; barriers between the kernel's phases gain nothing.
 template <bool HEAT, bool KIN, int NT = kFluxBlock, int MINB = 4>
 __global__ void __launch_bounds__(NT, MINB)
     k_face_flux_df(DeviceMesh d, const float *__restrict__ w2, const float *__restrict__ x2, double dt_const,
@@ -272,43 +277,36 @@ gks_status launch_flux_df(gks_mesh *m, const double *w, const double *x, double 
     const double K = 2.0 / (m->cfg.gamma - 1.0) - 2.0;
     const gks_config &c = m->cfg;
     const bool heat = c.prandtl != 1.0;
-    const unsigned g = blocks(2 * m->d.F, kFluxBlock);
-    {
-        // FP32 pairs of the state and the coefficients, then the double-FP32 flux
-        k_to_df<<<dim3(blocks(m->d.T, kBlock), 6), kBlock, 0, s>>>(w, x, m->wk.w2, m->wk.x2, m->d.T);
-        note_launch();
-        const lead::LeadConst lc = lead_const(c);
-        const df pr_fac = dfm::from_double(1.0 / c.prandtl - 1.0);
-        const bool kin = c.slope0_mode == 1;
-        auto go = [&](auto H, auto Kw) {
-            k_face_flux_df<decltype(H)::value, decltype(Kw)::value><<<g, kFluxBlock, 0, s>>>(
-                m->d, m->wk.w2, m->wk.x2, dt_const, dt_dev, lc, float(c.gamma), float(K), c.tau2_exact, pr_fac, flux,
-                m->wk.status);
-        };
-        using Y = std::true_type;
-        using N = std::false_type;
-        if (heat) {
-            kin ? go(Y{}, Y{}) : go(Y{}, N{});
-        } else if (kin) {
-            go(N{}, Y{});
-        } else {
-            const float gf = float(c.gamma), kf = float(K);
-            switch (c.flux_shape) {
-            case 1:
-                k_face_flux_df<false, false, 128, 3><<<g, 128, 0, s>>>(m->d, m->wk.w2, m->wk.x2, dt_const, dt_dev, lc,
-                                                                      gf, kf, c.tau2_exact, pr_fac, flux,
-                                                                      m->wk.status);
-                break;
-            case 2:
-                k_face_flux_df<false, false, 128, 2><<<g, 128, 0, s>>>(m->d, m->wk.w2, m->wk.x2, dt_const, dt_dev, lc,
-                                                                      gf, kf, c.tau2_exact, pr_fac, flux,
-                                                                      m->wk.status);
-                break;
-            default:
-                go(N{}, N{});
-                break;
-            }
-        }
+    // FP32 pairs of the state and the coefficients, then the double-FP32 flux
+    k_to_df<<<dim3(blocks(m->d.T, kBlock), 6), kBlock, 0, s>>>(w, x, m->wk.w2, m->wk.x2, m->d.T);
+    note_launch();
+    const lead::LeadConst lc = lead_const(c);
+    const df pr_fac = dfm::from_double(1.0 / c.prandtl - 1.0);
+    const bool kin = c.slope0_mode == 1;
+    const int64_t npts = 2 * m->d.F;
+    auto go = [&](auto H, auto Kw, auto NT, auto MINB) {
+        constexpr int nt = decltype(NT)::value;
+        k_face_flux_df<decltype(H)::value, decltype(Kw)::value, nt, decltype(MINB)::value>
+            <<<blocks(npts, nt), nt, 0, s>>>(m->d, m->wk.w2, m->wk.x2, dt_const, dt_dev, lc, float(c.gamma), float(K),
+                                             c.tau2_exact, pr_fac, flux, m->wk.status);
+    };
+    using Y = std::true_type;
+    using N = std::false_type;
+    // the launch shape: 256-thread blocks (flux_shape 1) unless they would leave a
+    // last wave nearly empty (fewer than four waves of the SMs' 512 points each)
+    const bool wide = c.flux_shape == 1 || npts >= 4 * 512 * (int64_t)m->wk.sm_count;
+    auto shaped = [&](auto H, auto Kw) {
+        if (wide) go(H, Kw, std::integral_constant<int, 256>{}, std::integral_constant<int, 2>{});
+        else go(H, Kw, std::integral_constant<int, kFluxBlock>{}, std::integral_constant<int, 4>{});
+    };
+    if (heat) {
+        kin ? shaped(Y{}, Y{}) : shaped(Y{}, N{});
+    } else if (kin) {
+        shaped(N{}, Y{});
+    } else if (c.flux_shape == 2) {
+        go(N{}, N{}, std::integral_constant<int, kFluxBlock>{}, std::integral_constant<int, 2>{});
+    } else {
+        shaped(N{}, N{});
     }
     GKS_CUDA(cudaGetLastError());
     return GKS_OK;
