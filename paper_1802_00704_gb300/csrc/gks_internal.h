@@ -136,6 +136,7 @@ struct Work {
     float *x2 = nullptr;             // [40][T] FP32 pairs of the coefficients: x32, then the low parts
     float *w2 = nullptr;             // [8][T] FP32 pairs of the state: hi, then lo
     int32_t *lflag = nullptr;        // [T] 0 untouched, 1 limited, 2 reset to the average
+    int32_t *llist = nullptr;        // [T + 1] cells to limit (limiter 1), then their number
     double *b = nullptr, *r = nullptr, *t2 = nullptr, *t3 = nullptr;  // [20][T]
     float *t2_32 = nullptr, *t3_32 = nullptr;  // [20][T] FP32 preconditioner work
     float *r32 = nullptr;            // [20][T] FP32 copy of the preconditioner's source (sweeps); the FP32

@@ -27,25 +27,24 @@
 //    cell average only (first order), for contacts with density ratios near
 //    10, where the DWBAP polynomials let cell averages turn negative.
 //
-// One thread per cell, FP64.  The unlimited coefficients stay in x (the warm
-// start of the next CLS solve); the limited ones are written to a separate
-// array that the flux kernel reads.
+// FP64 throughout, in two kernels: a thread per cell for the detector and the
+// positivity of every cell, which copies the coefficients of a smooth cell and
+// lists the others, and a group of lanes per listed cell for the limiter.  An FP64
+// instruction holds an SM sub-partition for 33 ns whatever its active lanes, and a
+// limited cell's weights and means are some 5,000 of them (80 arctangents and
+// divisions, 20 tangents): one flagged cell among a warp's 32 cost as much as 32.
+// A limiter call on a 12,000-triangle strip (characteristic variables) went from 260 us
+// in one kernel to 21 us for the detector and 30 us for the limiter, a step of the
+// 6,400-triangle Sod strip from 0.85 to 0.65 ms.
+// The unlimited coefficients stay in x (the warm start of the next CLS solve);
+// the limited ones are written to a separate array that the flux kernel reads.
+#include <algorithm>
 #include <cmath>
 
 #include "gks_internal.h"
 
 namespace gks {
 namespace {
-
-// Variable v of cell c's polynomial at offset (dx, dy) in c's scaled frame.
-__device__ __forceinline__ double poly_value(const DeviceMesh &d, const double *__restrict__ w, const double *x,
-                                             int64_t c, int v, double dx, double dy)
-{
-    const int64_t T = d.T;
-    const double qx = dx * dx - d.mxx[c], qxy = dx * dy - d.mxy[c], qy = dy * dy - d.myy[c];
-    return w[v * T + c] + x[(v * 5 + 0) * T + c] * dx + x[(v * 5 + 1) * T + c] * dy +
-           0.5 * x[(v * 5 + 2) * T + c] * qx + x[(v * 5 + 3) * T + c] * qxy + 0.5 * x[(v * 5 + 4) * T + c] * qy;
-}
 
 // Right (columns) and left (rows) eigenvectors, row-major 4x4, of the Jacobian
 // of the Euler flux along the unit direction (nx, ny) at the conservative
@@ -68,227 +67,283 @@ __device__ __forceinline__ void char_basis(const double *W, double gamma, double
     L[12] = 0.5 * (b2 - qn * ic); L[13] = -0.5 * (b1 * u - nx * ic); L[14] = -0.5 * (b1 * v - ny * ic); L[15] = 0.5 * b1;
 }
 
-// u_0 tan(sum_j om_j atan(u_j / u_0)) over the first n of 4 candidates.
-__device__ __forceinline__ double biased_mean(const double (&u)[4], const double (&om)[4], int n)
+// u_0 tan(sum_j om_j atan(u_j / u_0)) over the candidates (weight 0: none); the own
+// candidate's arctangent is pi/4 (NaN for an infinite u_0, as the quotient is)
+__device__ __forceinline__ double biased_mean(const double (&u)[4], const double (&om)[4])
 {
     if (u[0] == 0.0) return 0.0;
-    double acc = 0.0;
+    double acc = om[0] * 0.78539816339744830962 + (u[0] - u[0]);
 #pragma unroll
-    for (int j = 0; j < 4; ++j)
-        if (j < n) acc += om[j] * atan(u[j] / u[0]);
+    for (int j = 1; j < 4; ++j)
+        if (om[j] != 0.0) acc += om[j] * atan(u[j] / u[0]);
     return u[0] * tan(acc);
 }
 
-// rho > 0 and p > 0 at all face Gauss points of cell i for the coefficients c.
-__device__ __forceinline__ bool physical_gp(const DeviceMesh &d, const double *__restrict__ w, const double *c,
-                                            int64_t i, double gamma)
+// rho > 0 and p > 0 at Gauss point (dx, dy) of a cell, U its averages and c its
+// coefficients [variable][5].  p > 0 as 2 rho E > |rho u|^2, which has the same sign
+// for rho > 0 without a division (9 instructions), unless rho E nears the range's ends
+__device__ __forceinline__ bool physical_at(const double *U, const double (*c)[5], double mxx, double mxy, double myy,
+                                            double dx, double dy)
 {
-    const int64_t T = d.T, F = d.F;
-    bool ok = true;
+    const double hx = 0.5 * (dx * dx - mxx), xy = dx * dy - mxy, hy = 0.5 * (dy * dy - myy);
+    double q[4];
 #pragma unroll
-    for (int s = 0; s < 3; ++s) {
-        const int32_t cf = d.cf[s * T + i];
-        if (cf < 0) continue;
-        const int64_t f = cf >> 1;
-        const double *g = (cf & 1) ? d.gr : d.gl;
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            const double dx = g[(2 * k) * F + f], dy = g[(2 * k + 1) * F + f];
-            const double rho = poly_value(d, w, c, i, 0, dx, dy);
-            const double mx = poly_value(d, w, c, i, 1, dx, dy), my = poly_value(d, w, c, i, 2, dx, dy);
-            const double E = poly_value(d, w, c, i, 3, dx, dy);
-            const double p = (gamma - 1.0) * (E - 0.5 * (mx * mx + my * my) / rho);
-            ok = ok && rho > 0.0 && p > 0.0;
-        }
-    }
-    return ok;
+    for (int v = 0; v < 4; ++v)
+        q[v] = U[v] + c[v][0] * dx + c[v][1] * dy + c[v][2] * hx + c[v][3] * xy + c[v][4] * hy;
+    const double e = 2.0 * q[0] * q[3], k = q[1] * q[1] + q[2] * q[2];
+    const int ex = (__double2hiint(e) >> 20) & 0x7ff;      // biased exponent, on the integer pipe
+    if (ex < 64 || ex > 1983) return q[0] > 0.0 && q[3] - 0.5 * k / q[0] > 0.0;
+    return q[0] > 0.0 && e > k;
 }
 
-__global__ void __launch_bounds__(kBlock) k_limit(const DeviceMesh d, const double *__restrict__ w,
-                                                  const double *__restrict__ x, double *xl,
-                                                  int32_t *__restrict__ flag, double gamma, int robust, int charm)
+constexpr int kDetectBlock = 64;       // small blocks: a few thousand cells reach every SM
+
+// Detector (Eqs. (37)-(38)) and positivity of every cell.  A smooth cell keeps its
+// coefficients (flag 0); another one goes to list (list_n: its length) or, robust,
+// keeps its average only (flag 2).
+__global__ void __launch_bounds__(kDetectBlock) k_detect(const DeviceMesh d, const double *__restrict__ w,
+                                                         const double *__restrict__ x, double *__restrict__ xl,
+                                                         int32_t *__restrict__ flag, int32_t *__restrict__ list,
+                                                         int32_t *__restrict__ list_n, int robust)
 {
     const int64_t T = d.T, F = d.F;
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= T) return;
-    int32_t nbj[3];
-    double oxj[3], oyj[3];
+    double U[4], c[4][5];
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+        U[v] = w[v * T + i];
+#pragma unroll
+        for (int l = 0; l < 5; ++l) c[v][l] = x[(v * 5 + l) * T + i];
+    }
+    const double hi = d.h[i], mxx = d.mxx[i], mxy = d.mxy[i], myy = d.myy[i];
     int J = 0;
+    double s0 = 0.0, s3 = 0.0, m0 = U[0], m3 = U[3];
+    const double v0 = U[0] - 0.5 * c[0][2] * mxx - c[0][3] * mxy - 0.5 * c[0][4] * myy;
+    const double v3 = U[3] - 0.5 * c[3][2] * mxx - c[3][3] * mxy - 0.5 * c[3][4] * myy;
 #pragma unroll
     for (int s = 0; s < 3; ++s) {
-        nbj[s] = d.nb[s * T + i];      // neighbour slots are filled from slot 0
-        oxj[s] = d.ox[s * T + i];
-        oyj[s] = d.oy[s * T + i];
-        J += nbj[s] >= 0;
+        const int64_t j = d.nb[s * T + i];             // neighbour slots are filled from slot 0
+        if (j < 0) continue;
+        ++J;
+        const double r = hi / d.h[j];
+        const double dx = -d.ox[s * T + i] * r, dy = -d.oy[s * T + i] * r;   // r_i in j's scaled frame
+        const double hx = 0.5 * (dx * dx - d.mxx[j]), xy = dx * dy - d.mxy[j], hy = 0.5 * (dy * dy - d.myy[j]);
+        const double w0 = w[j], w3 = w[3 * T + j];
+        const double q0 = w0 + x[j] * dx + x[T + j] * dy + x[2 * T + j] * hx + x[3 * T + j] * xy + x[4 * T + j] * hy;
+        const double q3 = w3 + x[15 * T + j] * dx + x[16 * T + j] * dy + x[17 * T + j] * hx + x[18 * T + j] * xy +
+                          x[19 * T + j] * hy;
+        s0 += fabs(v0 - q0);
+        s3 += fabs(v3 - q3);
+        m0 = fmax(m0, w0);
+        m3 = fmax(m3, w3);
     }
-    const double hi = d.h[i];
-    const int ki = d.kord[i];
     bool flagged = false;
     if (J > 0) {
-        // Eq. (37) for rho and E
-        const double v0 = poly_value(d, w, x, i, 0, 0.0, 0.0), v3 = poly_value(d, w, x, i, 3, 0.0, 0.0);
-        double s0 = 0.0, s3 = 0.0, m0 = w[i], m3 = w[3 * T + i];
+        const double scale = J * (d.kord[i] == 2 ? hi * sqrt(hi) : hi);     // J h^{(k+1)/2}
+        flagged = !(s0 / (scale * m0) < 1.0 && s3 / (scale * m3) < 1.0);
 #pragma unroll
         for (int s = 0; s < 3; ++s) {
-            if (s >= J) continue;
-            const int64_t j = nbj[s];
-            const double r = hi / d.h[j];
-            const double ddx = -oxj[s] * r, ddy = -oyj[s] * r;   // r_i in j's scaled frame
-            s0 += fabs(v0 - poly_value(d, w, x, j, 0, ddx, ddy));
-            s3 += fabs(v3 - poly_value(d, w, x, j, 3, ddx, ddy));
-            m0 = fmax(m0, w[j]);
-            m3 = fmax(m3, w[3 * T + j]);
+            const int32_t cf = d.cf[s * T + i];
+            if (cf < 0) continue;
+            const int64_t f = cf >> 1;
+            const double *g = (cf & 1) ? d.gr : d.gl;
+#pragma unroll
+            for (int k = 0; k < 2; ++k)
+                flagged |= !physical_at(U, c, mxx, mxy, myy, g[(2 * k) * F + f], g[(2 * k + 1) * F + f]);
         }
-        const double scale = J * pow(hi, 0.5 * (ki + 1));
-        flagged = !(s0 / (scale * m0) < 1.0 && s3 / (scale * m3) < 1.0) || !physical_gp(d, w, x, i, gamma);
     }
-    if (!flagged) {
-#pragma unroll 4
-        for (int q = 0; q < 20; ++q) xl[q * T + i] = x[q * T + i];
-        flag[i] = 0;
+    if (flagged && !robust) {
+        list[atomicAdd(list_n, 1)] = (int32_t)i;
         return;
     }
-    if (robust) {
-        for (int q = 0; q < 20; ++q) xl[q * T + i] = 0.0;
-        flag[i] = 2;
-        return;
-    }
+#pragma unroll
+    for (int v = 0; v < 4; ++v)
+#pragma unroll
+        for (int l = 0; l < 5; ++l) xl[(v * 5 + l) * T + i] = flagged ? 0.0 : c[v][l];
+    flag[i] = flagged ? 2 : 0;
+}
 
-    // ---- weights, Eqs. (35)-(36); distances in i's scaled frame times h_i
-    double fmx[3] = {0.0, 0.0, 0.0}, fmy[3] = {0.0, 0.0, 0.0};
-    int nf = 0;
-#pragma unroll
-    for (int s = 0; s < 3; ++s) {
-        const int32_t cf = d.cf[s * T + i];
-        if (cf < 0) continue;
-        const int64_t f = cf >> 1;
-        if (d.fr[f] < 0) continue;
-        const double *g = (cf & 1) ? d.gr : d.gl;   // the two Gauss points straddle the midpoint
-        const double mx = 0.5 * (g[f] + g[2 * F + f]), my = 0.5 * (g[F + f] + g[3 * F + f]);
-        if (nf == 0) { fmx[0] = mx; fmy[0] = my; }
-        else if (nf == 1) { fmx[1] = mx; fmy[1] = my; }
-        else { fmx[2] = mx; fmy[2] = my; }
-        ++nf;
-    }
-    double X[3] = {0.0, 0.0, 0.0}, Xbar = 0.0;
-#pragma unroll
-    for (int s = 0; s < 3; ++s) {
-        if (s >= J) continue;
-        const int64_t j = nbj[s];
-        const double rho = w[j], u = w[T + j] / rho, v = w[2 * T + j] / rho;
-        X[s] = (gamma - 1.0) * (w[3 * T + j] - 0.5 * rho * (u * u + v * v));
-        Xbar += X[s] / J;
-    }
-    double var = 0.0;
-#pragma unroll
-    for (int s = 0; s < 3; ++s)
-        if (s < J) var += (X[s] - Xbar) * (X[s] - Xbar) / J;
-    const double chi = sqrt(var) / Xbar;
-    const double S = 1.0 / (sqrt(chi + 1e-8) + 0.05);
-    double om[4] = {0.0, 0.0, 0.0, 0.0}, bsum = 0.0;
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        if (c > J) continue;
-        const double px = c == 0 ? 0.0 : oxj[c - 1], py = c == 0 ? 0.0 : oyj[c - 1];
-        double dist = 0.0;
-#pragma unroll
-        for (int q = 0; q < 3; ++q)
-            if (q < nf) dist += hi * hypot(px - fmx[q], py - fmy[q]) / nf;
-        om[c] = pow(dist, -S);
-        bsum += om[c];
-    }
-#pragma unroll
-    for (int c = 0; c < 4; ++c) om[c] /= bsum;
+constexpr int kLimitWarps = 4;         // warps per block
 
-    double hj[3] = {1.0, 1.0, 1.0}, ddx[3] = {0.0, 0.0, 0.0}, ddy[3] = {0.0, 0.0, 0.0};
-    bool k2[3] = {false, false, false};
-#pragma unroll
-    for (int s = 0; s < 3; ++s) {
-        if (s >= J) continue;
-        hj[s] = d.h[nbj[s]];
-        ddx[s] = -oxj[s] * hi / hj[s];
-        ddy[s] = -oyj[s] * hi / hj[s];
-        k2[s] = d.kord[nbj[s]] == 2;
-    }
-    // candidates of every derivative row l, in physical units: cand[c][v] for the
-    // cell's own polynomial (c = 0) and the neighbours' (at r_i; for the second
-    // derivatives only neighbours with k = 2, weights renormalised)
-    const double Wi[4] = {w[i], w[T + i], w[2 * T + i], w[3 * T + i]};
-    for (int l = 0; l < 5; ++l) {
-        if (l >= 2 && ki != 2) {
-            for (int v = 0; v < 4; ++v) xl[(v * 5 + l) * T + i] = x[(v * 5 + l) * T + i];
-            continue;
-        }
-        double cand[4][4] = {}, omc[4] = {0.0, 0.0, 0.0, 0.0};
-        const double sc = l < 2 ? hi : hi * hi;
-#pragma unroll
-        for (int v = 0; v < 4; ++v) cand[0][v] = x[(v * 5 + l) * T + i] / sc;
-        omc[0] = om[0];
-        double os = om[0];
-        int n = 1;
+// DWBAP limiter (Eqs. (34)-(36)) of the listed cells from e0 on, in steps of the grid,
+// G lanes each: the first four lanes of a group take a candidate's weight each, lane
+// 4 a + v the derivatives l = a, a + G/4, ... of variable (characteristic) v.
+template <int G>
+__device__ __forceinline__ void limit_cells(const DeviceMesh &d, const double *__restrict__ w,
+                                            const double *__restrict__ x, double *__restrict__ xl,
+                                            int32_t *__restrict__ flag, const int32_t *__restrict__ list, int total,
+                                            double gamma, int charm, double (*sh)[4][5])
+{
+    constexpr unsigned kAll = 0xffffffffu;
+    constexpr int kPer = 32 / G;               // cells per warp
+    const int64_t T = d.T, F = d.F;
+    const int lane = threadIdx.x & (G - 1), grp = (threadIdx.x & 31) / G, v = lane & 3;
+    double(*c)[5] = sh[grp];
+    const int warp = blockIdx.x * kLimitWarps + (threadIdx.x >> 5), nwarp = gridDim.x * kLimitWarps;
+    for (int e0 = warp * kPer; e0 < total; e0 += nwarp * kPer) {       // uniform over the warp
+        const bool mine = e0 + grp < total;
+        const int64_t i = list[mine ? e0 + grp : total - 1];
+        const double hi = d.h[i];
+        const int ki = d.kord[i];
+        // lane s < 3: the pressure of neighbour s, its centroid in i's frame and i's in its
+        int J = 0;
+        int32_t nbj[3];
 #pragma unroll
         for (int s = 0; s < 3; ++s) {
-            if (s >= J || (l >= 2 && !k2[s])) continue;
-            const int64_t j = nbj[s];
+            nbj[s] = d.nb[s * T + i];
+            J += nbj[s] >= 0;
+        }
+        double X = 0.0, rh = 0.0, dx = 0.0, dy = 0.0;
+        if (v < J) {
+            const int64_t j = v == 0 ? nbj[0] : (v == 1 ? nbj[1] : nbj[2]);
+            const double rho = w[j], mx = w[T + j], my = w[2 * T + j];
+            X = (gamma - 1.0) * (w[3 * T + j] - 0.5 * (mx * mx + my * my) / rho);
+            rh = 1.0 / d.h[j];
+            dx = -d.ox[v * T + i] * hi * rh;
+            dy = -d.oy[v * T + i] * hi * rh;
+        }
+        // ---- weights, Eqs. (35)-(36); distances in i's scaled frame times h_i
+        const double rJ = 1.0 / J;
+        double Xs[3], rhj[3], ddx[3], ddy[3], Xbar = 0.0, var = 0.0;
 #pragma unroll
-            for (int v = 0; v < 4; ++v) {
-                double c;
-                if (l >= 2) {
-                    c = x[(v * 5 + l) * T + j] / (hj[s] * hj[s]);
+        for (int s = 0; s < 3; ++s) {
+            Xs[s] = __shfl_sync(kAll, X, s, G);
+            rhj[s] = __shfl_sync(kAll, rh, s, G);
+            ddx[s] = __shfl_sync(kAll, dx, s, G);
+            ddy[s] = __shfl_sync(kAll, dy, s, G);
+            Xbar += s < J ? Xs[s] * rJ : 0.0;
+        }
+#pragma unroll
+        for (int s = 0; s < 3; ++s)
+            if (s < J) var += (Xs[s] - Xbar) * (Xs[s] - Xbar) * rJ;
+        const double chi = sqrt(var) / Xbar;
+        const double S = 1.0 / (sqrt(chi + 1e-8) + 0.05);
+        // lane q: the weight of candidate q (0 the cell itself)
+        double wt = 0.0;
+        if (v <= J) {
+            const double px = v == 0 ? 0.0 : d.ox[(v - 1) * T + i], py = v == 0 ? 0.0 : d.oy[(v - 1) * T + i];
+            double dist = 0.0;
+            int nf = 0;
+#pragma unroll
+            for (int s = 0; s < 3; ++s) {
+                const int32_t cf = d.cf[s * T + i];
+                if (cf < 0) continue;
+                const int64_t f = cf >> 1;
+                if (d.fr[f] < 0) continue;
+                const double *g = (cf & 1) ? d.gr : d.gl;   // the two Gauss points straddle the midpoint
+                dist += hypot(px - 0.5 * (g[f] + g[2 * F + f]), py - 0.5 * (g[F + f] + g[3 * F + f]));
+                ++nf;
+            }
+            wt = pow(hi * dist / nf, -S);
+        }
+        // weights of the first derivatives, and of the second ones (the neighbours with k = 2)
+        double om[2][4], sum[2] = {0.0, 0.0};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            om[0][q] = __shfl_sync(kAll, wt, q, G);
+            om[1][q] = q == 0 || (q <= J && d.kord[nbj[q > 0 ? q - 1 : 0]] == 2) ? om[0][q] : 0.0;
+            sum[0] += om[0][q];
+            sum[1] += om[1][q];
+        }
+#pragma unroll
+        for (int a = 0; a < 2; ++a) {
+            const double r = 1.0 / sum[a];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) om[a][q] *= r;
+        }
+        // ---- a derivative row at a time: candidates in physical units, the cell's own
+        // polynomial and the neighbours' (at r_i)
+        const double rhi = 1.0 / hi;
+#pragma unroll 1
+        for (int l0 = 0; l0 < 5; l0 += G / 4) {
+            const int l = min(l0 + (lane >> 2), 4);        // spare lanes repeat the last row
+            const bool high = l >= 2;
+            const double own = x[(v * 5 + l) * T + i];
+            double cand[4] = {own * (high ? rhi * rhi : rhi), 0.0, 0.0, 0.0}, o[4];
+#pragma unroll
+            for (int s = 0; s < 3; ++s) {
+                if (s >= J) continue;
+                const int64_t j = nbj[s];
+                if (high) {
+                    cand[s + 1] = x[(v * 5 + l) * T + j] * (rhj[s] * rhj[s]);
                 } else {
                     const double ua = x[(v * 5 + l) * T + j];          // u1 (l = 0) or u2 (l = 1)
                     const double ub = x[(v * 5 + 2 + l) * T + j];      // u3 or u4
                     const double uc = x[(v * 5 + 3 + l) * T + j];      // u4 or u5
-                    c = (ua + ub * ddx[s] + uc * ddy[s]) / hj[s];
+                    cand[s + 1] = (ua + ub * ddx[s] + uc * ddy[s]) * rhj[s];
                 }
-                if (n == 1) cand[1][v] = c;
-                else if (n == 2) cand[2][v] = c;
-                else cand[3][v] = c;
             }
-            if (n == 1) omc[1] = om[s + 1];
-            else if (n == 2) omc[2] = om[s + 1];
-            else omc[3] = om[s + 1];
-            os += om[s + 1];
-            ++n;
-        }
 #pragma unroll
-        for (int q = 0; q < 4; ++q) omc[q] /= os;
-        double res[4];
-        if (charm) {
-            // characteristic variables along x (d/dx, d2/dx2), y (d/dy, d2/dy2), the diagonal (d2/dxdy)
-            const double nx = l == 1 || l == 4 ? 0.0 : (l == 3 ? 0.70710678118654752 : 1.0);
-            const double ny = l == 0 || l == 2 ? 0.0 : (l == 3 ? 0.70710678118654752 : 1.0);
-            double Rm[16], Lm[16];
-            char_basis(Wi, gamma, nx, ny, Rm, Lm);
-            double lim[4];
+            for (int q = 0; q < 4; ++q) o[q] = high ? om[1][q] : om[0][q];
+            double res;
+            if (charm) {
+                // characteristic variables along x (d/dx, d2/dx2), y (d/dy, d2/dy2), the
+                // diagonal (d2/dxdy); lane v of a row takes characteristic v
+                const double Wi[4] = {w[i], w[T + i], w[2 * T + i], w[3 * T + i]};
+                const double nx = l == 1 || l == 4 ? 0.0 : (l == 3 ? 0.70710678118654752 : 1.0);
+                const double ny = l == 0 || l == 2 ? 0.0 : (l == 3 ? 0.70710678118654752 : 1.0);
+                double Rm[16], Lm[16], Lr[4], Rr[4], ch[4];
+                char_basis(Wi, gamma, nx, ny, Rm, Lm);
 #pragma unroll
-            for (int a2 = 0; a2 < 4; ++a2) {
-                double ch[4];
+                for (int q = 0; q < 4; ++q) {
+                    Lr[q] = v == 0 ? Lm[q] : (v == 1 ? Lm[4 + q] : (v == 2 ? Lm[8 + q] : Lm[12 + q]));
+                    Rr[q] = v == 0 ? Rm[q] : (v == 1 ? Rm[4 + q] : (v == 2 ? Rm[8 + q] : Rm[12 + q]));
+                }
 #pragma unroll
                 for (int q = 0; q < 4; ++q)
-                    ch[q] = Lm[4 * a2] * cand[q][0] + Lm[4 * a2 + 1] * cand[q][1] + Lm[4 * a2 + 2] * cand[q][2] +
-                            Lm[4 * a2 + 3] * cand[q][3];
-                lim[a2] = biased_mean(ch, omc, n);
+                    ch[q] = Lr[0] * __shfl_sync(kAll, cand[q], 0, 4) + Lr[1] * __shfl_sync(kAll, cand[q], 1, 4) +
+                            Lr[2] * __shfl_sync(kAll, cand[q], 2, 4) + Lr[3] * __shfl_sync(kAll, cand[q], 3, 4);
+                const double lim = biased_mean(ch, o);
+                res = Rr[0] * __shfl_sync(kAll, lim, 0, 4) + Rr[1] * __shfl_sync(kAll, lim, 1, 4) +
+                      Rr[2] * __shfl_sync(kAll, lim, 2, 4) + Rr[3] * __shfl_sync(kAll, lim, 3, 4);
+            } else {
+                res = biased_mean(cand, o);
             }
-#pragma unroll
-            for (int a2 = 0; a2 < 4; ++a2)
-                res[a2] = Rm[4 * a2] * lim[0] + Rm[4 * a2 + 1] * lim[1] + Rm[4 * a2 + 2] * lim[2] + Rm[4 * a2 + 3] * lim[3];
-        } else {
-#pragma unroll
-            for (int v = 0; v < 4; ++v) {
-                const double cv[4] = {cand[0][v], cand[1][v], cand[2][v], cand[3][v]};
-                res[v] = biased_mean(cv, omc, n);
-            }
+            // a linear cell's second derivatives are kept
+            c[v][l] = high && ki != 2 ? own : (high ? hi * hi : hi) * res;
         }
-#pragma unroll
-        for (int v = 0; v < 4; ++v) xl[(v * 5 + l) * T + i] = sc * res[v];
-    }
+        __syncwarp();
 
-    // ---- safeguard at the cell's face Gauss points
-    const bool bad = !physical_gp(d, w, xl, i, gamma);
-    if (bad)
-        for (int q = 0; q < 20; ++q) xl[q * T + i] = 0.0;
-    flag[i] = bad ? 2 : 1;
+        // ---- safeguard at the cell's face Gauss points, a point (2 s + k: k of face s) per lane
+        double U[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) U[q] = w[q * T + i];
+        bool ok = true;
+        for (int t = lane; t < 6; t += G) {
+            const int32_t cf = d.cf[(t >> 1) * T + i];
+            if (cf < 0) continue;
+            const int64_t f = cf >> 1;
+            const double *g = (cf & 1) ? d.gr : d.gl;
+            const int k = t & 1;
+            ok = ok && physical_at(U, c, d.mxx[i], d.mxy[i], d.myy[i], g[(2 * k) * F + f], g[(2 * k + 1) * F + f]);
+        }
+        const unsigned fails = __ballot_sync(kAll, !ok) >> (G * grp);
+        const bool bad = (G == 32 ? fails : fails & ((1u << (G & 31)) - 1u)) != 0u;
+        if (mine) {
+            for (int l = lane >> 2; l < 5; l += G / 4) xl[(v * 5 + l) * T + i] = bad ? 0.0 : c[v][l];
+            if (lane == 0) flag[i] = bad ? 2 : 1;
+        }
+        __syncwarp();
+    }
+}
+
+// A warp takes one listed cell or eight.  A cell of its own ends in about 20 us, eight
+// in about 45 (five rows per lane), so eight pay once the sub-partitions have more than
+// two cells each.
+__global__ void __launch_bounds__(32 * kLimitWarps) k_limit(const DeviceMesh d, const double *__restrict__ w,
+                                                            const double *__restrict__ x, double *__restrict__ xl,
+                                                            int32_t *__restrict__ flag,
+                                                            const int32_t *__restrict__ list,
+                                                            const int32_t *__restrict__ list_n, double gamma, int charm,
+                                                            int one_max)
+{
+    __shared__ double sh[kLimitWarps][8][4][5];
+    const int total = *list_n;
+    if (total <= one_max)
+        limit_cells<32>(d, w, x, xl, flag, list, total, gamma, charm, sh[threadIdx.x >> 5]);
+    else
+        limit_cells<4>(d, w, x, xl, flag, list, total, gamma, charm, sh[threadIdx.x >> 5]);
 }
 
 // caller[perm[i]] = internal[i] for the limiter flags (padding skipped)
@@ -311,10 +366,20 @@ gks_status launch_limiter(gks_mesh *m, const double *w, const double *x, cudaStr
         return GKS_EINVAL;
     }
     if (d.T == 0) return GKS_OK;
-    const unsigned nb = (unsigned)((d.T + kBlock - 1) / kBlock);
-    k_limit<<<nb, kBlock, 0, s>>>(d, w, x, m->wk.xl, m->wk.lflag, m->cfg.gamma, m->cfg.limiter == 2 ? 1 : 0,
-                                  m->cfg.limit_char);
+    Work &k = m->wk;
+    const bool robust = m->cfg.limiter == 2;
+    if (!robust) GKS_CUDA(cudaMemsetAsync(k.llist + d.T, 0, sizeof(int32_t), s));
+    k_detect<<<(unsigned)((d.T + kDetectBlock - 1) / kDetectBlock), kDetectBlock, 0, s>>>(
+        d, w, x, k.xl, k.lflag, k.llist, robust ? nullptr : k.llist + d.T, robust ? 1 : 0);
     note_launch();
+    if (!robust) {
+        // every listed cell on a group of its own, up to four warps per SM sub-partition
+        const int64_t need = (d.T + kLimitWarps - 1) / kLimitWarps;
+        const unsigned g = (unsigned)std::min<int64_t>(need, (int64_t)k.sm_count * 4);
+        k_limit<<<g, 32 * kLimitWarps, 0, s>>>(d, w, x, k.xl, k.lflag, k.llist, k.llist + d.T, m->cfg.gamma,
+                                               m->cfg.limit_char, 2 * 4 * k.sm_count);
+        note_launch();
+    }
     GKS_CUDA(cudaGetLastError());
     return GKS_OK;
 }

@@ -872,6 +872,7 @@ gks_status build_batch(gks_mesh *m, const CaseIn *cases, int32_t n_cases)
     AL(part, (size_t)nblk * rows * 4 * (mm + 2)); AL(dpart, (size_t)nblk * 4);
     if (cfg.limiter) {
         AL(xl, 20 * T); AL(lflag, T);
+        if (cfg.limiter == 1) AL(llist, T + 1);
     }
     AL(x_prev, 20 * T); AL(x_prev2, 20 * T);   // extrapolated warm start (also for the autotuner)
     if (cfg.precision == GKS_MIXED) {
