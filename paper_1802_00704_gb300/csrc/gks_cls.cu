@@ -1408,8 +1408,8 @@ gks_status solve64_shared_limit(int mm)
     auto set = [&](auto C) -> gks_status {
         constexpr int c = decltype(C)::value;
         GKS_CUDA(cudaFuncSetAttribute(k64_apply_dots<c>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)acc64(mm - 1, kAccStride)));
-        GKS_CUDA(cudaFuncSetAttribute(k64_update_dots<c>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)acc64(mm, kAccStride)));
+        GKS_CUDA(cudaFuncSetAttribute(k64_update<c>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)acc64(mm - 1, kAccStride + 1)));
         return GKS_OK;
     };
@@ -1441,17 +1441,19 @@ void solve64_apply_dots(gks_mesh *m, const double *z, const double *V, double *y
 {
     const DeviceMesh &d = m->d;
     with_cells(m->wk.c64, [&](auto C) {
-        k64_apply_dots<decltype(C)::value><<<rows64(m), kW64, acc64(j, kAccStride), q>>>(
+        k64_apply_dots<decltype(C)::value><<<rows64(m), kW64, acc64(j + 1, kAccStride), q>>>(
             d.T, d.nb, d.D, d.off, d.blk_case, m->wk.ctl + kCtlRunning * m->wk.ns, z, y, V, j, m->wk.part);
     });
 }
 
-void solve64_update_dots(gks_mesh *m, const double *V, double *w, int j, int ps, cudaStream_t q)
+void solve64_update(gks_mesh *m, const double *V, double *w, int j, int ps, cudaStream_t q)
 {
     const DeviceMesh &d = m->d;
+    const Work &k = m->wk;
     with_cells(m->wk.c64, [&](auto C) {
-        k64_update_dots<decltype(C)::value><<<rows64(m), kW64, acc64(j, kAccStride + 1), q>>>(
-            d.T, d.blk_case, m->wk.ctl + kCtlRunning * m->wk.ns, V, w, j, m->wk.hco, ps, m->wk.part);
+        k64_update<decltype(C)::value><<<rows64(m), kW64, acc64(j, kAccStride + 1), q>>>(
+            d.T, d.blk_case, d.case_blk, k.ctl + kCtlRunning * k.ns, V, w, j, k.hcol, k.hco, ps,
+            k.ctl + kCtlTwice * k.ns, k.part);
     });
 }
 
@@ -1460,7 +1462,8 @@ void solve64_update_norm(gks_mesh *m, const double *V, double *w, int j, int ps,
     const DeviceMesh &d = m->d;
     with_cells(m->wk.c64, [&](auto C) {
         k64_update_norm<decltype(C)::value><<<rows64(m), kW64, 0, q>>>(
-            d.T, d.blk_case, m->wk.ctl + kCtlRunning * m->wk.ns, V, w, j, m->wk.hco, ps, m->wk.part);
+            d.T, d.blk_case, m->wk.ctl + kCtlRunning * m->wk.ns, m->wk.ctl + kCtlTwice * m->wk.ns, V, w, j, m->wk.hco,
+            ps, m->wk.part);
     });
 }
 
@@ -1929,6 +1932,7 @@ gks_status cls_solve_t(gks_mesh *m, TB *V, cudaStream_t s, int32_t *iters, doubl
     const int rs_rhs = C64 ? rs64 : (rhs_df ? rs32 : 1);
     const int rs_res = C64 ? rs64 : (std::is_same<TB, float>::value && d.D2 ? kResidRows : 1);
     const int rs = rs64;
+    const int32_t *twice = C64 ? k.ctl + kCtlTwice * ns : nullptr;
     auto residual = [&](cudaStream_t q, bool first) -> gks_status {
         const int32_t *act = first ? nullptr : k.ctl + kCtlActive * ns;
         if (C64) {
@@ -2009,7 +2013,7 @@ gks_status cls_solve_t(gks_mesh *m, TB *V, cudaStream_t s, int32_t *iters, doubl
         } else if (mixed) {
             spmv32(q, k.Z32 + j * vs, vj1);
         } else if (C64) {
-            // with the first Gram-Schmidt products
+            // V_{j+1} = K Z_j - V_j with the first Gram-Schmidt products
             solve64_apply_dots(m, k.Z + j * vs, reinterpret_cast<const double *>(V), reinterpret_cast<double *>(vj1),
                                j, q);
         } else {
@@ -2018,14 +2022,16 @@ gks_status cls_solve_t(gks_mesh *m, TB *V, cudaStream_t s, int32_t *iters, doubl
         if (!C64 && !fused_dots) note_launch();
         prof_stop(m, slot, q);
         slot = prof_start(m, kProfOrth, q);
-        // classical Gram-Schmidt: twice in FP64 mode; once in the mixed mode, whose
+        // classical Gram-Schmidt: twice in FP64 mode (per-cell equations: a second
+        // time where it is needed, see gks_solve64.cuh); once in the mixed mode, whose
         // cycles only reduce the residual by inner_rtol before an FP64 restart
         if (!fused_dots && !C64 && (st = dots<TB>(m, V, vj1, j, k.part, q)) != GKS_OK) return st;
-        k_reduce<<<dim3(j + 1, ns), kReduceThreads, 0, q>>>(k.part, rs * (int64_t)nb, d.case_blk, rs, k.hcol, ps, k.vn,
-                                                             mm + 1, k.hco, ps);
+        k_reduce<<<dim3(j + (C64 ? 2 : 1), ns), kReduceThreads, 0, q>>>(k.part, rs * (int64_t)nb, d.case_blk, rs,
+                                                                         k.hcol, ps, k.vn, mm + 1, k.hco, ps, j + 1,
+                                                                         nullptr);
         note_launch();
         if (C64) {
-            solve64_update_dots(m, reinterpret_cast<const double *>(V), reinterpret_cast<double *>(vj1), j, ps, q);
+            solve64_update(m, reinterpret_cast<const double *>(V), reinterpret_cast<double *>(vj1), j, ps, q);
         } else if (fused_dots) {
             solve32_update_norm(m, reinterpret_cast<const float *>(V), reinterpret_cast<float *>(vj1), j, ps, q);
         } else {
@@ -2033,10 +2039,10 @@ gks_status cls_solve_t(gks_mesh *m, TB *V, cudaStream_t s, int32_t *iters, doubl
             note_launch();
         }
         if (!mixed) {
-            // the second pass
+            // the second pass (the systems flagged in twice)
             if (!C64 && (st = dots<TB>(m, V, vj1, j, k.part, q)) != GKS_OK) return st;
             k_reduce<<<dim3(j + 1, ns), kReduceThreads, 0, q>>>(k.part, rs * (int64_t)nb, d.case_blk, rs, k.y, mm, k.vn,
-                                                                 mm + 1, k.hco, ps);
+                                                                 mm + 1, k.hco, ps, j + 1, twice);
             note_launch();
             if (C64) {
                 solve64_update_norm(m, reinterpret_cast<const double *>(V), reinterpret_cast<double *>(vj1), j, ps, q);
@@ -2047,7 +2053,7 @@ gks_status cls_solve_t(gks_mesh *m, TB *V, cudaStream_t s, int32_t *iters, doubl
         }
         // |V_{j+1}| and the Givens step of every system (and the end of a single mesh's cycle)
         k_arnoldi_end<<<ns, kReduceThreads, 0, q>>>(kry, k.part, rs * (int64_t)nb, d.case_blk, rs, j, k.hcol, ps,
-                                                        mixed ? nullptr : k.y, mm, cd);
+                                                        mixed ? nullptr : k.y, mm, twice, C64 ? 1.0 : 0.0, cd);
         note_launch();
         prof_stop(m, slot, q);
         GKS_CUDA(cudaGetLastError());

@@ -72,19 +72,21 @@ __device__ __forceinline__ double block_sum(const double *part, int q, int v, in
 
 // out[s][q] = sum over the rows of case(s) of column q, q < nq, and with vn given
 // co[s][q] = sum / vn[s][q]^2 (the Gram-Schmidt coefficient of the unnormalised
-// basis vector q).  Grid (nq, ns).
+// basis vector q; q < nco).  Grid (nq, ns).  on (may be NULL): the systems to sum.
 __global__ void __launch_bounds__(kReduceThreads) k_reduce(const double *__restrict__ part, int64_t R,
                                                            const int32_t *__restrict__ seg, int rs, double *out,
                                                            int ostride, const double *__restrict__ vn, int vstride,
-                                                           double *co, int cstride)
+                                                           double *co, int cstride, int nco,
+                                                           const int32_t *__restrict__ on)
 {
     __shared__ double sh[kReduceThreads / 32];
     const int q = blockIdx.x, sy = blockIdx.y, c = sy >> 2;
-    const double n = vn[sy * vstride + q];
+    if (on && !on[sy]) return;
+    const double n = q < nco ? vn[sy * vstride + q] : 0.0;
     const double acc = block_sum(part, q, sy & 3, R, rs * seg[c], rs * seg[c + 1], sh);
     if (threadIdx.x == 0) {
         out[sy * ostride + q] = acc;
-        co[sy * cstride + q] = n > 0.0 ? acc / (n * n) : 0.0;
+        if (q < nco) co[sy * cstride + q] = n > 0.0 ? acc / (n * n) : 0.0;
     }
 }
 
@@ -172,12 +174,13 @@ __device__ __forceinline__ double pow2_exact(int e)
 }
 
 // Arnoldi index j of system sy, by one warp: the new Hessenberg column from the
-// raw sums hc (plus h2 of the second Gram-Schmidt pass, if given), the earlier
+// raw sums hc (plus h2 of a second Gram-Schmidt pass, if given) and shift on its
+// diagonal (1 when V_j was taken off the new vector, else 0), the earlier
 // rotations applied, a new rotation, the rotated residual g and the stopping
 // test.  The column's divisions are done by the lanes together, and only the
 // chain of rotations (four FP64 instructions each) is serial.
 __device__ __forceinline__ void givens_step(const Krylov &k, int sy, int j, const double *hc, int hstride,
-                                            const double *h2, int h2stride, double hnext,
+                                            const double *h2, int h2stride, double shift, double hnext,
                                             double (*sh)[kMaxRestart + 1])
 {
     const int lane = threadIdx.x & 31, m = k.m;
@@ -187,7 +190,7 @@ __device__ __forceinline__ void givens_step(const Krylov &k, int sy, int j, cons
     const double nj = k.vn[sy * (m + 1) + j];
     for (int q = lane; q <= j + 1; q += 32) {
         const double a = q <= j ? hc[sy * hstride + q] + (h2 ? h2[sy * h2stride + q] : 0.0) : hnext;
-        h[q] = a / (q <= j ? k.vn[sy * (m + 1) + q] * nj : nj);
+        h[q] = a / (q <= j ? k.vn[sy * (m + 1) + q] * nj : nj) + (q == j ? shift : 0.0);
         if (q < j) {
             c0[q] = k.cs[sy * m + q];
             s0[q] = k.sn[sy * m + q];
@@ -290,18 +293,20 @@ __global__ void __launch_bounds__(32 * kSolveWarps) k_cycle_solve(Krylov k)
 }
 
 // End of Arnoldi index j, one block per system: |V_{j+1}| of a running system
-// from the summed partials and its Givens step; then the condition "any system
+// from the summed partials and its Givens step (twice, may be NULL: the systems
+// that ran the second Gram-Schmidt pass); then the condition "any system
 // still runs" and, for a single mesh, the solve of the cycle once none does.
 __global__ void __cluster_dims__(4, 1, 1) __launch_bounds__(kReduceThreads)
     k_arnoldi_end(Krylov k, const double *part, int64_t R, const int32_t *__restrict__ seg, int rs, int j,
-                  const double *hc, int hstride, const double *h2, int h2stride, Cond cd)
+                  const double *hc, int hstride, const double *h2, int h2stride, const int32_t *twice, double shift,
+                  Cond cd)
 {
     __shared__ double sh[kReduceThreads / 32];
     __shared__ double shg[4][kMaxRestart + 1];
     const int sy = blockIdx.x, c = sy >> 2;
     if (k.ctl[kCtlRunning * k.ns + sy] != 0) {
         const double acc = block_sum(part, 0, sy & 3, R, rs * seg[c], rs * seg[c + 1], sh);
-        if (threadIdx.x < 32) givens_step(k, sy, j, hc, hstride, h2, h2stride, sqrt(acc), shg);
+        if (threadIdx.x < 32) givens_step(k, sy, j, hc, hstride, twice && !twice[sy] ? nullptr : h2, h2stride, shift, sqrt(acc), shg);
     }
     bool last;
     const bool any = any_flag(k.ctl + kCtlRunning * k.ns, k.ns, cd.ticket, &last);

@@ -48,7 +48,7 @@ enum : int {
 enum : int { kStatusNonPhys = 1, kStatusNoConv = 2, kStatusTimeout = 4 };
 
 // GMRES control words, ctl[field * ns + system] with system = case * 4 + variable.
-enum : int { kCtlActive = 0, kCtlRunning = 1, kCtlJv = 2, kCtlIters = 3, kCtlFields = 4 };
+enum : int { kCtlActive = 0, kCtlRunning = 1, kCtlJv = 2, kCtlIters = 3, kCtlTwice = 4, kCtlFields = 5 };
 
 // Device data, all in internal (per-case RCM, padded) cell order.
 struct DeviceMesh {
@@ -154,7 +154,7 @@ struct Work {
     double *g = nullptr;             // [ns][m+1]
     double *y = nullptr;             // [ns][m]
     float *y32 = nullptr;            // [ns][m] FP32 copy of y (mixed mode)
-    double *hcol = nullptr;          // [ns][m+2] raw sums <V_k, u> of the current column, then |V_{j+1}|
+    double *hcol = nullptr;          // [ns][m+2] raw sums <V_k, u>, k <= j, of the current column (FP64 solve: then |u|^2)
     double *hco = nullptr;           // [ns][m+2] Gram-Schmidt coefficients <V_k, u> / vn_k^2
     double *vn = nullptr;            // [ns][m+1] norms vn_k of the stored basis vectors
     double *bnorm = nullptr, *beta = nullptr;  // [ns]

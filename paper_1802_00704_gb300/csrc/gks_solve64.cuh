@@ -19,7 +19,16 @@
 //    arithmetic of a triangular relation;
 //  - sums over cells start their FMA chains from the running sum in shared
 //    memory and are added across the lanes of a warp in transposed order, 7-31
-//    additions for all Arnoldi indices together instead of 5 for each.
+//    additions for all Arnoldi indices together instead of 5 for each;
+//  - the basis grows by w = K M^-1 V_j - V_j, which spans the same Krylov space (the
+//    Hessenberg diagonal gets its 1 back).  The preconditioner is close to the
+//    inverse, so nearly all of K M^-1 V_j is V_j itself: without it the part
+//    orthogonal to the basis is 0.63-0.99 of |w| instead of 0.02-0.26 (800- and
+//    1,200-triangle systems), one Gram-Schmidt pass loses no digits (V^T V - 1 is 4e-16
+//    as after two; one pass of the unshifted basis leaves 1e-4), and the second
+//    runs only where the orthogonal part is below half of |w| (the launches of the
+//    second are there and return).  Three steps at 399,424 triangles 46.2 -> 41.9 ms,
+//    ten at 6,400 6.56 -> 6.06 ms, at 800 6.05 -> 5.50 ms.
 // Measured on GB300 (the solve's classes, per Arnoldi index, events around each
 // class): preconditioner with two sweeps each way 80 -> 25 us at 800 triangles
 // and 680 -> 448 us at 399,424; operator with the first Gram-Schmidt products and
@@ -221,10 +230,11 @@ __global__ void __launch_bounds__(kW64) k64_bwd(int64_t T, const int32_t *__rest
     }
 }
 
-// acc = (K x)_i of variable v: diagonal block minus the off-diagonal ones
+// acc = (K x)_i of variable v, diagonal block minus the off-diagonal ones, minus
+// s_i (s may be NULL)
 __device__ __forceinline__ void apply64(int64_t T, const int32_t *__restrict__ nb, const double *__restrict__ D,
                                         const double *__restrict__ off, const double *__restrict__ xv, int64_t i,
-                                        double *acc)
+                                        double *acc, const double *__restrict__ s0 = nullptr)
 {
     int j[3];
     Off64 o[3];
@@ -247,7 +257,7 @@ __device__ __forceinline__ void apply64(int64_t T, const int32_t *__restrict__ n
                                 {4, 8, 11, 13, 14}};
 #pragma unroll
     for (int a = 0; a < 5; ++a) {
-        acc[a] = Dm[kIdx[a][0]] * x[0];
+        acc[a] = s0 ? fma(Dm[kIdx[a][0]], x[0], -s0[a * T + i]) : Dm[kIdx[a][0]] * x[0];
 #pragma unroll
         for (int c = 1; c < 5; ++c) acc[a] = fma(Dm[kIdx[a][c]], x[c], acc[a]);
     }
@@ -282,9 +292,9 @@ __device__ __forceinline__ double warp_sum(double s)
     return s;
 }
 
-// y = K z and the products <V_k, y>, k <= j, of the first Gram-Schmidt pass:
-// part[k][v][row] over the 32 C cells of the block.  Dynamic shared memory:
-// 4 (j + 1) kAccStride doubles.
+// y = K z - V_j, the products <V_k, y>, k <= j, of the first Gram-Schmidt pass and
+// |y|^2 (k = j + 1): part[k][v][row] over the 32 C cells of the block.  Dynamic
+// shared memory: 4 (j + 2) kAccStride doubles.
 template <int C>
 __global__ void __launch_bounds__(kW64) k64_apply_dots(int64_t T, const int32_t *__restrict__ nb,
                                                        const double *__restrict__ D, const double *__restrict__ off,
@@ -298,16 +308,20 @@ __global__ void __launch_bounds__(kW64) k64_apply_dots(int64_t T, const int32_t 
     const Warp64 w = warp64(blk_case, run, c0);
     if (!w.run) return;
     const int K = j + 1;
-    double *acc = sh64 + w.v * K * kAccStride;
+    double *acc = sh64 + w.v * (K + 1) * kAccStride;
     for (int k = 0; k < K; ++k) acc[k * kAccStride + w.lane] = 0.0;
     const int64_t vo = (int64_t)w.v * 5 * T, vs = 20 * T;
+    double nr = 0.0;
     for (int c = 0; c < C; ++c) {
         const int64_t i = c0 + 32 * c + w.lane;
         if (i >= T) break;
         double u[5];
-        apply64(T, nb, D, off, z + vo, i, u);
+        apply64(T, nb, D, off, z + vo, i, u, V + j * vs + vo);
 #pragma unroll
-        for (int l = 0; l < 5; ++l) y[vo + l * T + i] = u[l];
+        for (int l = 0; l < 5; ++l) {
+            y[vo + l * T + i] = u[l];
+            nr = fma(u[l], u[l], nr);
+        }
 #pragma unroll 4
         for (int k = 0; k < K; ++k) {
             const double *vk = V + k * vs + vo + i;
@@ -317,17 +331,22 @@ __global__ void __launch_bounds__(kW64) k64_apply_dots(int64_t T, const int32_t 
             acc[k * kAccStride + w.lane] = s;
         }
     }
+    acc[K * kAccStride + w.lane] = nr;
     __syncwarp();
-    warp_rows(acc, K, w.lane, part + w.v * (int64_t)gridDim.x + blockIdx.x, 4 * (int64_t)gridDim.x);
+    warp_rows(acc, K + 1, w.lane, part + w.v * (int64_t)gridDim.x + blockIdx.x, 4 * (int64_t)gridDim.x);
 }
 
-// w -= sum_k h_k V_k, then the products <V_k, w> of the second pass
+// First Gram-Schmidt update w -= sum_k h_k V_k, with the partial |w|^2 (column 0)
+// of a system that this leaves with at least half of its norm (hs: the sums <V_k, w>,
+// hc: the coefficients, hs[j + 1] = |w|^2), else the products <V_k, w> of a second
+// pass (twice[system] = 1, for the kernels after this one).
 template <int C>
-__global__ void __launch_bounds__(kW64) k64_update_dots(int64_t T, const int32_t *__restrict__ blk_case,
-                                                        const int32_t *__restrict__ run,
-                                                        const double *__restrict__ V, double *__restrict__ wn, int j,
-                                                        const double *__restrict__ hc, int hstride,
-                                                        double *__restrict__ part)
+__global__ void __launch_bounds__(kW64) k64_update(int64_t T, const int32_t *__restrict__ blk_case,
+                                                   const int32_t *__restrict__ case_blk,
+                                                   const int32_t *__restrict__ run, const double *__restrict__ V,
+                                                   double *__restrict__ wn, int j, const double *__restrict__ hs,
+                                                   const double *__restrict__ hc, int hstride,
+                                                   int32_t *__restrict__ twice, double *__restrict__ part)
 {
     extern __shared__ double sh64[];
     const int64_t c0 = blockIdx.x * (int64_t)(32 * C);
@@ -335,8 +354,18 @@ __global__ void __launch_bounds__(kW64) k64_update_dots(int64_t T, const int32_t
     if (!w.run) return;
     const int K = j + 1;
     double *acc = sh64 + w.v * K * (kAccStride + 1), *h = acc + K * kAccStride;
-    for (int k = w.lane; k < K; k += 32) h[k] = hc[w.sys * hstride + k];
+    double nr = 0.0;
+    for (int k = w.lane; k < K; k += 32) {
+        h[k] = hc[w.sys * hstride + k];
+        nr = fma(h[k], hs[w.sys * hstride + k], nr);      // |projection on V_k|^2
+    }
     for (int k = 0; k < K; ++k) acc[k * kAccStride + w.lane] = 0.0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) nr += __shfl_xor_sync(0xffffffffu, nr, o);
+    const double n2 = hs[w.sys * hstride + K];
+    const bool again = !(n2 > 0.0 && nr <= 0.75 * n2);
+    if (w.lane == 0 && c0 == (int64_t)case_blk[w.sys >> 2] * kBlock) twice[w.sys] = again;
+    nr = 0.0;
     __syncwarp();
     const int64_t vo = (int64_t)w.v * 5 * T, vs = 20 * T;
     for (int c = 0; c < C; ++c) {
@@ -354,6 +383,11 @@ __global__ void __launch_bounds__(kW64) k64_update_dots(int64_t T, const int32_t
         }
 #pragma unroll
         for (int l = 0; l < 5; ++l) wn[vo + l * T + i] = u[l];
+        if (!again) {
+#pragma unroll
+            for (int l = 0; l < 5; ++l) nr = fma(u[l], u[l], nr);
+            continue;
+        }
 #pragma unroll 4
         for (int k = 0; k < K; ++k) {
             const double *vk = V + k * vs + vo + i;
@@ -363,14 +397,21 @@ __global__ void __launch_bounds__(kW64) k64_update_dots(int64_t T, const int32_t
             acc[k * kAccStride + w.lane] = s;
         }
     }
+    double *out = part + w.v * (int64_t)gridDim.x + blockIdx.x;
+    if (!again) {
+        nr = warp_sum(nr);
+        if (w.lane == 0) *out = nr;
+        return;
+    }
     __syncwarp();
-    warp_rows(acc, K, w.lane, part + w.v * (int64_t)gridDim.x + blockIdx.x, 4 * (int64_t)gridDim.x);
+    warp_rows(acc, K, w.lane, out, 4 * (int64_t)gridDim.x);
 }
 
-// w -= sum_k h_k V_k and the partial |w|^2
+// The second pass of the systems that need it: w -= sum_k h_k V_k and the partial |w|^2
 template <int C>
 __global__ void __launch_bounds__(kW64) k64_update_norm(int64_t T, const int32_t *__restrict__ blk_case,
                                                         const int32_t *__restrict__ run,
+                                                        const int32_t *__restrict__ twice,
                                                         const double *__restrict__ V, double *__restrict__ wn, int j,
                                                         const double *__restrict__ hc, int hstride,
                                                         double *__restrict__ part)
@@ -378,7 +419,7 @@ __global__ void __launch_bounds__(kW64) k64_update_norm(int64_t T, const int32_t
     __shared__ double hs[4][kMaxRestart];
     const int64_t c0 = blockIdx.x * (int64_t)(32 * C);
     const Warp64 w = warp64(blk_case, run, c0);
-    if (!w.run) return;
+    if (!w.run || !twice[w.sys]) return;
     const int K = j + 1;
     for (int k = w.lane; k < K; k += 32) hs[w.v][k] = hc[w.sys * hstride + k];
     __syncwarp();
