@@ -1503,12 +1503,16 @@ void solve32_apply_dots(gks_mesh *m, const float *z, const float *V, float *y, i
     note_launch();
 }
 
-void solve32_update_norm(gks_mesh *m, const float *V, float *w, int j, int ps, cudaStream_t q)
+// the update with the end of Arnoldi index j
+void solve32_update(gks_mesh *m, const Krylov &kry, const float *V, float *w, int j, int ps, const Cond &cd,
+                    cudaStream_t q)
 {
     const DeviceMesh &d = m->d;
     const Work &k = m->wk;
-    const int32_t *run = k.ctl + kCtlRunning * k.ns;
-#define U32(J) k32_update_norm<J><<<k.nblk, kBlock, 0, q>>>(d.T, d.blk_case, run, V, w, j, k.hco, ps, k.part)
+    const unsigned g = (unsigned)(m->n_case + k.nblk);
+    const int32_t *ran = k.ctl + kCtlRan * k.ns;
+#define U32(J) \
+    k32_update<J><<<g, kBlock, 0, q>>>(d.T, d.blk_case, kry, m->n_case, V, w, j, k.hcol, k.hco, ps, ran, cd)
     switch (j) {
     case 0: U32(1); break;
     case 1: U32(2); break;
@@ -2026,14 +2030,18 @@ gks_status cls_solve_t(gks_mesh *m, TB *V, cudaStream_t s, int32_t *iters, doubl
         // time where it is needed, see gks_solve64.cuh); once in the mixed mode, whose
         // cycles only reduce the residual by inner_rtol before an FP64 restart
         if (!fused_dots && !C64 && (st = dots<TB>(m, V, vj1, j, k.part, q)) != GKS_OK) return st;
-        k_reduce<<<dim3(j + (C64 ? 2 : 1), ns), kReduceThreads, 0, q>>>(k.part, rs * (int64_t)nb, d.case_blk, rs,
-                                                                         k.hcol, ps, k.vn, mm + 1, k.hco, ps, j + 1,
-                                                                         nullptr);
+        // (C64, fused_dots: and |w|^2)
+        k_reduce<<<dim3(j + (C64 || fused_dots ? 2 : 1), ns), kReduceThreads, 0, q>>>(
+            k.part, rs * (int64_t)nb, d.case_blk, rs, k.hcol, ps, k.vn, mm + 1, k.hco, ps, j + 1, nullptr,
+            k.ctl + kCtlRunning * ns, fused_dots ? k.ctl + kCtlRan * ns : nullptr);
         note_launch();
         if (C64) {
             solve64_update(m, reinterpret_cast<const double *>(V), reinterpret_cast<double *>(vj1), j, ps, q);
         } else if (fused_dots) {
-            solve32_update_norm(m, reinterpret_cast<const float *>(V), reinterpret_cast<float *>(vj1), j, ps, q);
+            solve32_update(m, kry, reinterpret_cast<const float *>(V), reinterpret_cast<float *>(vj1), j, ps, cd, q);
+            prof_stop(m, slot, q);
+            GKS_CUDA(cudaGetLastError());
+            return GKS_OK;
         } else {
             launch_orth_update<TB>(d, nb, q, V, vj1, j, k.hco, ps, k.ctl, ns, k.part, mixed ? 1 : 0);
             note_launch();
@@ -2042,7 +2050,8 @@ gks_status cls_solve_t(gks_mesh *m, TB *V, cudaStream_t s, int32_t *iters, doubl
             // the second pass (the systems flagged in twice)
             if (!C64 && (st = dots<TB>(m, V, vj1, j, k.part, q)) != GKS_OK) return st;
             k_reduce<<<dim3(j + 1, ns), kReduceThreads, 0, q>>>(k.part, rs * (int64_t)nb, d.case_blk, rs, k.y, mm, k.vn,
-                                                                 mm + 1, k.hco, ps, j + 1, twice);
+                                                                 mm + 1, k.hco, ps, j + 1, twice,
+                                                                 nullptr, nullptr);
             note_launch();
             if (C64) {
                 solve64_update_norm(m, reinterpret_cast<const double *>(V), reinterpret_cast<double *>(vj1), j, ps, q);

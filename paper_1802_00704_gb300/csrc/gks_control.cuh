@@ -13,7 +13,9 @@
 // a case a cluster that its hardware barrier joins; the cluster (of a batch the
 // last one to finish) then sets the graph's condition: one launch for the norm, the Givens
 // step, the condition and a single mesh's end of the cycle, one for the residual's norm, the
-// masks, g and the condition.  One block with a case's four systems was slower
+// masks, g and the condition.  In the mixed solve the first of the two (8.2 us at
+// 41,000 triangles) is a block of the update's launch (control_end): ten
+// steps at 41,000 triangles 4.89 -> 4.55 ms, a batch of 64 19.1 -> 18.5 ms.  One block with a case's four systems was slower
 // (10.0 us for the first of the two at 41,000 triangles: four FP64 chains on one
 // SM, and 25 us for the sums at 1M).
 #pragma once
@@ -73,11 +75,13 @@ __device__ __forceinline__ double block_sum(const double *part, int q, int v, in
 // out[s][q] = sum over the rows of case(s) of column q, q < nq, and with vn given
 // co[s][q] = sum / vn[s][q]^2 (the Gram-Schmidt coefficient of the unnormalised
 // basis vector q; q < nco).  Grid (nq, ns).  on (may be NULL): the systems to sum.
+// ran (may be NULL) = run: the running systems, for a kernel that changes run.
 __global__ void __launch_bounds__(kReduceThreads) k_reduce(const double *__restrict__ part, int64_t R,
                                                            const int32_t *__restrict__ seg, int rs, double *out,
                                                            int ostride, const double *__restrict__ vn, int vstride,
                                                            double *co, int cstride, int nco,
-                                                           const int32_t *__restrict__ on)
+                                                           const int32_t *__restrict__ on, const int32_t *run,
+                                                           int32_t *ran)
 {
     __shared__ double sh[kReduceThreads / 32];
     const int q = blockIdx.x, sy = blockIdx.y, c = sy >> 2;
@@ -86,6 +90,7 @@ __global__ void __launch_bounds__(kReduceThreads) k_reduce(const double *__restr
     const double acc = block_sum(part, q, sy & 3, R, rs * seg[c], rs * seg[c + 1], sh);
     if (threadIdx.x == 0) {
         out[sy * ostride + q] = acc;
+        if (q == 0 && ran) ran[sy] = run[sy];
         if (q < nco) co[sy * cstride + q] = n > 0.0 ? acc / (n * n) : 0.0;
     }
 }
@@ -134,15 +139,20 @@ __device__ __forceinline__ bool any_flag(const int32_t *flag, int ns, uint32_t *
     return __syncthreads_or(a) != 0;
 }
 
-__device__ __forceinline__ void set_cond(const Cond &cd, bool any)
+__device__ __forceinline__ void put_cond(const Cond &cd, bool any)
 {
-    if (threadIdx.x != 0 || (blockIdx.x & 3) != 0) return;
     unsigned v = any ? 1u : 0u;
     if (cd.slot >= 0) cd.ctr[cd.slot] += 1;
     if (cd.begin) cd.ctr[kCtrGuard] = 0;
     if (cd.limit > 0 && cd.ctr[kCtrGuard] > cd.limit) v = 0u;
     if (cd.word) *cd.word = (int32_t)v;
     if (cd.set) cudaGraphSetConditional(cd.h, v);
+}
+
+// ... by the first thread of a cluster
+__device__ __forceinline__ void set_cond(const Cond &cd, bool any)
+{
+    if (threadIdx.x == 0 && (blockIdx.x & 3) == 0) put_cond(cd, any);
 }
 
 // A cycle of the device-controlled solve begins: counted for the launch and work
@@ -177,11 +187,11 @@ __device__ __forceinline__ double pow2_exact(int e)
 // raw sums hc (plus h2 of a second Gram-Schmidt pass, if given) and shift on its
 // diagonal (1 when V_j was taken off the new vector, else 0), the earlier
 // rotations applied, a new rotation, the rotated residual g and the stopping
-// test.  The column's divisions are done by the lanes together, and only the
+// test (stop: it ends the cycle here in any case).  The column's divisions are done by the lanes together, and only the
 // chain of rotations (four FP64 instructions each) is serial.
 __device__ __forceinline__ void givens_step(const Krylov &k, int sy, int j, const double *hc, int hstride,
                                             const double *h2, int h2stride, double shift, double hnext,
-                                            double (*sh)[kMaxRestart + 1])
+                                            bool stop, double (*sh)[kMaxRestart + 1])
 {
     const int lane = threadIdx.x & 31, m = k.m;
     // Hessenberg column of the normalised basis: h_kj = <V_k, u_j> / (vn_k vn_j),
@@ -233,7 +243,7 @@ __device__ __forceinline__ void givens_step(const Krylov &k, int sy, int j, cons
     // stop the cycle at the target, or (mixed precision, eta > 0) once the inner
     // residual has dropped by eta: the FP64 refinement residual then restarts it
     const double gn = fabs(s * gj);
-    if (gn <= k.rtol * bn || gn <= k.eta * be || !(hnext > 0.0) || it >= k.maxit || j + 1 == m)
+    if (gn <= k.rtol * bn || gn <= k.eta * be || !(hnext > 0.0) || it >= k.maxit || j + 1 == m || stop)
         k.ctl[kCtlRunning * k.ns + sy] = 0;
 }
 
@@ -306,13 +316,54 @@ __global__ void __cluster_dims__(4, 1, 1) __launch_bounds__(kReduceThreads)
     const int sy = blockIdx.x, c = sy >> 2;
     if (k.ctl[kCtlRunning * k.ns + sy] != 0) {
         const double acc = block_sum(part, 0, sy & 3, R, rs * seg[c], rs * seg[c + 1], sh);
-        if (threadIdx.x < 32) givens_step(k, sy, j, hc, hstride, twice && !twice[sy] ? nullptr : h2, h2stride, shift, sqrt(acc), shg);
+        if (threadIdx.x < 32) givens_step(k, sy, j, hc, hstride, twice && !twice[sy] ? nullptr : h2, h2stride, shift, sqrt(acc), false, shg);
     }
     bool last;
     const bool any = any_flag(k.ctl + kCtlRunning * k.ns, k.ns, cd.ticket, &last);
     if (!last) return;
     if (gridDim.x == 4 && !any && threadIdx.x < 32) cycle_solve(k, sy);
     set_cond(cd, any);
+}
+
+// End of Arnoldi index j inside the update's launch, a block per case with a warp
+// per system: the basis holds K Z_j - V_j, at least half of whose norm is orthogonal to it as
+// a rule (gks_solve64.cuh), so the new vector's norm follows from |w|^2 (n2 = hs[j + 1])
+// and the projections, and the Givens step needs no sum over the updated vector.
+// A system with little left (below 3 % of |w|, where the difference loses
+// its digits) ends its cycle.  ran: the running systems before this launch.
+__device__ __forceinline__ void control_end(const Krylov &k, int c, int ncase, int j, const double *hs, const double *hc,
+                                            int hstride, const int32_t *ran, const Cond &cd,
+                                            double (*shg)[4][kMaxRestart + 1])
+{
+    __shared__ int is_last;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, sy = 4 * c + (warp & 3);
+    if (warp < 4 && ran[sy] != 0) {
+        double s = 0.0;
+        for (int q = lane; q <= j; q += 32) s = fma(hc[sy * hstride + q], hs[sy * hstride + q], s);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        const double n2 = hs[sy * hstride + j + 1], r2 = n2 - s;
+        givens_step(k, sy, j, hs, hstride, nullptr, 0, 1.0, sqrt(fmax(r2, 1e-7 * n2)), !(r2 > 1e-3 * n2), shg[warp]);
+    }
+    bool any;
+    if (ncase == 1) {
+        __syncthreads();
+        any = __syncthreads_or(threadIdx.x < 4 && k.ctl[kCtlRunning * k.ns + threadIdx.x] != 0) != 0;
+        if (!any && warp < 4) cycle_solve(k, sy);
+    } else {
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            __threadfence();
+            is_last = atomicInc(cd.ticket, ncase - 1) == (unsigned)(ncase - 1);
+            __threadfence();
+        }
+        __syncthreads();
+        if (!is_last) return;
+        int a = 0;
+        for (int q = threadIdx.x; q < k.ns; q += blockDim.x) a |= __ldcg(k.ctl + kCtlRunning * k.ns + q);
+        any = __syncthreads_or(a) != 0;
+    }
+    if (threadIdx.x == 0) put_cond(cd, any);
 }
 
 // Start (first) or restart of a system, one block each: the norm of the stored
@@ -365,6 +416,67 @@ __global__ void __cluster_dims__(4, 1, 1) __launch_bounds__(kReduceThreads)
     bool last;
     const bool any = any_flag(k.ctl + kCtlActive * k.ns, k.ns, cd.ticket, &last);
     if (last) set_cond(cd, any);
+}
+
+// w -= sum_{k<=j} c_k V_k for the running systems, w = 0 for the others, and the end
+// of Arnoldi index j: the first ncase blocks are control_end's, the others take
+// kBlock cells each.  J as k32_apply_dots (the loads of all vectors first).
+template <int J>
+__global__ void __launch_bounds__(kBlock) k32_update(int64_t T, const int32_t *__restrict__ blk_case, Krylov kr,
+                                                     int ncase, const float *__restrict__ V, float *__restrict__ wn,
+                                                     int j, const double *__restrict__ hs_raw,
+                                                     const double *__restrict__ hc, int hstride,
+                                                     const int32_t *__restrict__ ran, Cond cd)
+{
+    if (J > 0) j = J - 1;
+    __shared__ double shg[4][4][kMaxRestart + 1];
+    __shared__ float hs[kMaxRestart][4];
+    if ((int)blockIdx.x < ncase) {
+        control_end(kr, blockIdx.x, ncase, j, hs_raw, hc, hstride, ran, cd, shg);
+        return;
+    }
+    const int64_t b = blockIdx.x - ncase, i = b * kBlock + threadIdx.x;
+    const int c = blk_case[b];
+    const int4 r = reinterpret_cast<const int4 *>(ran)[c];
+    if ((r.x | r.y | r.z | r.w) == 0) return;
+    for (int q = threadIdx.x; q < 4 * (j + 1); q += blockDim.x)
+        hs[q >> 2][q & 3] = -float(hc[(4 * c + (q & 3)) * hstride + (q >> 2)]);
+    const bool on[4] = {r.x != 0, r.y != 0, r.z != 0, r.w != 0};
+    __syncthreads();
+    if (i >= T) return;
+    const int64_t vs = 20 * T;
+    float w[5][4];
+#pragma unroll
+    for (int l = 0; l < 5; ++l) vload(wn, l, T, i, w[l]);
+    if constexpr (J > 0) {
+        float t[J][5][4];
+#pragma unroll
+        for (int k = 0; k < J; ++k)
+#pragma unroll
+            for (int l = 0; l < 5; ++l) vload(V + k * vs, l, T, i, t[k][l]);
+#pragma unroll
+        for (int k = 0; k < J; ++k)
+#pragma unroll
+            for (int l = 0; l < 5; ++l)
+#pragma unroll
+                for (int v = 0; v < 4; ++v) w[l][v] = fmaf(hs[k][v], t[k][l][v], w[l][v]);
+    } else {
+#pragma unroll 2
+        for (int k = 0; k <= j; ++k)
+#pragma unroll
+            for (int l = 0; l < 5; ++l) {
+                float t[4];
+                vload(V + k * vs, l, T, i, t);
+#pragma unroll
+                for (int v = 0; v < 4; ++v) w[l][v] = fmaf(hs[k][v], t[v], w[l][v]);
+            }
+    }
+#pragma unroll
+    for (int l = 0; l < 5; ++l) {
+#pragma unroll
+        for (int v = 0; v < 4; ++v) w[l][v] = on[v] ? w[l][v] : 0.0f;
+        vstore(wn, l, T, i, w[l]);
+    }
 }
 
 // Scale of the first residual of a solve, one block per system: |b|^2 from the

@@ -48,7 +48,7 @@ enum : int {
 enum : int { kStatusNonPhys = 1, kStatusNoConv = 2, kStatusTimeout = 4 };
 
 // GMRES control words, ctl[field * ns + system] with system = case * 4 + variable.
-enum : int { kCtlActive = 0, kCtlRunning = 1, kCtlJv = 2, kCtlIters = 3, kCtlTwice = 4, kCtlFields = 5 };
+enum : int { kCtlActive = 0, kCtlRunning = 1, kCtlJv = 2, kCtlIters = 3, kCtlTwice = 4, kCtlRan = 5, kCtlFields = 6 };
 
 // Device data, all in internal (per-case RCM, padded) cell order.
 struct DeviceMesh {

@@ -431,9 +431,10 @@ __device__ __forceinline__ void df_add(float x, float y, float &h, float &l)
 }
 
 // Block sums of K x 4 FP32 values per thread, sv[k][v]: FP32 within a warp (at
-// most 160 products each), added across the warps to 48 bits: part[k0 + k][v][row].
+// most 160 products each), added across the warps to 48 bits: part[k0 + k][v][row], k < n.
 template <int K>
-__device__ __forceinline__ void block_rows32(float (&sv)[K][4], float (*sh)[K][4], double *__restrict__ part, int k0)
+__device__ __forceinline__ void block_rows32(float (&sv)[K][4], float (*sh)[K][4], double *__restrict__ part, int k0,
+                                             int n = K)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
@@ -452,7 +453,7 @@ __device__ __forceinline__ void block_rows32(float (&sv)[K][4], float (*sh)[K][4
         if ((lane & 7) == 0) sh[warp][k][lane >> 3] = s;
     }
     __syncthreads();
-    if (threadIdx.x < 4 * K) {
+    if (threadIdx.x < 4 * min(K, n)) {
         const int k = threadIdx.x / 4, v = threadIdx.x % 4;
         float h = 0.0f, l = 0.0f;
 #pragma unroll
@@ -461,9 +462,9 @@ __device__ __forceinline__ void block_rows32(float (&sv)[K][4], float (*sh)[K][4
     }
 }
 
-// y = K z and the products <V_k, y>, k <= j, of the Gram-Schmidt pass; J > 0: the
-// Arnoldi index j = J - 1 is a compile-time constant (all products before one
-// block-wide pass), J = 0: two basis vectors at a time
+// y = K z - V_j (gks_solve64.cuh), the products <V_k, y>, k <= j, of the Gram-Schmidt
+// pass and |y|^2 (k = j + 1); J > 0: the Arnoldi index j = J - 1 is a compile-time
+// constant (all products before one block-wide pass), J = 0: two sums at a time
 template <int J>
 __global__ void __launch_bounds__(kBlock, 3) k32_apply_dots(int64_t T, const int32_t *__restrict__ nb,
                                                             const float4 *__restrict__ op,
@@ -473,96 +474,61 @@ __global__ void __launch_bounds__(kBlock, 3) k32_apply_dots(int64_t T, const int
                                                             const float *__restrict__ V, int j,
                                                             double *__restrict__ part)
 {
-    constexpr int N = J > 0 ? J : 2;
+    constexpr int N = J > 0 ? J + 1 : 2;
     __shared__ float sh[kBlock / 32][N][4];
     if (!case_runs(blk_case, run)) return;
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    float u[5][4] = {};
+    const int64_t vs = 20 * T;
+    if (J > 0) j = J - 1;
+    float u[5][4] = {}, sv[N][4] = {};
+    // the last two sums: <V_j, y> and |y|^2
     if (i < T) {
         apply32(T, nb, op, z, i, u);
 #pragma unroll
-        for (int l = 0; l < 5; ++l) vstore(y, l, T, i, u[l]);
+        for (int l = 0; l < 5; ++l) {
+            float t[4];
+            vload(V + j * vs, l, T, i, t);
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                u[l][v] -= t[v];
+                sv[N - 2][v] = fmaf(t[v], u[l][v], sv[N - 2][v]);
+                sv[N - 1][v] = fmaf(u[l][v], u[l][v], sv[N - 1][v]);
+            }
+            vstore(y, l, T, i, u[l]);
+        }
     }
-    const int64_t vs = 20 * T;
-    for (int k0 = 0; k0 <= (J > 0 ? 0 : j); k0 += N) {
-        float sv[N][4] = {};
+    if constexpr (J > 0) {
         if (i < T)
 #pragma unroll
-            for (int k = 0; k < N; ++k) {
-                if (J == 0 && k0 + k > j) continue;
-#pragma unroll
-                for (int l = 0; l < 5; ++l) {
-                    float t[4];
-                    vload(V + (k0 + k) * vs, l, T, i, t);
-#pragma unroll
-                    for (int v = 0; v < 4; ++v) sv[k][v] = fmaf(t[v], u[l][v], sv[k][v]);
-                }
-            }
-        if (J == 0 && k0 > 0) __syncthreads();
-        block_rows32<N>(sv, sh, part, k0);
-    }
-}
-
-// w -= sum_{k<=j} c_k V_k for the running systems, w = 0 for the others, and the
-// partial |w|^2.  J as k32_apply_dots (the loads of all vectors first).
-template <int J>
-__global__ void __launch_bounds__(kBlock) k32_update_norm(int64_t T, const int32_t *__restrict__ blk_case,
-                                                          const int32_t *__restrict__ run,
-                                                          const float *__restrict__ V, float *__restrict__ wn, int j,
-                                                          const double *__restrict__ hc, int hstride,
-                                                          double *__restrict__ part)
-{
-    if (J > 0) j = J - 1;
-    __shared__ float sh[kBlock / 32][1][4];
-    __shared__ float hs[kMaxRestart][4];
-    if (!case_runs(blk_case, run)) return;
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const int c = blk_case[(blockIdx.x * (int64_t)blockDim.x) / kBlock];
-    for (int q = threadIdx.x; q < 4 * (j + 1); q += blockDim.x)
-        hs[q >> 2][q & 3] = -float(hc[(4 * c + (q & 3)) * hstride + (q >> 2)]);
-    const int4 r = reinterpret_cast<const int4 *>(run)[c];
-    const bool on[4] = {r.x != 0, r.y != 0, r.z != 0, r.w != 0};
-    __syncthreads();
-    const int64_t vs = 20 * T;
-    float nrm[1][4] = {};
-    if (i < T) {
-        float w[5][4];
-#pragma unroll
-        for (int l = 0; l < 5; ++l) vload(wn, l, T, i, w[l]);
-        if constexpr (J > 0) {
-            float t[J][5][4];
-#pragma unroll
-            for (int k = 0; k < J; ++k)
-#pragma unroll
-                for (int l = 0; l < 5; ++l) vload(V + k * vs, l, T, i, t[k][l]);
-#pragma unroll
-            for (int k = 0; k < J; ++k)
-#pragma unroll
-                for (int l = 0; l < 5; ++l)
-#pragma unroll
-                    for (int v = 0; v < 4; ++v) w[l][v] = fmaf(hs[k][v], t[k][l][v], w[l][v]);
-        } else {
-#pragma unroll 2
-            for (int k = 0; k <= j; ++k)
+            for (int k = 0; k < J - 1; ++k)
 #pragma unroll
                 for (int l = 0; l < 5; ++l) {
                     float t[4];
                     vload(V + k * vs, l, T, i, t);
 #pragma unroll
-                    for (int v = 0; v < 4; ++v) w[l][v] = fmaf(hs[k][v], t[v], w[l][v]);
+                    for (int v = 0; v < 4; ++v) sv[k][v] = fmaf(t[v], u[l][v], sv[k][v]);
                 }
-        }
+        block_rows32<N>(sv, sh, part, 0);
+    } else {
+        block_rows32<N>(sv, sh, part, j);
+        for (int k0 = 0; k0 < j; k0 += N) {
+            float s2[N][4] = {};
+            if (i < T)
 #pragma unroll
-        for (int l = 0; l < 5; ++l) {
+                for (int k = 0; k < N; ++k) {
+                    if (k0 + k >= j) continue;
 #pragma unroll
-            for (int v = 0; v < 4; ++v) {
-                w[l][v] = on[v] ? w[l][v] : 0.0f;
-                nrm[0][v] = fmaf(w[l][v], w[l][v], nrm[0][v]);
-            }
-            vstore(wn, l, T, i, w[l]);
+                    for (int l = 0; l < 5; ++l) {
+                        float t[4];
+                        vload(V + (k0 + k) * vs, l, T, i, t);
+#pragma unroll
+                        for (int v = 0; v < 4; ++v) s2[k][v] = fmaf(t[v], u[l][v], s2[k][v]);
+                    }
+                }
+            __syncthreads();
+            block_rows32<N>(s2, sh, part, k0, j - k0);
         }
     }
-    block_rows32<1>(nrm, sh, part, 0);
 }
 
 }  // namespace

@@ -32,3 +32,22 @@ def test_reconstruction_matches_oracle(n, sweeps, gmres_m):
     coef, info = gm.cls_reconstruct(dev(c.w0))
     assert max(info["relres"]) <= 1e-12
     assert np.max(np.abs(host(coef) - ref)) <= 1e-9 * np.max(np.abs(ref))
+
+
+@pytest.mark.parametrize("n", [3, 4, 12])
+@pytest.mark.parametrize("inner_rtol,gmres_m", [(1e-3, 8), (1e-7, 8), (1e-7, 3), (1e-7, 30)])
+def test_mixed_reconstruction_matches_oracle(n, inner_rtol, gmres_m):
+    """The mixed solve ends each Arnoldi index in the update's launch, with the new
+    vector's norm from the projections: cycles that end early, at the restart
+    length, and beyond the indices that are unrolled (1e-7 takes five or six)."""
+    from oracle import oracle as O
+    from paper_1802_00704_gb300 import build, gks
+    O.build()
+    build.build()
+    c = I.advection_case(n)
+    ref, _, _, bad = O.OracleMesh(c.mesh).cls_solve(c.w0)
+    assert not bad
+    gm = gks.GksMesh(c.mesh, precision=gks.MIXED, basis_fp32=1, inner_rtol=inner_rtol, gmres_m=gmres_m, gmres_maxit=200)
+    coef, info = gm.cls_reconstruct(dev(c.w0))
+    assert max(info["relres"]) <= 1e-12
+    assert np.max(np.abs(host(coef) - ref)) <= 1e-9 * np.max(np.abs(ref))
