@@ -1446,14 +1446,17 @@ void solve64_apply_dots(gks_mesh *m, const double *z, const double *V, double *y
     });
 }
 
-void solve64_update(gks_mesh *m, const double *V, double *w, int j, int ps, cudaStream_t q)
+// the first update with the end of Arnoldi index j
+void solve64_update(gks_mesh *m, const Krylov &kry, const double *V, double *w, int j, int ps, const Cond &cd,
+                    cudaStream_t q)
 {
     const DeviceMesh &d = m->d;
     const Work &k = m->wk;
     with_cells(m->wk.c64, [&](auto C) {
-        k64_update<decltype(C)::value><<<rows64(m), kW64, acc64(j, kAccStride + 1), q>>>(
-            d.T, d.blk_case, d.case_blk, k.ctl + kCtlRunning * k.ns, V, w, j, k.hcol, k.hco, ps,
-            k.ctl + kCtlTwice * k.ns, k.part);
+        k64_update<decltype(C)::value>
+            <<<m->n_case + rows64(m), kW64, std::max(acc64(j, kAccStride + 1), 4 * sizeof(GivensRows)), q>>>(
+                d.T, d.blk_case, kry, m->n_case, V, w, j, k.hcol, k.hco, ps, k.ctl + kCtlRan * k.ns,
+                k.ctl + kCtlTwice * k.ns, cd, k.part);
     });
 }
 
@@ -2033,10 +2036,10 @@ gks_status cls_solve_t(gks_mesh *m, TB *V, cudaStream_t s, int32_t *iters, doubl
         // (C64, fused_dots: and |w|^2)
         k_reduce<<<dim3(j + (C64 || fused_dots ? 2 : 1), ns), kReduceThreads, 0, q>>>(
             k.part, rs * (int64_t)nb, d.case_blk, rs, k.hcol, ps, k.vn, mm + 1, k.hco, ps, j + 1, nullptr,
-            k.ctl + kCtlRunning * ns, fused_dots ? k.ctl + kCtlRan * ns : nullptr);
+            k.ctl + kCtlRunning * ns, C64 || fused_dots ? k.ctl + kCtlRan * ns : nullptr);
         note_launch();
         if (C64) {
-            solve64_update(m, reinterpret_cast<const double *>(V), reinterpret_cast<double *>(vj1), j, ps, q);
+            solve64_update(m, kry, reinterpret_cast<const double *>(V), reinterpret_cast<double *>(vj1), j, ps, cd, q);
         } else if (fused_dots) {
             solve32_update(m, kry, reinterpret_cast<const float *>(V), reinterpret_cast<float *>(vj1), j, ps, cd, q);
             prof_stop(m, slot, q);
@@ -2060,9 +2063,12 @@ gks_status cls_solve_t(gks_mesh *m, TB *V, cudaStream_t s, int32_t *iters, doubl
                 note_launch();
             }
         }
-        // |V_{j+1}| and the Givens step of every system (and the end of a single mesh's cycle)
+        // |V_{j+1}| and the Givens step of every system (and the end of a single mesh's cycle);
+        // C64: of the systems with a second pass, the index is counted already
+        Cond ce = cd;
+        if (C64) ce.slot = -1;
         k_arnoldi_end<<<ns, kReduceThreads, 0, q>>>(kry, k.part, rs * (int64_t)nb, d.case_blk, rs, j, k.hcol, ps,
-                                                        mixed ? nullptr : k.y, mm, twice, C64 ? 1.0 : 0.0, cd);
+                                                        mixed ? nullptr : k.y, mm, twice, C64 ? 1.0 : 0.0, ce);
         note_launch();
         prof_stop(m, slot, q);
         GKS_CUDA(cudaGetLastError());

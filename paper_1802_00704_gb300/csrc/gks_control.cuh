@@ -303,8 +303,9 @@ __global__ void __launch_bounds__(32 * kSolveWarps) k_cycle_solve(Krylov k)
 }
 
 // End of Arnoldi index j, one block per system: |V_{j+1}| of a running system
-// from the summed partials and its Givens step (twice, may be NULL: the systems
-// that ran the second Gram-Schmidt pass); then the condition "any system
+// from the summed partials and its Givens step (twice given: only of the systems
+// flagged there, which ran the second Gram-Schmidt pass, the others are done; no
+// such system: nothing to do); then the condition "any system
 // still runs" and, for a single mesh, the solve of the cycle once none does.
 __global__ void __cluster_dims__(4, 1, 1) __launch_bounds__(kReduceThreads)
     k_arnoldi_end(Krylov k, const double *part, int64_t R, const int32_t *__restrict__ seg, int rs, int j,
@@ -314,9 +315,14 @@ __global__ void __cluster_dims__(4, 1, 1) __launch_bounds__(kReduceThreads)
     __shared__ double sh[kReduceThreads / 32];
     __shared__ double shg[4][kMaxRestart + 1];
     const int sy = blockIdx.x, c = sy >> 2;
-    if (k.ctl[kCtlRunning * k.ns + sy] != 0) {
+    if (twice) {
+        int a = 0;
+        for (int q = threadIdx.x; q < k.ns; q += blockDim.x) a |= twice[q];
+        if (__syncthreads_or(a) == 0) return;
+    }
+    if (k.ctl[kCtlRunning * k.ns + sy] != 0 && (!twice || twice[sy])) {
         const double acc = block_sum(part, 0, sy & 3, R, rs * seg[c], rs * seg[c + 1], sh);
-        if (threadIdx.x < 32) givens_step(k, sy, j, hc, hstride, twice && !twice[sy] ? nullptr : h2, h2stride, shift, sqrt(acc), false, shg);
+        if (threadIdx.x < 32) givens_step(k, sy, j, hc, hstride, h2, h2stride, shift, sqrt(acc), false, shg);
     }
     bool last;
     const bool any = any_flag(k.ctl + kCtlRunning * k.ns, k.ns, cd.ticket, &last);
@@ -326,32 +332,55 @@ __global__ void __cluster_dims__(4, 1, 1) __launch_bounds__(kReduceThreads)
 }
 
 // End of Arnoldi index j inside the update's launch, a block per case with a warp
-// per system: the basis holds K Z_j - V_j, at least half of whose norm is orthogonal to it as
-// a rule (gks_solve64.cuh), so the new vector's norm follows from |w|^2 (n2 = hs[j + 1])
-// and the projections, and the Givens step needs no sum over the updated vector.
-// A system with little left (below 3 % of |w|, where the difference loses
-// its digits) ends its cycle.  ran: the running systems before this launch.
+// per system: the basis holds w = K Z_j - V_j, at least half of whose norm is
+// orthogonal to it as a rule (gks_solve64.cuh), so the new vector's norm follows from
+// |w|^2 (hs[j + 1]) and the projections, and the Givens step needs no sum over the
+// updated vector.  ran: the running systems before this launch.
+//  - FP64: the difference of the squares keeps its digits (within a factor of 4);
+//    a system with less than half of |w| left gets the second Gram-Schmidt pass and
+//    its Givens step from the launches that follow (twice[system] = 1);
+//  - mixed: a system with less than 3 % left, where an FP32 basis loses the digits,
+//    ends its cycle (twice NULL).
+
+// |w|^2 of system sy and the part of it that the projections take, to every lane
+__device__ __forceinline__ double projected(const double *hs, const double *hc, int hstride, int sy, int j, double *n2)
+{
+    double s = 0.0;
+    for (int q = threadIdx.x & 31; q <= j; q += 32) s = fma(hc[sy * hstride + q], hs[sy * hstride + q], s);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    *n2 = hs[sy * hstride + j + 1];
+    return s;
+}
+
+__device__ __forceinline__ bool needs_second(double s, double n2) { return !(n2 > 0.0 && s <= 0.75 * n2); }
+
+typedef double GivensRows[4][kMaxRestart + 1];
+
 __device__ __forceinline__ void control_end(const Krylov &k, int c, int ncase, int j, const double *hs, const double *hc,
-                                            int hstride, const int32_t *ran, const Cond &cd,
-                                            double (*shg)[4][kMaxRestart + 1])
+                                            int hstride, const int32_t *ran, int32_t *twice, const Cond &cd,
+                                            GivensRows *shg)
 {
     __shared__ int is_last;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, sy = 4 * c + (warp & 3);
-    if (warp < 4 && ran[sy] != 0) {
-        double s = 0.0;
-        for (int q = lane; q <= j; q += 32) s = fma(hc[sy * hstride + q], hs[sy * hstride + q], s);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        const double n2 = hs[sy * hstride + j + 1], r2 = n2 - s;
-        givens_step(k, sy, j, hs, hstride, nullptr, 0, 1.0, sqrt(fmax(r2, 1e-7 * n2)), !(r2 > 1e-3 * n2), shg[warp]);
+    const int warp = threadIdx.x >> 5, sy = 4 * c + (warp & 3);
+    if (warp < 4) {
+        bool again = false;
+        if (ran[sy] != 0) {
+            double n2;
+            const double s = projected(hs, hc, hstride, sy, j, &n2), r2 = n2 - s;
+            again = twice && needs_second(s, n2);
+            if (!again)
+                givens_step(k, sy, j, hs, hstride, nullptr, 0, 1.0, sqrt(fmax(r2, 1e-7 * n2)),
+                            !twice && !(r2 > 1e-3 * n2), shg[warp]);
+        }
+        if (twice && (threadIdx.x & 31) == 0) twice[sy] = again;
     }
     bool any;
+    __syncthreads();
     if (ncase == 1) {
-        __syncthreads();
         any = __syncthreads_or(threadIdx.x < 4 && k.ctl[kCtlRunning * k.ns + threadIdx.x] != 0) != 0;
         if (!any && warp < 4) cycle_solve(k, sy);
     } else {
-        __syncthreads();
         if (threadIdx.x == 0) {
             __threadfence();
             is_last = atomicInc(cd.ticket, ncase - 1) == (unsigned)(ncase - 1);
@@ -418,6 +447,63 @@ __global__ void __cluster_dims__(4, 1, 1) __launch_bounds__(kReduceThreads)
     if (last) set_cond(cd, any);
 }
 
+// First Gram-Schmidt update w -= sum_k h_k V_k of the FP64 solve (32 C cells per
+// block) and the end of Arnoldi index j (the first ncase blocks); a system that
+// needs the second pass also gets the products <V_k, w>.  Dynamic shared memory:
+// 4 (j + 1) (kAccStride + 1) doubles, at least four GivensRows.
+template <int C>
+__global__ void __launch_bounds__(kW64) k64_update(int64_t T, const int32_t *__restrict__ blk_case, Krylov kr, int ncase,
+                                                   const double *__restrict__ V, double *__restrict__ wn, int j,
+                                                   const double *__restrict__ hs, const double *__restrict__ hc,
+                                                   int hstride, const int32_t *__restrict__ ran, int32_t *twice,
+                                                   Cond cd, double *__restrict__ part)
+{
+    extern __shared__ double sh64[];
+    if ((int)blockIdx.x < ncase) {
+        control_end(kr, blockIdx.x, ncase, j, hs, hc, hstride, ran, twice, cd, reinterpret_cast<GivensRows *>(sh64));
+        return;
+    }
+    const int64_t b = blockIdx.x - ncase, R = gridDim.x - ncase, c0 = b * (32 * C);
+    const Warp64 w = warp64(blk_case, ran, c0);
+    if (!w.run) return;
+    const int K = j + 1;
+    double *acc = sh64 + w.v * K * (kAccStride + 1), *h = acc + K * kAccStride, n2;
+    const double s0 = projected(hs, hc, hstride, w.sys, j, &n2);
+    const bool again = needs_second(s0, n2);
+    for (int k = w.lane; k < K; k += 32) h[k] = hc[w.sys * hstride + k];
+    for (int k = 0; k < K; ++k) acc[k * kAccStride + w.lane] = 0.0;
+    __syncwarp();
+    const int64_t vo = (int64_t)w.v * 5 * T, vs = 20 * T;
+    for (int c = 0; c < C; ++c) {
+        const int64_t i = c0 + 32 * c + w.lane;
+        if (i >= T) break;
+        double u[5];
+#pragma unroll
+        for (int l = 0; l < 5; ++l) u[l] = wn[vo + l * T + i];
+#pragma unroll 4
+        for (int k = 0; k < K; ++k) {
+            const double *vk = V + k * vs + vo + i;
+            const double hk = -h[k];
+#pragma unroll
+            for (int l = 0; l < 5; ++l) u[l] = fma(hk, vk[l * T], u[l]);
+        }
+#pragma unroll
+        for (int l = 0; l < 5; ++l) wn[vo + l * T + i] = u[l];
+        if (!again) continue;
+#pragma unroll 4
+        for (int k = 0; k < K; ++k) {
+            const double *vk = V + k * vs + vo + i;
+            double s = acc[k * kAccStride + w.lane];
+#pragma unroll
+            for (int l = 0; l < 5; ++l) s = fma(vk[l * T], u[l], s);
+            acc[k * kAccStride + w.lane] = s;
+        }
+    }
+    if (!again) return;
+    __syncwarp();
+    warp_rows(acc, K, w.lane, part + w.v * R + b, 4 * R);
+}
+
 // w -= sum_{k<=j} c_k V_k for the running systems, w = 0 for the others, and the end
 // of Arnoldi index j: the first ncase blocks are control_end's, the others take
 // kBlock cells each.  J as k32_apply_dots (the loads of all vectors first).
@@ -429,10 +515,10 @@ __global__ void __launch_bounds__(kBlock) k32_update(int64_t T, const int32_t *_
                                                      const int32_t *__restrict__ ran, Cond cd)
 {
     if (J > 0) j = J - 1;
-    __shared__ double shg[4][4][kMaxRestart + 1];
+    __shared__ GivensRows shg[4];
     __shared__ float hs[kMaxRestart][4];
     if ((int)blockIdx.x < ncase) {
-        control_end(kr, blockIdx.x, ncase, j, hs_raw, hc, hstride, ran, cd, shg);
+        control_end(kr, blockIdx.x, ncase, j, hs_raw, hc, hstride, ran, nullptr, cd, shg);
         return;
     }
     const int64_t b = blockIdx.x - ncase, i = b * kBlock + threadIdx.x;

@@ -336,77 +336,6 @@ __global__ void __launch_bounds__(kW64) k64_apply_dots(int64_t T, const int32_t 
     warp_rows(acc, K + 1, w.lane, part + w.v * (int64_t)gridDim.x + blockIdx.x, 4 * (int64_t)gridDim.x);
 }
 
-// First Gram-Schmidt update w -= sum_k h_k V_k, with the partial |w|^2 (column 0)
-// of a system that this leaves with at least half of its norm (hs: the sums <V_k, w>,
-// hc: the coefficients, hs[j + 1] = |w|^2), else the products <V_k, w> of a second
-// pass (twice[system] = 1, for the kernels after this one).
-template <int C>
-__global__ void __launch_bounds__(kW64) k64_update(int64_t T, const int32_t *__restrict__ blk_case,
-                                                   const int32_t *__restrict__ case_blk,
-                                                   const int32_t *__restrict__ run, const double *__restrict__ V,
-                                                   double *__restrict__ wn, int j, const double *__restrict__ hs,
-                                                   const double *__restrict__ hc, int hstride,
-                                                   int32_t *__restrict__ twice, double *__restrict__ part)
-{
-    extern __shared__ double sh64[];
-    const int64_t c0 = blockIdx.x * (int64_t)(32 * C);
-    const Warp64 w = warp64(blk_case, run, c0);
-    if (!w.run) return;
-    const int K = j + 1;
-    double *acc = sh64 + w.v * K * (kAccStride + 1), *h = acc + K * kAccStride;
-    double nr = 0.0;
-    for (int k = w.lane; k < K; k += 32) {
-        h[k] = hc[w.sys * hstride + k];
-        nr = fma(h[k], hs[w.sys * hstride + k], nr);      // |projection on V_k|^2
-    }
-    for (int k = 0; k < K; ++k) acc[k * kAccStride + w.lane] = 0.0;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) nr += __shfl_xor_sync(0xffffffffu, nr, o);
-    const double n2 = hs[w.sys * hstride + K];
-    const bool again = !(n2 > 0.0 && nr <= 0.75 * n2);
-    if (w.lane == 0 && c0 == (int64_t)case_blk[w.sys >> 2] * kBlock) twice[w.sys] = again;
-    nr = 0.0;
-    __syncwarp();
-    const int64_t vo = (int64_t)w.v * 5 * T, vs = 20 * T;
-    for (int c = 0; c < C; ++c) {
-        const int64_t i = c0 + 32 * c + w.lane;
-        if (i >= T) break;
-        double u[5];
-#pragma unroll
-        for (int l = 0; l < 5; ++l) u[l] = wn[vo + l * T + i];
-#pragma unroll 4
-        for (int k = 0; k < K; ++k) {
-            const double *vk = V + k * vs + vo + i;
-            const double hk = -h[k];
-#pragma unroll
-            for (int l = 0; l < 5; ++l) u[l] = fma(hk, vk[l * T], u[l]);
-        }
-#pragma unroll
-        for (int l = 0; l < 5; ++l) wn[vo + l * T + i] = u[l];
-        if (!again) {
-#pragma unroll
-            for (int l = 0; l < 5; ++l) nr = fma(u[l], u[l], nr);
-            continue;
-        }
-#pragma unroll 4
-        for (int k = 0; k < K; ++k) {
-            const double *vk = V + k * vs + vo + i;
-            double s = acc[k * kAccStride + w.lane];
-#pragma unroll
-            for (int l = 0; l < 5; ++l) s = fma(vk[l * T], u[l], s);
-            acc[k * kAccStride + w.lane] = s;
-        }
-    }
-    double *out = part + w.v * (int64_t)gridDim.x + blockIdx.x;
-    if (!again) {
-        nr = warp_sum(nr);
-        if (w.lane == 0) *out = nr;
-        return;
-    }
-    __syncwarp();
-    warp_rows(acc, K, w.lane, out, 4 * (int64_t)gridDim.x);
-}
-
 // The second pass of the systems that need it: w -= sum_k h_k V_k and the partial |w|^2
 template <int C>
 __global__ void __launch_bounds__(kW64) k64_update_norm(int64_t T, const int32_t *__restrict__ blk_case,
