@@ -1330,15 +1330,15 @@ gks_status precond_t(gks_mesh *m, const TP *Pg, const TP *alg, const TP *exg, co
 }
 
 // The sweeps of the FP64 solve of the per-cell equations (a thread per cell and
-// variable): dst = M^{-1} src with the arithmetic of the sweeps of precond_t.
-// Sweeps that only feed another sweep form the rows 0 and 1 alone; their
-// results alternate between dst and t2 so that the last one is in t2, and the
-// full z is in t3 (or dst without backward sweeps).
+// variable, see gks_solve64.cuh): dst = M^{-1} src with the sweeps of precond_t.
 //
-// The block-diagonal pass is folded into the first forward sweep (ilu_fuse_first;
+// z = P src is in t3 (rows 0 and 1 of it are z^0).  The rows 0 and 1 of the other
+// intermediate results go to four pairs of rows, two in t2 and two in dst; what the
+// last launch reads of neighbours, z^{ns-1} and x^{nsb-1}, is in t3 or t2.
+//
+// The first forward sweep is folded into the pivot launch (ilu_fuse_first;
 // the same results bit for bit) where a launch costs more than the FP64 work it
-// repeats, up to kFuse64 triangles: ten steps take 6,307 against 6,403 us at 800
-// triangles, 8,839 against 8,949 at 6,400, 9,933 against 9,909 at 20,000.
+// repeats, up to kFuse64 triangles.
 constexpr int64_t kFuse64 = 16000;
 
 gks_status precond64(gks_mesh *m, const double *src, double *dst, cudaStream_t s)
@@ -1349,36 +1349,30 @@ gks_status precond64(gks_mesh *m, const double *src, double *dst, cudaStream_t s
     const unsigned g = (unsigned)((T + 31) / 32);
     const int32_t *run = k.ctl + kCtlRunning * k.ns;
     const int ns = m->cfg.ilu_sweeps, nsb = m->cfg.ilu_sweeps_bwd < 0 ? ns : m->cfg.ilu_sweeps_bwd;
-    const bool fuse = ns > 0 && m->cfg.ilu_fuse_first && T <= kFuse64;
-    double *z = nsb > 0 ? k.t3 : dst;
-    // buffer of the q-th of n intermediate results
-    auto mid = [&](int q, int n) { return (n - 1 - q) % 2 == 0 ? k.t2 : dst; };
-    auto fwd = [&](int nb, bool full, const double *zin, double *zout) {
-#define F64(NB, FULL) k64_fwd<NB, FULL><<<g, kW64, 0, s>>>(T, d.nb, d.P, d.off, d.blk_case, run, src, zin, zout)
-        if (nb == 0) full ? F64(0, true) : F64(0, false);
-        else if (nb == 1) full ? F64(1, true) : F64(1, false);
-        else full ? F64(2, true) : F64(2, false);
-#undef F64
+    // forward sweeps of the rows 0 and 1: z^ns is the start of the backward sweeps
+    const int nf = nsb > 0 ? ns : ns - 1;
+    const bool fuse = nf > 0 && m->cfg.ilu_fuse_first && T <= kFuse64;
+    double *z = ns + nsb > 0 ? k.t3 : dst;
+    double *t2a = k.t2, *t2b = k.t2 + 2 * T, *da = dst, *db = dst + 2 * T;
+    // z^q (0 < q <= nf), z^{ns-1} in t2a; z^ns in da (t2b where the last launch reads it as x^0)
+    auto zq = [&](int q) { return q == 0 ? z : (q == ns ? (nsb == 1 ? t2b : da) : ((ns - 1 - q) % 2 == 0 ? t2a : da)); };
+    // x^q (q < nsb), x^0 = z^ns, x^{nsb-1} in t2b
+    auto xq = [&](int q) { return q == 0 ? zq(ns) : ((nsb - 1 - q) % 2 == 0 ? t2b : db); };
+    if (fuse) k64_pivot<true><<<g, kW64, 0, s>>>(T, d.nb, d.P, d.w64, d.blk_case, run, src, z, zq(1));
+    else k64_pivot<false><<<g, kW64, 0, s>>>(T, d.nb, d.P, d.w64, d.blk_case, run, src, z, nullptr);
+    note_launch();
+    for (int q = fuse ? 1 : 0; q < nf; ++q) {
+        k64_sweep<false><<<g, kW64, 0, s>>>(T, d.nb, d.w64, d.blk_case, run, z, zq(q), zq(q + 1));
         note_launch();
-    };
-    // forward: z^0 = P r (a launch of its own unless folded in), z^{q+1} = F(z^q)
-    const int nf = fuse ? ns : ns + 1;                    // launches
-    const double *prev = nullptr;
-    for (int q = 0; q < nf; ++q) {
-        const bool last = q + 1 == nf;
-        double *out = last ? z : mid(q, nf - 1);
-        fwd(q == 0 ? (fuse ? 2 : 0) : 1, last, prev, out);
-        prev = out;
     }
-    // backward: x^0 = z, x^{q+1} = B(x^q)
-    const double *x = z;
-    for (int q = 0; q < nsb; ++q) {
-        const bool last = q + 1 == nsb;
-        double *out = last ? dst : mid(q, nsb - 1);
-        if (last) k64_bwd<true><<<g, kW64, 0, s>>>(T, d.nb, d.P, d.off, d.blk_case, run, z, x, out);
-        else k64_bwd<false><<<g, kW64, 0, s>>>(T, d.nb, d.P, d.off, d.blk_case, run, z, x, out);
+    for (int q = 0; q + 1 < nsb; ++q) {
+        k64_sweep<true><<<g, kW64, 0, s>>>(T, d.nb, d.w64, d.blk_case, run, zq(ns), xq(q), xq(q + 1));
         note_launch();
-        x = out;
+    }
+    if (ns + nsb > 0) {
+        k64_last<<<g, kW64, 0, s>>>(T, d.nb, d.w64, d.blk_case, run, z, ns > 0 ? zq(ns - 1) : nullptr,
+                                    nsb > 0 ? xq(nsb - 1) : nullptr, dst);
+        note_launch();
     }
     GKS_CUDA(cudaGetLastError());
     return GKS_OK;
@@ -2290,6 +2284,8 @@ gks_status launch_pack(gks_mesh *m)
     const unsigned g = nblocks(d.T);
     if (d.off) {
         k64_off<<<g, kBlock>>>(d.T, d.alpha, d.ex, d.ey, d.off);
+        k64_products<<<g, kBlock>>>(d.T, d.P, d.off, d.w64);
+        note_launch();
         note_launch();
     }
     if (d.op32) {

@@ -861,6 +861,7 @@ gks_status build_batch(gks_mesh *m, const CaseIn *cases, int32_t n_cases)
     if (!ext) {
         if (cfg.precision == GKS_FP64) {
             if ((st = dalloc(m, &d.off, (size_t)9 * T)) != GKS_OK) return st;
+            if ((st = dalloc(m, &d.w64, (size_t)30 * T)) != GKS_OK) return st;
         } else {
             if ((st = dalloc(m, &d.op32, (size_t)24 * T)) != GKS_OK) return st;
             if (cfg.precond == GKS_PC_ILU_SWEEP &&

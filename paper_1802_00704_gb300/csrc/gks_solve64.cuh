@@ -11,12 +11,16 @@
 // warps of a variable whose system has stopped return at once.
 //
 // Three more things keep the instruction count down:
-//  - a sweep whose result only feeds another sweep forms the gradient rows 0
-//    and 1 of each cell alone, all that an off-diagonal block reads (10 of the
-//    25 products with the pivot inverse);
-//  - the off-diagonal blocks are stored multiplied out (off: alpha, alpha dx,
-//    alpha dy per slot), and only the lower (upper) slots of a cell enter the
-//    arithmetic of a triangular relation;
+//  - the sweeps work on the products W = P O of the pivot inverse and the
+//    off-diagonal blocks (set-up; 5 x 2, a block reads the gradient rows 0 and 1 of a
+//    neighbour alone): z = P r once, then rows 0 and 1 of z + sum W z per sweep (12
+//    multiply-adds; rows 0 and 1 are all that the next sweep reads), and the last
+//    sweep adds the lower and the upper neighbours' terms together, three slots
+//    of 10.  With P applied in every sweep, and the lower and upper slots
+//    apart (a warp's lanes have up to three of each), two sweeps each way
+//    took 152 multiply-adds, now 91;
+//  - the operator's off-diagonal blocks are stored multiplied out (off: alpha,
+//    alpha dx, alpha dy per slot);
 //  - sums over cells start their FMA chains from the running sum in shared
 //    memory and are added across the lanes of a warp in transposed order, 7-31
 //    additions for all Arnoldi indices together instead of 5 for each;
@@ -30,10 +34,10 @@
 //    second are there and return).  Three steps at 399,424 triangles 46.2 -> 41.9 ms,
 //    ten at 6,400 6.56 -> 6.06 ms, at 800 6.05 -> 5.50 ms.
 // Measured on GB300 (the solve's classes, per Arnoldi index, events around each
-// class): preconditioner with two sweeps each way 80 -> 25 us at 800 triangles
-// and 680 -> 448 us at 399,424; operator with the first Gram-Schmidt products and
-// the rest of the Gram-Schmidt passes 83 -> 46 us and 610 -> 528 us.  Two
-// backward sweeps in one launch, each thread forming its upper neighbours' first
+// class) against a thread per cell: preconditioner with two sweeps each way 80 -> 25 us
+// at 6,400 triangles and 680 -> 266 us at 399,424 (436 with P in every sweep);
+// operator with the first Gram-Schmidt products and the rest of the Gram-Schmidt
+// passes 83 -> 39 us and 610 -> 363 us.  Two backward sweeps in one launch, each thread forming its upper neighbours' first
 // sweep itself, were no faster at any size (6,323 against 6,307 us for ten steps
 // at 800 triangles, 10,285 against 9,933 at 20,000) and are not there.
 #pragma once
@@ -61,26 +65,6 @@ __device__ __forceinline__ void off_acc(double a, double ax, double ay, double g
     acc[4] = fma(ay, g2, acc[4]);
 }
 
-// The lower (UP = false: 0 <= j < i) or upper (j > i) neighbours of cell i, in
-// slot order: js[q], their slots ss[q], q < the returned number.
-template <bool UP>
-__device__ __forceinline__ int side_slots(const int32_t *__restrict__ nb, int64_t T, int64_t i, int *js, int *ss)
-{
-    int n = 0;
-    js[0] = js[1] = js[2] = (int)i;
-    ss[0] = ss[1] = ss[2] = 0;
-#pragma unroll
-    for (int s = 0; s < 3; ++s) {
-        const int j = nb[s * T + i];
-        if (!(UP ? j > (int)i : (j >= 0 && j < (int)i))) continue;
-        if (n == 0) { js[0] = j; ss[0] = s; }
-        else if (n == 1) { js[1] = j; ss[1] = s; }
-        else { js[2] = j; ss[2] = s; }
-        ++n;
-    }
-    return n;
-}
-
 struct Off64 {
     double a, ax, ay;
 };
@@ -105,6 +89,25 @@ __global__ void k64_off(int64_t T, const double *__restrict__ al, const double *
     }
 }
 
+// W = P O per slot (set-up): w[10 s + 2 a + c], row a, column c (the neighbour's row c)
+__global__ void k64_products(int64_t T, const double *__restrict__ P, const double *__restrict__ off,
+                             double *__restrict__ w)
+{
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= T) return;
+#pragma unroll
+    for (int s = 0; s < 3; ++s) {
+        const Off64 o = off_load(off, T, s, i);
+        for (int a = 0; a < 5; ++a) {
+            double p[5];
+#pragma unroll
+            for (int c = 0; c < 5; ++c) p[c] = P[(a * 5 + c) * T + i];
+            w[(10 * s + 2 * a) * T + i] = fma(p[0], o.a, fma(p[2], o.ax, p[3] * o.ay));
+            w[(10 * s + 2 * a + 1) * T + i] = fma(p[1], o.a, fma(p[3], o.ax, p[4] * o.ay));
+        }
+    }
+}
+
 // What every kernel of the solve knows about its warp: the variable, the first
 // cell of the block, and whether the system still runs.
 struct Warp64 {
@@ -123,111 +126,141 @@ __device__ __forceinline__ Warp64 warp64(const int32_t *__restrict__ blk_case, c
     return w;
 }
 
-// Forward relation z_i = P_i (r_i + sum_{k<i} O_ik zin_k).  NB 0: no neighbours
-// (z = P r); 1: zin as given; 2: zin_k = P_k r_k formed here (the first sweep).
-// FULL: all five rows of z, else the rows 0 and 1 that the next sweep reads.
-template <int NB, bool FULL>
-__global__ void __launch_bounds__(kW64) k64_fwd(int64_t T, const int32_t *__restrict__ nb,
-                                                const double *__restrict__ P, const double *__restrict__ off,
-                                                const int32_t *__restrict__ blk_case, const int32_t *__restrict__ run,
-                                                const double *__restrict__ r, const double *__restrict__ zin,
-                                                double *__restrict__ zout)
+// z = P r, all five rows, into zout; FIRST: also the rows 0 and 1 of the first
+// forward sweep, z_i + sum_{k<i} W_ik z_k with the neighbours' z formed here, into z1
+template <bool FIRST>
+__global__ void __launch_bounds__(kW64, FIRST ? 3 : 6)
+    k64_pivot(int64_t T, const int32_t *__restrict__ nb, const double *__restrict__ P, const double *__restrict__ W,
+              const int32_t *__restrict__ blk_case, const int32_t *__restrict__ run, const double *__restrict__ r,
+              double *__restrict__ zout, double *__restrict__ z1)
 {
+    constexpr int NS = FIRST ? 3 : 0;
     const int64_t c0 = blockIdx.x * (int64_t)32;
     const Warp64 w = warp64(blk_case, run, c0);
-    const int64_t i = c0 + w.lane;
+    const int64_t i = c0 + w.lane, vo = (int64_t)w.v * 5 * T;
     if (!w.run || i >= T) return;
-    const double *rv = r + (int64_t)w.v * 5 * T;
-    constexpr int NR = FULL ? 5 : 2;
-    double y[5], Pm[NR * 5];
+    const double *rv = r + vo;
+    double y[5], Pm[25], rj[NS + 1][5], pj[NS + 1][10], wj[NS + 1][4], o[2];
+    int js[NS + 1];
+#pragma unroll
+    for (int s = 0; s < NS; ++s) {
+        // a slot that is not a lower neighbour reads the cell's own values, times zero
+        const int j = nb[s * T + i];
+        js[s] = j >= 0 && j < (int)i ? j : (int)i;
+    }
 #pragma unroll
     for (int k = 0; k < 5; ++k) y[k] = rv[k * T + i];
 #pragma unroll
-    for (int k = 0; k < NR * 5; ++k) Pm[k] = P[k * T + i];
-    if (NB) {
-        int js[3], ss[3];
-        const int n = side_slots<false>(nb, T, i, js, ss);
-        // the loads of all neighbours first, then the sums
-        Off64 o[3];
-        double z[3][2], rj[NB == 2 ? 3 : 1][5], pj[NB == 2 ? 3 : 1][10];
+    for (int k = 0; k < 25; ++k) Pm[k] = P[k * T + i];
 #pragma unroll
-        for (int q = 0; q < 3; ++q)
-            if (q < n) {
-                const int64_t j = js[q];
-                o[q] = off_load(off, T, ss[q], i);
-                if (NB == 2) {
+    for (int s = 0; s < NS; ++s) {
 #pragma unroll
-                    for (int k = 0; k < 5; ++k) rj[q][k] = rv[k * T + j];
+        for (int k = 0; k < 5; ++k) rj[s][k] = rv[k * T + js[s]];
 #pragma unroll
-                    for (int k = 0; k < 10; ++k) pj[q][k] = P[k * T + j];
-                } else {
+        for (int k = 0; k < 10; ++k) pj[s][k] = P[k * T + js[s]];
 #pragma unroll
-                    for (int a = 0; a < 2; ++a) z[q][a] = zin[(w.v * 5 + a) * T + j];
-                }
-            }
-#pragma unroll
-        for (int q = 0; q < 3; ++q)
-            if (q < n) {
-                if (NB == 2)
-#pragma unroll
-                    for (int a = 0; a < 2; ++a) {
-                        double t = 0.0;
-#pragma unroll
-                        for (int c = 0; c < 5; ++c) t = fma(pj[q][a * 5 + c], rj[q][c], t);
-                        z[q][a] = t;
-                    }
-                off_acc(o[q].a, o[q].ax, o[q].ay, z[q][0], z[q][1], y);
-            }
+        for (int k = 0; k < 4; ++k) wj[s][k] = W[(10 * s + k) * T + i];
     }
 #pragma unroll
-    for (int a = 0; a < NR; ++a) {
+    for (int a = 0; a < 5; ++a) {
         double s = 0.0;
 #pragma unroll
         for (int c = 0; c < 5; ++c) s = fma(Pm[a * 5 + c], y[c], s);
-        zout[(w.v * 5 + a) * T + i] = s;
+        zout[vo + a * T + i] = s;
+        if (a < 2) o[a] = s;
     }
+#pragma unroll
+    for (int s = 0; s < NS; ++s) {
+        double z[2];
+#pragma unroll
+        for (int a = 0; a < 2; ++a) {
+            double t = 0.0;
+#pragma unroll
+            for (int c = 0; c < 5; ++c) t = fma(pj[s][a * 5 + c], rj[s][c], t);
+            z[a] = t;
+        }
+        const bool low = js[s] != (int)i;
+#pragma unroll
+        for (int a = 0; a < 2; ++a)
+            o[a] = fma(low ? wj[s][2 * a] : 0.0, z[0], fma(low ? wj[s][2 * a + 1] : 0.0, z[1], o[a]));
+    }
+    if (FIRST)
+#pragma unroll
+        for (int a = 0; a < 2; ++a) z1[vo + a * T + i] = o[a];
 }
 
-// Backward relation x_i = z_i + P_i sum_{j>i} O_ij xin_j (rows 0 and 1 alone
-// unless FULL)
-template <bool FULL>
-__global__ void __launch_bounds__(kW64) k64_bwd(int64_t T, const int32_t *__restrict__ nb,
-                                                const double *__restrict__ P, const double *__restrict__ off,
-                                                const int32_t *__restrict__ blk_case, const int32_t *__restrict__ run,
-                                                const double *__restrict__ z, const double *__restrict__ xin,
-                                                double *__restrict__ xout)
+// A sweep that only feeds another one, rows 0 and 1: out_i = base_i + sum_j W_ij
+// in_j over the lower (UP = false) or upper neighbours j
+template <bool UP>
+__global__ void __launch_bounds__(kW64) k64_sweep(int64_t T, const int32_t *__restrict__ nb,
+                                                  const double *__restrict__ W, const int32_t *__restrict__ blk_case,
+                                                  const int32_t *__restrict__ run, const double *__restrict__ base,
+                                                  const double *__restrict__ in, double *__restrict__ out)
 {
     const int64_t c0 = blockIdx.x * (int64_t)32;
     const Warp64 w = warp64(blk_case, run, c0);
-    const int64_t i = c0 + w.lane;
+    const int64_t i = c0 + w.lane, vo = (int64_t)w.v * 5 * T;
     if (!w.run || i >= T) return;
-    constexpr int NR = FULL ? 5 : 2;
-    double y[5] = {0.0, 0.0, 0.0, 0.0, 0.0}, zi[NR], Pm[NR * 5];
+    int js[3];
+    double wj[3][4], z[3][2], o[2];
 #pragma unroll
-    for (int k = 0; k < NR; ++k) zi[k] = z[(w.v * 5 + k) * T + i];
+    for (int s = 0; s < 3; ++s) js[s] = nb[s * T + i];
 #pragma unroll
-    for (int k = 0; k < NR * 5; ++k) Pm[k] = P[k * T + i];
-    int js[3], ss[3];
-    const int n = side_slots<true>(nb, T, i, js, ss);
-    Off64 o[3];
-    double x[3][2];
+    for (int a = 0; a < 2; ++a) o[a] = base[vo + a * T + i];
+    // the loads of all neighbours first, then the sums
 #pragma unroll
-    for (int q = 0; q < 3; ++q)
-        if (q < n) {
-            o[q] = off_load(off, T, ss[q], i);
+    for (int s = 0; s < 3; ++s) {
+        const int64_t j = js[s];
+        if (!(UP ? j > i : (j >= 0 && j < i))) continue;
 #pragma unroll
-            for (int a = 0; a < 2; ++a) x[q][a] = xin[(w.v * 5 + a) * T + js[q]];
-        }
+        for (int k = 0; k < 4; ++k) wj[s][k] = W[(10 * s + k) * T + i];
 #pragma unroll
-    for (int q = 0; q < 3; ++q)
-        if (q < n) off_acc(o[q].a, o[q].ax, o[q].ay, x[q][0], x[q][1], y);
-#pragma unroll
-    for (int a = 0; a < NR; ++a) {
-        double s = zi[a];
-#pragma unroll
-        for (int c = 0; c < 5; ++c) s = fma(Pm[a * 5 + c], y[c], s);
-        xout[(w.v * 5 + a) * T + i] = s;
+        for (int a = 0; a < 2; ++a) z[s][a] = in[vo + a * T + j];
     }
+#pragma unroll
+    for (int s = 0; s < 3; ++s) {
+        const int64_t j = js[s];
+        if (!(UP ? j > i : (j >= 0 && j < i))) continue;
+#pragma unroll
+        for (int a = 0; a < 2; ++a) o[a] = fma(wj[s][2 * a], z[s][0], fma(wj[s][2 * a + 1], z[s][1], o[a]));
+    }
+#pragma unroll
+    for (int a = 0; a < 2; ++a) out[vo + a * T + i] = o[a];
+}
+
+// The last sweep, x_i = z_i + sum_{j<i} W_ij low_j + sum_{j>i} W_ij up_j, all five
+// rows (low, up: the last sweep's sources; NULL: no sweeps that way)
+__global__ void __launch_bounds__(kW64, 4) k64_last(int64_t T, const int32_t *__restrict__ nb,
+                                                 const double *__restrict__ W, const int32_t *__restrict__ blk_case,
+                                                 const int32_t *__restrict__ run, const double *__restrict__ z,
+                                                 const double *__restrict__ low, const double *__restrict__ up,
+                                                 double *__restrict__ x)
+{
+    const int64_t c0 = blockIdx.x * (int64_t)32;
+    const Warp64 w = warp64(blk_case, run, c0);
+    const int64_t i = c0 + w.lane, vo = (int64_t)w.v * 5 * T;
+    if (!w.run || i >= T) return;
+    double o[5], g[3][2], wj[3][10];
+    int js[3];
+#pragma unroll
+    for (int s = 0; s < 3; ++s) js[s] = nb[s * T + i];
+#pragma unroll
+    for (int a = 0; a < 5; ++a) o[a] = z[vo + a * T + i];
+#pragma unroll
+    for (int s = 0; s < 3; ++s) {
+        const int64_t j = js[s];
+        const double *src = j < 0 ? nullptr : (j < i ? low : up);
+#pragma unroll
+        for (int a = 0; a < 2; ++a) g[s][a] = src ? src[vo + a * T + j] : 0.0;
+#pragma unroll
+        for (int k = 0; k < 10; ++k) wj[s][k] = W[(10 * s + k) * T + i];
+    }
+#pragma unroll
+    for (int s = 0; s < 3; ++s)
+#pragma unroll
+        for (int a = 0; a < 5; ++a) o[a] = fma(wj[s][2 * a], g[s][0], fma(wj[s][2 * a + 1], g[s][1], o[a]));
+#pragma unroll
+    for (int a = 0; a < 5; ++a) x[vo + a * T + i] = o[a];
 }
 
 // acc = (K x)_i of variable v, diagonal block minus the off-diagonal ones, minus
