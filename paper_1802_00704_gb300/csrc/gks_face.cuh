@@ -10,48 +10,37 @@ namespace {
 
 constexpr int kFluxBlock = 128;
 
-// Value and derivatives (global frame) of cell c's reconstruction (Eq. (19))
-// at the point whose scaled offsets from the centroid are (dx, dy).
-// o[6][4]: W, W_x, W_y, W_xx, W_xy, W_yy.
-__device__ __forceinline__ void recon(const DeviceMesh &d, const double *__restrict__ w,
-                                      const double *__restrict__ x, int c, double dx, double dy, double *o)
+// Value and derivatives of cell c's reconstruction (Eq. (19)) at the point whose
+// scaled offsets from the centroid are (dx, dy), in the face frame (n = (nx, ny),
+// t = (-ny, nx)): f[6][4], W, W_n, W_t, W_nn, W_nt, W_tt.  The rotation carries
+// the 1/h of the derivatives (21 instead of 32 multiply-adds per variable).
+__device__ __forceinline__ void recon_face(const DeviceMesh &d, const double *__restrict__ w,
+                                           const double *__restrict__ x, int c, double dx, double dy, double nx,
+                                           double ny, double *f)
 {
     const int64_t T = d.T;
     const double ih = 1.0 / d.h[c];
-    const double qx = dx * dx - d.mxx[c], qxy = dx * dy - d.mxy[c], qy = dy * dy - d.myy[c];
+    const double hx = 0.5 * (dx * dx - d.mxx[c]), xy = dx * dy - d.mxy[c], hy = 0.5 * (dy * dy - d.myy[c]);
+    const double cn = nx * ih, sn = ny * ih, cc = cn * cn, ss = sn * sn, cs = cn * sn, tr = ih * ih;
+    const double cs2 = 2.0 * cs, cd = cc - ss;
 #pragma unroll
     for (int v = 0; v < 4; ++v) {
         const double u1 = x[(v * 5 + 0) * T + c], u2 = x[(v * 5 + 1) * T + c], u3 = x[(v * 5 + 2) * T + c];
         const double u4 = x[(v * 5 + 3) * T + c], u5 = x[(v * 5 + 4) * T + c];
-        o[v] = w[v * T + c] + u1 * dx + u2 * dy + 0.5 * u3 * qx + u4 * qxy + 0.5 * u5 * qy;
-        o[4 + v] = (u1 + u3 * dx + u4 * dy) * ih;
-        o[8 + v] = (u2 + u4 * dx + u5 * dy) * ih;
-        o[12 + v] = u3 * ih * ih;
-        o[16 + v] = u4 * ih * ih;
-        o[20 + v] = u5 * ih * ih;
-    }
-}
-
-// Global rows -> face frame (n = (nx, ny), t = (-ny, nx)): directions of the
-// derivatives and the momentum components of every row.
-__device__ __forceinline__ void to_face(const double *g, double nx, double ny, double *f)
-{
-    const double tx = -ny, ty = nx;
-#pragma unroll
-    for (int v = 0; v < 4; ++v) {
-        const double gx = g[4 + v], gy = g[8 + v], gxx = g[12 + v], gxy = g[16 + v], gyy = g[20 + v];
-        f[v] = g[v];
-        f[4 + v] = nx * gx + ny * gy;
-        f[8 + v] = tx * gx + ty * gy;
-        f[12 + v] = nx * nx * gxx + 2.0 * nx * ny * gxy + ny * ny * gyy;
-        f[16 + v] = nx * tx * gxx + (nx * ty + ny * tx) * gxy + ny * ty * gyy;
-        f[20 + v] = tx * tx * gxx + 2.0 * tx * ty * gxy + ty * ty * gyy;
+        f[v] = w[v * T + c] + u1 * dx + u2 * dy + u3 * hx + u4 * xy + u5 * hy;
+        const double gx = u1 + u3 * dx + u4 * dy, gy = u2 + u4 * dx + u5 * dy;
+        f[4 + v] = cn * gx + sn * gy;
+        f[8 + v] = cn * gy - sn * gx;
+        const double nn = cc * u3 + cs2 * u4 + ss * u5;
+        f[12 + v] = nn;
+        f[16 + v] = cs * (u5 - u3) + cd * u4;
+        f[20 + v] = tr * (u3 + u5) - nn;
     }
 #pragma unroll
     for (int r = 0; r < 6; ++r) {
         const double mx = f[4 * r + 1], my = f[4 * r + 2];
         f[4 * r + 1] = nx * mx + ny * my;
-        f[4 * r + 2] = tx * mx + ty * my;
+        f[4 * r + 2] = nx * my - ny * mx;
     }
 }
 

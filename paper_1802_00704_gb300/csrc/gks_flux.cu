@@ -68,12 +68,10 @@ __global__ void __launch_bounds__(kFluxBlock, MIXED ? 4 : 1) k_face_flux(DeviceM
             }
             ok = kin::gp_flux_mixed_split<HEAT, KIN>(vl, vr, dl, dr, dt, gamma, K, mu, tau2, fk, prandtl);
         } else {
-            double gl[24], wl[24], wr[24];
-            recon(d, w, x, l, d.gl[(2 * k) * F + f], d.gl[(2 * k + 1) * F + f], gl);
-            to_face(gl, nx, ny, wl);
+            double wl[24], wr[24];
+            recon_face(d, w, x, l, d.gl[(2 * k) * F + f], d.gl[(2 * k + 1) * F + f], nx, ny, wl);
             if (r >= 0) {
-                recon(d, w, x, r, d.gr[(2 * k) * F + f], d.gr[(2 * k + 1) * F + f], gl);
-                to_face(gl, nx, ny, wr);
+                recon_face(d, w, x, r, d.gr[(2 * k) * F + f], d.gr[(2 * k + 1) * F + f], nx, ny, wr);
             } else {
                 const double bc[4] = {d.bc[f], d.bc[F + f], d.bc[2 * F + f], d.bc[3 * F + f]};
                 ghost(d.ftag[f], bc, nx, ny, gamma, wl, wr);

@@ -205,8 +205,9 @@ __device__ __forceinline__ bool case_runs(const int32_t *__restrict__ blk_case, 
     return (r.x | r.y | r.z | r.w) != 0;
 }
 
-// Forward relation z_i = P_i (r_i + sum_{k<i} O_ik zin_k); NB and FULL as
-// k64_fwd.  rc (may be NULL): also store float(r_i) for the later sweeps of a
+// Forward relation z_i = P_i (r_i + sum_{k<i} O_ik zin_k); NB 0: no neighbours
+// (z = P r); 1: zin as given; 2: zin_k = P_k r_k formed here (the first sweep).
+// FULL: all five rows of z, else the rows 0 and 1 that the next sweep reads.  rc (may be NULL): also store float(r_i) for the later sweeps of a
 // wider source.
 template <int NB, bool FULL, typename TR, typename TP>
 __global__ void __launch_bounds__(kW32, 5) k32_fwd(int64_t T, const int32_t *__restrict__ nb,
@@ -300,7 +301,7 @@ __device__ __forceinline__ void bwd_finish(const TP *__restrict__ pk, int64_t T,
     }
 }
 
-// Backward relation x_i = z_i + P_i sum_{j>i} O_ij xin_j; FULL as k64_bwd
+// Backward relation x_i = z_i + P_i sum_{j>i} O_ij xin_j; FULL as k32_fwd
 template <bool FULL, typename TP>
 __global__ void __launch_bounds__(kW32, 5) k32_bwd(int64_t T, const int32_t *__restrict__ nb,
                                                    const TP *__restrict__ pk, const int32_t *__restrict__ blk_case,

@@ -37,9 +37,7 @@
 // class) against a thread per cell: preconditioner with two sweeps each way 80 -> 25 us
 // at 6,400 triangles and 680 -> 266 us at 399,424 (436 with P in every sweep);
 // operator with the first Gram-Schmidt products and the rest of the Gram-Schmidt
-// passes 83 -> 39 us and 610 -> 363 us.  Two backward sweeps in one launch, each thread forming its upper neighbours' first
-// sweep itself, were no faster at any size (6,323 against 6,307 us for ten steps
-// at 800 triangles, 10,285 against 9,933 at 20,000) and are not there.
+// passes 83 -> 39 us and 610 -> 363 us.
 #pragma once
 
 #include "gks_internal.h"
