@@ -183,8 +183,9 @@ typedef struct gks_config {
     int32_t ilu_fuse_first; /* GKS_PC_ILU_SWEEP with ilu_sweeps > 0: 1 (default) the
                               block-diagonal pass z^0 = P r is folded into the first
                               forward sweep (each cell forms its lower neighbours'
-                              z^0 itself; GKS_FP64: on small meshes only); 0 a
-                              separate pass.  Same arithmetic, same results            */
+                              z^0 itself; GKS_FP64 with the per-cell equations: not
+                              folded); 0 a separate pass.  Same arithmetic, same
+                              results                                                 */
     int32_t flux_split;    /* mixed precision without the Prandtl correction: 1 (default)
                               half of the warps of the persistent face flux kernel
                               form the FP64 part (values, interface state, collision

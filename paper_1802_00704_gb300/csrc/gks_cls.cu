@@ -1336,10 +1336,12 @@ gks_status precond_t(gks_mesh *m, const TP *Pg, const TP *alg, const TP *exg, co
 // intermediate results go to four pairs of rows, two in t2 and two in dst; what the
 // last launch reads of neighbours, z^{ns-1} and x^{nsb-1}, is in t3 or t2.
 //
-// The first forward sweep is folded into the pivot launch (ilu_fuse_first;
-// the same results bit for bit) where a launch costs more than the FP64 work it
-// repeats, up to kFuse64 triangles.
-constexpr int64_t kFuse64 = 16000;
+// Up to this many triangles the second Gram-Schmidt pass of the systems that need it is a
+// block per system inside k_arnoldi_end; above, two launches over the whole GPU, which return
+// at once (about 1.3 us each) when no system needs them.
+// 800 triangles (no second passes): ten steps 5.02 -> 4.88 ms; 6,400 (a shock tube, where
+// they are common): 5.53 -> 5.96 ms.
+constexpr int64_t kSolo64 = 2000;
 
 gks_status precond64(gks_mesh *m, const double *src, double *dst, cudaStream_t s)
 {
@@ -1351,17 +1353,15 @@ gks_status precond64(gks_mesh *m, const double *src, double *dst, cudaStream_t s
     const int ns = m->cfg.ilu_sweeps, nsb = m->cfg.ilu_sweeps_bwd < 0 ? ns : m->cfg.ilu_sweeps_bwd;
     // forward sweeps of the rows 0 and 1: z^ns is the start of the backward sweeps
     const int nf = nsb > 0 ? ns : ns - 1;
-    const bool fuse = nf > 0 && m->cfg.ilu_fuse_first && T <= kFuse64;
     double *z = ns + nsb > 0 ? k.t3 : dst;
     double *t2a = k.t2, *t2b = k.t2 + 2 * T, *da = dst, *db = dst + 2 * T;
     // z^q (0 < q <= nf), z^{ns-1} in t2a; z^ns in da (t2b where the last launch reads it as x^0)
     auto zq = [&](int q) { return q == 0 ? z : (q == ns ? (nsb == 1 ? t2b : da) : ((ns - 1 - q) % 2 == 0 ? t2a : da)); };
     // x^q (q < nsb), x^0 = z^ns, x^{nsb-1} in t2b
     auto xq = [&](int q) { return q == 0 ? zq(ns) : ((nsb - 1 - q) % 2 == 0 ? t2b : db); };
-    if (fuse) k64_pivot<true><<<g, kW64, 0, s>>>(T, d.nb, d.P, d.w64, d.blk_case, run, src, z, zq(1));
-    else k64_pivot<false><<<g, kW64, 0, s>>>(T, d.nb, d.P, d.w64, d.blk_case, run, src, z, nullptr);
+    k64_pivot<<<g, kW64, 0, s>>>(T, d.P, d.blk_case, run, src, z);
     note_launch();
-    for (int q = fuse ? 1 : 0; q < nf; ++q) {
+    for (int q = 0; q < nf; ++q) {
         k64_sweep<false><<<g, kW64, 0, s>>>(T, d.nb, d.w64, d.blk_case, run, z, zq(q), zq(q + 1));
         note_launch();
     }
@@ -2043,7 +2043,9 @@ gks_status cls_solve_t(gks_mesh *m, TB *V, cudaStream_t s, int32_t *iters, doubl
             launch_orth_update<TB>(d, nb, q, V, vj1, j, k.hco, ps, k.ctl, ns, k.part, mixed ? 1 : 0);
             note_launch();
         }
-        if (!mixed) {
+        // small meshes: the second pass inside the last kernel
+        const bool solo = C64 && T <= kSolo64;
+        if (!mixed && !solo) {
             // the second pass (the systems flagged in twice)
             if (!C64 && (st = dots<TB>(m, V, vj1, j, k.part, q)) != GKS_OK) return st;
             k_reduce<<<dim3(j + 1, ns), kReduceThreads, 0, q>>>(k.part, rs * (int64_t)nb, d.case_blk, rs, k.y, mm, k.vn,
@@ -2062,7 +2064,10 @@ gks_status cls_solve_t(gks_mesh *m, TB *V, cudaStream_t s, int32_t *iters, doubl
         Cond ce = cd;
         if (C64) ce.slot = -1;
         k_arnoldi_end<<<ns, kReduceThreads, 0, q>>>(kry, k.part, rs * (int64_t)nb, d.case_blk, rs, j, k.hcol, ps,
-                                                        mixed ? nullptr : k.y, mm, twice, C64 ? 1.0 : 0.0, ce);
+                                                        mixed ? nullptr : k.y, mm, twice, C64 ? 1.0 : 0.0,
+                                                        Solo{reinterpret_cast<const double *>(V),
+                                                             solo ? reinterpret_cast<double *>(vj1) : nullptr, T},
+                                                        ce);
         note_launch();
         prof_stop(m, slot, q);
         GKS_CUDA(cudaGetLastError());

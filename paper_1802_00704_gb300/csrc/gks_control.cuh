@@ -53,12 +53,9 @@ __device__ __forceinline__ double strided_sum(int t, int b0, int b1, F &&at)
     return acc;
 }
 
-// The block's sum of column q of the partial sums for variable v, rows b0..b1:
-// every lane of the first warp gets it.  sh: one value per warp.
-__device__ __forceinline__ double block_sum(const double *part, int q, int v, int64_t R, int b0, int b1, double *sh)
+// The sum of acc over the block, to every lane of the first warp.  sh: one value per warp.
+__device__ __forceinline__ double block_total(double acc, double *sh)
 {
-    const double *p = part + ((int64_t)q * 4 + v) * R;
-    double acc = strided_sum(threadIdx.x, b0, b1, [&](int b) { return p[b]; });
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
     if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
@@ -70,6 +67,14 @@ __device__ __forceinline__ double block_sum(const double *part, int q, int v, in
         for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     }
     return s;
+}
+
+// The block's sum of column q of the partial sums for variable v, rows b0..b1:
+// every lane of the first warp gets it.  sh: one value per warp.
+__device__ __forceinline__ double block_sum(const double *part, int q, int v, int64_t R, int b0, int b1, double *sh)
+{
+    const double *p = part + ((int64_t)q * 4 + v) * R;
+    return block_total(strided_sum(threadIdx.x, b0, b1, [&](int b) { return p[b]; }), sh);
 }
 
 // out[s][q] = sum over the rows of case(s) of column q, q < nq, and with vn given
@@ -302,14 +307,54 @@ __global__ void __launch_bounds__(32 * kSolveWarps) k_cycle_solve(Krylov k)
     if (sy < k.ns) cycle_solve(k, sy);
 }
 
+// The second Gram-Schmidt pass of a system by one block: h2 = the products' sums,
+// w -= sum_k h2_k / vn_k^2 V_k over the case's cells; the first warp gets |w|^2.
+struct Solo {
+    const double *V;
+    double *w;              // NULL: the pass has launches of its own
+    int64_t T;
+};
+
+__device__ __forceinline__ double solo_pass(const Krylov &k, const Solo &o, int sy, int j, const double *part, int64_t R,
+                                            int b0, int b1, int c0, int c1, double *h2, double *hk, double *sh)
+{
+    for (int q = 0; q <= j; ++q) {
+        const double s = block_sum(part, q, sy & 3, R, b0, b1, sh);
+        if (threadIdx.x == 0) {
+            const double n = k.vn[sy * (k.m + 1) + q];
+            h2[q] = s;
+            hk[q] = n > 0.0 ? s / (n * n) : 0.0;
+        }
+        __syncthreads();
+    }
+    const int64_t vo = (int64_t)(sy & 3) * 5 * o.T, vs = 20 * o.T;
+    double nr = 0.0;
+    for (int64_t i = c0 + threadIdx.x; i < min((int64_t)c1, o.T); i += kReduceThreads) {
+        double u[5];
+#pragma unroll
+        for (int l = 0; l < 5; ++l) u[l] = o.w[vo + l * o.T + i];
+        for (int q = 0; q <= j; ++q)
+#pragma unroll
+            for (int l = 0; l < 5; ++l) u[l] = fma(-hk[q], o.V[q * vs + vo + l * o.T + i], u[l]);
+#pragma unroll
+        for (int l = 0; l < 5; ++l) {
+            o.w[vo + l * o.T + i] = u[l];
+            nr = fma(u[l], u[l], nr);
+        }
+    }
+    return block_total(nr, sh);
+}
+
 // End of Arnoldi index j, one block per system: |V_{j+1}| of a running system
 // from the summed partials and its Givens step (twice given: only of the systems
 // flagged there, which ran the second Gram-Schmidt pass, the others are done; no
-// such system: nothing to do); then the condition "any system
+// such system: nothing to do); with solo.w the block also does that pass for its
+// system, from the products' partial sums on (small meshes: one launch that
+// returns as a rule instead of three); then the condition "any system
 // still runs" and, for a single mesh, the solve of the cycle once none does.
 __global__ void __cluster_dims__(4, 1, 1) __launch_bounds__(kReduceThreads)
     k_arnoldi_end(Krylov k, const double *part, int64_t R, const int32_t *__restrict__ seg, int rs, int j,
-                  const double *hc, int hstride, const double *h2, int h2stride, const int32_t *twice, double shift,
+                  const double *hc, int hstride, double *h2, int h2stride, const int32_t *twice, double shift, Solo solo,
                   Cond cd)
 {
     __shared__ double sh[kReduceThreads / 32];
@@ -321,7 +366,11 @@ __global__ void __cluster_dims__(4, 1, 1) __launch_bounds__(kReduceThreads)
         if (__syncthreads_or(a) == 0) return;
     }
     if (k.ctl[kCtlRunning * k.ns + sy] != 0 && (!twice || twice[sy])) {
-        const double acc = block_sum(part, 0, sy & 3, R, rs * seg[c], rs * seg[c + 1], sh);
+        const int b0 = rs * seg[c], b1 = rs * seg[c + 1];
+        const double acc = solo.w ? solo_pass(k, solo, sy, j, part, R, b0, b1, kBlock * seg[c], kBlock * seg[c + 1],
+                                              h2 + sy * h2stride, shg[0], sh)
+                                  : block_sum(part, 0, sy & 3, R, b0, b1, sh);
+        __syncthreads();
         if (threadIdx.x < 32) givens_step(k, sy, j, hc, hstride, h2, h2stride, shift, sqrt(acc), false, shg);
     }
     bool last;

@@ -51,3 +51,22 @@ def test_mixed_reconstruction_matches_oracle(n, inner_rtol, gmres_m):
     coef, info = gm.cls_reconstruct(dev(c.w0))
     assert max(info["relres"]) <= 1e-12
     assert np.max(np.abs(host(coef) - ref)) <= 1e-9 * np.max(np.abs(ref))
+
+
+def test_second_pass_on_either_side_of_its_size_rule():
+    """The 3 x 3 mesh needs the second pass (above); alone it runs inside the last
+    kernel of the index, in a batch with 16,200 triangles in launches of its own.
+    Both give the same step (1e-13, as the batch tests: sums over other blocks)."""
+    from paper_1802_00704_gb300 import build, gks
+    build.build()
+    cases = [I.advection_case(3), I.advection_case(90), I.advection_case(4)]
+    t_end = np.array([0.01, 0.002, 0.01])
+    w = dev(np.concatenate([c.w0 for c in cases], axis=1))
+    gks.GksMesh.batch([c.mesh for c in cases]).batch_run(w, t_final=t_end, max_steps=2)
+    got, o = host(w), 0
+    for q, c in enumerate(cases):
+        ws = dev(c.w0)
+        gks.GksMesh(c.mesh).run(ws, t_final=float(t_end[q]), max_steps=2)
+        T = c.w0.shape[1]
+        assert np.max(np.abs(got[:, o:o + T] - host(ws))) <= 1e-13 * np.max(np.abs(host(ws)))
+        o += T
