@@ -13,11 +13,12 @@
 // a case a cluster that its hardware barrier joins; the cluster (of a batch the
 // last one to finish) then sets the graph's condition: one launch for the norm, the Givens
 // step, the condition and a single mesh's end of the cycle, one for the residual's norm, the
-// masks, g and the condition.  In the mixed solve the first of the two (8.2 us at
-// 41,000 triangles) is a block of the update's launch (control_end): ten
-// steps at 41,000 triangles 4.89 -> 4.55 ms, a batch of 64 19.1 -> 18.5 ms.  One block with a case's four systems was slower
-// (10.0 us for the first of the two at 41,000 triangles: four FP64 chains on one
-// SM, and 25 us for the sums at 1M).
+// masks, g and the condition.  With the per-cell equations the first of the two (8.2 us
+// at 41,000 triangles) is a block of the update's launch (control_end): ten steps at
+// 41,000 triangles, mixed, 4.89 -> 4.55 ms, at 800, FP64, 5.44 -> 5.14 ms, a batch of 64
+// 19.1 -> 18.5 ms.  One block with a case's four systems was slower (10.0 us for the
+// first of the two at 41,000 triangles: four FP64 chains on one SM, and 25 us for the
+// sums at 1M).
 #pragma once
 
 #include <cuda_runtime.h>

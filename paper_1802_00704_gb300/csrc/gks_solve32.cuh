@@ -207,8 +207,8 @@ __device__ __forceinline__ bool case_runs(const int32_t *__restrict__ blk_case, 
 
 // Forward relation z_i = P_i (r_i + sum_{k<i} O_ik zin_k); NB 0: no neighbours
 // (z = P r); 1: zin as given; 2: zin_k = P_k r_k formed here (the first sweep).
-// FULL: all five rows of z, else the rows 0 and 1 that the next sweep reads.  rc (may be NULL): also store float(r_i) for the later sweeps of a
-// wider source.
+// FULL: all five rows of z, else the rows 0 and 1 that the next sweep reads.  rc
+// (may be NULL): also store float(r_i) for the later sweeps of a wider source.
 template <int NB, bool FULL, typename TR, typename TP>
 __global__ void __launch_bounds__(kW32, 5) k32_fwd(int64_t T, const int32_t *__restrict__ nb,
                                                    const TP *__restrict__ pk, const int32_t *__restrict__ blk_case,

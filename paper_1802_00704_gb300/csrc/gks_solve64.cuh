@@ -10,7 +10,7 @@
 // warps with a quarter of the instructions each, no block-wide barrier, and the
 // warps of a variable whose system has stopped return at once.
 //
-// Three more things keep the instruction count down:
+// What else keeps the instruction count down:
 //  - the sweeps work on the products W = P O of the pivot inverse and the
 //    off-diagonal blocks (set-up; 5 x 2, a block reads the gradient rows 0 and 1 of a
 //    neighbour alone): z = P r once, then rows 0 and 1 of z + sum W z per sweep (12
