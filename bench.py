@@ -379,7 +379,9 @@ def class_bytes(cls: str, prof: dict, T: int, F: int, steps: int, sweeps: int, e
     or 2 with FP16 copies).  With the block-diagonal pass folded into the first
     forward sweep the neighbours' z^0 comes from their own factors and right-hand
     sides, already counted as those cells' reads; with backward sweep pairs
-    likewise the neighbours' first-sweep values."""
+    likewise the neighbours' first-sweep values.  The FP64 solve of the per-cell
+    equations moves less (products in the operator kernel, a second Gram-Schmidt
+    pass only where needed, sweeps on P O): its counts are an upper bound."""
     sM = 4 if mixed else 8
     sZ = 4 if mixed else 8
     sB = 4 if basis32 else 8
