@@ -1396,15 +1396,17 @@ inline unsigned rows64(const gks_mesh *m) { return (unsigned)(m->wk.nblk * (kRow
 // dynamic shared memory of the product kernels at Arnoldi index j
 inline size_t acc64(int j, int stride) { return sizeof(double) * 4 * (j + 1) * stride; }
 
-// Beyond 48 KiB (restart lengths above 45) the kernels have to ask for it.
-gks_status solve64_shared_limit(int mm)
+// Beyond 48 KiB (restart lengths above 45) the kernels have to ask for it.  The limit
+// is the process's, not the handle's: always that of the longest restart, so that a
+// handle never lowers it between another's call and launch.
+gks_status solve64_shared_limit()
 {
     auto set = [&](auto C) -> gks_status {
         constexpr int c = decltype(C)::value;
         GKS_CUDA(cudaFuncSetAttribute(k64_apply_dots<c>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)acc64(mm, kAccStride)));
+                                      (int)acc64(kMaxRestart, kAccStride)));
         GKS_CUDA(cudaFuncSetAttribute(k64_update<c>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)acc64(mm - 1, kAccStride + 1)));
+                                      (int)acc64(kMaxRestart - 1, kAccStride + 1)));
         return GKS_OK;
     };
     gks_status st = set(std::integral_constant<int, 1>{});
@@ -1895,7 +1897,7 @@ gks_status cls_solve_t(gks_mesh *m, TB *V, cudaStream_t s, int32_t *iters, doubl
     // (gks_solve64.cuh), C64 cells per thread, rs partial-sum rows per cell block
     const int C64 = k.c64;
     if (C64 && mm > 45) {
-        if ((st = solve64_shared_limit(mm)) != GKS_OK) return st;
+        if ((st = solve64_shared_limit()) != GKS_OK) return st;
     }
 
     // FP32 basis: first basis vector scaled by a power of two; exponents per
