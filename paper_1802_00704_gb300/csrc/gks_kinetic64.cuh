@@ -65,21 +65,25 @@ struct State {
     R a, b;                // U / sqrt(h), V / sqrt(h)
 };
 
-// Primitive variables of a state (rho, rho U, rho V, E); false unless rho > 0 and p > 0.
-template <typename R>
+// Primitive variables of a state (rho, rho U, rho V, E); false unless rho > 0 and p > 0,
+// and for a SIDE of the face unless four times its internal energy is in range (the
+// sums over both sides would overflow; tested on the exponent, off the FP64 pipe).
+template <bool SIDE = false, typename R>
 __device__ __forceinline__ bool prim(const R *w, R gamma, State<R> &s)
 {
     s.rho = w[0];
     s.ir = R(1) / w[0];
     s.U = w[1] * s.ir;
     s.V = w[2] * s.ir;
-    s.p = (gamma - R(1)) * (w[3] - R(0.5) * (w[1] * s.U + w[2] * s.V));
+    const R eint = w[3] - R(0.5) * (w[1] * s.U + w[2] * s.V);
+    s.p = (gamma - R(1)) * eint;
     s.h = s.p * s.ir;
     s.isg = rsqrt(s.h);
     s.sg = s.h * s.isg;
     s.a = s.U * s.isg;
     s.b = s.V * s.isg;
-    return s.rho > R(0) && s.p > R(0);
+    const bool fits = !SIDE || (__double2hiint(eint) & 0x7ff00000) < 0x7fd00000;     // |eint| < 2^1022
+    return s.rho > R(0) && s.p > R(0) && fits;
 }
 
 // Moments <x^k>, k < 10, over u > 0 (sign = +1: x > -a) or u < 0 (sign = -1),
@@ -549,7 +553,7 @@ template <typename R>
 __device__ __forceinline__ bool interface_state(const R *wl, const R *wr, R dt, R gamma, R mu, const Gas<R> &c,
                                                 int tau2_exact, Iface<R> &I)
 {
-    if (!(prim(wl, gamma, I.L) & prim(wr, gamma, I.Rs))) return false;
+    if (!(prim<true>(wl, gamma, I.L) & prim<true>(wr, gamma, I.Rs))) return false;
 #pragma unroll
     for (int q = 0; q < 4; ++q) I.w0[q] = R(0);
 #pragma unroll
