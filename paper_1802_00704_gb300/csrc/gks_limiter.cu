@@ -197,8 +197,9 @@ __device__ __forceinline__ void limit_cells(const DeviceMesh &d, const double *_
         double X = 0.0, rh = 0.0, dx = 0.0, dy = 0.0;
         if (v < J) {
             const int64_t j = v == 0 ? nbj[0] : (v == 1 ? nbj[1] : nbj[2]);
-            const double rho = w[j], mx = w[T + j], my = w[2 * T + j];
-            X = (gamma - 1.0) * (w[3 * T + j] - 0.5 * (mx * mx + my * my) / rho);
+            // in velocities: an infinite density gives no pressure (NaN), as an infinite energy does
+            const double rho = w[j], ir = 1.0 / rho, u = w[T + j] * ir, vv = w[2 * T + j] * ir;
+            X = (gamma - 1.0) * (w[3 * T + j] - 0.5 * rho * (u * u + vv * vv));
             rh = 1.0 / d.h[j];
             dx = -d.ox[v * T + i] * hi * rh;
             dy = -d.oy[v * T + i] * hi * rh;
