@@ -46,25 +46,51 @@
 namespace gks {
 namespace {
 
-// Right (columns) and left (rows) eigenvectors, row-major 4x4, of the Jacobian
-// of the Euler flux along the unit direction (nx, ny) at the conservative
-// state W (eigenvalues q_n - c, q_n, q_n, q_n + c).
-__device__ __forceinline__ void char_basis(const double *W, double gamma, double nx, double ny, double *R, double *L)
+// The Euler flux Jacobian's eigenvectors at a conservative state: what does not depend
+// on the direction, once per cell.
+struct EulerState {
+    double u, v, ke, c, ic, H, b1, b2;
+};
+
+__device__ __forceinline__ EulerState euler_state(const double *W, double gamma)
 {
-    const double rho = W[0], u = W[1] / rho, v = W[2] / rho;
-    const double ke = 0.5 * (u * u + v * v);
-    const double p = (gamma - 1.0) * (W[3] - rho * ke);
-    const double c = sqrt(gamma * p / rho), H = (W[3] + p) / rho;
-    const double qn = u * nx + v * ny, qt = -u * ny + v * nx;
-    const double b1 = (gamma - 1.0) / (c * c), b2 = b1 * ke, ic = 1.0 / c;
-    R[0] = 1.0;             R[1] = 1.0; R[2] = 0.0; R[3] = 1.0;
-    R[4] = u - c * nx;      R[5] = u;   R[6] = -ny; R[7] = u + c * nx;
-    R[8] = v - c * ny;      R[9] = v;   R[10] = nx; R[11] = v + c * ny;
-    R[12] = H - qn * c;     R[13] = ke; R[14] = qt; R[15] = H + qn * c;
-    L[0] = 0.5 * (b2 + qn * ic);  L[1] = -0.5 * (b1 * u + nx * ic); L[2] = -0.5 * (b1 * v + ny * ic); L[3] = 0.5 * b1;
-    L[4] = 1.0 - b2;              L[5] = b1 * u;                    L[6] = b1 * v;                    L[7] = -b1;
-    L[8] = -qt;                   L[9] = -ny;                       L[10] = nx;                       L[11] = 0.0;
-    L[12] = 0.5 * (b2 - qn * ic); L[13] = -0.5 * (b1 * u - nx * ic); L[14] = -0.5 * (b1 * v - ny * ic); L[15] = 0.5 * b1;
+    EulerState e;
+    e.u = W[1] / W[0];
+    e.v = W[2] / W[0];
+    e.ke = 0.5 * (e.u * e.u + e.v * e.v);
+    const double p = (gamma - 1.0) * (W[3] - W[0] * e.ke);
+    e.c = sqrt(gamma * p / W[0]);
+    e.H = (W[3] + p) / W[0];
+    e.b1 = (gamma - 1.0) / (e.c * e.c);
+    e.b2 = e.b1 * e.ke;
+    e.ic = 1.0 / e.c;
+    return e;
+}
+
+// Row q of the left eigenvectors (eigenvalues q_n - c, q_n, q_n, q_n + c), and row q of
+// the right ones (columns), of the Jacobian along the unit direction (nx, ny).
+__device__ __forceinline__ void char_rows(const EulerState &e, int q, double nx, double ny, double *R, double *L)
+{
+    const double qn = e.u * nx + e.v * ny, qt = -e.u * ny + e.v * nx;
+    const double s = q == 0 ? e.ic : -e.ic;
+    const double bu = e.b1 * e.u, bv = e.b1 * e.v;
+    if (q == 0 || q == 3) {
+        L[0] = 0.5 * (e.b2 + qn * s);
+        L[1] = -0.5 * (bu + nx * s);
+        L[2] = -0.5 * (bv + ny * s);
+        L[3] = 0.5 * e.b1;
+    } else {
+        L[0] = q == 1 ? 1.0 - e.b2 : -qt;
+        L[1] = q == 1 ? bu : -ny;
+        L[2] = q == 1 ? bv : nx;
+        L[3] = q == 1 ? -e.b1 : 0.0;
+    }
+    const double mid = q == 0 ? 1.0 : (q == 1 ? e.u : (q == 2 ? e.v : e.H));
+    const double dif = e.c * (q == 0 ? 0.0 : (q == 1 ? nx : (q == 2 ? ny : qn)));
+    R[0] = mid - dif;
+    R[1] = q == 3 ? e.ke : mid;
+    R[2] = q == 0 ? 0.0 : (q == 1 ? -ny : (q == 2 ? nx : qt));
+    R[3] = mid + dif;
 }
 
 // u_0 tan(sum_j om_j atan(u_j / u_0)) over the candidates (weight 0: none); the own
@@ -256,6 +282,11 @@ __device__ __forceinline__ void limit_cells(const DeviceMesh &d, const double *_
         // ---- a derivative row at a time: candidates in physical units, the cell's own
         // polynomial and the neighbours' (at r_i)
         const double rhi = 1.0 / hi;
+        EulerState es = {};
+        if (charm) {
+            const double Wi[4] = {w[i], w[T + i], w[2 * T + i], w[3 * T + i]};
+            es = euler_state(Wi, gamma);
+        }
 #pragma unroll 1
         for (int l0 = 0; l0 < 5; l0 += G / 4) {
             const int l = min(l0 + (lane >> 2), 4);        // spare lanes repeat the last row
@@ -281,16 +312,10 @@ __device__ __forceinline__ void limit_cells(const DeviceMesh &d, const double *_
             if (charm) {
                 // characteristic variables along x (d/dx, d2/dx2), y (d/dy, d2/dy2), the
                 // diagonal (d2/dxdy); lane v of a row takes characteristic v
-                const double Wi[4] = {w[i], w[T + i], w[2 * T + i], w[3 * T + i]};
                 const double nx = l == 1 || l == 4 ? 0.0 : (l == 3 ? 0.70710678118654752 : 1.0);
                 const double ny = l == 0 || l == 2 ? 0.0 : (l == 3 ? 0.70710678118654752 : 1.0);
-                double Rm[16], Lm[16], Lr[4], Rr[4], ch[4];
-                char_basis(Wi, gamma, nx, ny, Rm, Lm);
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    Lr[q] = v == 0 ? Lm[q] : (v == 1 ? Lm[4 + q] : (v == 2 ? Lm[8 + q] : Lm[12 + q]));
-                    Rr[q] = v == 0 ? Rm[q] : (v == 1 ? Rm[4 + q] : (v == 2 ? Rm[8 + q] : Rm[12 + q]));
-                }
+                double Lr[4], Rr[4], ch[4];
+                char_rows(es, v, nx, ny, Rr, Lr);
 #pragma unroll
                 for (int q = 0; q < 4; ++q)
                     ch[q] = Lr[0] * __shfl_sync(kAll, cand[q], 0, 4) + Lr[1] * __shfl_sync(kAll, cand[q], 1, 4) +
@@ -331,8 +356,11 @@ __device__ __forceinline__ void limit_cells(const DeviceMesh &d, const double *_
 
 // A warp takes one listed cell or eight.  A cell of its own ends in about 20 us, eight
 // in about 45 (five rows per lane), so eight pay once the sub-partitions have more than
-// two cells each.
-__global__ void __launch_bounds__(32 * kLimitWarps) k_limit(const DeviceMesh d, const double *__restrict__ w,
+// two cells each.  Long lists need the grid's four blocks per SM resident: 128 registers
+// with 28 bytes of spills, where 151 left a quarter of the grid for a second round (a call with
+// 480,000 flagged cells, conservative / characteristic: 6.4 / 8.0 -> 4.5 / 5.6 ms, 5.8 / 6.3
+// with a thread per cell; 240,000: 2.7 / 3.4 -> 2.3 / 2.8, 3.1 / 3.4; 24,000 or fewer the same).
+__global__ void __launch_bounds__(32 * kLimitWarps, 4) k_limit(const DeviceMesh d, const double *__restrict__ w,
                                                             const double *__restrict__ x, double *__restrict__ xl,
                                                             int32_t *__restrict__ flag,
                                                             const int32_t *__restrict__ list,
