@@ -327,6 +327,17 @@ __device__ __noinline__ void resid64_cell(const DeviceMesh &d, const double *__r
 
 constexpr int kResidRows = NV;          // residual blocks (partial-sum rows) per cell block
 
+// (h, l) += (x, y), sums of FP32 numbers to about 48 bits (TwoSum): on GB300 an
+// FP64 addition costs a warp 33 ns, this seven FP32 operations
+__device__ __forceinline__ void df_add(float x, float y, float &h, float &l)
+{
+    const float t = __fadd_rn(h, x);
+    const float z = __fsub_rn(t, h);
+    const float e = __fadd_rn(__fsub_rn(h, __fsub_rn(t, z)), __fsub_rn(x, z));
+    l = __fadd_rn(l, __fadd_rn(e, y));
+    h = t;
+}
+
 // (h, l) of every lane summed over the warp (lane 0 gets the pair)
 __device__ __forceinline__ void df_warp_sum(float &h, float &l)
 {
@@ -357,7 +368,7 @@ __device__ __forceinline__ void load4(const float4 *__restrict__ p, int q, int64
 // of 256 cells the operator came from L2 four times; in different warps of a
 // block it was no faster.)  A value outside the split range sends
 // the thread to the FP64 operator.  Each thread's five squares are summed in
-// FP32 (the scaled vector is near unit size), the threads' sums to 48 bits.
+// FP32 (the scaled vector is near unit size), the threads' sums in FP64.
 // act (NULL on a solve's first residual): a case without an active system keeps
 // its V_0 and norms.  G: global normal equations, the
 // transpose form from the reverse-slot pairs SR2 ([6][T][4]: 9 values and their
@@ -372,7 +383,7 @@ __global__ void __launch_bounds__(kBlock, 4) k_resid_df(const __grid_constant__ 
                                                         const int32_t *__restrict__ act,
                                                         const float4 *__restrict__ SR2 = nullptr)
 {
-    __shared__ float2 sh[kBlock / 32][NV];
+    __shared__ double sh[kBlock / 32][NV];
     const int64_t T = d.T;
     const int cs = d.blk_case[blockIdx.x / kResidRows];
     if (act) {
@@ -381,7 +392,7 @@ __global__ void __launch_bounds__(kBlock, 4) k_resid_df(const __grid_constant__ 
     }
     const int v = threadIdx.x & 3;
     const int64_t i = blockIdx.x * (int64_t)(kBlock / NV) + (threadIdx.x >> 2);
-    float nh = 0.0f, nl = 0.0f;
+    double nr = 0.0;
     if (i < T) {
         const int e = sexp[4 * cs + v];
         int64_t jn[3];
@@ -467,17 +478,9 @@ __global__ void __launch_bounds__(kBlock, 4) k_resid_df(const __grid_constant__ 
             y[(l * T + i) * NV + v] = out[l];
             sq = __fmaf_rn(out[l], out[l], sq);
         }
-        nh = sq;
+        nr = double(sq);
     }
-    // over the warp's eight cells, then the warps
-#pragma unroll
-    for (int o = 16; o >= NV; o >>= 1) df_add(__shfl_down_sync(0xffffffffu, nh, o), __shfl_down_sync(0xffffffffu, nl, o), nh, nl);
-    if ((threadIdx.x & 31) < NV) sh[threadIdx.x >> 5][threadIdx.x & 31] = make_float2(nh, nl);
-    __syncthreads();
-    if (threadIdx.x < NV) {
-        for (int w = 1; w < kBlock / 32; ++w) df_add(sh[w][threadIdx.x].x, sh[w][threadIdx.x].y, nh, nl);
-        part[threadIdx.x * (int64_t)gridDim.x + blockIdx.x] = double(nh) + double(nl);
-    }
+    block_quads(nr, sh, part);
 }
 
 // 2^e f as an FP64 value, formed on the integer pipe (exact; an FP32 subnormal

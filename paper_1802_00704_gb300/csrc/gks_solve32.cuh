@@ -420,19 +420,9 @@ __device__ __forceinline__ void apply32(int64_t T, const int32_t *__restrict__ n
     for (int s = 0; s < 3; ++s) off_acc4(-c[15 + s], c[18 + s], c[21 + s], g[s][0], g[s][1], u);
 }
 
-// (h, l) += (x, y), sums of FP32 numbers to about 48 bits (TwoSum): on GB300 an
-// FP64 addition costs a warp 33 ns, this seven FP32 operations
-__device__ __forceinline__ void df_add(float x, float y, float &h, float &l)
-{
-    const float t = __fadd_rn(h, x);
-    const float z = __fsub_rn(t, h);
-    const float e = __fadd_rn(__fsub_rn(h, __fsub_rn(t, z)), __fsub_rn(x, z));
-    l = __fadd_rn(l, __fadd_rn(e, y));
-    h = t;
-}
-
 // Block sums of K x 4 FP32 values per thread, sv[k][v]: FP32 within a warp (at
-// most 160 products each), added across the warps to 48 bits: part[k0 + k][v][row], k < n.
+// most 160 products each), FP64 across the warps: part[k0 + k][v][row], k < n.  A warp
+// per k adds its four sums, eight lanes each (four FP64 instructions).
 template <int K>
 __device__ __forceinline__ void block_rows32(float (&sv)[K][4], float (*sh)[K][4], double *__restrict__ part, int k0,
                                              int n = K)
@@ -454,12 +444,29 @@ __device__ __forceinline__ void block_rows32(float (&sv)[K][4], float (*sh)[K][4
         if ((lane & 7) == 0) sh[warp][k][lane >> 3] = s;
     }
     __syncthreads();
-    if (threadIdx.x < 4 * min(K, n)) {
-        const int k = threadIdx.x / 4, v = threadIdx.x % 4;
-        float h = 0.0f, l = 0.0f;
+    if (warp < min(K, n)) {
+        const int v = lane >> 3;
+        double s = double(sh[lane & 7][warp][v]);
 #pragma unroll
-        for (int w = 0; w < kBlock / 32; ++w) df_add(sh[w][k][v], 0.0f, h, l);
-        part[((k0 + k) * 4 + v) * (int64_t)gridDim.x + blockIdx.x] = double(h) + double(l);
+        for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if ((lane & 7) == 0) part[((k0 + warp) * 4 + v) * (int64_t)gridDim.x + blockIdx.x] = s;
+    }
+}
+
+// Block sums of one value per thread, the variable of a thread being its index mod 4:
+// FP64 from the thread on, part[variable][row].
+__device__ __forceinline__ void block_quads(double s, double (*sh)[4], double *__restrict__ part)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int o = 16; o >= 4; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane < 4) sh[warp][lane] = s;
+    __syncthreads();
+    if (warp == 0) {
+        s = sh[lane >> 2][lane & 3];
+#pragma unroll
+        for (int o = 16; o >= 4; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane < 4) part[lane * (int64_t)gridDim.x + blockIdx.x] = s;
     }
 }
 
