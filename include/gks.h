@@ -218,10 +218,13 @@ typedef struct gks_config {
                               would limit the agreement with the FP64 path         */
     int32_t flux_shape;    /* launch shape of the double-FP32 flux kernel: 0 (default)
                               128 threads x 4 blocks per SM on small meshes, 256 x 2
-                              on large ones (128 registers), 1 256 x 2, 2 128 x 2
-                              (255 registers).  The same source, compiled once per
-                              shape, so results of two shapes may differ in the last
-                              bits; the autotuner's last stage picks one               */
+                              on large ones (128 registers), 1 256 x 2 (128 x 3, 168
+                              registers, until it was the fastest at no size any
+                              more), 2 128 x 2 (255 registers; the shape of 0 with the
+                              Prandtl correction or kinetic slopes).  The same source,
+                              compiled once per shape, so results of two shapes may
+                              differ in the last bits; the autotuner's last stage
+                              picks one                                                */
     int32_t reserved;      /* must be 0                                                */
 } gks_config;
 

@@ -271,6 +271,16 @@ inline unsigned blocks(int64_t n, int b) { return (unsigned)((n + b - 1) / b); }
 
 }  // namespace
 
+// The launch that a flux_shape stands for: 0 128 threads x 4 blocks per SM, 1 256 x 2, 2 128 x 2.
+// Shape 0 takes 256-thread blocks unless they would leave a last wave nearly empty (fewer
+// than four waves of the SMs' 512 points each, 104,000 triangles on 152 SMs).  us, 128 x 4 / 256 x 2 / 128
+// x 2: 41,000 triangles 69.7 / 74.4 / 85.4, 90,000 149 / 148 / 156, 131,000 214 / 203 / 236, 1M 1,394 / 1,240
+// / 1,545; at 1,600 and 10,000, one wave, 128 x 2 is the best of them (27.2 against 31.1, 29.3 against 31.5).
+int flux_df_launch(const gks_mesh *m, int shape)
+{
+    return shape == 0 && 2 * m->d.F >= 4 * 512 * (int64_t)m->wk.sm_count ? 1 : shape;
+}
+
 gks_status launch_flux_df(gks_mesh *m, const double *w, const double *x, double dt_const, const double *dt_dev,
                           double *flux, cudaStream_t s)
 {
@@ -292,9 +302,8 @@ gks_status launch_flux_df(gks_mesh *m, const double *w, const double *x, double 
     };
     using Y = std::true_type;
     using N = std::false_type;
-    // the launch shape: 256-thread blocks (flux_shape 1) unless they would leave a
-    // last wave nearly empty (fewer than four waves of the SMs' 512 points each)
-    const bool wide = c.flux_shape == 1 || npts >= 4 * 512 * (int64_t)m->wk.sm_count;
+    // (shape 2 is compiled for the flux without the Prandtl correction and with mean slopes)
+    const bool wide = flux_df_launch(m, heat || kin ? c.flux_shape % 2 : c.flux_shape) == 1;
     auto shaped = [&](auto H, auto Kw) {
         if (wide) go(H, Kw, std::integral_constant<int, 256>{}, std::integral_constant<int, 2>{});
         else go(H, Kw, std::integral_constant<int, kFluxBlock>{}, std::integral_constant<int, 4>{});

@@ -305,6 +305,8 @@ gks_status launch_update(gks_mesh *m, double *w, const double *flux, cudaStream_
 // the autotuner may choose from for the flux without the Prandtl correction
 // and with mean interface slopes
 constexpr int kFluxDfVariants = 3;
+// ... and the launch that a shape stands for on this handle (shape 0 goes by the mesh's size)
+int flux_df_launch(const gks_mesh *m, int shape);
 gks_status launch_flux_df(gks_mesh *m, const double *w, const double *x, double dt_const, const double *dt_dev,
                           double *flux, cudaStream_t s);
 gks_status launch_point_flux_df(int64_t n, const double *wl, const double *wr, double dt, const gks_config &cfg,

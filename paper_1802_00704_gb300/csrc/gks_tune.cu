@@ -11,7 +11,7 @@
 // combination and keeps the fastest; then it times shorter GMRES restarts with
 // those knobs (a shorter restart orthogonalises against fewer vectors per
 // iteration but may need more iterations), and the launch shapes of the
-// double-FP32 flux kernel (its register budget against the warps per SM).
+// double-FP32 flux kernel (threads per block and register budget).
 #include <cfloat>
 #include <vector>
 
@@ -106,7 +106,7 @@ extern "C" gks_status gks_autotune(gks_mesh *m, const double *w, int32_t trial_s
     std::vector<Candidate> cand;
     // (forward, backward) sweeps: the same number each way (bwd -1), one
     // backward sweep after two or three forward ones, and one forward sweep
-    // before a backward pair (one launch, k_ilu_bwd2)
+    // before a backward pair (one launch, k32_bwd2)
     const int32_t pairs[6][2] = {{1, -1}, {2, -1}, {3, -1}, {2, 1}, {3, 1}, {1, 2}};
     for (const auto &pr : pairs) {
         const int32_t sw = pr[0], bwd = pr[1];
@@ -153,15 +153,18 @@ extern "C" gks_status gks_autotune(gks_mesh *m, const double *w, int32_t trial_s
         c.m = mr;
         try_one(c);
     }
-    // third stage: the launch shape (register budget) of the double-FP32 flux
-    // kernel, with the best knobs and restart length
+    // third stage: the launch shape of the double-FP32 flux kernel, with the best
+    // knobs and restart length; each launch once (on large meshes shape 0 is shape 1's)
     const int32_t v0 = m->cfg.flux_shape;
     int32_t vpick = v0;
     const bool df_flux = mixed && m->cfg.flux_lead == 1 && m->cfg.prandtl == 1.0 && m->cfg.slope0_mode == 0;
     if (df_flux && st == GKS_OK) {
         apply(m, pick);
+        unsigned timed = 1u << flux_df_launch(m, v0);
         for (int32_t v = 0; v < kFluxDfVariants && st == GKS_OK; ++v) {
-            if (v == v0) continue;
+            const unsigned launch = 1u << flux_df_launch(m, v);
+            if (timed & launch) continue;
+            timed |= launch;
             m->cfg.flux_shape = v;
             double ms = DBL_MAX;
             st = time_candidate(m, w, trial_steps, s, e0, e1, &ms);
