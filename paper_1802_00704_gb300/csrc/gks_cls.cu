@@ -1338,14 +1338,6 @@ gks_status precond_t(gks_mesh *m, const TP *Pg, const TP *alg, const TP *exg, co
 // z = P src is in t3 (rows 0 and 1 of it are z^0).  The rows 0 and 1 of the other
 // intermediate results go to four pairs of rows, two in t2 and two in dst; what the
 // last launch reads of neighbours, z^{ns-1} and x^{nsb-1}, is in t3 or t2.
-//
-// Up to this many triangles the second Gram-Schmidt pass of the systems that need it is a
-// block per system inside k_arnoldi_end; above, two launches over the whole GPU, which return
-// at once (about 1.3 us each) when no system needs them.
-// 800 triangles (no second passes): ten steps 5.02 -> 4.88 ms; 6,400 (a shock tube, where
-// they are common): 5.53 -> 5.96 ms.
-constexpr int64_t kSolo64 = 2000;
-
 gks_status precond64(gks_mesh *m, const double *src, double *dst, cudaStream_t s)
 {
     const DeviceMesh &d = m->d;
@@ -1380,6 +1372,16 @@ gks_status precond64(gks_mesh *m, const double *src, double *dst, cudaStream_t s
     GKS_CUDA(cudaGetLastError());
     return GKS_OK;
 }
+
+// Up to this many triangles the second Gram-Schmidt pass of the FP64 solve is a block per
+// system inside k_arnoldi_end; above, three launches over the whole GPU, which return at once
+// (about 1.3 us each) when no system needs them.  Timed both ways on 148 systems (cells stretched
+// up to 300 : 1, no to four sweeps, restarts of 8 and 30; passes in none to two thirds of the
+// indices): up to 968 triangles the block is the faster one for every solve that converged
+// (0.5 to 8 %; exact triangular solves, bound by their waits, within 4 % either way), at 1,800-1,922 it
+// is 2 to 7 % faster where passes are rare and up to 11 % slower where they are not, at 6,400 (a
+// shock tube) 30 % slower.
+constexpr int64_t kSolo64 = 1000;
 
 // A launch with c cells per thread.
 template <typename F>

@@ -309,7 +309,9 @@ __global__ void __launch_bounds__(32 * kSolveWarps) k_cycle_solve(Krylov k)
 }
 
 // The second Gram-Schmidt pass of a system by one block: h2 = the products' sums,
-// w -= sum_k h2_k / vn_k^2 V_k over the case's cells; the first warp gets |w|^2.
+// w -= sum_k h2_k / vn_k^2 V_k over the case's cells; the first warp gets |w|^2.  A block's
+// latency: with the block on one sum after another and a thread per cell, steps on 50 triangles
+// stretched 50 : 1 (a pass in two indices of three) took 15.7 ms, now 12.0 (launches 13.0).
 struct Solo {
     const double *V;
     double *w;              // NULL: the pass has launches of its own
@@ -319,29 +321,31 @@ struct Solo {
 __device__ __forceinline__ double solo_pass(const Krylov &k, const Solo &o, int sy, int j, const double *part, int64_t R,
                                             int b0, int b1, int c0, int c1, double *h2, double *hk, double *sh)
 {
-    for (int q = 0; q <= j; ++q) {
-        const double s = block_sum(part, q, sy & 3, R, b0, b1, sh);
-        if (threadIdx.x == 0) {
+    // the products' sums: a warp per basis vector
+    const int lane = threadIdx.x & 31;
+    for (int q = threadIdx.x >> 5; q <= j; q += kReduceThreads / 32) {
+        const double *p = part + ((int64_t)q * 4 + (sy & 3)) * R;
+        double s = 0.0;
+        for (int b = b0 + lane; b < b1; b += 32) s += p[b];
+        s = warp_sum(s);
+        if (lane == 0) {
             const double n = k.vn[sy * (k.m + 1) + q];
             h2[q] = s;
             hk[q] = n > 0.0 ? s / (n * n) : 0.0;
         }
-        __syncthreads();
     }
+    __syncthreads();
+    // the update: a thread per cell and unknown
     const int64_t vo = (int64_t)(sy & 3) * 5 * o.T, vs = 20 * o.T;
+    const int n = int(min((int64_t)c1, o.T) - c0);
     double nr = 0.0;
-    for (int64_t i = c0 + threadIdx.x; i < min((int64_t)c1, o.T); i += kReduceThreads) {
-        double u[5];
-#pragma unroll
-        for (int l = 0; l < 5; ++l) u[l] = o.w[vo + l * o.T + i];
-        for (int q = 0; q <= j; ++q)
-#pragma unroll
-            for (int l = 0; l < 5; ++l) u[l] = fma(-hk[q], o.V[q * vs + vo + l * o.T + i], u[l]);
-#pragma unroll
-        for (int l = 0; l < 5; ++l) {
-            o.w[vo + l * o.T + i] = u[l];
-            nr = fma(u[l], u[l], nr);
-        }
+    for (int e = threadIdx.x; e < 5 * n; e += kReduceThreads) {
+        const int l = e / n;
+        const int64_t at = vo + l * o.T + c0 + (e - l * n);
+        double u = o.w[at];
+        for (int q = 0; q <= j; ++q) u = fma(-hk[q], o.V[q * vs + at], u);
+        o.w[at] = u;
+        nr = fma(u, u, nr);
     }
     return block_total(nr, sh);
 }
