@@ -1476,7 +1476,7 @@ gks_status precond(gks_mesh *m, const TR *src, double *dst, cudaStream_t s)
 {
     DeviceMesh &d = m->d;
     if constexpr (std::is_same_v<TR, double>)
-        if (m->wk.c64 && m->cfg.precond == GKS_PC_ILU_SWEEP) return precond64(m, src, dst, s);
+        if (d.w64) return precond64(m, src, dst, s);
     return precond_t<TR, double, double>(m, d.P, d.alpha, d.ex, d.ey, src, dst, m->wk.t2, m->wk.t3, nullptr, s,
                                          {d.alr, d.exr, d.eyr, d.bdg});
 }
@@ -1580,8 +1580,8 @@ template <typename TR>
 gks_status precond32(gks_mesh *m, const TR *src, float *dst, cudaStream_t s)
 {
     DeviceMesh &d = m->d;
-    if (m->cfg.precond == GKS_PC_ILU_SWEEP && d.pk16) return precond32s<TR, __half>(m, d.pk16, src, dst, s);
-    if (m->cfg.precond == GKS_PC_ILU_SWEEP && d.pk32) return precond32s<TR, float>(m, d.pk32, src, dst, s);
+    if (d.pk16) return precond32s<TR, __half>(m, d.pk16, src, dst, s);
+    if (d.pk32) return precond32s<TR, float>(m, d.pk32, src, dst, s);
     if (d.P16)   // FP16 factors (ilu_fp16), FP32 arithmetic
         return precond_t<TR, float, float, __half>(m, d.P16, d.alpha16, d.ex16, d.ey16, src, dst, m->wk.t2_32,
                                                    m->wk.t3_32, m->wk.r32, s, {d.alr16, d.exr16, d.eyr16, d.bdg16});
@@ -2296,8 +2296,10 @@ gks_status launch_pack(gks_mesh *m)
     const unsigned g = nblocks(d.T);
     if (d.off) {
         k64_off<<<g, kBlock>>>(d.T, d.alpha, d.ex, d.ey, d.off);
-        k64_products<<<g, kBlock>>>(d.T, d.P, d.off, d.w64);
         note_launch();
+    }
+    if (d.w64) {
+        k64_products<<<g, kBlock>>>(d.T, d.P, d.off, d.w64);
         note_launch();
     }
     if (d.op32) {

@@ -66,6 +66,19 @@ gks_status dalloc(gks_mesh *m, T **p, size_t n)
     return GKS_OK;
 }
 
+// Give back an array of n values that nothing reads any more (kernels that read it
+// have been launched on the null stream; cudaFree waits for them).
+template <typename T>
+gks_status drop(gks_mesh *m, T **p, size_t n)
+{
+    if (!*p) return GKS_OK;
+    m->allocations.erase(std::find(m->allocations.begin(), m->allocations.end(), (void *)*p));
+    m->device_bytes -= (int64_t)(std::max<size_t>(n, 1) * sizeof(T));
+    GKS_CUDA(cudaFree(*p));
+    *p = nullptr;
+    return GKS_OK;
+}
+
 template <typename T>
 gks_status upload(gks_mesh *m, T **p, const std::vector<T> &h)
 {
@@ -834,6 +847,42 @@ gks_status build_batch(gks_mesh *m, const CaseIn *cases, int32_t n_cases)
     }
 #undef UP
 
+    // ---- the per-cell equations' own layouts, and what they are read instead of
+    if (!ext) {
+        const bool sweep = cfg.precond == GKS_PC_ILU_SWEEP;
+        // the triangular solves that read the off-diagonal blocks as uploaded
+        const bool solves = cfg.precond == GKS_PC_ILU_EXACT || cfg.precond == GKS_PC_ILU_LEVELS;
+        const bool fused = cfg.basis_fp32 && cfg.spmv_dots;      // the operator with the products
+        if (cfg.precision == GKS_FP64) {
+            if ((st = dalloc(m, &d.off, (size_t)9 * T)) != GKS_OK) return st;
+            if (sweep && (st = dalloc(m, &d.w64, (size_t)30 * T)) != GKS_OK) return st;
+        } else {
+            if (fused && (st = dalloc(m, &d.op32, (size_t)24 * T)) != GKS_OK) return st;
+            if (sweep && (st = d.P16 ? dalloc(m, &d.pk16, (size_t)34 * T) : dalloc(m, &d.pk32, (size_t)34 * T)) != GKS_OK)
+                return st;
+        }
+        if ((st = launch_pack(m)) != GKS_OK) return st;
+#define DROP(ptr, n) \
+    if ((st = drop(m, &d.ptr, (size_t)(n) * T)) != GKS_OK) return st
+        if (cfg.precision == GKS_FP64) {
+            if (!solves) {
+                DROP(alpha, 3); DROP(ex, 3); DROP(ey, 3);
+            }
+        } else {
+            DROP(P, 25);
+            if (fused) DROP(D32, 15);
+            if (fused && (!solves || d.P16)) {
+                DROP(alpha32, 3); DROP(ex32, 3); DROP(ey32, 3);
+            }
+            if (sweep || d.P16) DROP(P32, 25);
+            if (sweep) DROP(P16, 25);
+            if (!solves) {
+                DROP(alpha16, 3); DROP(ex16, 3); DROP(ey16, 3);
+            }
+        }
+#undef DROP
+    }
+
     // ---- work buffers
     Work &k = m->wk;
     k.m = cfg.gmres_m;
@@ -858,18 +907,6 @@ gks_status build_batch(gks_mesh *m, const CaseIn *cases, int32_t n_cases)
     }
     int rows = 1;
     if (cfg.precision == GKS_MIXED || !ext) plan_solve(m, &rows);
-    if (!ext) {
-        if (cfg.precision == GKS_FP64) {
-            if ((st = dalloc(m, &d.off, (size_t)9 * T)) != GKS_OK) return st;
-            if ((st = dalloc(m, &d.w64, (size_t)30 * T)) != GKS_OK) return st;
-        } else {
-            if ((st = dalloc(m, &d.op32, (size_t)24 * T)) != GKS_OK) return st;
-            if (cfg.precond == GKS_PC_ILU_SWEEP &&
-                (st = d.P16 ? dalloc(m, &d.pk16, (size_t)34 * T) : dalloc(m, &d.pk32, (size_t)34 * T)) != GKS_OK)
-                return st;
-        }
-        if ((st = launch_pack(m)) != GKS_OK) return st;
-    }
     AL(part, (size_t)nblk * rows * 4 * (mm + 2)); AL(dpart, (size_t)nblk * 4);
     if (cfg.limiter) {
         AL(xl, 20 * T); AL(lflag, T);
