@@ -604,12 +604,12 @@ __global__ void __launch_bounds__(kW32) k_rhs_df(DeviceMesh d, const float *__re
 
 // Forward block-ILU relation for the listed rows (or all rows when rows == nullptr):
 //   z_i = P_i (r_i + sum_{k<i} O_ik zin_k)      (use_nb = 0: z_i = P_i r_i)
-// use_nb = 2: the first sweep with the block-diagonal pass folded in, zin_k =
+// use_nb = 2 (G): the first sweep with the block-diagonal pass folded in, zin_k =
 // P_k r_k formed here from the lower neighbours' factors and right-hand sides
 // (rounded to TZ as the separate pass stores them), which saves the write and
 // the re-read of that pass; the neighbours' data mostly comes from L2.
 // TR: type of r, TZ: type of z, TM: type of the factors and of the arithmetic.
-// rcopy (may be NULL): also store TZ(r_i), so that later sweeps read r in the
+// rcopy (G, may be NULL): also store TZ(r_i), so that later sweeps read r in the
 // working precision (same values as converting r again).  Own data (r, P) is
 // loaded before the neighbour gathers so that the two overlap.
 // TP: storage type of the factors (TM, or FP16 for the mixed mode's FP32
@@ -638,7 +638,7 @@ __device__ __forceinline__ void ilu_fwd_row(const DeviceMesh &d, const TP *__res
     for (int l = 0; l < ND; ++l) {
         TM t[NV];
         vload(r, l, T, i, t);
-        if (rcopy) vstore(rcopy, l, T, i, t);
+        if (G && rcopy) vstore(rcopy, l, T, i, t);
 #pragma unroll
         for (int v = 0; v < NV; ++v) y[v * ND + l] = t[v];
     }
@@ -668,7 +668,7 @@ __device__ __forceinline__ void ilu_fwd_row(const DeviceMesh &d, const TP *__res
             const int64_t j = lower ? jn : i;
             const TM sa = TM(alg[s * T + i]), sax = sa * TM(exg[s * T + i]), say = sa * TM(eyg[s * T + i]);
             TM zn[NV][NA];
-            if (use_nb == 2) {
+            if (G && use_nb == 2) {
                 TM rj[ND][NV];
 #pragma unroll
                 for (int l = 0; l < ND; ++l) vload(r, l, T, j, rj[l]);
@@ -1252,14 +1252,16 @@ gks_status precond_t(gks_mesh *m, const TP *Pg, const TP *alg, const TP *exg, co
     DeviceMesh &d = m->d;
     const int64_t T = d.T;
     // forward / backward relation, the global variant when reverse slots are given
-    auto fwd = [&](int64_t n, const int32_t *rows, auto r, const TZ *zin, TZ *zout, int use_nb, TZ *rc) {
+    auto fwd_global = [&](int64_t n, const int32_t *rows, auto r, const TZ *zin, TZ *zout, int use_nb, TZ *rc) {
         using TRx = std::remove_cv_t<std::remove_pointer_t<decltype(r)>>;
-        if (rev.a)
-            k_ilu_fwd<TRx, TZ, TM, TP, true><<<nblocks(n), kBlock, 0, s>>>(d, Pg, alg, exg, eyg, rows, n, r, zin, zout,
-                                                                          use_nb, rc, rev.a, rev.x, rev.y, rev.b);
-        else
-            k_ilu_fwd<TRx, TZ, TM, TP, false><<<nblocks(n), kBlock, 0, s>>>(d, Pg, alg, exg, eyg, rows, n, r, zin,
-                                                                           zout, use_nb, rc);
+        k_ilu_fwd<TRx, TZ, TM, TP, true><<<nblocks(n), kBlock, 0, s>>>(d, Pg, alg, exg, eyg, rows, n, r, zin, zout,
+                                                                      use_nb, rc, rev.a, rev.x, rev.y, rev.b);
+        note_launch();
+    };
+    auto fwd = [&](int64_t n, const int32_t *rows, const TR *r, const TZ *zin, TZ *zout, int use_nb) {
+        if (rev.a) return fwd_global(n, rows, r, zin, zout, use_nb, nullptr);
+        k_ilu_fwd<TR, TZ, TM, TP, false><<<nblocks(n), kBlock, 0, s>>>(d, Pg, alg, exg, eyg, rows, n, r, zin, zout,
+                                                                      use_nb, nullptr);
         note_launch();
     };
     auto bwd = [&](int64_t n, const int32_t *rows, const TZ *z, const TZ *xin, TZ *xout) {
@@ -1292,13 +1294,14 @@ gks_status precond_t(gks_mesh *m, const TP *Pg, const TP *alg, const TP *exg, co
     } else if (m->cfg.precond == GKS_PC_ILU_LEVELS) {
         const auto &lp = m->lvl_lo_ptr;
         for (size_t l = 0; l + 1 < lp.size(); ++l)
-            fwd(lp[l + 1] - lp[l], d.lvl_lo + lp[l], src, dst, dst, 1, (TZ *)nullptr);
+            fwd(lp[l + 1] - lp[l], d.lvl_lo + lp[l], src, dst, dst, 1);
         const auto &up = m->lvl_up_ptr;
         for (size_t l = 0; l + 1 < up.size(); ++l) bwd(up[l + 1] - up[l], d.lvl_up + up[l], dst, dst, dst);
     } else if (m->cfg.precond == GKS_PC_BJACOBI) {
-        fwd(T, nullptr, src, nullptr, dst, 0, (TZ *)nullptr);     // z = P r, the block-diagonal inverse
+        fwd(T, nullptr, src, nullptr, dst, 0);     // z = P r, the block-diagonal inverse
     } else {
-        // sweeps: forward z^0 = P r, z^{q+1} = F(z^q); backward x^0 = z, x^{q+1} = B(x^q)
+        // sweeps of the global normal equations (those of the per-cell equations:
+        // precond64, precond32s): forward z^0 = P r, z^{q+1} = F(z^q); backward x^0 = z, x^{q+1} = B(x^q)
         const int ns = m->cfg.ilu_sweeps;
         const int nsb = m->cfg.ilu_sweeps_bwd < 0 ? ns : m->cfg.ilu_sweeps_bwd;
         // z^0 folded into the first sweep (ilu_fuse_first) or a pass of its own
@@ -1308,12 +1311,12 @@ gks_status precond_t(gks_mesh *m, const TP *Pg, const TP *alg, const TP *exg, co
         TZ *zb = (nf % 2 == 1) ? dst : tA;
         // a wider source is rounded to TZ once, in the first pass, for the sweeps
         TZ *rc = (sizeof(TR) > sizeof(TZ) && ns > 0) ? rz : nullptr;
-        fwd(T, nullptr, src, nullptr, za, fuse ? 2 : 0, rc);
+        fwd_global(T, nullptr, src, nullptr, za, fuse ? 2 : 0, rc);
         for (int q = fuse ? 1 : 0; q < ns; ++q) {
             if (rc)
-                fwd(T, nullptr, (const TZ *)rc, za, zb, 1, (TZ *)nullptr);
+                fwd_global(T, nullptr, (const TZ *)rc, za, zb, 1, (TZ *)nullptr);
             else
-                fwd(T, nullptr, src, za, zb, 1, (TZ *)nullptr);
+                fwd_global(T, nullptr, src, za, zb, 1, (TZ *)nullptr);
             std::swap(za, zb);
         }
         if (nsb == 0) {
