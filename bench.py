@@ -367,7 +367,7 @@ def errors_vs_oracle(case, w_oracle, dts, dev, mixed_kw: dict) -> dict:
 
 def class_bytes(cls: str, prof: dict, T: int, F: int, steps: int, sweeps: int, exact: bool, mixed: bool,
                 basis32: bool, ilu16: bool = False, sweeps_bwd: int = -1, fuse_first: bool = True,
-                pairs: bool = False, fused_dots: bool = False) -> float:
+                pairs: bool = False, fused_dots: bool = False, percell64: bool = False) -> float:
     """Algorithmic DRAM bytes moved by one kernel class over the timed region,
     from the solver's work counters (Arnoldi iterations n, sum of j + 1 over
     them, preconditioner applications).  Per cell: operator = diagonal block 15
@@ -379,21 +379,26 @@ def class_bytes(cls: str, prof: dict, T: int, F: int, steps: int, sweeps: int, e
     or 2 with FP16 copies).  With the block-diagonal pass folded into the first
     forward sweep the neighbours' z^0 comes from their own factors and right-hand
     sides, already counted as those cells' reads; with backward sweep pairs
-    likewise the neighbours' first-sweep values.  The FP64 solve of the per-cell
-    equations moves less (products in the operator kernel, a second Gram-Schmidt
-    pass only where needed, sweeps on P O): its counts are an upper bound."""
+    likewise the neighbours' first-sweep values.  percell64: the FP64 solve of the
+    per-cell equations, which forms the Gram-Schmidt products in the operator kernel,
+    makes one pass (the second, of the systems that need it, is not counted) and
+    sweeps on the products P O of pivot inverse and off-diagonal block, 30 values: z =
+    P r once, rows 0 and 1 of z (8 values) per sweep with the 6 products of its
+    triangle, all five rows in the last launch, which covers a sweep each way."""
     sM = 4 if mixed else 8
     sZ = 4 if mixed else 8
     sB = 4 if basis32 else 8
     sP = 2 if ilu16 else sM
     n, jsum = prof["arnoldi"], prof["arnoldi_jsum"]
+    fused_dots = fused_dots or percell64
     op = sM * (15 + 9) + 12
     if cls == "orth":
         # per iteration j: dots read V_0..V_j and w, the update reads them again and
-        # writes w: (2 j + 5) vectors; FP64 mode runs the pair twice (CGS2); with the
-        # products formed in the operator kernel only the update's (j + 3) remain
+        # writes w: (2 j + 5) vectors; FP64 mode on the extended stencils runs the pair
+        # twice (CGS2); with the products formed in the operator kernel only the update's
+        # (j + 3) remain
         vecs = (jsum + 2 * n) if fused_dots else (2 * jsum + 3 * n)
-        return T * 20 * sB * vecs * (1 if mixed else 2)
+        return T * 20 * sB * vecs * (1 if mixed or percell64 else 2)
     if cls == "spmv":                   # y = K z: z (own + neighbour values), operator, y (basis)
         # (+ V_0..V_j when the operator kernel also forms the Gram-Schmidt products)
         return T * ((op + 20 * sZ + 20 * sB) * n + (20 * sB * jsum if fused_dots else 0))
@@ -403,10 +408,14 @@ def class_bytes(cls: str, prof: dict, T: int, F: int, steps: int, sweeps: int, e
             fwd = 20 * sB + 8 * sZ + sP * (25 + 9) + 12 + 20 * sZ
             bwd = 20 * sZ + 8 * sZ + sP * (25 + 9) + 12 + 20 * sZ
             return T * (fwd + bwd) * pc
+        nbwd = sweeps if sweeps_bwd < 0 else sweeps_bwd
+        if percell64:
+            mid = (sweeps if nbwd > 0 else max(sweeps - 1, 0)) + max(nbwd - 1, 0)
+            last = 12 + 8 * (20 + 30 + 20) + 64 * (sweeps > 0) + 64 * (nbwd > 0) if sweeps + nbwd else 0
+            return T * (8 * (20 + 25 + 20) + mid * (12 + 8 * (8 + 6 + 8 + 8)) + last) * pc
         first = 20 * sB + sP * 25 + 20 * sZ
         fwd = 20 * sB + 8 * sZ + sP * (25 + 9) + 12 + 20 * sZ
         bwd = 20 * sZ + 8 * sZ + sP * (25 + 9) + 12 + 20 * sZ
-        nbwd = sweeps if sweeps_bwd < 0 else sweeps_bwd
         # with sweep pairs a launch covers two sweeps and moves a single sweep's
         # bytes (the neighbours' first-sweep inputs are other cells' reads)
         nbl = (nbwd // 2 + nbwd % 2) if pairs else nbwd
@@ -520,7 +529,7 @@ def run_gks(args, world, rank, local):
             by = class_bytes(nm, prof, T, F, args.steps, main["knobs"]["ilu_sweeps"], exact, mixed, basis32,
                              mixed and args.ilu16 == "on", main["knobs"]["ilu_sweeps_bwd"],
                              bool(main["knobs"]["ilu_fuse_first"]), bool(main["knobs"]["ilu_sweep_pairs"]),
-                             bool(main["knobs"]["spmv_dots"]) and basis32)
+                             bool(main["knobs"]["spmv_dots"]) and basis32, percell64=not mixed)
             gbs = by / (ms_c / 1e3) / 1e9
             ent.update({"bytes": by, "gbs": round(gbs, 1), "frac": round(gbs / hbm_peak, 3)})
         classes[nm] = ent
@@ -694,7 +703,7 @@ def run_batch(args, world, rank, local):
             by = class_bytes(nm, prof, T, F, args.steps, knobs["ilu_sweeps"], False, mixed,
                              mixed and args.basis == "fp32", mixed and args.ilu16 == "on", knobs["ilu_sweeps_bwd"],
                              bool(knobs["ilu_fuse_first"]), bool(knobs["ilu_sweep_pairs"]),
-                             bool(knobs["spmv_dots"]) and mixed and args.basis == "fp32")
+                             bool(knobs["spmv_dots"]) and mixed and args.basis == "fp32", percell64=not mixed)
             gbs = by / (prof["ms"][q] / 1e3) / 1e9
             ent.update({"bytes": by, "gbs": round(gbs, 1), "frac": round(gbs / hbm_peak, 3)})
         classes[nm] = ent
