@@ -367,7 +367,8 @@ def errors_vs_oracle(case, w_oracle, dts, dev, mixed_kw: dict) -> dict:
 
 def class_bytes(cls: str, prof: dict, T: int, F: int, steps: int, sweeps: int, exact: bool, mixed: bool,
                 basis32: bool, ilu16: bool = False, sweeps_bwd: int = -1, fuse_first: bool = True,
-                pairs: bool = False, fused_dots: bool = False, percell64: bool = False) -> float:
+                pairs: bool = False, fused_dots: bool = False, percell64: bool = False,
+                packed32: bool = False) -> float:
     """Algorithmic DRAM bytes moved by one kernel class over the timed region,
     from the solver's work counters (Arnoldi iterations n, sum of j + 1 over
     them, preconditioner applications).  Per cell: operator = diagonal block 15
@@ -384,7 +385,10 @@ def class_bytes(cls: str, prof: dict, T: int, F: int, steps: int, sweeps: int, e
     makes one pass (the second, of the systems that need it, is not counted) and
     sweeps on the products P O of pivot inverse and off-diagonal block, 30 values: z =
     P r once, rows 0 and 1 of z (8 values) per sweep with the 6 products of its
-    triangle, all five rows in the last launch, which covers a sweep each way."""
+    triangle, all five rows in the last launch, which covers a sweep each way.
+    packed32: the mixed solve's sweeps of the per-cell equations on packed factors,
+    where a launch that feeds another one writes rows 0 and 1 alone and reads 24 of
+    the 34 factor values (16 without neighbours), and a backward one starts from z."""
     sM = 4 if mixed else 8
     sZ = 4 if mixed else 8
     sB = 4 if basis32 else 8
@@ -413,6 +417,19 @@ def class_bytes(cls: str, prof: dict, T: int, F: int, steps: int, sweeps: int, e
             mid = (sweeps if nbwd > 0 else max(sweeps - 1, 0)) + max(nbwd - 1, 0)
             last = 12 + 8 * (20 + 30 + 20) + 64 * (sweeps > 0) + 64 * (nbwd > 0) if sweeps + nbwd else 0
             return T * (8 * (20 + 25 + 20) + mid * (12 + 8 * (8 + 6 + 8 + 8)) + last) * pc
+        if packed32:
+            fuse = fuse_first and sweeps > 0
+            nfwd = sweeps if fuse else sweeps + 1
+            nbl = (nbwd // 2 + nbwd % 2) if pairs else nbwd
+            by = 20 * sZ if sB > sZ and sweeps > 0 else 0          # the source rounded once
+            for q in range(nfwd):
+                full, nb = q == nfwd - 1, q > 0 or fuse
+                by += 20 * (sB if q == 0 else sZ) + 8 * sZ * (q > 0) + 12 * nb
+                by += sP * (34 if full else (24 if nb else 16)) + sZ * (20 if full else 8)
+            for q in range(nbl):
+                full = q == nbl - 1
+                by += 12 + 8 * sZ * (q > 0) + sP * (34 if full else 24) + 2 * sZ * (20 if full else 8)
+            return T * by * pc
         first = 20 * sB + sP * 25 + 20 * sZ
         fwd = 20 * sB + 8 * sZ + sP * (25 + 9) + 12 + 20 * sZ
         bwd = 20 * sZ + 8 * sZ + sP * (25 + 9) + 12 + 20 * sZ
@@ -529,7 +546,8 @@ def run_gks(args, world, rank, local):
             by = class_bytes(nm, prof, T, F, args.steps, main["knobs"]["ilu_sweeps"], exact, mixed, basis32,
                              mixed and args.ilu16 == "on", main["knobs"]["ilu_sweeps_bwd"],
                              bool(main["knobs"]["ilu_fuse_first"]), bool(main["knobs"]["ilu_sweep_pairs"]),
-                             bool(main["knobs"]["spmv_dots"]) and basis32, percell64=not mixed)
+                             bool(main["knobs"]["spmv_dots"]) and basis32, percell64=not mixed,
+                             packed32=mixed)
             gbs = by / (ms_c / 1e3) / 1e9
             ent.update({"bytes": by, "gbs": round(gbs, 1), "frac": round(gbs / hbm_peak, 3)})
         classes[nm] = ent
@@ -703,7 +721,8 @@ def run_batch(args, world, rank, local):
             by = class_bytes(nm, prof, T, F, args.steps, knobs["ilu_sweeps"], False, mixed,
                              mixed and args.basis == "fp32", mixed and args.ilu16 == "on", knobs["ilu_sweeps_bwd"],
                              bool(knobs["ilu_fuse_first"]), bool(knobs["ilu_sweep_pairs"]),
-                             bool(knobs["spmv_dots"]) and mixed and args.basis == "fp32", percell64=not mixed)
+                             bool(knobs["spmv_dots"]) and mixed and args.basis == "fp32", percell64=not mixed,
+                             packed32=mixed)
             gbs = by / (prof["ms"][q] / 1e3) / 1e9
             ent.update({"bytes": by, "gbs": round(gbs, 1), "frac": round(gbs / hbm_peak, 3)})
         classes[nm] = ent
