@@ -1,12 +1,17 @@
 // CLS reconstruction on the device (Sec. III): right-hand side, operator
 // application, block ILU(0) preconditioner and restarted GMRES.
 //
-// Four independent systems (rho, rho u, rho v, E) share one operator; every
-// kernel handles one cell and all four variables, so each block of the
-// operator is read once per application.  FP64 vectors are [var][dof][cell] in
-// RCM order, FP32 vectors [dof][cell][var] (vload, vstore).  GMRES (Saad & Schultz 1986) is right-preconditioned, uses
-// classical Gram-Schmidt (twice, CGS2, in FP64 mode), and keeps per-variable
-// state on the device (running/converged masks); reductions go through
+// Four independent systems (rho, rho u, rho v, E) share one operator.  This file
+// holds the generic kernels, a cell and all four variables per thread (extended
+// stencils, exact triangular solves, FP64 basis of the mixed mode), the mixed
+// mode's right-hand side, residual and correction, and the launches; the per-cell
+// equations' own kernels are in gks_solve64.cuh (FP64, a thread per cell and
+// variable) and gks_solve32.cuh (mixed), sums and control in gks_control.cuh.
+// FP64 vectors are [var][dof][cell] in RCM order, FP32 vectors [dof][cell][var]
+// (vload, vstore).  GMRES (Saad & Schultz 1986) is right-preconditioned with
+// classical Gram-Schmidt: one pass on the shifted basis in FP64, a second where it is
+// needed; two on the extended stencils; one in the mixed mode.  Per-variable state
+// stays on the device (running/converged masks); reductions go through
 // per-block partial sums and a fixed-order second pass, so results are
 // deterministic.  The Krylov basis is stored unnormalised, V_k = vn_k v_k,
 // with the norms vn_k on the device: the normalisation is folded into the
@@ -27,10 +32,6 @@ namespace {
 constexpr int NV = 4, ND = 5, NX = 20;
 constexpr int kDotThreads = 256;       // threads per block of the dot-product kernel
 constexpr int kDotMaxTiles = 65535;    // grid.y limit of the dot-product kernel
-
-// Per-variable control words ctl[16]: [0..3] active (needs more work), [4..7]
-// running (iterating in the current cycle), [8..11] Krylov vectors in the
-// cycle, [12..15] iterations so far.
 
 // acc += sa [e1 + dx e3 + dy e4 | e2 + dx e4 + dy e5] (g1, g2): the off-diagonal
 // block O_ij = alpha [...] applied to the gradient entries (g1, g2) of

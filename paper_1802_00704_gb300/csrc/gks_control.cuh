@@ -394,7 +394,10 @@ __global__ void __cluster_dims__(4, 1, 1) __launch_bounds__(kReduceThreads)
 //    a system with less than half of |w| left gets the second Gram-Schmidt pass and
 //    its Givens step from the launches that follow (twice[system] = 1);
 //  - mixed: a system with less than 3 % left, where an FP32 basis loses the digits,
-//    ends its cycle (twice NULL).
+//    ends its cycle (twice NULL).  The norm is then good to FP32's digits over |w| / |V_{j+1}|;
+//    with it the basis is still nearer to orthonormal than without the shift and with a norm
+//    of its own: largest entry of V^T V - 1 over eight indices on 60 systems (32 to 1,800
+//    triangles, aspects 1 to 200, no to two sweeps) 4e-8 to 3e-6 against 5e-7 to 0.2.
 
 // |w|^2 of system sy and the part of it that the projections take, to every lane
 __device__ __forceinline__ double projected(const double *hs, const double *hc, int hstride, int sy, int j, double *n2)

@@ -47,7 +47,9 @@ enum : int {
 // Device status bits (per case words the kernels OR into).
 enum : int { kStatusNonPhys = 1, kStatusNoConv = 2, kStatusTimeout = 4 };
 
-// GMRES control words, ctl[field * ns + system] with system = case * 4 + variable.
+// GMRES control words, ctl[field * ns + system] with system = case * 4 + variable: needs
+// more work, iterates in the current cycle, Krylov vectors in the cycle, iterations so
+// far, needs the second Gram-Schmidt pass, ran at the start of the Arnoldi index.
 enum : int { kCtlActive = 0, kCtlRunning = 1, kCtlJv = 2, kCtlIters = 3, kCtlTwice = 4, kCtlRan = 5, kCtlFields = 6 };
 
 // Device data, all in internal (per-case RCM, padded) cell order.

@@ -26,13 +26,14 @@
 //    additions for all Arnoldi indices together instead of 5 for each;
 //  - the basis grows by w = K M^-1 V_j - V_j, which spans the same Krylov space (the
 //    Hessenberg diagonal gets its 1 back).  The preconditioner is close to the
-//    inverse, so nearly all of K M^-1 V_j is V_j itself: without it the part
-//    orthogonal to the basis is 0.63-0.99 of |w| instead of 0.02-0.26 (800- and
-//    1,200-triangle systems), one Gram-Schmidt pass loses no digits (V^T V - 1 is 4e-16
-//    as after two; one pass of the unshifted basis leaves 1e-4), and the second
-//    runs only where the orthogonal part is below half of |w| (the launches of the
-//    second are there and return).  Three steps at 399,424 triangles 46.2 -> 41.9 ms,
-//    ten at 6,400 6.56 -> 6.06 ms, at 800 6.05 -> 5.50 ms.
+//    inverse, so nearly all of K M^-1 V_j is V_j itself: without the shift the part
+//    orthogonal to the basis is 0.02-0.36 of the vector, with it 0.3 or more and mostly
+//    0.5-0.99 of |w|, so one Gram-Schmidt pass loses few digits and the second runs only
+//    where the orthogonal part is below half of |w|.  Largest entry of V^T V - 1 (128 to 800
+//    triangles, aspects 1 to 300, no to two sweeps, 28 vectors): 4e-15, with a second pass in
+//    none to 13 of the indices; two passes of the unshifted basis 1e-15, one 2e-13 to 1.
+//    Three steps at 399,424 triangles 46.2 -> 41.9 ms, ten at 6,400 6.56 -> 6.06 ms, at 800
+//    6.05 -> 5.50 ms.
 // Measured on GB300 (the solve's classes, per Arnoldi index, events around each
 // class) against a thread per cell: preconditioner with two sweeps each way 80 -> 25 us
 // at 6,400 triangles and 680 -> 266 us at 399,424 (436 with P in every sweep);
